@@ -3,6 +3,8 @@
 
 #include <cuda_runtime.h>
 
+#include "packed.cuh"
+
 namespace ws {
 
 // Stack layout of one w-plane: column blocks of CB = 4 grid columns, each
@@ -32,10 +34,11 @@ __host__ __device__ constexpr double quarter_turn_coef(int n) {
     return v;
 }
 
-// sin and cos of (pi/2) r for |r| <= 1/2 + 2^-11, i.e. |angle| < 0.787: the
+// (sin, cos) of (pi/2) r for |r| <= 1/2 + 2^-11, i.e. |angle| < 0.787: the
 // Taylor series of sin through the r^9 term and of cos through r^10, whose
-// first omitted terms are below 1.8e-9 and 1.2e-10.
-__device__ __forceinline__ void sincos_quarter(float r, float *s, float *c) {
+// first omitted terms are below 1.8e-9 and 1.2e-10.  Both run as one packed
+// Horner chain; the last step is (ps r + 0, pc r^2 + 1).
+__device__ __forceinline__ float2 sincos_quarter(float r) {
     constexpr float s1 = (float)quarter_turn_coef(1), s3 = (float)-quarter_turn_coef(3),
                     s5 = (float)quarter_turn_coef(5), s7 = (float)-quarter_turn_coef(7),
                     s9 = (float)quarter_turn_coef(9);
@@ -43,16 +46,11 @@ __device__ __forceinline__ void sincos_quarter(float r, float *s, float *c) {
                     c6 = (float)-quarter_turn_coef(6), c8 = (float)quarter_turn_coef(8),
                     c10 = (float)-quarter_turn_coef(10);
     const float r2 = r * r;
-    float ps = fmaf(s9, r2, s7);
-    ps = fmaf(ps, r2, s5);
-    ps = fmaf(ps, r2, s3);
-    ps = fmaf(ps, r2, s1);
-    float pc = fmaf(c10, r2, c8);
-    pc = fmaf(pc, r2, c6);
-    pc = fmaf(pc, r2, c4);
-    pc = fmaf(pc, r2, c2);
-    *s = ps * r;
-    *c = fmaf(pc, r2, 1.0f);
+    float2 p = fma2(make_float2(s9, c10), dup2(r2), make_float2(s7, c8));
+    p = fma2(p, dup2(r2), make_float2(s5, c6));
+    p = fma2(p, dup2(r2), make_float2(s3, c4));
+    p = fma2(p, dup2(r2), make_float2(s1, c2));
+    return fma2(p, make_float2(r, r2), make_float2(0.f, 1.f));
 }
 
 // exp(2 pi i t z) with z = hi + lo split so that t * hi is exact in FP32
@@ -69,8 +67,8 @@ __device__ __forceinline__ void phase_tz(float t, float2 z, float *s, float *c) 
     const float q = a - kRound;
     const float r = fmaf(t4, z.y, h4 - q);
     const unsigned k = __float_as_uint(a);           // q mod 4 in bits 0 and 1
-    float ps, pc;
-    sincos_quarter(r, &ps, &pc);
+    const float2 sc = sincos_quarter(r);
+    const float ps = sc.x, pc = sc.y;
     // quadrant k: sin = (S, C, -S, -C)[k], cos = (C, -S, -C, S)[k]
     const bool odd = k & 1u;
     const float sv = odd ? pc : ps, cv = odd ? ps : pc;
@@ -78,10 +76,11 @@ __device__ __forceinline__ void phase_tz(float t, float2 z, float *s, float *c) 
     *c = __uint_as_float(__float_as_uint(cv) ^ (((k + 1u) << 30) & 0x80000000u));
 }
 
-__device__ __forceinline__ void kahan_add(float &sum, float &comp, float v) {
-    float y = v - comp;
-    float t = sum + y;
-    comp = (t - sum) - y;
+// Compensated sums of the two components: sum += v with the rounding error kept in comp.
+__device__ __forceinline__ void kahan_add(float2 &sum, float2 &comp, float2 v) {
+    const float2 y = csub(v, comp);
+    const float2 t = cadd(sum, y);
+    comp = csub(csub(t, sum), y);
     sum = t;
 }
 

@@ -8,33 +8,35 @@
 // to digit-reversed positions; every later stage reads, twiddles, transforms
 // and writes back the same R positions, so a thread holds one butterfly at a
 // time and a stage needs a single barrier; the last stage hands its outputs
-// straight back (global stores, crops, accumulations).  Radices: 16, 8, 4
-// (power-of-two part) and 7, 5, 3.  Twiddles come from a table of
-// exp(-2 pi i m / n) computed in double precision on the host.
+// straight back (global stores, crops, accumulations).  Twiddles come from a
+// table of exp(-2 pi i m / n) computed in double precision on the host.
 //
-// Shared-memory addressing inserts one pad slot after every n / radix[0]
-// elements (a power of two), which removes the bank conflicts of the
-// digit-reversed scatter for the main sizes; two transforms of a CTA sit
-// 8 (mod 16) slots apart so interleaved lanes use different banks.
+// The forward and the inverse transforms of a size have plans of their own
+// (fft_make_plan in plan.cpp).
+//
+// Shared-memory addressing inserts one pad slot after every `chunk` elements,
+// which removes most bank conflicts of the digit-reversed scatter; two
+// transforms of a CTA sit 8 (mod 16) slots apart so interleaved lanes use
+// different banks.
 #pragma once
 
 #include <cuda_runtime.h>
+#include <stdint.h>
+
+#include <type_traits>
 
 #include "fft_plan.hpp"
+#include "packed.cuh"
 
 namespace ws {
 
 namespace fftdev {
 
-__device__ __forceinline__ float2 cadd(float2 a, float2 b) { return make_float2(a.x + b.x, a.y + b.y); }
-__device__ __forceinline__ float2 csub(float2 a, float2 b) { return make_float2(a.x - b.x, a.y - b.y); }
-__device__ __forceinline__ float2 cmul(float2 a, float2 b) {
-    return make_float2(fmaf(a.x, b.x, -a.y * b.y), fmaf(a.x, b.y, a.y * b.x));
-}
-// multiply by -i (forward) or +i (inverse)
-__device__ __forceinline__ float2 rot_q(float2 a, bool inv) {
-    return inv ? make_float2(-a.y, a.x) : make_float2(a.y, -a.x);
-}
+template <int R>
+struct Radix {
+    static constexpr int value = R;
+};
+
 // exp(-+ 2 pi i m / n) from the forward table
 __device__ __forceinline__ float2 twiddle(const float2 *__restrict__ tw, int m, bool inv) {
     float2 w = __ldg(tw + m);
@@ -42,11 +44,20 @@ __device__ __forceinline__ float2 twiddle(const float2 *__restrict__ tw, int m, 
 }
 
 __device__ __forceinline__ void dft4(float2 &a0, float2 &a1, float2 &a2, float2 &a3, bool inv) {
-    const float2 t0 = cadd(a0, a2), t1 = csub(a0, a2), t2 = cadd(a1, a3), t3 = rot_q(csub(a1, a3), inv);
+    const float2 t0 = cadd(a0, a2), t1 = csub(a0, a2), t2 = cadd(a1, a3), d = csub(a1, a3);
     a0 = cadd(t0, t2);
     a2 = csub(t0, t2);
-    a1 = cadd(t1, t3);
-    a3 = csub(t1, t3);
+    a1 = add_rot(t1, d, inv);
+    a3 = sub_rot(t1, d, inv);
+}
+
+// the same with a2 to be taken times -i (forward) or +i (inverse) first
+__device__ __forceinline__ void dft4_rot2(float2 &a0, float2 &a1, float2 &a2, float2 &a3, bool inv) {
+    const float2 t0 = add_rot(a0, a2, inv), t1 = sub_rot(a0, a2, inv), t2 = cadd(a1, a3), d = csub(a1, a3);
+    a0 = cadd(t0, t2);
+    a2 = csub(t0, t2);
+    a1 = add_rot(t1, d, inv);
+    a3 = sub_rot(t1, d, inv);
 }
 
 // cos and sin of 2 pi m / 16 for m = 1, 2, 3 (exact decimal expansions)
@@ -54,64 +65,55 @@ constexpr float kC1 = 0.92387953251128674f;   // cos(pi/8)
 constexpr float kS1 = 0.38268343236508978f;   // sin(pi/8)
 constexpr float kR2 = 0.70710678118654752f;   // sqrt(1/2)
 
-// exp(-+ 2 pi i m / 16) for m in 0..9 (the products q*k1 of the 4x4 split)
-__device__ __forceinline__ float2 w16(int m, bool inv) {
-    float c, s;
-    switch (m) {
-        case 0: c = 1.f; s = 0.f; break;
-        case 1: c = kC1; s = kS1; break;
-        case 2: c = kR2; s = kR2; break;
-        case 3: c = kS1; s = kC1; break;
-        case 4: c = 0.f; s = 1.f; break;
-        case 6: c = -kR2; s = kR2; break;
-        case 9: c = -kC1; s = -kS1; break;
-        default: c = 1.f; s = 0.f; break;   // not reached
-    }
-    return make_float2(c, inv ? s : -s);
+// a times exp(-+ 2 pi i m / 16), m = 1, 2, 3, 6 or 9 (products q*k1 of the 4x4 split; 4 is a quarter turn)
+__device__ __forceinline__ float2 mul_w16(float2 a, int m, bool inv) {
+    const float c = m == 1 ? kC1 : m == 2 ? kR2 : m == 3 ? kS1 : m == 6 ? -kR2 : -kC1;
+    const float s = m == 1 ? kS1 : m == 2 ? kR2 : m == 3 ? kC1 : m == 6 ? kR2 : -kS1;
+    return inv ? cmul_rot(a, make_float2(c, s), make_float2(-s, c)) : cmul_rot(a, make_float2(c, -s), make_float2(s, c));
 }
 
 template <int R>
-__device__ __forceinline__ void dft(float2 *v, bool inv, const float2 *__restrict__ tw, int n);
+__device__ __forceinline__ void dft(float2 *v, bool inv);
 
 template <>
-__device__ __forceinline__ void dft<4>(float2 *v, bool inv, const float2 *__restrict__, int) {
+__device__ __forceinline__ void dft<4>(float2 *v, bool inv) {
     dft4(v[0], v[1], v[2], v[3], inv);
 }
 
 template <>
-__device__ __forceinline__ void dft<8>(float2 *v, bool inv, const float2 *__restrict__, int) {
+__device__ __forceinline__ void dft<8>(float2 *v, bool inv) {
     float2 e0 = v[0], e1 = v[2], e2 = v[4], e3 = v[6];
     float2 o0 = v[1], o1 = v[3], o2 = v[5], o3 = v[7];
     dft4(e0, e1, e2, e3, inv);
     dft4(o0, o1, o2, o3, inv);
-    const float sg = inv ? 1.f : -1.f;
-    o1 = cmul(o1, make_float2(kR2, sg * kR2));
-    o2 = rot_q(o2, inv);
-    o3 = cmul(o3, make_float2(-kR2, sg * kR2));
+    o1 = mul_w16(o1, 2, inv);
+    o3 = mul_w16(o3, 6, inv);
     v[0] = cadd(e0, o0);
     v[4] = csub(e0, o0);
     v[1] = cadd(e1, o1);
     v[5] = csub(e1, o1);
-    v[2] = cadd(e2, o2);
-    v[6] = csub(e2, o2);
+    v[2] = add_rot(e2, o2, inv);
+    v[6] = sub_rot(e2, o2, inv);
     v[3] = cadd(e3, o3);
     v[7] = csub(e3, o3);
 }
 
-template <>
-__device__ __forceinline__ void dft<16>(float2 *v, bool inv, const float2 *__restrict__, int) {
-    // X[k1 + 4 k2] = sum_q w16^(q k1) w4^(q k2) sum_s v[q + 4 s] w4^(s k1)
-#pragma unroll
-    for (int q = 0; q < 4; ++q) dft4(v[q], v[q + 4], v[q + 8], v[q + 12], inv);
+// Second level of the 4 x 4 split of radix 16: the twiddles w16^(q k1), then the
+// 4-point DFTs over q, in natural output order.
+__device__ __forceinline__ void dft16_second(float2 *v, bool inv) {
 #pragma unroll
     for (int q = 1; q < 4; ++q)
 #pragma unroll
-        for (int k1 = 1; k1 < 4; ++k1) v[q + 4 * k1] = cmul(v[q + 4 * k1], w16(q * k1, inv));
+        for (int k1 = 1; k1 < 4; ++k1)
+            if (q * k1 != 4) v[q + 4 * k1] = mul_w16(v[q + 4 * k1], q * k1, inv);
     float2 o[16];
 #pragma unroll
     for (int k1 = 0; k1 < 4; ++k1) {
         float2 a0 = v[0 + 4 * k1], a1 = v[1 + 4 * k1], a2 = v[2 + 4 * k1], a3 = v[3 + 4 * k1];
-        dft4(a0, a1, a2, a3, inv);
+        if (k1 == 2)
+            dft4_rot2(a0, a1, a2, a3, inv);
+        else
+            dft4(a0, a1, a2, a3, inv);
         o[k1] = a0;
         o[k1 + 4] = a1;
         o[k1 + 8] = a2;
@@ -119,6 +121,14 @@ __device__ __forceinline__ void dft<16>(float2 *v, bool inv, const float2 *__res
     }
 #pragma unroll
     for (int i = 0; i < 16; ++i) v[i] = o[i];
+}
+
+template <>
+__device__ __forceinline__ void dft<16>(float2 *v, bool inv) {
+    // X[k1 + 4 k2] = sum_q w16^(q k1) w4^(q k2) sum_s v[q + 4 s] w4^(s k1)
+#pragma unroll
+    for (int q = 0; q < 4; ++q) dft4(v[q], v[q + 4], v[q + 8], v[q + 12], inv);
+    dft16_second(v, inv);
 }
 
 // Radix 16 whose middle half of inputs, v[4] .. v[11], is zero (the centred
@@ -128,28 +138,13 @@ __device__ __forceinline__ void dft<16>(float2 *v, bool inv, const float2 *__res
 __device__ __forceinline__ void dft16_zero_middle(float2 *v, bool inv) {
 #pragma unroll
     for (int q = 0; q < 4; ++q) {
-        const float2 a = v[q], d = v[q + 12], rd = rot_q(d, inv);
+        const float2 a = v[q], d = v[q + 12];
         v[q] = cadd(a, d);
         v[q + 8] = csub(a, d);
-        v[q + 4] = csub(a, rd);
-        v[q + 12] = cadd(a, rd);
+        v[q + 4] = sub_rot(a, d, inv);
+        v[q + 12] = add_rot(a, d, inv);
     }
-#pragma unroll
-    for (int q = 1; q < 4; ++q)
-#pragma unroll
-        for (int k1 = 1; k1 < 4; ++k1) v[q + 4 * k1] = cmul(v[q + 4 * k1], w16(q * k1, inv));
-    float2 o[16];
-#pragma unroll
-    for (int k1 = 0; k1 < 4; ++k1) {
-        float2 a0 = v[0 + 4 * k1], a1 = v[1 + 4 * k1], a2 = v[2 + 4 * k1], a3 = v[3 + 4 * k1];
-        dft4(a0, a1, a2, a3, inv);
-        o[k1] = a0;
-        o[k1 + 4] = a1;
-        o[k1 + 8] = a2;
-        o[k1 + 12] = a3;
-    }
-#pragma unroll
-    for (int i = 0; i < 16; ++i) v[i] = o[i];
+    dft16_second(v, inv);
 }
 
 // cos and sin of 2 pi m / R for the odd radices R = 3, 5, 7 and 0 <= m < R
@@ -194,110 +189,131 @@ __device__ __forceinline__ void dft_odd(float2 *v, bool inv) {
 #pragma unroll
         for (int r = 1; r <= h; ++r) {
             const float c = (float)odd_cos(R, (r * k) % R), sn = (float)odd_sin(R, (r * k) % R);
-            A.x = fmaf(c, a[r].x, A.x);
-            A.y = fmaf(c, a[r].y, A.y);
-            B.x = fmaf(sn, b[r].x, B.x);
-            B.y = fmaf(sn, b[r].y, B.y);
+            A = fma2(a[r], dup2(c), A);
+            B = r == 1 ? mul2(b[r], dup2(sn)) : fma2(b[r], dup2(sn), B);
         }
-        const float2 minus = make_float2(A.x + B.y, A.y - B.x);   // A - i B
-        const float2 plus = make_float2(A.x - B.y, A.y + B.x);    // A + i B
-        v[k] = inv ? plus : minus;
-        v[R - k] = inv ? minus : plus;
+        v[k] = add_rot(A, B, inv);          // A - i B forward, A + i B inverse
+        v[R - k] = sub_rot(A, B, inv);
     }
 }
 template <>
-__device__ __forceinline__ void dft<3>(float2 *v, bool inv, const float2 *__restrict__, int) {
+__device__ __forceinline__ void dft<3>(float2 *v, bool inv) {
     dft_odd<3>(v, inv);
 }
 template <>
-__device__ __forceinline__ void dft<5>(float2 *v, bool inv, const float2 *__restrict__, int) {
+__device__ __forceinline__ void dft<5>(float2 *v, bool inv) {
     dft_odd<5>(v, inv);
 }
 template <>
-__device__ __forceinline__ void dft<7>(float2 *v, bool inv, const float2 *__restrict__, int) {
+__device__ __forceinline__ void dft<7>(float2 *v, bool inv) {
     dft_odd<7>(v, inv);
 }
-// 10 = 2 x 5: five-point DFTs of the even and of the odd inputs, then
-// X_k = E_k + w10^k O_k and X_{k+5} = E_k - w10^k O_k, w10 = exp(-+ 2 pi i / 10).
 template <>
-__device__ __forceinline__ void dft<10>(float2 *v, bool inv, const float2 *__restrict__, int) {
-    float2 e[5] = {v[0], v[2], v[4], v[6], v[8]}, o[5] = {v[1], v[3], v[5], v[7], v[9]};
-    dft_odd<5>(e, inv);
-    dft_odd<5>(o, inv);
-    // cos and sin of 2 pi k / 10, k = 1..4 (cos(pi/5) = (sqrt 5 + 1) / 4, cos(2 pi/5) = (sqrt 5 - 1) / 4)
-    constexpr float c[5] = {1.f, 0.80901699437494742f, 0.30901699437494742f, -0.30901699437494742f,
-                            -0.80901699437494742f};
-    constexpr float sn[5] = {0.f, 0.58778525229247313f, 0.95105651629515357f, 0.95105651629515357f,
-                             0.58778525229247313f};
-#pragma unroll
-    for (int k = 0; k < 5; ++k) {
-        const float2 t = k == 0 ? o[0] : cmul(o[k], make_float2(c[k], inv ? sn[k] : -sn[k]));
-        v[k] = cadd(e[k], t);
-        v[k + 5] = csub(e[k], t);
-    }
+__device__ __forceinline__ void dft<2>(float2 *v, bool) {
+    const float2 a = v[0], b = v[1];
+    v[0] = cadd(a, b);
+    v[1] = csub(a, b);
 }
 
-// v[m] *= w^m for m = 1..R-1, w = exp(-+ 2 pi i e / n).  The table holds w^m
-// to half an ulp, but a warp's loads of w^m for m > 1 scatter over many
-// sectors; so only w and w^4 are read and the other powers are products of
-// them (at most five roundings: RMS error about 7e-8 against 2e-8 for the
-// table, far below the FP32 transform's own rounding).
-// The same with w and w^4 given (R = 16 or 8).
+// R = A B with coprime A and B, by the prime factor form (Good, Thomas): with
+// n = (B a + A b) mod R the kernel w_R^(n k) is w_A^(a k) w_B^(b k), so the DFT
+// is an A x B two-dimensional one without twiddles; output k sits at (k mod A, k mod B).
+template <int A, int B>
+__device__ __forceinline__ void dft_pfa(float2 *v, bool inv) {
+    float2 y[A][B];
+#pragma unroll
+    for (int b = 0; b < B; ++b) {
+        float2 c[A];
+#pragma unroll
+        for (int a = 0; a < A; ++a) c[a] = v[(B * a + A * b) % (A * B)];
+        dft<A>(c, inv);
+#pragma unroll
+        for (int a = 0; a < A; ++a) y[a][b] = c[a];
+    }
+#pragma unroll
+    for (int a = 0; a < A; ++a) dft<B>(y[a], inv);
+#pragma unroll
+    for (int k = 0; k < A * B; ++k) v[k] = y[k % A][k % B];
+}
+template <>
+__device__ __forceinline__ void dft<6>(float2 *v, bool inv) {
+    dft_pfa<2, 3>(v, inv);
+}
+template <>
+__device__ __forceinline__ void dft<10>(float2 *v, bool inv) {
+    dft_pfa<2, 5>(v, inv);
+}
+template <>
+__device__ __forceinline__ void dft<12>(float2 *v, bool inv) {
+    dft_pfa<4, 3>(v, inv);
+}
+template <>
+__device__ __forceinline__ void dft<14>(float2 *v, bool inv) {
+    dft_pfa<2, 7>(v, inv);
+}
+template <>
+__device__ __forceinline__ void dft<20>(float2 *v, bool inv) {
+    dft_pfa<4, 5>(v, inv);
+}
+template <>
+__device__ __forceinline__ void dft<21>(float2 *v, bool inv) {
+    dft_pfa<3, 7>(v, inv);
+}
+template <>
+__device__ __forceinline__ void dft<28>(float2 *v, bool inv) {
+    dft_pfa<4, 7>(v, inv);
+}
+template <>
+__device__ __forceinline__ void dft<24>(float2 *v, bool inv) {
+    dft_pfa<8, 3>(v, inv);
+}
+
+// A twiddle and the pair its products need.
+struct Tw {
+    float2 w, rot;
+    __device__ __forceinline__ explicit Tw(float2 v) : w(v), rot(turn2(v)) {}
+    __device__ __forceinline__ float2 times(float2 a) const { return cmul_rot(a, w, rot); }
+};
+
+// v[m] *= w^m for m = 1..R-1, w = exp(-+ 2 pi i e / n), given w and w^4.  The
+// table holds w^m to half an ulp, but a warp's loads of w^m for m > 1 scatter
+// over many sectors; so only w and, from R = 8 on, w^4 are read and the
+// other powers are products of them (at most five roundings: RMS error about 7e-8 against 2e-8
+// for the table, far below the FP32 transform's own rounding).
 template <int R>
 __device__ __forceinline__ void twiddle_powers(float2 *v, float2 w1, float2 w4) {
-    static_assert(R == 16 || R == 8, "radix 16 or 8");
-    const float2 w2 = cmul(w1, w1), w3 = cmul(w2, w1);
-    v[1] = cmul(v[1], w1);
-    v[2] = cmul(v[2], w2);
-    v[3] = cmul(v[3], w3);
-    v[4] = cmul(v[4], w4);
-    v[5] = cmul(v[5], cmul(w4, w1));
-    v[6] = cmul(v[6], cmul(w4, w2));
-    v[7] = cmul(v[7], cmul(w4, w3));
-    if constexpr (R == 16) {
-        const float2 w8 = cmul(w4, w4), w12 = cmul(w8, w4);
-        v[8] = cmul(v[8], w8);
-        v[9] = cmul(v[9], cmul(w8, w1));
-        v[10] = cmul(v[10], cmul(w8, w2));
-        v[11] = cmul(v[11], cmul(w8, w3));
-        v[12] = cmul(v[12], w12);
-        v[13] = cmul(v[13], cmul(w12, w1));
-        v[14] = cmul(v[14], cmul(w12, w2));
-        v[15] = cmul(v[15], cmul(w12, w3));
-    }
-}
-
-template <int R>
-__device__ __forceinline__ void twiddle_all(float2 *v, const float2 *__restrict__ tw, int e, bool inv) {
-    if constexpr (R == 16 || R == 8) {
-        twiddle_powers<R>(v, twiddle(tw, e, inv), twiddle(tw, 4 * e, inv));
-    } else if constexpr (R == 10) {
-        // w^m from w and w^4, products at most two deep
-        const float2 w1 = twiddle(tw, e, inv), w4 = twiddle(tw, 4 * e, inv);
-        const float2 w2 = cmul(w1, w1), w3 = cmul(w2, w1), w8 = cmul(w4, w4);
-        v[1] = cmul(v[1], w1);
-        v[2] = cmul(v[2], w2);
-        v[3] = cmul(v[3], w3);
-        v[4] = cmul(v[4], w4);
-        v[5] = cmul(v[5], cmul(w4, w1));
-        v[6] = cmul(v[6], cmul(w4, w2));
-        v[7] = cmul(v[7], cmul(w4, w3));
-        v[8] = cmul(v[8], w8);
-        v[9] = cmul(v[9], cmul(w8, w1));
-    } else {
-        // R <= 7: w^m from w by products, at most three roundings deep
-        static_assert(R <= 7, "radices 3 to 7");
-        const float2 w1 = twiddle(tw, e, inv), w2 = cmul(w1, w1);
-        v[1] = cmul(v[1], w1);
-        v[2] = cmul(v[2], w2);
-        if constexpr (R >= 4) v[3] = cmul(v[3], cmul(w2, w1));
-        if constexpr (R >= 5) v[4] = cmul(v[4], cmul(w2, w2));
-        if constexpr (R >= 6) v[5] = cmul(v[5], cmul(cmul(w2, w2), w1));
-        if constexpr (R >= 7) {
-            const float2 w3 = cmul(w2, w1);
-            v[6] = cmul(v[6], cmul(w3, w3));
+    static_assert(R >= 3 && R <= 28, "powers up to w^27");
+    const Tw t1(w1);
+    v[1] = t1.times(v[1]);
+    const Tw t2(t1.times(w1));
+    v[2] = t2.times(v[2]);
+    if constexpr (R >= 4) {
+        const Tw t3(t1.times(t2.w));
+        v[3] = t3.times(v[3]);
+        if constexpr (R > 4) {
+            const Tw t4(R <= 7 ? t2.times(t2.w) : w4);
+            float2 base = t4.w, w8 = t4.w;
+#pragma unroll
+            for (int a = 1; 4 * a < R; ++a) {
+                if (a == 2) base = w8 = t4.times(t4.w);
+                if (a == 3 || a >= 5) base = t4.times(base);
+                if (a == 4) base = Tw(w8).times(w8);
+                v[4 * a] = Tw(base).times(v[4 * a]);
+                if (4 * a + 1 < R) v[4 * a + 1] = Tw(t1.times(base)).times(v[4 * a + 1]);
+                if (4 * a + 2 < R) v[4 * a + 2] = Tw(R == 7 ? t3.times(t3.w) : t2.times(base)).times(v[4 * a + 2]);
+                if (4 * a + 3 < R) v[4 * a + 3] = Tw(t3.times(base)).times(v[4 * a + 3]);
+            }
         }
     }
+}
+template <int R>
+__device__ __forceinline__ void twiddle_all(float2 *v, const float2 *__restrict__ tw, int e, bool inv) {
+    twiddle_powers<R>(v, twiddle(tw, e, inv), R >= 8 ? twiddle(tw, 4 * e, inv) : make_float2(1.f, 0.f));
+}
+
+// x / d for 0 <= x < 2^16, 1 <= d < 2^13, with mul = div_mul(d) (fft_plan.hpp)
+__device__ __forceinline__ int div_small(int x, unsigned mul) {
+    return mul ? (int)__umulhi((unsigned)x, mul) : x;
 }
 
 // In-place decimation-in-time stage of radix R: for every block b of R*L
@@ -306,84 +322,150 @@ __device__ __forceinline__ void twiddle_all(float2 *v, const float2 *__restrict_
 // to the same positions.  Butterflies own disjoint positions, so a thread
 // can do them one after another and a stage needs no barrier between its
 // reads and writes.  Work item q -> transform t = q % COUNT, butterfly q / COUNT.
-// POW2: n, R and L are powers of two and the index arithmetic uses shifts.
-// x / d for 0 <= x < 2^16, 1 <= d < 2^13, with mul = div_mul(d) (fft_plan.hpp)
-__device__ __forceinline__ int div_small(int x, unsigned mul) {
-    return mul ? (int)__umulhi((unsigned)x, mul) : x;
-}
-
-template <int R, int COUNT, bool POW2, class Store>
-__device__ __forceinline__ void dit_stage(float2 *buf, const FftPlan &P, int L, unsigned Lmul, bool last,
-                                          const float2 *__restrict__ tw, bool inv, int tid, int nthr,
-                                          Store &store) {
-    const int n = P.n, nb = n / R, total = COUNT * nb;
-    int logL = 0, lgtw = 0;
-    if constexpr (POW2) {
-        logL = __ffs(L) - 1;
-        lgtw = P.logn - logL - (__ffs(R) - 1);
-    }
-    const int twstep = POW2 ? 0 : n / (R * L);
+//
+// A butterfly's slots are one base plus multiples of P.step[s] (FftPlan), so the
+// slot arithmetic costs once per butterfly.
+template <int R, int COUNT, bool LAST, class Store>
+__device__ __forceinline__ void dit_stage(float2 *buf, const FftPlan &P, int s, const float2 *__restrict__ tw,
+                                          bool inv, int tid, int nthr, Store &store) {
+    const int L = P.L[s], total = COUNT * P.nb[s], twstep = P.twstep[s];
+    const int step = P.step[s];
     for (int q = tid; q < total; q += nthr) {
         const int t = q % COUNT, bq = q / COUNT;
-        int blk, k;
-        if constexpr (POW2) {
-            blk = bq >> logL;
-            k = bq & (L - 1);
-        } else {
-            blk = div_small(bq, Lmul);
-            k = bq - blk * L;
-        }
+        const int blk = LAST ? 0 : div_small(bq, P.L_mul[s]), k = bq - blk * L;
         const int base = blk * R * L + k;
-        float2 *x = buf + t * P.stride;
+        float2 *x = buf + t * P.stride + base + div_small(base, P.chunk_mul);
         float2 v[R];
 #pragma unroll
-        for (int m = 0; m < R; ++m) v[m] = x[fft_pad(base + m * L, P.padshift)];
-        if (k > 0) twiddle_all<R>(v, tw, POW2 ? k << lgtw : k * twstep, inv);
-        dft<R>(v, inv, tw, n);
-        if (last) {
+        for (int m = 0; m < R; ++m) v[m] = x[m * step];
+        if (k > 0) twiddle_all<R>(v, tw, k * twstep, inv);
+        dft<R>(v, inv);
+        if constexpr (LAST) {
 #pragma unroll
             for (int m = 0; m < R; ++m) store(t, base + m * L, v[m]);
         } else {
 #pragma unroll
-            for (int m = 0; m < R; ++m) x[fft_pad(base + m * L, P.padshift)] = v[m];
+            for (int m = 0; m < R; ++m) x[m * step] = v[m];
         }
     }
-    if (!last) __syncthreads();
+    if constexpr (!LAST) __syncthreads();
+}
+
+// The slot where butterfly j of the first stage puts its R outputs: that of
+// position g*R, g = the digits of j in reverse order.
+__device__ __forceinline__ int first_slot(const FftPlan &P, int j) {
+    int g = 0;
+    for (int i = 1; i < P.nstages; ++i) {
+        const int a = div_small(j, P.xw_mul[i]);
+        g += (a - div_small(a, P.r_mul[i]) * P.radix[i]) * P.gw[i];
+    }
+    g *= P.radix[0];
+    return g + div_small(g, P.chunk_mul);
 }
 
 // First stage: butterfly j of each transform reads inputs m*(n/R) + j, m < R,
 // straight from load(t, e), and writes them to the digit-reversed positions
-// g*R + m that the later in-place stages expect (g = the digits of j in
-// reverse order).  A one-stage transform stores directly.
-template <int R, int COUNT, bool POW2, class Load, class Store>
-__device__ __forceinline__ void dit_first(float2 *buf, const FftPlan &P, const float2 *__restrict__ tw,
-                                          bool inv, int tid, int nthr, Load &load, Store &store) {
-    const int n = P.n, nb = n / R, total = COUNT * nb;
+// g*R + m that the later in-place stages expect.
+template <int R, int COUNT, class Load>
+__device__ __forceinline__ void dit_first(float2 *buf, const FftPlan &P, bool inv, int tid, int nthr, Load &load) {
+    const int nb = P.nb[0], total = COUNT * nb;
     for (int q = tid; q < total; q += nthr) {
         const int t = q % COUNT, j = q / COUNT;
         float2 v[R];
 #pragma unroll
         for (int m = 0; m < R; ++m) v[m] = load(t, m * nb + j);
-        dft<R>(v, inv, tw, n);
-        if (P.nstages == 1) {
+        dft<R>(v, inv);
+        float2 *x = buf + t * P.stride + first_slot(P, j);
 #pragma unroll
-            for (int m = 0; m < R; ++m) store(t, m, v[m]);
-            continue;
-        }
-        int g = 0;
-        for (int i = 1; i < P.nstages; ++i) {
-            if constexpr (POW2) {
-                g += ((j >> P.lxw[i]) & (P.radix[i] - 1)) << P.lgw[i];
-            } else {
-                const int a = div_small(j, P.xw_mul[i]);
-                g += (a - div_small(a, P.r_mul[i]) * P.radix[i]) * P.gw[i];
-            }
-        }
-        float2 *x = buf + t * P.stride;
-#pragma unroll
-        for (int m = 0; m < R; ++m) x[fft_pad(g * R + m, P.padshift)] = v[m];
+        for (int m = 0; m < R; ++m) x[m] = v[m];
     }
-    if (P.nstages > 1) __syncthreads();
+    __syncthreads();
+}
+
+// First stage of one transform whose input sits in the buffer in natural order
+// at 0..n-1 (n / R <= nthr: one butterfly per thread); input m of a thread is
+// zero where bit m of live is clear, whatever the buffer holds.
+template <int R>
+__device__ __forceinline__ void dit_first_inplace(float2 *buf, const FftPlan &P, bool inv, int tid, uint32_t live) {
+    // threads past nb read the last butterfly's inputs and drop them: a value that
+    // exists only under a condition, kept across the barrier, made the compiler spill
+    const int nb = P.nb[0], at = min(tid, nb - 1);
+    float2 v[R];
+#pragma unroll
+    for (int m = 0; m < R; ++m) {
+        const float2 x = buf[m * nb + at];
+        v[m] = (live >> m) & 1u ? x : make_float2(0.f, 0.f);
+    }
+    __syncthreads();
+    if (tid < nb) {
+        dft<R>(v, inv);
+        float2 *x = buf + first_slot(P, tid);
+#pragma unroll
+        for (int m = 0; m < R; ++m) x[m] = v[m];
+    }
+    __syncthreads();
+}
+
+// Calls f(Radix<r>) for the first or a later radix of a forward plan, and for the
+// first, a middle or the last radix of an inverse plan (the sets that
+// fft_make_plan chooses from).
+template <class F>
+__device__ __forceinline__ void with_forward_first(int r, F f) {
+    if (r == 16)
+        f(Radix<16>{});
+    else
+        f(Radix<8>{});
+}
+template <class F>
+__device__ __forceinline__ void with_forward_later(int r, F f) {
+    switch (r) {
+        case 16: f(Radix<16>{}); break;
+        case 10: f(Radix<10>{}); break;
+        case 8: f(Radix<8>{}); break;
+        case 7: f(Radix<7>{}); break;
+        case 5: f(Radix<5>{}); break;
+        case 4: f(Radix<4>{}); break;
+        default: f(Radix<3>{}); break;
+    }
+}
+template <class F>
+__device__ __forceinline__ void with_first_radix(int r, F f) {
+    switch (r) {
+        case 28: f(Radix<28>{}); break;
+        case 24: f(Radix<24>{}); break;
+        case 20: f(Radix<20>{}); break;
+        case 16: f(Radix<16>{}); break;
+        case 14: f(Radix<14>{}); break;
+        case 12: f(Radix<12>{}); break;
+        case 10: f(Radix<10>{}); break;
+        default: f(Radix<8>{}); break;
+    }
+}
+template <class F>
+__device__ __forceinline__ void with_middle_radix(int r, F f) {
+    switch (r) {
+        case 21: f(Radix<21>{}); break;
+        case 20: f(Radix<20>{}); break;
+        case 16: f(Radix<16>{}); break;
+        case 14: f(Radix<14>{}); break;
+        case 12: f(Radix<12>{}); break;
+        case 10: f(Radix<10>{}); break;
+        case 8: f(Radix<8>{}); break;
+        default: f(Radix<6>{}); break;
+    }
+}
+template <class F>
+__device__ __forceinline__ void with_last_radix(int r, F f) {
+    switch (r) {
+        case 16: f(Radix<16>{}); break;
+        case 14: f(Radix<14>{}); break;
+        case 12: f(Radix<12>{}); break;
+        case 10: f(Radix<10>{}); break;
+        case 8: f(Radix<8>{}); break;
+        case 7: f(Radix<7>{}); break;
+        case 6: f(Radix<6>{}); break;
+        default: f(Radix<4>{}); break;
+    }
 }
 
 }  // namespace fftdev
@@ -391,49 +473,52 @@ __device__ __forceinline__ void dit_first(float2 *buf, const FftPlan &P, const f
 // Transform COUNT sequences of length P.n from load(t, e) to store(t, e, v)
 // (t < COUNT), using the shared buffers buf + t * P.stride between stages.
 // All threads of the CTA must call it; shared buffers may be reused after the
-// caller's next barrier.  MIXED enables the odd radices (and integer
-// division in the index arithmetic); without it n is a power of two and only
-// radices 16, 8 and 4 are compiled.
-template <bool MIXED, int COUNT, class Load, class Store>
-__device__ __forceinline__ void fft_many(float2 *buf, const FftPlan &P, const float2 *__restrict__ tw, bool inv,
-                                         int tid, int nthr, Load load, Store store) {
-    constexpr bool POW2 = !MIXED;
-    switch (P.radix[0]) {
-        case 16: fftdev::dit_first<16, COUNT, POW2>(buf, P, tw, inv, tid, nthr, load, store); break;
-        case 8: fftdev::dit_first<8, COUNT, POW2>(buf, P, tw, inv, tid, nthr, load, store); break;
-        case 4: fftdev::dit_first<4, COUNT, POW2>(buf, P, tw, inv, tid, nthr, load, store); break;
-        default:
-            if constexpr (MIXED) {
-                if (P.radix[0] == 10) fftdev::dit_first<10, COUNT, POW2>(buf, P, tw, inv, tid, nthr, load, store);
-                else if (P.radix[0] == 7) fftdev::dit_first<7, COUNT, POW2>(buf, P, tw, inv, tid, nthr, load, store);
-                else if (P.radix[0] == 5) fftdev::dit_first<5, COUNT, POW2>(buf, P, tw, inv, tid, nthr, load, store);
-                else fftdev::dit_first<3, COUNT, POW2>(buf, P, tw, inv, tid, nthr, load, store);
-            }
-            break;
+// caller's next barrier.
+template <int COUNT, bool INV, class Store>
+__device__ __forceinline__ void fft_later_stages(float2 *buf, const FftPlan &P, const float2 *__restrict__ tw,
+                                                 int tid, int nthr, Store &store) {
+    const int last = P.nstages - 1;
+    auto middle = [&](int s) {
+        return [&, s](auto r) {
+            fftdev::dit_stage<decltype(r)::value, COUNT, false>(buf, P, s, tw, INV, tid, nthr, store);
+        };
+    };
+    auto final = [&](auto r) {
+        fftdev::dit_stage<decltype(r)::value, COUNT, true>(buf, P, last, tw, INV, tid, nthr, store);
+    };
+    for (int s = 1; s < last; ++s) {
+        if constexpr (INV)
+            fftdev::with_middle_radix(P.radix[s], middle(s));
+        else
+            fftdev::with_forward_later(P.radix[s], middle(s));
     }
-    int L = P.radix[0];
-    for (int s = 1; s < P.nstages; ++s) {
-        const int R = P.radix[s];
-        const bool last = s == P.nstages - 1;
-        switch (R) {
-            case 16: fftdev::dit_stage<16, COUNT, POW2>(buf, P, L, P.L_mul[s], last, tw, inv, tid, nthr, store); break;
-            case 8: fftdev::dit_stage<8, COUNT, POW2>(buf, P, L, P.L_mul[s], last, tw, inv, tid, nthr, store); break;
-            case 4: fftdev::dit_stage<4, COUNT, POW2>(buf, P, L, P.L_mul[s], last, tw, inv, tid, nthr, store); break;
-            default:
-                if constexpr (MIXED) {
-                    if (R == 10)
-                        fftdev::dit_stage<10, COUNT, POW2>(buf, P, L, P.L_mul[s], last, tw, inv, tid, nthr, store);
-                    else if (R == 7)
-                        fftdev::dit_stage<7, COUNT, POW2>(buf, P, L, P.L_mul[s], last, tw, inv, tid, nthr, store);
-                    else if (R == 5)
-                        fftdev::dit_stage<5, COUNT, POW2>(buf, P, L, P.L_mul[s], last, tw, inv, tid, nthr, store);
-                    else
-                        fftdev::dit_stage<3, COUNT, POW2>(buf, P, L, P.L_mul[s], last, tw, inv, tid, nthr, store);
-                }
-                break;
-        }
-        L *= R;
-    }
+    if constexpr (INV)
+        fftdev::with_last_radix(P.radix[last], final);
+    else
+        fftdev::with_forward_later(P.radix[last], final);
+}
+
+template <int COUNT, bool INV, class Load, class Store>
+__device__ __forceinline__ void fft_many(float2 *buf, const FftPlan &P, const float2 *__restrict__ tw, int tid,
+                                         int nthr, Load load, Store store) {
+    auto first = [&](auto r) {
+        fftdev::dit_first<decltype(r)::value, COUNT>(buf, P, INV, tid, nthr, load);
+    };
+    if constexpr (INV)
+        fftdev::with_first_radix(P.radix[0], first);
+    else
+        fftdev::with_forward_first(P.radix[0], first);
+    fft_later_stages<COUNT, INV>(buf, P, tw, tid, nthr, store);
+}
+
+// One inverse transform whose input sits in buf in natural order (see dit_first_inplace).
+template <class Store>
+__device__ __forceinline__ void fft_inplace(float2 *buf, const FftPlan &P, const float2 *__restrict__ tw, int tid,
+                                            int nthr, Store store, uint32_t live) {
+    fftdev::with_first_radix(P.radix[0], [&](auto r) {
+        fftdev::dit_first_inplace<decltype(r)::value>(buf, P, true, tid, live);
+    });
+    fft_later_stages<1, true>(buf, P, tw, tid, nthr, store);
 }
 
 // -- compile-time plans for the power-of-two sizes -----------------------------
@@ -467,17 +552,16 @@ template <int N> struct Layout {
 // R0/4 <= m < 3 R0/4; in the last stage, output k + m (N/R) likewise.
 constexpr int PRUNE_IN = 1, PRUNE_OUT = 2;
 
-// First stage (radix R0): inputs m*(N/R0) + j, outputs to digit-reversed g*R0 + m.
-template <int N, int COUNT, class Load, int PRUNE = 0>
-__device__ __forceinline__ void first(float2 *buf, const float2 *__restrict__ tw, bool inv, int tid, int nthr,
-                                      Load &load) {
+// First stage (radix R0) of COUNT transforms by T threads: inputs m*(N/R0) + j, outputs to digit-reversed g*R0 + m.
+template <int N, int COUNT, int T, int PRUNE, class Load>
+__device__ __forceinline__ void first(float2 *buf, bool inv, int tid, Load &load) {
     using Rd = Radices<N>;
     using Ly = Layout<N>;
     constexpr int R = Rd::r0, nb = N / R, total = COUNT * nb;
     constexpr bool pin = (PRUNE & PRUNE_IN) != 0;
     static_assert(!pin || R == 16, "input pruning is written for a radix-16 first stage");
     // j = d1 * r2 + d2 (x-order); g = d1 + d2 * r1 (position order)
-    for (int q = tid; q < total; q += nthr) {
+    for (int q = tid; q < total; q += T) {
         const int t = q % COUNT, j = q / COUNT;
         float2 v[R];
 #pragma unroll
@@ -486,7 +570,7 @@ __device__ __forceinline__ void first(float2 *buf, const float2 *__restrict__ tw
         if constexpr (pin)
             fftdev::dft16_zero_middle(v, inv);
         else
-            fftdev::dft<R>(v, inv, tw, N);
+            fftdev::dft<R>(v, inv);
         const int d1 = j >> ilog2(Rd::r2), d2 = j & (Rd::r2 - 1);
         const int g = d1 + d2 * Rd::r1;
         float2 *x = buf + t * Ly::stride + Ly::pad(g * R);     // R divides 2^shift: one base
@@ -496,28 +580,38 @@ __device__ __forceinline__ void first(float2 *buf, const float2 *__restrict__ tw
     __syncthreads();
 }
 
-// Later stage of radix R over span L (constant): in place, or to store() if LAST.
-// Twiddle bases w, w^4 of the one butterfly a thread owns in a later stage
-// (one transform, nthr >= N / R): they do not change from transform to
-// transform, so a kernel that loops over many transforms reads them once.
+// Twiddle bases w, w^4 of the butterflies a thread owns in a later stage of one
+// transform by T threads (butterflies tid + i T): they do not change from
+// transform to transform, so a kernel that loops over many transforms reads
+// them once.  Where T is a multiple of L every round has the same ones.
+template <int N, int R, int L, int T>
 struct StageTw {
-    float2 w1, w4;
+    static constexpr int rounds = (N / R + T - 1) / T, kept = T % L == 0 ? 1 : rounds;
+    float2 w1[kept], w4[kept];
+    __device__ __forceinline__ void load(const float2 *__restrict__ tw, bool inv, int tid) {
+        constexpr int lgtw = ilog2(N / (R * L));
+#pragma unroll
+        for (int i = 0; i < kept; ++i) {
+            const int k = (tid + i * T) & (L - 1);
+            w1[i] = fftdev::twiddle(tw, k << lgtw, inv);
+            w4[i] = R >= 8 ? fftdev::twiddle(tw, (4 * k) << lgtw, inv) : make_float2(1.f, 0.f);
+        }
+    }
 };
+struct NoTw {};
 
-template <int N, int R, int L>
-__device__ __forceinline__ StageTw stage_twiddles(const float2 *__restrict__ tw, bool inv, int tid) {
-    constexpr int lgtw = ilog2(N / (R * L));
-    const int k = tid & (L - 1);
-    return StageTw{fftdev::twiddle(tw, k << lgtw, inv), fftdev::twiddle(tw, (4 * k) << lgtw, inv)};
-}
-
-template <int N, int COUNT, int R, int L, bool LAST, class Store, int PRUNE = 0>
-__device__ __forceinline__ void later(float2 *buf, const float2 *__restrict__ tw, bool inv, int tid, int nthr,
-                                      Store &store, const StageTw *pre = nullptr) {
+// Later stage of radix R over span L (constants) of COUNT transforms by T
+// threads: in place, or to store() if LAST.  PRE holds the thread's twiddle
+// bases (COUNT = 1), or is NoTw.
+template <int N, int COUNT, int T, int R, int L, bool LAST, int PRUNE, class Pre, class Store>
+__device__ __forceinline__ void later(float2 *buf, const float2 *__restrict__ tw, bool inv, int tid, const Pre &pre,
+                                      Store &store) {
     constexpr bool pout = LAST && (PRUNE & PRUNE_OUT) != 0;
     static_assert(!pout || (R % 4 == 0 && R * L == N), "output pruning needs the last stage, R a multiple of 4");
+    constexpr bool kept_tw = !std::is_same<Pre, NoTw>::value;
+    static_assert(!kept_tw || COUNT == 1, "kept twiddle bases belong to one transform");
     using Ly = Layout<N>;
-    constexpr int nb = N / R, total = COUNT * nb;
+    constexpr int nb = N / R, total = COUNT * nb, rounds = (total + T - 1) / T;
     constexpr int lgL = ilog2(L), lgtw = ilog2(N / (R * L));
     // pad(base + m L) with base = blk R L + k, k < L, is pad_base + m * step when
     //  (a) L is a multiple of 2^shift (the pad of m L is exact), or
@@ -530,7 +624,10 @@ __device__ __forceinline__ void later(float2 *buf, const float2 *__restrict__ tw
     auto at = [&](int pbase, int base, int m) {
         return affine ? pbase + m * step : Ly::pad(base + m * L);
     };
-    for (int q = tid; q < total; q += nthr) {
+#pragma unroll(kept_tw ? rounds : 1)
+    for (int i = 0; i < rounds; ++i) {
+        const int q = tid + i * T;
+        if (total % T != 0 && q >= total) break;
         const int t = q % COUNT, bq = q / COUNT;
         const int blk = bq >> lgL, k = bq & (L - 1);
         const int base = blk * R * L + k;
@@ -540,14 +637,12 @@ __device__ __forceinline__ void later(float2 *buf, const float2 *__restrict__ tw
 #pragma unroll
         for (int m = 0; m < R; ++m) v[m] = x[at(pbase, base, m)];
         if (k > 0) {
-            if constexpr (R == 16 || R == 8) {
-                if (pre) fftdev::twiddle_powers<R>(v, pre->w1, pre->w4);
-                else fftdev::twiddle_all<R>(v, tw, k << lgtw, inv);
-            } else {
+            if constexpr (kept_tw)
+                fftdev::twiddle_powers<R>(v, pre.w1[Pre::kept == 1 ? 0 : i], pre.w4[Pre::kept == 1 ? 0 : i]);
+            else
                 fftdev::twiddle_all<R>(v, tw, k << lgtw, inv);
-            }
         }
-        fftdev::dft<R>(v, inv, tw, N);
+        fftdev::dft<R>(v, inv);
         if constexpr (LAST) {
 #pragma unroll
             for (int m = 0; m < R; ++m)
@@ -561,67 +656,72 @@ __device__ __forceinline__ void later(float2 *buf, const float2 *__restrict__ tw
 }
 
 // First stage for inputs already in the buffer, in natural order at 0..N-1
-// (one transform, at most one butterfly per thread: nthr >= N / R0).  Each
-// thread reads the R0 inputs m (N/R0) + tid (input m is zero where bit m of
-// live is clear, whatever the buffer holds), the CTA synchronises, between()
-// runs (the buffer's old contents are dead by then), and the outputs go to
-// their padded digit-reversed slots.
-template <int N, class Between>
-__device__ __forceinline__ void first_inplace(float2 *buf, const float2 *__restrict__ tw, bool inv, int tid,
-                                              Between &between, uint32_t live) {
+// (one transform, N / R0 threads).  Each thread reads the R0 inputs m (N/R0) +
+// tid (input m is zero where bit m of live is clear, whatever the buffer holds),
+// the CTA synchronises, and the outputs go to their padded digit-reversed slots.
+template <int N>
+__device__ __forceinline__ void first_inplace(float2 *buf, bool inv, int tid, uint32_t live) {
     using Rd = Radices<N>;
     using Ly = Layout<N>;
     constexpr int R = Rd::r0, nb = N / R;
-    const bool active = tid < nb;
     float2 v[R];
-    if (active) {
 #pragma unroll
-        for (int m = 0; m < R; ++m) {
-            const float2 x = buf[m * nb + tid];
-            v[m] = (live >> m) & 1u ? x : make_float2(0.f, 0.f);
-        }
+    for (int m = 0; m < R; ++m) {
+        const float2 x = buf[m * nb + tid];
+        v[m] = (live >> m) & 1u ? x : make_float2(0.f, 0.f);
     }
     __syncthreads();
-    between();
-    if (active) {
-        fftdev::dft<R>(v, inv, tw, N);
-        const int d1 = tid >> ilog2(Rd::r2), d2 = tid & (Rd::r2 - 1);
-        float2 *x = buf + Ly::pad((d1 + d2 * Rd::r1) * R);
+    fftdev::dft<R>(v, inv);
+    const int d1 = tid >> ilog2(Rd::r2), d2 = tid & (Rd::r2 - 1);
+    float2 *x = buf + Ly::pad((d1 + d2 * Rd::r1) * R);
 #pragma unroll
-        for (int m = 0; m < R; ++m) x[m] = v[m];
-    }
+    for (int m = 0; m < R; ++m) x[m] = v[m];
     __syncthreads();
 }
+
+// Twiddle bases of both later stages of one transform by T threads.
+template <int N, int T>
+struct RowTw {
+    using Rd = Radices<N>;
+    StageTw<N, Rd::r1, Rd::r0, T> s2;
+    StageTw<N, Rd::r2, Rd::r0 * Rd::r1, T> s3;
+    __device__ __forceinline__ RowTw(const float2 *__restrict__ tw, bool inv, int tid) {
+        s2.load(tw, inv, tid);
+        s3.load(tw, inv, tid);
+    }
+};
 
 }  // namespace fftst
 
-// One transform of the compile-time size N whose input sits in buf in natural
-// order (see first_inplace for live); later stages as in fft_static.
-template <int N, int PRUNE = 0, class Between, class Store>
-__device__ __forceinline__ void fft_static_inplace(float2 *buf, const float2 *__restrict__ tw, bool inv, int tid,
-                                                   int nthr, Between between, Store store,
-                                                   const fftst::StageTw &s2, const fftst::StageTw &s3,
-                                                   uint32_t live = 0xffffffffu) {
+// One transform of the compile-time size N by T threads: input in buf in
+// natural order (see first_inplace for live), or read through load.
+template <int N, int T, int PRUNE = 0, class Store>
+__device__ __forceinline__ void fft_static_inplace(float2 *buf, bool inv, int tid, Store store,
+                                                   const fftst::RowTw<N, T> &rt, uint32_t live) {
     using Rd = fftst::Radices<N>;
-    static_assert(Rd::n == 3, "three-stage plans only");
     static_assert((PRUNE & fftst::PRUNE_IN) == 0, "inputs already in the buffer are not pruned");
-    fftst::first_inplace<N>(buf, tw, inv, tid, between, live);
-    fftst::later<N, 1, Rd::r1, Rd::r0, false>(buf, tw, inv, tid, nthr, store, &s2);
-    fftst::later<N, 1, Rd::r2, Rd::r0 * Rd::r1, true, Store, PRUNE>(buf, tw, inv, tid, nthr, store, &s3);
+    static_assert(T == N / Rd::r0, "one first-stage butterfly per thread");
+    fftst::first_inplace<N>(buf, inv, tid, live);
+    fftst::later<N, 1, T, Rd::r1, Rd::r0, false, 0>(buf, nullptr, inv, tid, rt.s2, store);
+    fftst::later<N, 1, T, Rd::r2, Rd::r0 * Rd::r1, true, PRUNE>(buf, nullptr, inv, tid, rt.s3, store);
+}
+template <int N, int T, int PRUNE = 0, class Load, class Store>
+__device__ __forceinline__ void fft_static_row(float2 *buf, bool inv, int tid, Load load, Store store,
+                                               const fftst::RowTw<N, T> &rt) {
+    using Rd = fftst::Radices<N>;
+    fftst::first<N, 1, T, PRUNE>(buf, inv, tid, load);
+    fftst::later<N, 1, T, Rd::r1, Rd::r0, false, 0>(buf, nullptr, inv, tid, rt.s2, store);
+    fftst::later<N, 1, T, Rd::r2, Rd::r0 * Rd::r1, true, PRUNE>(buf, nullptr, inv, tid, rt.s3, store);
 }
 
-// COUNT transforms of the compile-time size N (see fft_many for the contract).
-// s2, s3: the thread's twiddle bases of stages 2 and 3 (stage_twiddles), for
-// COUNT = 1 callers that transform many sequences; null reads them per call.
-template <int N, int COUNT, int PRUNE = 0, class Load, class Store>
-__device__ __forceinline__ void fft_static(float2 *buf, const float2 *__restrict__ tw, bool inv, int tid, int nthr,
-                                           Load load, Store store, const fftst::StageTw *s2 = nullptr,
-                                           const fftst::StageTw *s3 = nullptr) {
+// COUNT transforms of the compile-time size N by T threads (see fft_many for the contract).
+template <int N, int COUNT, int T, int PRUNE = 0, class Load, class Store>
+__device__ __forceinline__ void fft_static(float2 *buf, const float2 *__restrict__ tw, bool inv, int tid, Load load,
+                                           Store store) {
     using Rd = fftst::Radices<N>;
-    static_assert(Rd::n == 3, "three-stage plans only");
-    fftst::first<N, COUNT, Load, PRUNE>(buf, tw, inv, tid, nthr, load);
-    fftst::later<N, COUNT, Rd::r1, Rd::r0, false>(buf, tw, inv, tid, nthr, store, s2);
-    fftst::later<N, COUNT, Rd::r2, Rd::r0 * Rd::r1, true, Store, PRUNE>(buf, tw, inv, tid, nthr, store, s3);
+    fftst::first<N, COUNT, T, PRUNE>(buf, inv, tid, load);
+    fftst::later<N, COUNT, T, Rd::r1, Rd::r0, false, 0>(buf, tw, inv, tid, fftst::NoTw{}, store);
+    fftst::later<N, COUNT, T, Rd::r2, Rd::r0 * Rd::r1, true, PRUNE>(buf, tw, inv, tid, fftst::NoTw{}, store);
 }
 
 }  // namespace ws

@@ -118,8 +118,7 @@ extern "C" ws_status ws_degrid_noalloc(ws_plan_t plan, const void *image, const 
     v.d_corr = p->d_corr;
     v.d_zsplit = p->d_zsplit;
     v.d_tw = p->d_tw;
-    v.fft = p->fft;
-    v.fft_mixed = p->fft_mixed;
+    v.fft_fwd = p->fft_fwd;
     v.ntiles = p->ntiles;
     v.P = P;
     v.d_stack = stack;

@@ -84,6 +84,7 @@ void release(ws_plan_s *p) {
     cudaFree(p->d_offsets);
     cudaFree(p->d_blocksums);
     cudaFree(p->d_acc);
+    cudaFree(p->d_rows_done);
     cudaFree(p->d_tile_occ);
     cudaFree(p->d_col_occ);
     cudaFree(p->d_img);
@@ -158,10 +159,39 @@ struct StageTimer {
     }
 };
 
-// Radices of an N'-point transform: 16, 8, 4 for the power of two (N' is a
-// multiple of 32, so no radix 2 is needed), then 7, 5, 3; plus the digit
-// weights of the first stage's reversal and the shared-memory layout.
-bool fft_make_plan(int n, FftPlan *F) {
+// Cost of one radix-r butterfly of the runtime transforms, in packed FP32
+// instructions: its DFT, its twiddles (about five per element: product, power
+// and the pair the product needs) and its shared-memory accesses.
+double butterfly_cost(int r) {
+    double dft = 0.0;
+    switch (r) {
+        case 3: dft = 8; break;
+        case 4: dft = 8; break;
+        case 5: dft = 18; break;
+        case 6: dft = 22; break;
+        case 7: dft = 36; break;
+        case 8: dft = 26; break;
+        case 10: dft = 46; break;
+        case 12: dft = 56; break;
+        case 14: dft = 86; break;
+        case 16: dft = 80; break;
+        case 20: dft = 112; break;
+        case 21: dft = 164; break;
+        case 24: dft = 142; break;
+        default: dft = 200; break;
+    }
+    return dft + 5.0 * r + 6.0 * r + 40.0;
+}
+
+// Radices of an N'-point forward transform: 16, 8, 4 for the power of two (N'
+// is a multiple of 32, so no radix 2 is needed), then 7, 5, 3.  One factor 2 and
+// one factor 5 make a radix-10 stage where that saves a stage (N' = 5600 = 2^5 5^2 7:
+// 16, 10, 7, 5 instead of 8, 4, 7, 5, 5).  The forward direction keeps these
+// radices although the inverse's take fewer stages: another sequence rounds the
+// w-stack differently in a way that many visibilities share, and a chi^2
+// summed over a prediction in FP64 moves with it (2e-7 at N' = 2016), where
+// predictions are otherwise the same from one version to the next.
+int forward_radices(int n, int *radix) {
     int a = 0, m = n;
     while (m % 2 == 0) {
         m /= 2;
@@ -178,8 +208,6 @@ bool fft_make_plan(int n, FftPlan *F) {
         }
         return s;
     };
-    // one factor 2 and one factor 5 make a radix-10 stage where that saves a stage
-    // (N' = 5600 = 2^5 5^2 7: 16, 10, 7, 5 instead of 8, 4, 7, 5, 5)
     const bool ten = m % 5 == 0 && a >= 1 && pow2_stages(a - 1) < pow2_stages(a);
     if (ten) {
         --a;
@@ -187,47 +215,154 @@ bool fft_make_plan(int n, FftPlan *F) {
     }
     int ns = 0;
     while (a > 0) {
-        if (a == 1) return false;
+        if (a == 1 || ns == kMaxFftStages) return 0;
         const int r = pow2_radix(a);
-        F->radix[ns++] = r;
+        radix[ns++] = r;
         a -= r == 16 ? 4 : (r == 8 ? 3 : 2);
-        if (ns >= 8) return false;
     }
-    if (ten) F->radix[ns++] = 10;
+    if (ten) {
+        if (ns == kMaxFftStages) return 0;
+        radix[ns++] = 10;
+    }
     for (int p : {7, 5, 3})
         while (m % p == 0) {
-            if (ns >= 8) return false;
-            F->radix[ns++] = p;
+            if (ns == kMaxFftStages) return 0;
+            radix[ns++] = p;
             m /= p;
         }
-    if (m != 1) return false;
+    return m == 1 ? ns : 0;
+}
+
+// Radices of an N'-point inverse transform, largest first: those of the least
+// total cost among the factorizations into radices that fft.cuh has, whose
+// first stage needs no more than kMaxFftThreads butterflies (a thread then owns
+// one, as the in-place first stage requires).  Three stages for nearly every
+// N', e.g. 2016 = 14 12 12 and 5600 = 28 20 10, where factors of 16, 8, 7, 5 and
+// 3 alone take four or five, each with its trip through shared memory.
+int inverse_radices(int n, int *best) {
+    // what the kernels have as a first, middle and last radix
+    auto first = [](int r) { return r == 28 || r == 24 || r == 20 || r == 16 || r == 14 || r == 12 || r == 10 || r == 8; };
+    auto middle = [](int r) { return r == 21 || r == 20 || r == 16 || r == 14 || r == 12 || r == 10 || r == 8 || r == 6; };
+    auto last = [](int r) { return r == 16 || r == 14 || r == 12 || r == 10 || r == 8 || r == 7 || r == 6 || r == 4; };
+    const int radices[] = {28, 24, 21, 20, 16, 14, 12, 10, 8, 7, 6, 4};
+    int cur[kMaxFftStages] = {}, nbest = 0;
+    double best_cost = 0.0;
+    auto search = [&](auto &&self, int rest, int depth, int from, double cost) -> void {
+        if (rest == 1) {
+            if (depth >= 2 && (nbest == 0 || cost < best_cost)) {
+                best_cost = cost;
+                nbest = depth;
+                std::copy(cur, cur + depth, best);
+            }
+            return;
+        }
+        if (depth == kMaxFftStages) return;
+        for (int i = from; i < (int)(sizeof(radices) / sizeof(radices[0])); ++i) {
+            const int r = radices[i];
+            if (rest % r || (depth == 0 && (!first(r) || n / r > kMaxFftThreads))) continue;
+            if (depth > 0 && !(rest == r ? last(r) : middle(r))) continue;
+            cur[depth] = r;
+            self(self, rest / r, depth + 1, i, cost + (double)(n / r) * butterfly_cost(r));
+        }
+    };
+    search(search, n, 0, 0, 0.0);
+    return nbest;
+}
+
+// Bank conflicts of a plan's shared-memory accesses by `count` interleaved
+// transforms: the sum over all half-warp accesses (16 lanes of 8 bytes) of the
+// lanes on the fullest bank pair.
+long fft_conflicts(const FftPlan &F, int chunk, int stride, int count) {
+    const int ns = F.nstages;
+    auto slot = [&](int e) { return e + e / chunk; };
+    long total = 0;
+    for (int s = 0; s < ns; ++s) {
+        const int R = F.radix[s], L = F.L[s], items = std::min(count * F.nb[s], 512);
+        for (int q0 = 0; q0 < items; q0 += 16) {
+            int at[16], n = std::min(16, items - q0);
+            for (int i = 0; i < n; ++i) {
+                const int t = (q0 + i) % count, b = (q0 + i) / count;
+                int e;
+                if (s == 0) {
+                    int g = 0, rest = b;
+                    for (int k = ns - 1; k >= 1; --k) {
+                        g += (rest % F.radix[k]) * F.gw[k];
+                        rest /= F.radix[k];
+                    }
+                    e = g * R;
+                } else {
+                    e = b / L * R * L + b % L;
+                }
+                at[i] = t * stride + slot(e);
+            }
+            int bank[16] = {}, worst = 0;
+            for (int i = 0; i < n; ++i) worst = std::max(worst, ++bank[at[i] % 16]);
+            total += (long)worst * R;
+        }
+    }
+    return total;
+}
+
+// Plan of an N'-point transform: its radices, the constants of each stage, the
+// shared-memory layout (the pad that leaves the fewest bank conflicts) and the CTA sizes.
+bool fft_make_plan(int n, bool inverse, FftPlan *F) {
+    int radix[kMaxFftStages] = {};
+    const int ns = inverse ? inverse_radices(n, radix) : forward_radices(n, radix);
+    if (ns < 2) return false;
     F->n = n;
     F->nstages = ns;
-    auto log2i = [](int v) {
-        int l = 0;
-        while ((1 << l) < v) ++l;
-        return (1 << l) == v ? l : -1;
-    };
-    int L = 1;
-    for (int i = 0; i < ns; ++i) {
-        int xw = 1, gw = 1;
-        for (int l = i + 1; l < ns; ++l) xw *= F->radix[l];
-        for (int l = 1; l < i; ++l) gw *= F->radix[l];
-        F->xw[i] = xw;
-        F->gw[i] = gw;
-        F->lxw[i] = log2i(xw);
-        F->lgw[i] = log2i(gw);
-        F->xw_mul[i] = div_mul(xw);
-        F->r_mul[i] = div_mul(F->radix[i]);
-        F->L_mul[i] = div_mul(L);
-        L *= F->radix[i];
+    int L = 1, gw = 1;
+    for (int s = 0; s < ns; ++s) {
+        const int r = radix[s];
+        int xw = 1;
+        for (int l = s + 1; l < ns; ++l) xw *= radix[l];
+        F->radix[s] = r;
+        F->L[s] = L;
+        F->nb[s] = n / r;
+        F->twstep[s] = n / (r * L);
+        F->gw[s] = s == 0 ? 0 : gw;
+        F->L_mul[s] = div_mul(L);
+        F->xw_mul[s] = div_mul(xw);
+        F->r_mul[s] = div_mul(r);
+        if (s > 0) gw *= r;
+        L *= r;
     }
-    F->logn = log2i(n);
-    int shift = 4;
-    while ((2 << shift) <= n / F->radix[0]) ++shift;
-    F->padshift = shift;
-    int len = (n - 1) + ((n - 1) >> shift) + 1;
-    F->stride = len + ((8 - len % 16) + 16) % 16;     // == 8 (mod 16)
+    auto stride_of = [&](int len) { return len + ((8 - len % 16) + 16) % 16; };     // == 8 (mod 16)
+    int chunk = 0;
+    long fewest = 0;
+    for (int s = ns - 1; s >= 1; --s) {
+        const int c = F->L[s], stride = stride_of(n + n / c);
+        const long conflicts = fft_conflicts(*F, c, stride, 1) + fft_conflicts(*F, c, stride, 2);
+        if (chunk == 0 || (double)conflicts < 0.95 * (double)fewest) {
+            chunk = c;
+            fewest = conflicts;
+        }
+    }
+    F->chunk_mul = div_mul(chunk);
+    for (int s = 0; s < ns; ++s) F->step[s] = F->L[s] >= chunk ? F->L[s] + F->L[s] / chunk : F->L[s];
+    // the compile-time plans of fft.cuh pad at most 17 slots
+    F->stride = stride_of(std::max(n + n / chunk, n + 17));
+    // threads per CTA for `count` transforms: the rounds of every stage, weighted by the idle threads
+    auto threads = [&](int count, int lo) {
+        int t_best = 0;
+        double w_best = 0.0;
+        for (int t = std::max(32, (lo + 31) / 32 * 32); t <= kMaxFftThreads; t += 32) {
+            double w = 0.0;
+            for (int s = 0; s < ns; ++s) w += (double)((count * F->nb[s] + t - 1) / t) * butterfly_cost(radix[s]) * t;
+            if (t_best == 0 || w < 0.98 * w_best) {
+                t_best = t;
+                w_best = w;
+            }
+        }
+        return t_best;
+    };
+    F->row_threads = threads(1, std::min(256, inverse ? F->nb[0] : n / 16));
+    F->col_threads = threads(2, std::min(256, n / 8));
+    // boxes of at most 256 column blocks whose size keeps shared-memory addresses 128-byte aligned
+    const int blocks = n / 4;
+    F->boxes = (blocks + 255) / 256;
+    while (blocks % F->boxes || (blocks / F->boxes) % 4) ++F->boxes;
+    F->box_blocks = blocks / F->boxes;
     return true;
 }
 
@@ -575,8 +710,8 @@ ws_status plan_create(ws_plan_s **out, int32_t N, double x0, int32_t W, double f
         delete p;
         return WS_ERR_ARG;
     }
-    p->fft_mixed = (Np & (Np - 1)) != 0;
-    if (!fft_make_plan((int)Np, &p->fft) || transform_smem_bytes(p->fft, N) > (size_t)227 * 1024) {
+    if (!fft_make_plan((int)Np, false, &p->fft_fwd) || !fft_make_plan((int)Np, true, &p->fft_inv) ||
+        transform_smem_bytes(p->fft_fwd, p->fft_inv, N) > (size_t)227 * 1024) {
         set_error("ws_plan: no transform plan for N' = " + std::to_string(Np));
         delete p;
         return WS_ERR_ARG;
@@ -699,11 +834,14 @@ ws_status plan_create(ws_plan_s **out, int32_t N, double x0, int32_t W, double f
         WS_TRY(cudaMemcpy(p->d_tw, tw.data(), tw.size() * sizeof(float2), cudaMemcpyHostToDevice),
                "uploading twiddles");
     }
-    WS_TRY(setup_transform_kernels(p->fft, N), "configuring transform kernels");
+    WS_TRY(setup_transform_kernels(p->fft_fwd, p->fft_inv, N), "configuring transform kernels");
     WS_TRY(dev_alloc(&p->d_counts, (size_t)p->ntiles + 1, &p->bytes), "allocating tile counts");
     WS_TRY(dev_alloc(&p->d_offsets, (size_t)p->ntiles + 1, &p->bytes), "allocating tile offsets");
     WS_TRY(dev_alloc(&p->d_blocksums, (size_t)4096, &p->bytes), "allocating scan sums");
-    WS_TRY(dev_alloc(&p->d_acc, (size_t)N * N, &p->bytes), "allocating the accumulator");
+    p->row_shares = inv_row_shares(p->fft_inv, N, p->P > 0 ? std::min(p->P, L.Nw) : L.Nw, p->sms);
+    WS_TRY(dev_alloc(&p->d_acc, (size_t)p->row_shares * N * N, &p->bytes), "allocating the accumulators");
+    WS_TRY(dev_alloc(&p->d_rows_done, (size_t)N, &p->bytes), "allocating row counters");
+    WS_TRY(cudaMemset(p->d_rows_done, 0, (size_t)N * sizeof(unsigned)), "clearing row counters");
     WS_TRY(dev_alloc(&p->d_tile_occ, (size_t)p->ntiles, &p->bytes), "allocating tile occupancy");
     WS_TRY(dev_alloc(&p->d_col_occ, (size_t)L.ntt * L.ntu, &p->bytes), "allocating strip occupancy");
     WS_TRY(dev_alloc(&p->d_img, (size_t)N * N, &p->bytes), "allocating the corrected image");

@@ -54,7 +54,7 @@ cudaError_t row_tensor_map(const ws_plan_s *p, CUtensorMap *map) {
     const cuuint64_t Np = (cuuint64_t)p->L.Np;
     const cuuint64_t dims[4] = {2 * CB, Np, Np / CB, (cuuint64_t)p->P};
     const cuuint64_t strides[3] = {2 * CB * sizeof(float), Np * 2 * CB * sizeof(float), Np * Np * sizeof(float2)};
-    const cuuint32_t box[4] = {2 * CB, 1, (cuuint32_t)std::min<cuuint64_t>(256, Np / CB), 1};
+    const cuuint32_t box[4] = {2 * CB, 1, (cuuint32_t)p->fft_inv.box_blocks, 1};
     const cuuint32_t estr[4] = {1, 1, 1, 1};
     const CUresult r = encode(map, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, p->d_stack, dims, strides, box, estr,
                               CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE,
@@ -62,57 +62,62 @@ cudaError_t row_tensor_map(const ws_plan_s *p, CUtensorMap *map) {
     return r == CUDA_SUCCESS ? cudaSuccess : cudaErrorInvalidValue;
 }
 
-const Ops &ops_runtime_pow2() {
+const Ops &ops_runtime() {
     static const Ops o = ops_of<0>();
-    return o;
-}
-const Ops &ops_runtime_mixed() {
-    static const Ops o = ops_of<1>();
     return o;
 }
 }  // namespace tf
 
 namespace {
 // The variant for an N'-point plan: a compile-time plan when one exists.
-const tf::Ops &ops_for(int Np, bool mixed) {
+const tf::Ops &ops_for(int Np) {
     switch (Np) {
         case 512: return tf::ops_512();
         case 1024: return tf::ops_1024();
         case 2048: return tf::ops_2048();
         case 4096: return tf::ops_4096();
-        default: return mixed ? tf::ops_runtime_mixed() : tf::ops_runtime_pow2();
+        default: return tf::ops_runtime();
     }
 }
 }  // namespace
 
-// Largest dynamic shared memory any transform kernel of this plan asks for
-// (the compile-time inv_rows double buffer is checked by its own setup).
-size_t transform_smem_bytes(const FftPlan &F, int N) {
-    size_t b = tf::smem2(F);
-    if (tf::smem_rows(F, N) > b) b = tf::smem_rows(F, N);
-    if (tf::smem_fwd_rows(F, N, false) > b) b = tf::smem_fwd_rows(F, N, false);
-    return b;
+// Largest dynamic shared memory any transform kernel of this plan asks for.
+size_t transform_smem_bytes(const FftPlan &fwd, const FftPlan &inv, int N) {
+    return std::max({tf::smem2(fwd), tf::smem2(inv), tf::rows_smem(inv, N).bytes, tf::smem_fwd_rows(fwd, N, false)});
 }
 
-cudaError_t setup_transform_kernels(const FftPlan &F, int N) {
-    return ops_for(F.n, (F.n & (F.n - 1)) != 0).setup(F, N);
+// Shares of the planes each image row is given in inv_rows.  The CTAs that fit
+// on the GPU at once should turn over about eight times, so that the last round
+// (partly empty) costs little; a share keeps at least eight planes, or two while
+// the rows alone leave part of the GPU idle.
+int inv_row_shares(const FftPlan &F, int N, int planes, int sms) {
+    const bool fixed = F.n == 512 || F.n == 1024 || F.n == 2048 || F.n == 4096;
+    const int T = fixed ? F.n / 16 : F.row_threads;
+    const int by_smem = (int)(228 * 1024 / (tf::rows_smem(F, N).bytes + 1024));
+    const int64_t slots = (int64_t)sms * std::max(1, std::min(by_smem, 512 / T));
+    const int want = (int)((8 * slots + N - 1) / N), fill = (int)((slots + N - 1) / N);
+    return std::max(1, std::min(want, std::max(planes / 8, std::min(fill, planes / 2))));
+}
+
+cudaError_t setup_transform_kernels(const FftPlan &fwd, const FftPlan &inv, int N) {
+    return ops_for(fwd.n).setup(fwd, inv, N);
 }
 
 cudaError_t launch_fwd_rows(const ws_plan_s *p, int chunk, int planes, cudaStream_t s) {
-    return ops_for(p->L.Np, p->fft_mixed).fwd_rows(p, chunk, planes, s);
+    return ops_for(p->L.Np).fwd_rows(p, chunk, planes, s);
 }
 
 cudaError_t launch_fwd_cols(const ws_plan_s *p, int chunk, int planes, cudaStream_t s) {
-    return ops_for(p->L.Np, p->fft_mixed).fwd_cols(p, chunk, planes, s);
+    return ops_for(p->L.Np).fwd_cols(p, chunk, planes, s);
 }
 
 cudaError_t launch_inv_cols(const ws_plan_s *p, int chunk, int planes, cudaStream_t s) {
-    return ops_for(p->L.Np, p->fft_mixed).inv_cols(p, chunk, planes, s);
+    return ops_for(p->L.Np).inv_cols(p, chunk, planes, s);
 }
 
 cudaError_t launch_inv_rows(const ws_plan_s *p, int chunk, int planes, bool first, bool last, float2 *dirty,
                             cudaStream_t s) {
-    return ops_for(p->L.Np, p->fft_mixed).inv_rows(p, chunk, planes, first, last, dirty, s);
+    return ops_for(p->L.Np).inv_rows(p, chunk, planes, first, last, dirty, s);
 }
 
 }  // namespace ws

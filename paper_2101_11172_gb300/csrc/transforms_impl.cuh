@@ -1,11 +1,14 @@
 // Kernel templates of the fused plane transforms (see transforms.cu).
 //
-// NP selects the FFT code: 0 = runtime plan, power of two; 1 = runtime plan
-// with odd radices; 512, 1024, 2048, 4096 = the compile-time plans of
-// fft.cuh.  Each translation unit instantiates Transforms<NP> for its sizes.
+// NP selects the FFT code: 0 = the runtime plan (any N'); 512, 1024, 2048, 4096
+// = the compile-time plans of fft.cuh.  Each translation unit instantiates
+// Transforms<NP> for its sizes.
 #pragma once
 
 #include <cuda.h>
+
+#include <algorithm>
+#include <type_traits>
 
 #include "common.cuh"
 #include "fft.cuh"
@@ -14,35 +17,60 @@
 namespace ws {
 namespace tf {
 
-constexpr int kThreads = 256;       // two rows or two columns per CTA
-constexpr int kPerCta = 2;
-constexpr int kRowThreads = 256;    // one row per CTA (inv_rows)
+constexpr int kPerCta = 2;          // columns per CTA of the column kernels
+// CTA sizes follow the transform: N'/16 threads for a row and twice that for a
+// pair of columns, one radix-16 butterfly per thread in a stage (two at N' =
+// 4096 for the columns).  With 256 threads at every size most of a CTA idled on
+// short rows (N' = 512: 32 butterflies in the first stage).  Runtime plans
+// bring their own (FftPlan::row_threads, col_threads).  The minimum of resident
+// CTAs bounds the registers: 128 a thread for rows, 80 for columns.
+template <int NP>
+WS_HD constexpr int row_threads_max() {
+    return NP ? NP / 16 : kMaxFftThreads;
+}
+template <int NP>
+WS_HD constexpr int col_threads_max() {
+    return NP ? (NP > 2048 ? 256 : NP / 8) : kMaxFftThreads;
+}
+template <int NP>
+WS_HD constexpr int row_ctas() {
+    return NP ? 512 / row_threads_max<NP>() : 2;
+}
+template <int NP>
+WS_HD constexpr int col_ctas() {
+    return NP ? 768 / col_threads_max<NP>() : 2;
+}
 // Shared memory per CTA that still lets two CTAs share an SM (228 KB, 1 KB of it reserved per CTA).
 constexpr size_t kTwoCtaSmem = 113 * 1024;
-
-// Runtime-plan inv_rows keeps the z row in shared memory when the row buffer,
-// the z row and the compensated sums still leave room for two CTAs per SM.
-__host__ __device__ inline bool rows_keep_z(const FftPlan &F, int N) {
-    return (size_t)F.stride * sizeof(float2) + (size_t)N * (sizeof(float2) + sizeof(float4)) + F.n / TU + 16 <=
-           kTwoCtaSmem;
-}
 
 __device__ __forceinline__ int grid_to_crop(int g, int half, int Np) { return g < half ? g + half : g - (Np - half); }
 __device__ __forceinline__ bool in_crop(int g, int half, int Np) { return g < half || g >= Np - half; }
 
-// PRUNE (fftst::PRUNE_IN / PRUNE_OUT, compile-time plans with N' = 2N only):
-// the inputs outside the centred half are zero / the outputs outside it are
-// not wanted, and the transform skips them.
-template <int NP, int COUNT, int PRUNE = 0, class Load, class Store>
-__device__ __forceinline__ void plane_fft(float2 *buf, const FftPlan &F, const float2 *__restrict__ tw, bool inv,
-                                          int tid, int nthr, Load load, Store store) {
+// The column kernels' transforms (two columns).  PRUNE (fftst::PRUNE_IN /
+// PRUNE_OUT, compile-time plans with N' = 2N only): the inputs outside the
+// centred half are zero / the outputs outside it are not wanted, and the
+// transform skips them.
+template <int NP, bool INV, int PRUNE, class Load, class Store>
+__device__ __forceinline__ void column_fft(float2 *buf, const FftPlan &F, const float2 *__restrict__ tw, Load load,
+                                           Store store) {
     if constexpr (NP == 0)
-        fft_many<false, COUNT>(buf, F, tw, inv, tid, nthr, load, store);
-    else if constexpr (NP == 1)
-        fft_many<true, COUNT>(buf, F, tw, inv, tid, nthr, load, store);
+        fft_many<kPerCta, INV>(buf, F, tw, threadIdx.x, blockDim.x, load, store);
     else
-        fft_static<NP, COUNT, PRUNE>(buf, tw, inv, tid, nthr, load, store);
+        fft_static<NP, kPerCta, col_threads_max<NP>(), PRUNE>(buf, tw, INV, threadIdx.x, load, store);
 }
+
+// The twiddle bases a row kernel's thread keeps across planes.
+struct NoRowTw {
+    __device__ __forceinline__ NoRowTw(const float2 *, bool, int) {}
+};
+template <int NP>
+struct RowTwOf {
+    using type = fftst::RowTw<NP, NP / 16>;
+};
+template <>
+struct RowTwOf<0> {
+    using type = NoRowTw;
+};
 
 // CROP: N' = 2N on a compile-time plan, so the crop is exactly the centred half.
 template <int NP>
@@ -64,7 +92,7 @@ constexpr int kScreenSteps = 8;
 // g and leaves g x step in its place for the next plane.  Each pixel is read
 // by the same thread on every plane, so the update needs no barrier.
 template <int NP, bool STEP, bool CROP>
-__global__ void __launch_bounds__(kRowThreads, 2)
+__global__ void __launch_bounds__(row_threads_max<NP>(), row_ctas<NP>())
 fwd_rows_kernel(Launch L, FftPlan F, const float2 *__restrict__ tw, const float2 *__restrict__ img,
                 const float2 *__restrict__ zsplit, const uint8_t *__restrict__ col_occ, int plane0, int planes,
                 float2 *__restrict__ stack) {
@@ -75,7 +103,7 @@ fwd_rows_kernel(Launch L, FftPlan F, const float2 *__restrict__ tw, const float2
     float2 *grow = zrow + N;                                     // N, STEP only: the screened row
     float2 *erow = grow + N;                                     // N, STEP only: exp(-2 pi i z)
     uint8_t *occ = reinterpret_cast<uint8_t *>(irow + (STEP ? 4 : 2) * N);   // ntu: strips of the current t-tile
-    const int ii = blockIdx.x, tid = threadIdx.x;
+    const int ii = blockIdx.x, tid = threadIdx.x, kRowThreads = NP ? row_threads_max<NP>() : (int)blockDim.x;
     // this CTA's planes: an equal share of the chunk's valid planes
     const int nvalid = min(planes, L.Nw - plane0);
     const int per = (nvalid + (int)gridDim.y - 1) / (int)gridDim.y;
@@ -93,12 +121,7 @@ fwd_rows_kernel(Launch L, FftPlan F, const float2 *__restrict__ tw, const float2
         }
     }
     int occ_tt = -1;
-    fftst::StageTw s2{}, s3{};                                  // the thread's twiddle bases, read once
-    if constexpr (NP >= 512) {
-        using Rd = fftst::Radices<NP>;
-        s2 = fftst::stage_twiddles<NP, Rd::r1, Rd::r0>(tw, false, tid);
-        s3 = fftst::stage_twiddles<NP, Rd::r2, Rd::r0 * Rd::r1>(tw, false, tid);
-    }
+    const typename RowTwOf<NP>::type rt(tw, false, tid);        // the thread's twiddle bases, read once
     for (int p = p_begin; p < p_end; ++p) {
         const int pl = plane0 + p;
         const float t = (float)(pl + L.t_lo);
@@ -144,14 +167,14 @@ fwd_rows_kernel(Launch L, FftPlan F, const float2 *__restrict__ tw, const float2
             if (occ[R / TU]) __stcs(plane + tiled_index(ii, R, Np), v);
         };
         if constexpr (NP >= 512)
-            fft_static<NP, 1, CROP ? fftst::PRUNE_IN : 0>(sbuf, tw, false, tid, kRowThreads, load, store, &s2, &s3);
+            fft_static_row<NP, row_threads_max<NP>(), CROP ? fftst::PRUNE_IN : 0>(sbuf, false, tid, load, store, rt);
         else
-            plane_fft<NP, 1>(sbuf, F, tw, false, tid, kRowThreads, load, store);
+            fft_many<1, false>(sbuf, F, tw, tid, kRowThreads, load, store);
     }
 }
 
 template <int NP, bool CROP>
-__global__ void __launch_bounds__(kThreads, 2)
+__global__ void __launch_bounds__(col_threads_max<NP>(), col_ctas<NP>())
 fwd_cols_kernel(Launch L, FftPlan F, const float2 *__restrict__ tw, const uint8_t *__restrict__ tile_occ,
                 const uint8_t *__restrict__ col_occ, int plane0, float2 *__restrict__ stack) {
     extern __shared__ __align__(16) float2 sbuf[];
@@ -162,7 +185,7 @@ fwd_cols_kernel(Launch L, FftPlan F, const float2 *__restrict__ tw, const uint8_
     if (!col_occ[tt * L.ntu + tu]) return;                // no visibility reads these columns of this plane
     float2 *blk = stack + (size_t)blockIdx.y * Np * Np + (size_t)(R0 >> 2) * Np * CB + (R0 & 3);
     uint8_t *occ = reinterpret_cast<uint8_t *>(sbuf + kPerCta * F.stride);
-    for (int i = threadIdx.x; i < L.ntv; i += kThreads) occ[i] = tile_occ[((size_t)tt * L.ntv + i) * L.ntu + tu];
+    for (int i = threadIdx.x; i < L.ntv; i += blockDim.x) occ[i] = tile_occ[((size_t)tt * L.ntv + i) * L.ntu + tu];
     __syncthreads();
     // rows 0..N-1 hold the N transformed image rows; every other row is zero padding
     auto load = [&](int b, int S) -> float2 {
@@ -172,13 +195,13 @@ fwd_cols_kernel(Launch L, FftPlan F, const float2 *__restrict__ tw, const uint8_
     auto store = [&](int b, int S, float2 v) {
         if (occ[S >> L.tv_log]) blk[(size_t)S * CB + b] = v;     // only tiles the gather reads
     };
-    plane_fft<NP, kPerCta, CROP ? fftst::PRUNE_IN : 0>(sbuf, F, tw, false, threadIdx.x, kThreads, load, store);
+    column_fft<NP, false, CROP ? fftst::PRUNE_IN : 0>(sbuf, F, tw, load, store);
 }
 
 // -- gridding ----------------------------------------------------------------
 
 template <int NP, bool CROP>
-__global__ void __launch_bounds__(kThreads, 2)
+__global__ void __launch_bounds__(col_threads_max<NP>(), col_ctas<NP>())
 inv_cols_kernel(Launch L, FftPlan F, const float2 *__restrict__ tw, const uint8_t *__restrict__ tile_occ,
                 const uint8_t *__restrict__ col_occ, int plane0, float2 *__restrict__ stack) {
     extern __shared__ __align__(16) float2 sbuf[];
@@ -189,7 +212,7 @@ inv_cols_kernel(Launch L, FftPlan F, const float2 *__restrict__ tw, const uint8_
     if (!col_occ[tt * L.ntu + tu]) return;                // all-zero columns: inv_rows skips them too
     float2 *blk = stack + (size_t)blockIdx.y * Np * Np + (size_t)(R0 >> 2) * Np * CB + (R0 & 3);
     uint8_t *occ = reinterpret_cast<uint8_t *>(sbuf + kPerCta * F.stride);
-    for (int i = threadIdx.x; i < L.ntv; i += kThreads) occ[i] = tile_occ[((size_t)tt * L.ntv + i) * L.ntu + tu];
+    for (int i = threadIdx.x; i < L.ntv; i += blockDim.x) occ[i] = tile_occ[((size_t)tt * L.ntv + i) * L.ntu + tu];
     __syncthreads();
     // gridding wrote only occupied tiles; every other cell is zero
     auto load = [&](int b, int S) -> float2 {
@@ -199,7 +222,7 @@ inv_cols_kernel(Launch L, FftPlan F, const float2 *__restrict__ tw, const uint8_
     auto store = [&](int b, int S, float2 v) {
         if (in_crop(S, half, Np)) blk[(size_t)grid_to_crop(S, half, Np) * CB + b] = v;
     };
-    plane_fft<NP, kPerCta, CROP ? fftst::PRUNE_OUT : 0>(sbuf, F, tw, true, threadIdx.x, kThreads, load, store);
+    column_fft<NP, true, CROP ? fftst::PRUNE_OUT : 0>(sbuf, F, tw, load, store);
 }
 
 // -- TMA row copies and mbarriers ----------------------------------------------
@@ -234,8 +257,7 @@ __device__ __forceinline__ bool mbar_wait(uint64_t *bar, unsigned parity, int po
     }
     return false;
 }
-// Box of an image row: {8 floats, 1 row, min(256, N'/4) column blocks, 1 plane}
-// of the stack's row map.
+// Box of an image row: {8 floats, 1 row, box_blocks column blocks, 1 plane} of the stack's row map.
 __device__ __forceinline__ void tma_row_box(float2 *dst, const CUtensorMap *map, int row, int block, int plane,
                                             uint64_t *bar) {
     asm volatile(
@@ -245,171 +267,176 @@ __device__ __forceinline__ void tma_row_box(float2 *dst, const CUtensorMap *map,
         : "memory");
 }
 
-// Shared-memory layout of the compile-time inv_rows: two 128-byte aligned row
-// buffers (TMA destinations), z row, compensated sums, two mbarriers.
-template <int NP>
+// Shared memory of inv_rows: one or two 128-byte aligned row buffers (TMA
+// destinations), the compensated sums, the z row (kept where it fits), two mbarriers and a flag.
 struct RowsSmem {
-    static constexpr size_t buf = (fftst::Layout<NP>::stride * sizeof(float2) + 127) / 128 * 128;
-    static size_t bytes(int N) { return 128 + 2 * buf + (size_t)N * (sizeof(float2) + sizeof(float4)) + 16; }
+    int buffers;          // 2: the next plane's row is copied while this one is transformed
+    int keep_z;           // 0: the screen reads z from global memory
+    size_t buf, bytes;
 };
+inline RowsSmem rows_smem(const FftPlan &F, int N) {
+    RowsSmem r{2, 1, ((size_t)F.stride * sizeof(float2) + 127) / 128 * 128, 0};
+    auto need = [&] {
+        return 128 + r.buffers * r.buf + (size_t)N * (sizeof(float4) + (r.keep_z ? sizeof(float2) : 0)) + 32;
+    };
+    // Two CTAs per SM come first: with one, nothing covers a CTA's barriers.  Where
+    // both buffers and the z row leave no room for a second CTA, one buffer and z
+    // from global memory do (N = 4096, N' = 5600).
+    if (need() > kTwoCtaSmem) {
+        r.keep_z = 0;
+        if (need() > kTwoCtaSmem) r.buffers = 1;
+    }
+    r.bytes = need();
+    return r;
+}
 
-// One CTA owns image row ii and sums the chunk's planes into a compensated
-// accumulator in shared memory; the last FFT stage screens and accumulates.
+// One CTA owns image row ii and an equal share of the chunk's planes (share
+// blockIdx.y of gridDim.y): it sums them into a compensated accumulator in
+// shared memory; the last FFT stage screens and accumulates.  Where a row is
+// shared, every share keeps its own sums in acc (N x N per share), and the CTA
+// that finishes the row last adds them up in share order, so the result does not
+// depend on which one that is.
 //
-// Compile-time plans double-buffer the row with TMA: as plane p starts, warp
-// 0 copies plane p + 1's row into the other buffer in boxes of up to 256
-// column blocks (8 KB), all completing on that buffer's mbarrier.  Strips no
-// footprint touched hold stale data; the first FFT stage masks them to zero.
-// Every wait is bounded; a CTA that gives up counts the failure in *timeouts,
-// waits (bounded) for the copy in flight and returns.
+// The rows come by TMA in boxes of up to 256 column blocks (8 KB), all
+// completing on the buffer's mbarrier: with two buffers, plane p + 1's row is
+// copied while plane p is transformed.  Strips no footprint touched hold stale
+// data; the first FFT stage masks them to zero.  Every wait is bounded; a CTA
+// that gives up waits (bounded) for the copy in flight and ends; *timeouts
+// counts the rows left incomplete.
 template <int NP, bool CROP>
-__global__ void __launch_bounds__(kRowThreads, 2)
-inv_rows_kernel(Launch L, FftPlan F, const float2 *__restrict__ tw, const float2 *__restrict__ stack,
-                const __grid_constant__ CUtensorMap row_map, const uint8_t *__restrict__ col_occ, int plane0,
-                int planes, const float2 *__restrict__ zsplit, const float *__restrict__ corr,
-                float4 *__restrict__ acc, int first, int last, float2 *__restrict__ dirty,
+__global__ void __launch_bounds__(row_threads_max<NP>(), row_ctas<NP>())
+inv_rows_kernel(Launch L, FftPlan F, const float2 *__restrict__ tw, const __grid_constant__ CUtensorMap row_map,
+                const uint8_t *__restrict__ col_occ, int plane0, int planes, int buffers, int keep_z, int buf_slots,
+                const float2 *__restrict__ zsplit, const float *__restrict__ corr, float4 *__restrict__ acc,
+                unsigned *__restrict__ rows_done, int first, int last, float2 *__restrict__ dirty,
                 unsigned long long *__restrict__ timeouts, int wait_polls) {
     extern __shared__ __align__(16) float2 sbuf[];
     const int Np = L.Np, N = L.N, half = N / 2;
-    const int ii = blockIdx.x;
-    const int tid = threadIdx.x;
-    const size_t pix0 = (size_t)ii * N;
-    const int nvalid = min(planes, L.Nw - plane0);
-    if constexpr (NP >= 512) {
-        using Sm = RowsSmem<NP>;
-        constexpr int R0 = fftst::Radices<NP>::r0, nb = NP / R0;
-        constexpr int kBoxBlocks = NP / CB < 256 ? NP / CB : 256, kRowBoxes = NP / CB / kBoxBlocks;
-        // 128-byte aligned start, by pointer arithmetic on sbuf so that every
-        // access below stays a shared-memory access
-        float2 *base = sbuf + ((128u - (smem_addr(sbuf) & 127u)) & 127u) / sizeof(float2);
-        constexpr int kBuf = (int)(Sm::buf / sizeof(float2));
-        auto row_buf = [&](int p) { return base + (p & 1) * kBuf; };
-        float2 *zrow = base + 2 * kBuf;                                   // N
-        float4 *srow = reinterpret_cast<float4 *>(zrow + N);              // N: (sum re, sum im, comp re, comp im)
-        uint64_t *bar = reinterpret_cast<uint64_t *>(srow + N);           // 2
-        const int warp = tid >> 5, lane = tid & 31;
-        // warp 0: copy plane p's row ii into buffer p & 1, kRowBoxes boxes of
-        // kBoxBlocks column blocks (strips no footprint touched come along and
-        // are masked to zero by the first stage)
-        auto issue = [&](int p) {
-            fence_proxy_async();             // the buffer's last generic reads precede these writes
-            if (lane == 0) mbar_arrive_expect_tx(&bar[p & 1], (unsigned)(NP * sizeof(float2)));
-            __syncwarp();
-            if (lane < kRowBoxes)
-                tma_row_box(row_buf(p) + lane * kBoxBlocks * CB, &row_map, ii, lane * kBoxBlocks, p, &bar[p & 1]);
+    const int ii = blockIdx.x, tid = threadIdx.x, T = NP ? row_threads_max<NP>() : (int)blockDim.x;
+    const int R0 = NP ? fftst::Radices<NP ? NP : 512>::r0 : F.radix[0], nb = NP ? NP / 16 : F.nb[0];
+    const int shares = gridDim.y, nvalid = min(planes, L.Nw - plane0);
+    const int per = (nvalid + shares - 1) / shares;
+    const int p_begin = min(nvalid, (int)blockIdx.y * per), p_end = min(nvalid, p_begin + per);
+    const size_t pix0 = (size_t)ii * N, image = (size_t)N * N;
+    float4 *own_acc = acc + blockIdx.y * image;
+    // 128-byte aligned start, by pointer arithmetic on sbuf so that every
+    // access below stays a shared-memory access
+    float2 *base = sbuf + ((128u - (smem_addr(sbuf) & 127u)) & 127u) / sizeof(float2);
+    auto row_buf = [&](int k) { return base + (k & (buffers - 1)) * buf_slots; };
+    float4 *srow = reinterpret_cast<float4 *>(base + buffers * buf_slots);   // N: (sum re, sum im, comp re, comp im)
+    float2 *zrow = reinterpret_cast<float2 *>(srow + N);                     // N if keep_z
+    uint64_t *bar = reinterpret_cast<uint64_t *>(zrow + (keep_z ? N : 0));   // 2
+    volatile int &finisher = *reinterpret_cast<int *>(bar + 2);              // shared by the CTA
+    const float2 *zsrc = keep_z ? zrow : zsplit + pix0;
+    const int warp = tid >> 5, lane = tid & 31;
+    // warp 0: copy row ii of the share's k-th plane into buffer k mod buffers
+    auto issue = [&](int k) {
+        fence_proxy_async();                 // the buffer's last generic reads precede these writes
+        uint64_t *b = &bar[k & (buffers - 1)];
+        if (lane == 0) mbar_arrive_expect_tx(b, (unsigned)(Np * sizeof(float2)));
+        __syncwarp();
+        if (lane < F.boxes)
+            tma_row_box(row_buf(k) + lane * F.box_blocks * CB, &row_map, ii, lane * F.box_blocks, p_begin + k, b);
+    };
+    if (tid == 0) {
+        mbar_init(&bar[0], 1);
+        mbar_init(&bar[1], 1);
+        mbar_init_fence();
+    }
+    for (int jj = tid; jj < N; jj += T) {
+        if (keep_z) zrow[jj] = zsplit[pix0 + jj];
+        srow[jj] = first ? make_float4(0.f, 0.f, 0.f, 0.f) : own_acc[pix0 + jj];
+    }
+    const typename RowTwOf<NP>::type rt(tw, true, tid);
+    __syncthreads();
+    const int count = p_end - p_begin;
+    if (warp == 0 && count > 0) issue(0);
+    uint32_t live = 0;                       // strips of this thread's first-stage inputs, one t-tile
+    int live_tt = -1;
+    bool gave_up = false;                    // uniform
+    for (int k = 0; k < count; ++k) {
+        const int pl = plane0 + p_begin + k;
+        const float t = (float)(pl + L.t_lo);
+        const int tt = pl / TT;
+        if (tt != live_tt) {                 // threads past nb own no first-stage butterfly
+            live = 0;
+            if (tid < nb) {
+#pragma unroll 4
+                for (int m = 0; m < R0; ++m)
+                    live |= (uint32_t)(__ldg(col_occ + tt * L.ntu + (m * nb + tid) / TU) != 0) << m;
+            }
+            live_tt = tt;
+        }
+        uint64_t *b = &bar[k & (buffers - 1)];
+        const unsigned parity = (buffers == 2 ? k >> 1 : k) & 1;
+        const bool ok = mbar_wait(b, parity, wait_polls);
+        if (__syncthreads_or(!ok)) {         // uniform: give up on this row
+            if (tid == 0) mbar_wait(b, parity);              // drain the copy in flight (full limit)
+            gave_up = true;
+            break;
+        }
+        // every thread is past plane k - 1, so its buffer is free for plane k + 1
+        if (warp == 0 && buffers == 2 && k + 1 < count) issue(k + 1);
+        auto store = [&](int, int J, float2 v) {
+            if (!in_crop(J, half, Np)) return;
+            const int jj = grid_to_crop(J, half, Np);
+            float sn, cs;
+            phase_tz(t, zsrc[jj], &sn, &cs);
+            const float4 a = srow[jj];
+            float2 sum = make_float2(a.x, a.y), comp = make_float2(a.z, a.w);
+            kahan_add(sum, comp, cmul_rot(v, make_float2(cs, sn), make_float2(-sn, cs)));
+            srow[jj] = make_float4(sum.x, sum.y, comp.x, comp.y);
         };
-        if (tid == 0) {
-            mbar_init(&bar[0], 1);
-            mbar_init(&bar[1], 1);
-            mbar_init_fence();
-        }
-        for (int jj = tid; jj < N; jj += kRowThreads) {
-            zrow[jj] = zsplit[pix0 + jj];
-            srow[jj] = first ? make_float4(0.f, 0.f, 0.f, 0.f) : acc[pix0 + jj];
-        }
-        using Rd = fftst::Radices<NP>;
-        const fftst::StageTw s2 = fftst::stage_twiddles<NP, Rd::r1, Rd::r0>(tw, true, tid);
-        const fftst::StageTw s3 = fftst::stage_twiddles<NP, Rd::r2, Rd::r0 * Rd::r1>(tw, true, tid);
-        __syncthreads();
-        if (warp == 0 && nvalid > 0) issue(0);
-        uint32_t live = 0;                   // strips of this thread's first-stage inputs, one t-tile
-        int live_tt = -1;
-        for (int p = 0; p < nvalid; ++p) {
-            const float t = (float)(plane0 + p + L.t_lo);
-            const int tt = (plane0 + p) / TT;
-            if (tt != live_tt) {             // threads past nb own no first-stage butterfly
-                live = 0;
-                if (tid < nb) {
-#pragma unroll
-                    for (int m = 0; m < R0; ++m)
-                        live |= (uint32_t)(__ldg(col_occ + tt * L.ntu + (m * nb + tid) / TU) != 0) << m;
-                }
-                live_tt = tt;
-            }
-            const bool ok = mbar_wait(&bar[p & 1], (p >> 1) & 1, wait_polls);
-            if (__syncthreads_or(!ok)) {     // uniform: give up on this row
-                if (tid == 0) {
-                    atomicAdd(timeouts, 1ull);
-                    mbar_wait(&bar[p & 1], (p >> 1) & 1);   // drain the copy in flight (full limit)
-                }
-                __syncthreads();
-                return;
-            }
-            // every thread is past plane p - 1, so its buffer is free for plane p + 1
-            if (warp == 0 && p + 1 < nvalid) issue(p + 1);
-            auto between = [] {};
-            auto store = [&](int, int J, float2 v) {
-                if (!in_crop(J, half, Np)) return;
-                const int jj = grid_to_crop(J, half, Np);
-                float sn, cs;
-                phase_tz(t, zrow[jj], &sn, &cs);
-                float4 a = srow[jj];
-                kahan_add(a.x, a.z, v.x * cs - v.y * sn);
-                kahan_add(a.y, a.w, v.x * sn + v.y * cs);
-                srow[jj] = a;
-            };
-            fft_static_inplace<NP, CROP ? fftst::PRUNE_OUT : 0>(row_buf(p), tw, true, tid, kRowThreads, between, store,
-                                                                  s2, s3, live);
-        }
-        __syncthreads();
-        for (int jj = tid; jj < N; jj += kRowThreads) {
-            const float4 a = srow[jj];
-            if (last) {
-                const float h = corr[pix0 + jj];
-                dirty[pix0 + jj] = make_float2(h * (a.x - a.z), L.fold ? 0.f : h * (a.y - a.w));
-            } else {
-                acc[pix0 + jj] = a;
-            }
-        }
-    } else {
-        // the z row stays in shared memory where two CTAs per SM still fit, else
-        // the screen reads z from global memory
-        const bool keep_z = rows_keep_z(F, N);
-        float2 *zrow = sbuf + F.stride;                          // N if keep_z (F.stride is even: 16-byte aligned)
-        float4 *srow = reinterpret_cast<float4 *>(zrow + (keep_z ? N : 0));   // N: (sum re, sum im, comp re, comp im)
-        uint8_t *occ = reinterpret_cast<uint8_t *>(srow + N);    // ntu: strips of the current t-tile
-        const float2 *zsrc = keep_z ? zrow : zsplit + pix0;
-        int occ_tt = -1;
-        for (int jj = tid; jj < N; jj += kRowThreads) {
-            if (keep_z) zrow[jj] = zsplit[pix0 + jj];
-            srow[jj] = first ? make_float4(0.f, 0.f, 0.f, 0.f) : acc[pix0 + jj];
-        }
-        __syncthreads();
-        for (int p = 0; p < nvalid; ++p) {
-            const float2 *plane = stack + (size_t)p * Np * Np;
-            const float t = (float)(plane0 + p + L.t_lo);
-            const int tt = (plane0 + p) / TT;
-            if (tt != occ_tt) {                  // uniform across the CTA; the previous plane ended with a barrier
-                for (int i = tid; i < L.ntu; i += kRowThreads) occ[i] = col_occ[tt * L.ntu + i];
-                __syncthreads();
-                occ_tt = tt;
-            }
-            // column strips no footprint touched were never transformed: they are zero
-            auto load = [&](int, int R) -> float2 {
-                return occ[R / TU] ? __ldcs(plane + tiled_index(ii, R, Np)) : make_float2(0.f, 0.f);
-            };
-            auto store = [&](int, int J, float2 v) {
-                if (!in_crop(J, half, Np)) return;
-                const int jj = grid_to_crop(J, half, Np);
-                float sn, cs;
-                phase_tz(t, zsrc[jj], &sn, &cs);
-                float4 a = srow[jj];
-                kahan_add(a.x, a.z, v.x * cs - v.y * sn);
-                kahan_add(a.y, a.w, v.x * sn + v.y * cs);
-                srow[jj] = a;
-            };
-            plane_fft<NP, 1>(sbuf, F, tw, true, tid, kRowThreads, load, store);
+        if constexpr (NP >= 512)
+            fft_static_inplace<NP, row_threads_max<NP>(), CROP ? fftst::PRUNE_OUT : 0>(row_buf(k), true, tid, store,
+                                                                                     rt, live);
+        else
+            fft_inplace(row_buf(k), F, tw, tid, T, store, live);
+        if (buffers == 1 && k + 1 < count) {
             __syncthreads();
+            if (warp == 0) issue(k + 1);
         }
-        for (int jj = tid; jj < N; jj += kRowThreads) {
-            const float4 a = srow[jj];
-            if (last) {
-                const float h = corr[pix0 + jj];
-                dirty[pix0 + jj] = make_float2(h * (a.x - a.z), L.fold ? 0.f : h * (a.y - a.w));
-            } else {
-                acc[pix0 + jj] = a;
+    }
+    __syncthreads();
+    if (shares == 1 || !last) {
+        if (gave_up) {
+            if (tid == 0) atomicAdd(timeouts, 1ull);
+            return;
+        }
+    }
+    if (!(last && shares == 1))
+        for (int jj = tid; jj < N; jj += T) own_acc[pix0 + jj] = srow[jj];
+    if (!last) return;
+    if (shares > 1) {
+        // the row's counter holds the finished shares and, above bit 16, those that
+        // gave up; the last one to finish leaves it zero for the next call
+        __threadfence();
+        __syncthreads();
+        if (tid == 0) {
+            const unsigned mine = gave_up ? 0x10001u : 1u, all = atomicAdd(&rows_done[ii], mine) + mine;
+            finisher = (all & 0xffffu) == (unsigned)shares ? 1 : 0;
+            if (finisher) {
+                rows_done[ii] = 0u;
+                if (all >> 16) {                 // an incomplete row counts once
+                    atomicAdd(timeouts, 1ull);
+                    finisher = 0;
+                }
             }
+            __threadfence();
         }
+        __syncthreads();
+        if (!finisher) return;
+    }
+    for (int jj = tid; jj < N; jj += T) {
+        float4 a = shares == 1 ? srow[jj] : __ldcg(acc + pix0 + jj);
+        float2 sum = make_float2(a.x, a.y), comp = make_float2(a.z, a.w);
+        for (int g = 1; g < shares; ++g) {
+            a = __ldcg(acc + g * image + pix0 + jj);
+            kahan_add(sum, comp, make_float2(a.x, a.y));
+            kahan_add(sum, comp, make_float2(-a.z, -a.w));
+        }
+        const float h = corr[pix0 + jj];
+        dirty[pix0 + jj] = make_float2(h * (sum.x - comp.x), L.fold ? 0.f : h * (sum.y - comp.y));
     }
 }
 
@@ -422,25 +449,12 @@ inline size_t smem_fwd_rows(const FftPlan &F, int N, bool step) {
 // CTAs per SM
 inline bool fwd_rows_step(const FftPlan &F, int N) { return smem_fwd_rows(F, N, true) <= kTwoCtaSmem; }
 // CTAs per image row in fwd_rows (each takes an equal share of the planes):
-// enough rows x groups for about 32 CTAs per SM over the launch, so the SMs
-// that finish first in the last round idle for a short CTA, not a long one
+// enough rows x groups for about 32 CTAs per SM over the launch,
+// so the SMs that finish first in the last round idle for a short CTA, not a long one
 inline int row_groups(int N, int planes, int sms) {
     const int want = (32 * sms + N - 1) / N;
     return want < 1 ? 1 : (want > planes ? (planes > 0 ? planes : 1) : want);
 }
-inline size_t smem_rows(const FftPlan &F, int N) {
-    return (size_t)F.stride * sizeof(float2) + (size_t)N * ((rows_keep_z(F, N) ? sizeof(float2) : 0) + sizeof(float4)) +
-           F.n / TU + 16;
-}
-// inv_rows: compile-time plans keep two aligned row buffers and two mbarriers
-template <int NP>
-inline size_t smem_inv_rows(const FftPlan &F, int N) {
-    if constexpr (NP >= 512)
-        return RowsSmem<NP>::bytes(N);
-    else
-        return smem_rows(F, N);
-}
-
 // Raise a kernel's dynamic shared-memory limit to the device's opt-in maximum
 // (after checking that this plan's need fits): kernels are shared by every
 // plan, so a limit set to one plan's need could be too low for another's.
@@ -455,75 +469,90 @@ cudaError_t allow_smem(K kernel, size_t bytes) {
 }
 
 // The stack as a 4-D FP32 tensor for TMA row copies: {8 floats of a column
-// block's row, N' rows, N'/4 blocks, P planes}, boxes of min(256, N'/4) blocks of one row.
+// block's row, N' rows, N'/4 blocks, P planes}, boxes of box_blocks (FftPlan) blocks of one row.
 cudaError_t row_tensor_map(const ws_plan_s *p, CUtensorMap *map);
 
 // Launchers of one FFT variant.
 template <int NP>
 struct Transforms {
-    static cudaError_t setup(const FftPlan &F, int N) {
+    static cudaError_t setup(const FftPlan &F, const FftPlan &inv, int N) {
         cudaError_t e;
         const bool step = fwd_rows_step(F, N);
         if ((e = allow_smem(fwd_rows_kernel<NP, false, false>, smem_fwd_rows(F, N, false))) != cudaSuccess) return e;
-        if ((e = allow_smem(fwd_rows_kernel<NP, false, true>, smem_fwd_rows(F, N, false))) != cudaSuccess) return e;
         if (step && (e = allow_smem(fwd_rows_kernel<NP, true, false>, smem_fwd_rows(F, N, true))) != cudaSuccess)
             return e;
-        if (step && (e = allow_smem(fwd_rows_kernel<NP, true, true>, smem_fwd_rows(F, N, true))) != cudaSuccess)
-            return e;
+        if constexpr (NP != 0) {
+            if ((e = allow_smem(fwd_rows_kernel<NP, false, true>, smem_fwd_rows(F, N, false))) != cudaSuccess) return e;
+            if (step && (e = allow_smem(fwd_rows_kernel<NP, true, true>, smem_fwd_rows(F, N, true))) != cudaSuccess)
+                return e;
+        }
         if ((e = allow_smem(fwd_cols_kernel<NP, false>, smem2(F))) != cudaSuccess) return e;
-        if ((e = allow_smem(fwd_cols_kernel<NP, true>, smem2(F))) != cudaSuccess) return e;
-        if ((e = allow_smem(inv_cols_kernel<NP, false>, smem2(F))) != cudaSuccess) return e;
-        if ((e = allow_smem(inv_cols_kernel<NP, true>, smem2(F))) != cudaSuccess) return e;
-        if ((e = allow_smem(inv_rows_kernel<NP, false>, smem_inv_rows<NP>(F, N))) != cudaSuccess) return e;
-        return allow_smem(inv_rows_kernel<NP, true>, smem_inv_rows<NP>(F, N));
+        if constexpr (NP != 0)
+            if ((e = allow_smem(fwd_cols_kernel<NP, true>, smem2(F))) != cudaSuccess) return e;
+        if ((e = allow_smem(inv_cols_kernel<NP, false>, smem2(inv))) != cudaSuccess) return e;
+        if constexpr (NP != 0)
+            if ((e = allow_smem(inv_cols_kernel<NP, true>, smem2(inv))) != cudaSuccess) return e;
+        if ((e = allow_smem(inv_rows_kernel<NP, false>, rows_smem(inv, N).bytes)) != cudaSuccess) return e;
+        if constexpr (NP != 0) e = allow_smem(inv_rows_kernel<NP, true>, rows_smem(inv, N).bytes);
+        return e;
     }
+    // Runs go(std::bool_constant): whether the crop is the centred half (compile-time plans only).
+    template <class Go>
+    static void with_crop(const Launch &L, Go go) {
+        if constexpr (NP != 0) {
+            if (crop_half<NP>(L)) {
+                go(std::true_type{});
+                return;
+            }
+        }
+        go(std::false_type{});
+    }
+    static int row_threads(const FftPlan &F) { return NP ? row_threads_max<NP>() : F.row_threads; }
+    static int col_threads(const FftPlan &F) { return NP ? col_threads_max<NP>() : F.col_threads; }
     static cudaError_t fwd_rows(const ws_plan_s *p, int chunk, int planes, cudaStream_t s) {
-        const bool step = fwd_rows_step(p->fft, p->L.N), crop = crop_half<NP>(p->L);
+        const bool step = fwd_rows_step(p->fft_fwd, p->L.N);
+        const int T = row_threads(p->fft_fwd);
         const dim3 grid(p->L.N, row_groups(p->L.N, planes, p->sms));
-        const size_t smem = smem_fwd_rows(p->fft, p->L.N, step);
+        const size_t smem = smem_fwd_rows(p->fft_fwd, p->L.N, step);
         auto go = [&](auto kernel) {
-            kernel<<<grid, kRowThreads, smem, s>>>(p->L, p->fft, p->d_tw, p->d_img, p->d_zsplit, p->d_col_occ,
-                                                   chunk * p->P, planes, p->d_stack);
+            kernel<<<grid, T, smem, s>>>(p->L, p->fft_fwd, p->d_tw, p->d_img, p->d_zsplit, p->d_col_occ, chunk * p->P,
+                                         planes, p->d_stack);
         };
-        if (step)
-            crop ? go(fwd_rows_kernel<NP, true, true>) : go(fwd_rows_kernel<NP, true, false>);
-        else
-            crop ? go(fwd_rows_kernel<NP, false, true>) : go(fwd_rows_kernel<NP, false, false>);
+        with_crop(p->L, [&](auto crop) {
+            constexpr bool C = decltype(crop)::value;
+            step ? go(fwd_rows_kernel<NP, true, C>) : go(fwd_rows_kernel<NP, false, C>);
+        });
         return cudaGetLastError();
     }
     static cudaError_t fwd_cols(const ws_plan_s *p, int chunk, int planes, cudaStream_t s) {
         const dim3 grid(p->L.Np / kPerCta, planes);
-        if (crop_half<NP>(p->L))
-            fwd_cols_kernel<NP, true><<<grid, kThreads, smem2(p->fft), s>>>(p->L, p->fft, p->d_tw, p->d_tile_occ,
-                                                                         p->d_col_occ, chunk * p->P, p->d_stack);
-        else
-            fwd_cols_kernel<NP, false><<<grid, kThreads, smem2(p->fft), s>>>(p->L, p->fft, p->d_tw, p->d_tile_occ,
-                                                                          p->d_col_occ, chunk * p->P, p->d_stack);
+        with_crop(p->L, [&](auto crop) {
+            fwd_cols_kernel<NP, decltype(crop)::value><<<grid, col_threads(p->fft_fwd), smem2(p->fft_fwd), s>>>(
+                p->L, p->fft_fwd, p->d_tw, p->d_tile_occ, p->d_col_occ, chunk * p->P, p->d_stack);
+        });
         return cudaGetLastError();
     }
     static cudaError_t inv_cols(const ws_plan_s *p, int chunk, int planes, cudaStream_t s) {
         const dim3 grid(p->L.Np / kPerCta, planes);
-        if (crop_half<NP>(p->L))
-            inv_cols_kernel<NP, true><<<grid, kThreads, smem2(p->fft), s>>>(p->L, p->fft, p->d_tw, p->d_tile_occ,
-                                                                         p->d_col_occ, chunk * p->P, p->d_stack);
-        else
-            inv_cols_kernel<NP, false><<<grid, kThreads, smem2(p->fft), s>>>(p->L, p->fft, p->d_tw, p->d_tile_occ,
-                                                                          p->d_col_occ, chunk * p->P, p->d_stack);
+        with_crop(p->L, [&](auto crop) {
+            inv_cols_kernel<NP, decltype(crop)::value><<<grid, col_threads(p->fft_inv), smem2(p->fft_inv), s>>>(
+                p->L, p->fft_inv, p->d_tw, p->d_tile_occ, p->d_col_occ, chunk * p->P, p->d_stack);
+        });
         return cudaGetLastError();
     }
     static cudaError_t inv_rows(const ws_plan_s *p, int chunk, int planes, bool first, bool last, float2 *dirty,
                                 cudaStream_t s) {
         CUtensorMap map{};
-        if constexpr (NP >= 512) {
-            const cudaError_t e = row_tensor_map(p, &map);
-            if (e != cudaSuccess) return e;
-        }
-        auto go = [&](auto kernel) {
-            kernel<<<p->L.N, kRowThreads, smem_inv_rows<NP>(p->fft, p->L.N), s>>>(
-                p->L, p->fft, p->d_tw, p->d_stack, map, p->d_col_occ, chunk * p->P, planes, p->d_zsplit, p->d_corr,
-                p->d_acc, first ? 1 : 0, last ? 1 : 0, dirty, p->d_drop + 2, p->wait_polls);
-        };
-        crop_half<NP>(p->L) ? go(inv_rows_kernel<NP, true>) : go(inv_rows_kernel<NP, false>);
+        const cudaError_t e = row_tensor_map(p, &map);
+        if (e != cudaSuccess) return e;
+        const RowsSmem sm = rows_smem(p->fft_inv, p->L.N);
+        with_crop(p->L, [&](auto crop) {
+            inv_rows_kernel<NP, decltype(crop)::value>
+                <<<dim3(p->L.N, p->row_shares), row_threads(p->fft_inv), sm.bytes, s>>>(
+                    p->L, p->fft_inv, p->d_tw, map, p->d_col_occ, chunk * p->P, planes, sm.buffers, sm.keep_z,
+                    (int)(sm.buf / sizeof(float2)), p->d_zsplit, p->d_corr, p->d_acc, p->d_rows_done, first ? 1 : 0,
+                    last ? 1 : 0, dirty, p->d_drop + 2, p->wait_polls);
+        });
         return cudaGetLastError();
     }
 };
@@ -531,7 +560,7 @@ struct Transforms {
 // Entry points of one variant, exported by the translation unit that
 // instantiates it (so every kernel is compiled exactly once).
 struct Ops {
-    cudaError_t (*setup)(const FftPlan &, int);
+    cudaError_t (*setup)(const FftPlan &, const FftPlan &, int);
     cudaError_t (*fwd_rows)(const ws_plan_s *, int, int, cudaStream_t);
     cudaError_t (*fwd_cols)(const ws_plan_s *, int, int, cudaStream_t);
     cudaError_t (*inv_cols)(const ws_plan_s *, int, int, cudaStream_t);
@@ -544,8 +573,7 @@ constexpr Ops ops_of() {
                &Transforms<NP>::inv_cols, &Transforms<NP>::inv_rows};
 }
 
-const Ops &ops_runtime_pow2();
-const Ops &ops_runtime_mixed();
+const Ops &ops_runtime();
 const Ops &ops_512();
 const Ops &ops_1024();
 const Ops &ops_2048();

@@ -129,8 +129,7 @@ struct ws_plan_s {
     int P = 0;                     // planes per chunk (multiple of TT)
     float2 *d_stack = nullptr;     // P x N' x N', column-block layout (common.cuh)
     float2 *d_tw = nullptr;        // N' twiddles exp(-2 pi i m / N')
-    ws::FftPlan fft{};             // the N'-point plane transform
-    bool fft_mixed = false;        // N' has a factor 3, 5 or 7
+    ws::FftPlan fft_fwd{}, fft_inv{};   // the N'-point plane transforms
     // per-call buffers (grow on demand)
     ws::VisRec *d_rec = nullptr;
     int64_t rec_cap = 0;
@@ -142,7 +141,9 @@ struct ws_plan_s {
     int64_t ntiles = 0;
     uint8_t *d_tile_occ = nullptr; // ntiles: 1 if any visibility footprint touches the tile
     uint8_t *d_col_occ = nullptr;  // ntt x ntu: 1 if any tile of that (t-tile, u-tile) strip is touched
-    float4 *d_acc = nullptr;       // N x N: (sum re, sum im, comp re, comp im)
+    int row_shares = 1;            // shares of the planes per image row in inv_rows (transforms.cu)
+    float4 *d_acc = nullptr;       // row_shares x N x N: (sum re, sum im, comp re, comp im)
+    unsigned *d_rows_done = nullptr;   // N: shares of the row that are done, zero between calls
     float2 *d_img = nullptr;       // N x N: corrected image (degridding)
     unsigned long long *d_drop = nullptr;   // kCounters: [0] non-finite uv, [1] w out of range, [2] timed-out waits
     unsigned long long *h_drop = nullptr;   // pinned mirror
@@ -242,8 +243,9 @@ cudaError_t launch_degrid_chunk(const ws_plan_s *p, int chunk, int planes, int64
                                 float2 *vis, cudaStream_t s);
 
 // Plane transforms (transforms.cu).
-size_t transform_smem_bytes(const FftPlan &F, int N);
-cudaError_t setup_transform_kernels(const FftPlan &F, int N);
+size_t transform_smem_bytes(const FftPlan &fwd, const FftPlan &inv, int N);
+int inv_row_shares(const FftPlan &F, int N, int planes, int sms);
+cudaError_t setup_transform_kernels(const FftPlan &fwd, const FftPlan &inv, int N);
 cudaError_t launch_fwd_rows(const ws_plan_s *p, int chunk, int planes, cudaStream_t s);
 cudaError_t launch_fwd_cols(const ws_plan_s *p, int chunk, int planes, cudaStream_t s);
 cudaError_t launch_inv_cols(const ws_plan_s *p, int chunk, int planes, cudaStream_t s);
