@@ -306,11 +306,6 @@ __device__ __forceinline__ void twiddle_powers(float2 *v, float2 w1, float2 w4) 
         }
     }
 }
-template <int R>
-__device__ __forceinline__ void twiddle_all(float2 *v, const float2 *__restrict__ tw, int e, bool inv) {
-    twiddle_powers<R>(v, twiddle(tw, e, inv), R >= 8 ? twiddle(tw, 4 * e, inv) : make_float2(1.f, 0.f));
-}
-
 // x / d for 0 <= x < 2^16, 1 <= d < 2^13, with mul = div_mul(d) (fft_plan.hpp)
 __device__ __forceinline__ int div_small(int x, unsigned mul) {
     return mul ? (int)__umulhi((unsigned)x, mul) : x;
@@ -325,30 +320,82 @@ __device__ __forceinline__ int div_small(int x, unsigned mul) {
 //
 // A butterfly's slots are one base plus multiples of P.step[s] (FftPlan), so the
 // slot arithmetic costs once per butterfly.
+//
+// The barrier that completes the previous stage comes after the first round's
+// twiddles have been asked for, and each round asks for the next one's: the table
+// mostly comes from L2 (the buffers leave little L1), and a stage that waited for
+// it after the barrier spent a third of its time there.
 template <int R, int COUNT, bool LAST, class Store>
 __device__ __forceinline__ void dit_stage(float2 *buf, const FftPlan &P, int s, const float2 *__restrict__ tw,
                                           bool inv, int tid, int nthr, Store &store) {
     const int L = P.L[s], total = COUNT * P.nb[s], twstep = P.twstep[s];
     const int step = P.step[s];
+    float2 w1, w4;
+    int base = 0, k = 0;
+    auto fetch = [&](int q) {                // butterfly q's first position and twiddles (q past the end: the last one's)
+        const int bq = min(q, total - 1) / COUNT;
+        const int blk = LAST ? 0 : div_small(bq, P.L_mul[s]);
+        k = bq - blk * L;
+        base = blk * R * L + k;
+        w1 = twiddle(tw, k * twstep, inv);
+        w4 = R >= 8 ? twiddle(tw, 4 * k * twstep, inv) : make_float2(1.f, 0.f);
+    };
+    fetch(tid);
+    __syncthreads();
     for (int q = tid; q < total; q += nthr) {
-        const int t = q % COUNT, bq = q / COUNT;
-        const int blk = LAST ? 0 : div_small(bq, P.L_mul[s]), k = bq - blk * L;
-        const int base = blk * R * L + k;
-        float2 *x = buf + t * P.stride + base + div_small(base, P.chunk_mul);
+        const int t = q % COUNT, b = base, kq = k;
+        const float2 v1 = w1, v4 = w4;
+        float2 *x = buf + t * P.stride + b + div_small(b, P.chunk_mul);
         float2 v[R];
 #pragma unroll
         for (int m = 0; m < R; ++m) v[m] = x[m * step];
-        if (k > 0) twiddle_all<R>(v, tw, k * twstep, inv);
+        fetch(q + nthr);
+        if (kq > 0) twiddle_powers<R>(v, v1, v4);
         dft<R>(v, inv);
         if constexpr (LAST) {
 #pragma unroll
-            for (int m = 0; m < R; ++m) store(t, base + m * L, v[m]);
+            for (int m = 0; m < R; ++m) store(t, b + m * L, v[m]);
         } else {
 #pragma unroll
             for (int m = 0; m < R; ++m) x[m * step] = v[m];
         }
     }
-    if constexpr (!LAST) __syncthreads();
+}
+
+// The last stage of one transform, its inputs all read before between() runs
+// (the buffer is free from then on): up to ROUNDS butterflies a thread in
+// registers, R ROUNDS <= 32.
+template <int R, class Between, class Store>
+__device__ __forceinline__ void dit_last_held(float2 *buf, const FftPlan &P, const float2 *__restrict__ tw, bool inv,
+                                              int tid, int nthr, Between &between, Store &store) {
+    constexpr int ROUNDS = 32 / R;
+    const int s = P.nstages - 1, L = P.L[s], nb = P.nb[s], step = P.step[s];
+    float2 v[ROUNDS][R], w1[ROUNDS], w4[ROUNDS];
+#pragma unroll
+    for (int i = 0; i < ROUNDS; ++i) {
+        const int e = min(tid + i * nthr, nb - 1) * P.twstep[s];
+        w1[i] = twiddle(tw, e, inv);
+        w4[i] = R >= 8 ? twiddle(tw, 4 * e, inv) : make_float2(1.f, 0.f);
+    }
+    __syncthreads();
+#pragma unroll
+    for (int i = 0; i < ROUNDS; ++i) {
+        const int k = min(tid + i * nthr, nb - 1);
+        const float2 *x = buf + k + div_small(k, P.chunk_mul);
+#pragma unroll
+        for (int m = 0; m < R; ++m) v[i][m] = x[m * step];
+    }
+    __syncthreads();
+    between();
+#pragma unroll
+    for (int i = 0; i < ROUNDS; ++i) {
+        const int k = tid + i * nthr;
+        if (k >= nb) break;
+        if (k > 0) twiddle_powers<R>(v[i], w1[i], w4[i]);
+        dft<R>(v[i], inv);
+#pragma unroll
+        for (int m = 0; m < R; ++m) store(0, k + m * L, v[i][m]);
+    }
 }
 
 // The slot where butterfly j of the first stage puts its R outputs: that of
@@ -379,7 +426,6 @@ __device__ __forceinline__ void dit_first(float2 *buf, const FftPlan &P, bool in
 #pragma unroll
         for (int m = 0; m < R; ++m) x[m] = v[m];
     }
-    __syncthreads();
 }
 
 // First stage of one transform whose input sits in the buffer in natural order
@@ -403,7 +449,6 @@ __device__ __forceinline__ void dit_first_inplace(float2 *buf, const FftPlan &P,
 #pragma unroll
         for (int m = 0; m < R; ++m) x[m] = v[m];
     }
-    __syncthreads();
 }
 
 // Calls f(Radix<r>) for the first or a later radix of a forward plan, and for the
@@ -474,28 +519,32 @@ __device__ __forceinline__ void with_last_radix(int r, F f) {
 // (t < COUNT), using the shared buffers buf + t * P.stride between stages.
 // All threads of the CTA must call it; shared buffers may be reused after the
 // caller's next barrier.
-template <int COUNT, bool INV, class Store>
-__device__ __forceinline__ void fft_later_stages(float2 *buf, const FftPlan &P, const float2 *__restrict__ tw,
-                                                 int tid, int nthr, Store &store) {
-    const int last = P.nstages - 1;
-    auto middle = [&](int s) {
-        return [&, s](auto r) {
-            fftdev::dit_stage<decltype(r)::value, COUNT, false>(buf, P, s, tw, INV, tid, nthr, store);
+template <int COUNT, bool INV>
+__device__ __forceinline__ void fft_middle_stages(float2 *buf, const FftPlan &P, const float2 *__restrict__ tw, int tid,
+                                                  int nthr) {
+    auto none = [](int, int, float2) {};
+    for (int s = 1; s < P.nstages - 1; ++s) {
+        auto stage = [&](auto r) {
+            fftdev::dit_stage<decltype(r)::value, COUNT, false>(buf, P, s, tw, INV, tid, nthr, none);
         };
-    };
-    auto final = [&](auto r) {
+        if constexpr (INV)
+            fftdev::with_middle_radix(P.radix[s], stage);
+        else
+            fftdev::with_forward_later(P.radix[s], stage);
+    }
+}
+
+template <int COUNT, bool INV, class Store>
+__device__ __forceinline__ void fft_last_stage(float2 *buf, const FftPlan &P, const float2 *__restrict__ tw, int tid,
+                                               int nthr, Store &store) {
+    const int last = P.nstages - 1;
+    auto stage = [&](auto r) {
         fftdev::dit_stage<decltype(r)::value, COUNT, true>(buf, P, last, tw, INV, tid, nthr, store);
     };
-    for (int s = 1; s < last; ++s) {
-        if constexpr (INV)
-            fftdev::with_middle_radix(P.radix[s], middle(s));
-        else
-            fftdev::with_forward_later(P.radix[s], middle(s));
-    }
     if constexpr (INV)
-        fftdev::with_last_radix(P.radix[last], final);
+        fftdev::with_last_radix(P.radix[last], stage);
     else
-        fftdev::with_forward_later(P.radix[last], final);
+        fftdev::with_forward_later(P.radix[last], stage);
 }
 
 template <int COUNT, bool INV, class Load, class Store>
@@ -508,17 +557,26 @@ __device__ __forceinline__ void fft_many(float2 *buf, const FftPlan &P, const fl
         fftdev::with_first_radix(P.radix[0], first);
     else
         fftdev::with_forward_first(P.radix[0], first);
-    fft_later_stages<COUNT, INV>(buf, P, tw, tid, nthr, store);
+    fft_middle_stages<COUNT, INV>(buf, P, tw, tid, nthr);
+    fft_last_stage<COUNT, INV>(buf, P, tw, tid, nthr, store);
 }
 
-// One inverse transform whose input sits in buf in natural order (see dit_first_inplace).
-template <class Store>
+// One inverse transform whose input sits in buf in natural order (see
+// dit_first_inplace).  HELD: between() runs once the buffer's last contents are
+// read (the plan's last stage has at most 32 / radix rounds).
+template <bool HELD, class Between, class Store>
 __device__ __forceinline__ void fft_inplace(float2 *buf, const FftPlan &P, const float2 *__restrict__ tw, int tid,
-                                            int nthr, Store store, uint32_t live) {
+                                            int nthr, Between between, Store store, uint32_t live) {
     fftdev::with_first_radix(P.radix[0], [&](auto r) {
         fftdev::dit_first_inplace<decltype(r)::value>(buf, P, true, tid, live);
     });
-    fft_later_stages<1, true>(buf, P, tw, tid, nthr, store);
+    fft_middle_stages<1, true>(buf, P, tw, tid, nthr);
+    if constexpr (HELD)
+        fftdev::with_last_radix(P.radix[P.nstages - 1], [&](auto r) {
+            fftdev::dit_last_held<decltype(r)::value>(buf, P, tw, true, tid, nthr, between, store);
+        });
+    else
+        fft_last_stage<1, true>(buf, P, tw, tid, nthr, store);
 }
 
 // -- compile-time plans for the power-of-two sizes -----------------------------
@@ -577,7 +635,6 @@ __device__ __forceinline__ void first(float2 *buf, bool inv, int tid, Load &load
 #pragma unroll
         for (int m = 0; m < R; ++m) x[m] = v[m];
     }
-    __syncthreads();
 }
 
 // Twiddle bases w, w^4 of the butterflies a thread owns in a later stage of one
@@ -624,6 +681,16 @@ __device__ __forceinline__ void later(float2 *buf, const float2 *__restrict__ tw
     auto at = [&](int pbase, int base, int m) {
         return affine ? pbase + m * step : Ly::pad(base + m * L);
     };
+    // the previous stage is complete after the barrier; twiddles that are not kept
+    // are asked for before it, the next round's ahead of this one's arithmetic
+    float2 w1, w4;
+    auto fetch = [&](int i) {
+        const int e = ((min(tid + i * T, total - 1) / COUNT) & (L - 1)) << lgtw;
+        w1 = fftdev::twiddle(tw, e, inv);
+        w4 = R >= 8 ? fftdev::twiddle(tw, 4 * e, inv) : make_float2(1.f, 0.f);
+    };
+    if constexpr (!kept_tw) fetch(0);
+    __syncthreads();
 #pragma unroll(kept_tw ? rounds : 1)
     for (int i = 0; i < rounds; ++i) {
         const int q = tid + i * T;
@@ -633,15 +700,18 @@ __device__ __forceinline__ void later(float2 *buf, const float2 *__restrict__ tw
         const int base = blk * R * L + k;
         const int pbase = wide ? Ly::pad(base) : base + ((blk * R * L) >> Ly::shift);
         float2 *x = buf + t * Ly::stride;
-        float2 v[R];
+        float2 v[R], v1, v4;
 #pragma unroll
         for (int m = 0; m < R; ++m) v[m] = x[at(pbase, base, m)];
-        if (k > 0) {
-            if constexpr (kept_tw)
-                fftdev::twiddle_powers<R>(v, pre.w1[Pre::kept == 1 ? 0 : i], pre.w4[Pre::kept == 1 ? 0 : i]);
-            else
-                fftdev::twiddle_all<R>(v, tw, k << lgtw, inv);
+        if constexpr (kept_tw) {
+            v1 = pre.w1[Pre::kept == 1 ? 0 : i];
+            v4 = pre.w4[Pre::kept == 1 ? 0 : i];
+        } else {
+            v1 = w1;
+            v4 = w4;
+            if (i + 1 < rounds) fetch(i + 1);
         }
+        if (k > 0) fftdev::twiddle_powers<R>(v, v1, v4);
         fftdev::dft<R>(v, inv);
         if constexpr (LAST) {
 #pragma unroll
@@ -652,7 +722,35 @@ __device__ __forceinline__ void later(float2 *buf, const float2 *__restrict__ tw
             for (int m = 0; m < R; ++m) x[at(pbase, base, m)] = v[m];
         }
     }
-    if constexpr (!LAST) __syncthreads();
+}
+
+// The last stage of one transform with all its inputs read before between() runs
+// (the buffer is free from then on).
+template <int N, int T, int R, int L, int PRUNE, class Pre, class Between, class Store>
+__device__ __forceinline__ void last_held(float2 *buf, int tid, bool inv, const Pre &pre, Between &between,
+                                          Store &store) {
+    constexpr bool pout = (PRUNE & PRUNE_OUT) != 0;
+    using Ly = Layout<N>;
+    constexpr int rounds = N / R / T;
+    static_assert(R * L == N && rounds * T * R == N && (L >> Ly::shift) > 0, "a last stage in whole rounds");
+    constexpr int step = L + (L >> Ly::shift);
+    float2 v[rounds][R];
+    __syncthreads();
+#pragma unroll
+    for (int i = 0; i < rounds; ++i)
+#pragma unroll
+        for (int m = 0; m < R; ++m) v[i][m] = buf[Ly::pad(tid + i * T) + m * step];
+    __syncthreads();
+    between();
+#pragma unroll
+    for (int i = 0; i < rounds; ++i) {
+        const int k = tid + i * T;
+        if (k > 0) fftdev::twiddle_powers<R>(v[i], pre.w1[Pre::kept == 1 ? 0 : i], pre.w4[Pre::kept == 1 ? 0 : i]);
+        fftdev::dft<R>(v[i], inv);
+#pragma unroll
+        for (int m = 0; m < R; ++m)
+            if (!pout || m < R / 4 || m >= 3 * R / 4) store(0, k + m * L, v[i][m]);
+    }
 }
 
 // First stage for inputs already in the buffer, in natural order at 0..N-1
@@ -676,7 +774,6 @@ __device__ __forceinline__ void first_inplace(float2 *buf, bool inv, int tid, ui
     float2 *x = buf + Ly::pad((d1 + d2 * Rd::r1) * R);
 #pragma unroll
     for (int m = 0; m < R; ++m) x[m] = v[m];
-    __syncthreads();
 }
 
 // Twiddle bases of both later stages of one transform by T threads.
@@ -694,16 +791,19 @@ struct RowTw {
 }  // namespace fftst
 
 // One transform of the compile-time size N by T threads: input in buf in
-// natural order (see first_inplace for live), or read through load.
-template <int N, int T, int PRUNE = 0, class Store>
-__device__ __forceinline__ void fft_static_inplace(float2 *buf, bool inv, int tid, Store store,
+// natural order (see first_inplace for live; HELD as in fft_inplace), or read through load.
+template <int N, int T, bool HELD, int PRUNE = 0, class Between, class Store>
+__device__ __forceinline__ void fft_static_inplace(float2 *buf, bool inv, int tid, Between between, Store store,
                                                    const fftst::RowTw<N, T> &rt, uint32_t live) {
     using Rd = fftst::Radices<N>;
     static_assert((PRUNE & fftst::PRUNE_IN) == 0, "inputs already in the buffer are not pruned");
     static_assert(T == N / Rd::r0, "one first-stage butterfly per thread");
     fftst::first_inplace<N>(buf, inv, tid, live);
     fftst::later<N, 1, T, Rd::r1, Rd::r0, false, 0>(buf, nullptr, inv, tid, rt.s2, store);
-    fftst::later<N, 1, T, Rd::r2, Rd::r0 * Rd::r1, true, PRUNE>(buf, nullptr, inv, tid, rt.s3, store);
+    if constexpr (HELD)
+        fftst::last_held<N, T, Rd::r2, Rd::r0 * Rd::r1, PRUNE>(buf, tid, inv, rt.s3, between, store);
+    else
+        fftst::later<N, 1, T, Rd::r2, Rd::r0 * Rd::r1, true, PRUNE>(buf, nullptr, inv, tid, rt.s3, store);
 }
 template <int N, int T, int PRUNE = 0, class Load, class Store>
 __device__ __forceinline__ void fft_static_row(float2 *buf, bool inv, int tid, Load load, Store store,

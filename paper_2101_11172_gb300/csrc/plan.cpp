@@ -233,12 +233,42 @@ int forward_radices(int n, int *radix) {
     return m == 1 ? ns : 0;
 }
 
-// Radices of an N'-point inverse transform, largest first: those of the least
-// total cost among the factorizations into radices that fft.cuh has, whose
-// first stage needs no more than kMaxFftThreads butterflies (a thread then owns
-// one, as the in-place first stage requires).  Three stages for nearly every
-// N', e.g. 2016 = 14 12 12 and 5600 = 28 20 10, where factors of 16, 8, 7, 5 and
-// 3 alone take four or five, each with its trip through shared memory.
+// Time of the stages of `count` transforms by CTAs of t threads, in relative
+// units: the rounds of every stage, over the CTAs an SM holds (512 threads of
+// 128 registers, and what shared memory allows).  A CTA of 192 threads, for
+// instance, is a poor fit: two of them leave a quarter of the registers idle.
+double stage_time(const int *radix, int ns, int n, int count, size_t smem, int t) {
+    double w = 0.0;
+    for (int s = 0; s < ns; ++s) w += (double)((count * (n / radix[s]) + t - 1) / t) * butterfly_cost(radix[s]);
+    return w / (double)std::max<size_t>(1, std::min<size_t>(512 / t, 228 * 1024 / (smem + 1024)));
+}
+
+// The CTA size with the least stage_time, at least lo threads.
+int best_threads(const int *radix, int ns, int n, int count, size_t smem, int lo, double *time) {
+    int t_best = 0;
+    double w_best = 0.0;
+    for (int t = std::max(32, (lo + 31) / 32 * 32); t <= kMaxFftThreads; t += 32) {
+        const double w = stage_time(radix, ns, n, count, smem, t);
+        if (t_best == 0 || w < w_best) {
+            t_best = t;
+            w_best = w;
+        }
+    }
+    if (time) *time = w_best;
+    return t_best;
+}
+
+// Shared memory of a row's CTA for an image of N'/2: the transform's buffer and
+// four more values per pixel; inverse, two buffers and three values.
+size_t row_smem(int n, bool inverse) { return inverse ? 28 * (size_t)n : 24 * (size_t)n; }
+
+// Radices of an N'-point inverse transform, largest first: the factorization
+// into radices that fft.cuh has, with a first stage of at most kMaxFftThreads
+// butterflies (a thread then owns one, as the in-place first stage requires),
+// that takes a row the least time with the CTA size that suits it best.  Three
+// stages for nearly every N', e.g. 2016 = 21 16 6 and 5600 = 28 20 10, where
+// factors of 16, 8, 7, 5 and 3 alone take four or five, each with its trip
+// through shared memory.
 int inverse_radices(int n, int *best) {
     // what the kernels have as a first, middle and last radix
     auto first = [](int r) { return r == 28 || r == 24 || r == 20 || r == 16 || r == 14 || r == 12 || r == 10 || r == 8; };
@@ -246,26 +276,27 @@ int inverse_radices(int n, int *best) {
     auto last = [](int r) { return r == 16 || r == 14 || r == 12 || r == 10 || r == 8 || r == 7 || r == 6 || r == 4; };
     const int radices[] = {28, 24, 21, 20, 16, 14, 12, 10, 8, 7, 6, 4};
     int cur[kMaxFftStages] = {}, nbest = 0;
-    double best_cost = 0.0;
-    auto search = [&](auto &&self, int rest, int depth, int from, double cost) -> void {
+    double best_time = 0.0;
+    auto search = [&](auto &&self, int rest, int depth) -> void {
         if (rest == 1) {
-            if (depth >= 2 && (nbest == 0 || cost < best_cost)) {
-                best_cost = cost;
+            double time = 0.0;
+            best_threads(cur, depth, n, 1, row_smem(n, true), n / cur[0], &time);
+            if (depth >= 2 && (nbest == 0 || time < best_time)) {
+                best_time = time;
                 nbest = depth;
                 std::copy(cur, cur + depth, best);
             }
             return;
         }
         if (depth == kMaxFftStages) return;
-        for (int i = from; i < (int)(sizeof(radices) / sizeof(radices[0])); ++i) {
-            const int r = radices[i];
-            if (rest % r || (depth == 0 && (!first(r) || n / r > kMaxFftThreads))) continue;
-            if (depth > 0 && !(rest == r ? last(r) : middle(r))) continue;
+        for (int r : radices) {
+            if (rest % r || (depth == 0 ? !first(r) || n / r > kMaxFftThreads : !(rest == r ? last(r) : middle(r))))
+                continue;
             cur[depth] = r;
-            self(self, rest / r, depth + 1, i, cost + (double)(n / r) * butterfly_cost(r));
+            self(self, rest / r, depth + 1);
         }
     };
-    search(search, n, 0, 0, 0.0);
+    search(search, n, 0);
     return nbest;
 }
 
@@ -342,22 +373,8 @@ bool fft_make_plan(int n, bool inverse, FftPlan *F) {
     for (int s = 0; s < ns; ++s) F->step[s] = F->L[s] >= chunk ? F->L[s] + F->L[s] / chunk : F->L[s];
     // the compile-time plans of fft.cuh pad at most 17 slots
     F->stride = stride_of(std::max(n + n / chunk, n + 17));
-    // threads per CTA for `count` transforms: the rounds of every stage, weighted by the idle threads
-    auto threads = [&](int count, int lo) {
-        int t_best = 0;
-        double w_best = 0.0;
-        for (int t = std::max(32, (lo + 31) / 32 * 32); t <= kMaxFftThreads; t += 32) {
-            double w = 0.0;
-            for (int s = 0; s < ns; ++s) w += (double)((count * F->nb[s] + t - 1) / t) * butterfly_cost(radix[s]) * t;
-            if (t_best == 0 || w < 0.98 * w_best) {
-                t_best = t;
-                w_best = w;
-            }
-        }
-        return t_best;
-    };
-    F->row_threads = threads(1, std::min(256, inverse ? F->nb[0] : n / 16));
-    F->col_threads = threads(2, std::min(256, n / 8));
+    F->row_threads = best_threads(radix, ns, n, 1, row_smem(n, inverse), inverse ? F->nb[0] : 32, nullptr);
+    F->col_threads = best_threads(radix, ns, n, 2, 16 * (size_t)n, 32, nullptr);
     // boxes of at most 256 column blocks whose size keeps shared-memory addresses 128-byte aligned
     const int blocks = n / 4;
     F->boxes = (blocks + 255) / 256;

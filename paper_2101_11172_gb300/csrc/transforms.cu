@@ -83,7 +83,7 @@ const tf::Ops &ops_for(int Np) {
 
 // Largest dynamic shared memory any transform kernel of this plan asks for.
 size_t transform_smem_bytes(const FftPlan &fwd, const FftPlan &inv, int N) {
-    return std::max({tf::smem2(fwd), tf::smem2(inv), tf::rows_smem(inv, N).bytes, tf::smem_fwd_rows(fwd, N, false)});
+    return std::max({tf::smem2(fwd), tf::smem2(inv), tf::rows_smem(inv, N).bytes, tf::smem_fwd_rows(fwd, N, tf::fwd_rows_keep(fwd, N))});
 }
 
 // Shares of the planes each image row is given in inv_rows.  The CTAs that fit
@@ -91,10 +91,8 @@ size_t transform_smem_bytes(const FftPlan &fwd, const FftPlan &inv, int N) {
 // (partly empty) costs little; a share keeps at least eight planes, or two while
 // the rows alone leave part of the GPU idle.
 int inv_row_shares(const FftPlan &F, int N, int planes, int sms) {
-    const bool fixed = F.n == 512 || F.n == 1024 || F.n == 2048 || F.n == 4096;
-    const int T = fixed ? F.n / 16 : F.row_threads;
     const int by_smem = (int)(228 * 1024 / (tf::rows_smem(F, N).bytes + 1024));
-    const int64_t slots = (int64_t)sms * std::max(1, std::min(by_smem, 512 / T));
+    const int64_t slots = (int64_t)sms * std::max(1, std::min(by_smem, tf::row_cta_limit(F)));
     const int want = (int)((8 * slots + N - 1) / N), fill = (int)((slots + N - 1) / N);
     return std::max(1, std::min(want, std::max(planes / 8, std::min(fill, planes / 2))));
 }

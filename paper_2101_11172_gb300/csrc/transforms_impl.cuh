@@ -18,12 +18,17 @@ namespace ws {
 namespace tf {
 
 constexpr int kPerCta = 2;          // columns per CTA of the column kernels
+// Whether N' has a compile-time plan.
+inline bool compile_time_size(int Np) { return Np == 512 || Np == 1024 || Np == 2048 || Np == 4096; }
 // CTA sizes follow the transform: N'/16 threads for a row and twice that for a
 // pair of columns, one radix-16 butterfly per thread in a stage (two at N' =
 // 4096 for the columns).  With 256 threads at every size most of a CTA idled on
 // short rows (N' = 512: 32 butterflies in the first stage).  Runtime plans
 // bring their own (FftPlan::row_threads, col_threads).  The minimum of resident
-// CTAs bounds the registers: 128 a thread for rows, 80 for columns.
+// CTAs bounds the registers: 128 a thread for rows and runtime plans, 80 for columns.
+// (Rows at 80 registers and three CTAs of 256 threads per SM, with one row buffer
+// and z read from global memory to fit, were slower: inv_rows 13.6 against 9.5 ms and
+// fwd_rows 9.2 against 8.6 on 366 planes of N' = 4096.)
 template <int NP>
 WS_HD constexpr int row_threads_max() {
     return NP ? NP / 16 : kMaxFftThreads;
@@ -40,8 +45,11 @@ template <int NP>
 WS_HD constexpr int col_ctas() {
     return NP ? 768 / col_threads_max<NP>() : 2;
 }
-// Shared memory per CTA that still lets two CTAs share an SM (228 KB, 1 KB of it reserved per CTA).
-constexpr size_t kTwoCtaSmem = 113 * 1024;
+// Row CTAs that an SM can hold by threads and registers, and the shared memory
+// that each may have for `ctas` of them to fit (228 KB per SM, 1 KB of it reserved per CTA).
+inline int row_threads_of(const FftPlan &F) { return compile_time_size(F.n) ? F.n / 16 : F.row_threads; }
+inline int row_cta_limit(const FftPlan &F) { return 512 / row_threads_of(F); }
+inline size_t cta_smem(int ctas) { return (size_t)228 * 1024 / ctas - 1024; }
 
 __device__ __forceinline__ int grid_to_crop(int g, int half, int Np) { return g < half ? g + half : g - (Np - half); }
 __device__ __forceinline__ bool in_crop(int g, int half, int Np) { return g < half || g >= Np - half; }
@@ -82,44 +90,46 @@ inline bool crop_half(const Launch &L) { return NP >= 512 && 2 * L.N == L.Np; }
 // pixel's screened value advances one plane by a product with exp(-2 pi i z).
 constexpr int kScreenSteps = 8;
 
-// One CTA owns image row ii for a run of planes: the corrected row and its z
-// stay in shared memory, so each plane costs the screen, one FFT and the
-// stores of the strips some footprint reads.
-//
-// STEP keeps two more shared rows, the screened row g = row x exp(-2 pi i t z)
-// and the step exp(-2 pi i z).  g is evaluated exactly on every kScreenSteps-th
-// plane of the CTA's share; on the planes between, the FFT's first stage reads
-// g and leaves g x step in its place for the next plane.  Each pixel is read
-// by the same thread on every plane, so the update needs no barrier.
-template <int NP, bool STEP, bool CROP>
+// One CTA owns image row ii for a run of planes.  Shared memory keeps the
+// screened row g = row x exp(-2 pi i t z) and the step exp(-2 pi i z), so each
+// plane costs the step, one FFT and the stores of the strips some footprint
+// reads.  g is evaluated exactly on every kScreenSteps-th plane of the CTA's
+// share; on the planes between, the FFT's first stage reads g and leaves g x step
+// in its place for the next plane.  Each pixel is read by the same thread on
+// every plane, so the update needs no barrier.  The exact evaluations read the
+// corrected row and its z from shared memory too (keep_rows), or, where that
+// would leave one CTA per SM, from global memory (N = 4096: evaluating the
+// screen exactly on every plane instead cost 12 % of the kernel there).
+template <int NP, bool CROP>
 __global__ void __launch_bounds__(row_threads_max<NP>(), row_ctas<NP>())
 fwd_rows_kernel(Launch L, FftPlan F, const float2 *__restrict__ tw, const float2 *__restrict__ img,
                 const float2 *__restrict__ zsplit, const uint8_t *__restrict__ col_occ, int plane0, int planes,
-                float2 *__restrict__ stack) {
+                int keep_rows, float2 *__restrict__ stack) {
     extern __shared__ __align__(16) float2 sbuf[];
     const int Np = L.Np, N = L.N, half = N / 2;
-    float2 *irow = sbuf + F.stride;                              // N (F.stride is even: 16-byte aligned)
-    float2 *zrow = irow + N;                                     // N
-    float2 *grow = zrow + N;                                     // N, STEP only: the screened row
-    float2 *erow = grow + N;                                     // N, STEP only: exp(-2 pi i z)
-    uint8_t *occ = reinterpret_cast<uint8_t *>(irow + (STEP ? 4 : 2) * N);   // ntu: strips of the current t-tile
-    const int ii = blockIdx.x, tid = threadIdx.x, kRowThreads = NP ? row_threads_max<NP>() : (int)blockDim.x;
+    float2 *grow = sbuf + F.stride;                              // N: the screened row (F.stride is even: 16-byte aligned)
+    float2 *erow = grow + N;                                     // N: exp(-2 pi i z)
+    float2 *irow = erow + N;                                     // N if keep_rows
+    float2 *zrow = irow + N;                                     // N if keep_rows
+    uint8_t *occ = reinterpret_cast<uint8_t *>(erow + (keep_rows ? 3 : 1) * N);   // ntu: strips of the current t-tile
+    const int ii = blockIdx.x, tid = threadIdx.x, T = NP ? row_threads_max<NP>() : (int)blockDim.x;
     // this CTA's planes: an equal share of the chunk's valid planes
     const int nvalid = min(planes, L.Nw - plane0);
     const int per = (nvalid + (int)gridDim.y - 1) / (int)gridDim.y;
     const int p_begin = (int)blockIdx.y * per, p_end = min(nvalid, p_begin + per);
     if (p_begin >= p_end) return;
     const size_t pix0 = (size_t)ii * N;
-    for (int jj = tid; jj < N; jj += kRowThreads) {
-        irow[jj] = img[pix0 + jj];
+    for (int jj = tid; jj < N; jj += T) {
         const float2 z = zsplit[pix0 + jj];
-        zrow[jj] = z;
-        if constexpr (STEP) {
-            float sn, cs;
-            phase_tz(1.f, z, &sn, &cs);
-            erow[jj] = make_float2(cs, -sn);
+        if (keep_rows) {
+            irow[jj] = img[pix0 + jj];
+            zrow[jj] = z;
         }
+        float sn, cs;
+        phase_tz(1.f, z, &sn, &cs);
+        erow[jj] = make_float2(cs, -sn);
     }
+    const float2 *isrc = keep_rows ? irow : img + pix0, *zsrc = keep_rows ? zrow : zsplit + pix0;
     int occ_tt = -1;
     const typename RowTwOf<NP>::type rt(tw, false, tid);        // the thread's twiddle bases, read once
     for (int p = p_begin; p < p_end; ++p) {
@@ -129,38 +139,30 @@ fwd_rows_kernel(Launch L, FftPlan F, const float2 *__restrict__ tw, const float2
         const int tt = pl / TT;
         __syncthreads();                     // row and z visible; the previous plane's last stage is done
         if (tt != occ_tt) {                  // uniform across the CTA
-            for (int i = tid; i < L.ntu; i += kRowThreads) occ[i] = col_occ[tt * L.ntu + i];
+            for (int i = tid; i < L.ntu; i += T) occ[i] = col_occ[tt * L.ntu + i];
             occ_tt = tt;
             __syncthreads();
         }
-        // row x exp(-i phi), phi = 2 pi t z
-        auto screened = [&](int jj) -> float2 {
-            const float2 f = irow[jj];
-            float sn, cs;
-            phase_tz(t, zrow[jj], &sn, &cs);
-            return make_float2(f.x * cs + f.y * sn, f.y * cs - f.x * sn);
-        };
-        bool step = false;                   // uniform: advance g to the next plane
-        if constexpr (STEP) {
-            if ((p - p_begin) % kScreenSteps == 0) {
-                for (int jj = tid; jj < N; jj += kRowThreads) grow[jj] = screened(jj);
-                __syncthreads();
+        if ((p - p_begin) % kScreenSteps == 0) {
+            for (int jj = tid; jj < N; jj += T) {
+                // row x exp(-i phi), phi = 2 pi t z
+                const float2 f = isrc[jj];
+                float sn, cs;
+                phase_tz(t, zsrc[jj], &sn, &cs);
+                grow[jj] = make_float2(f.x * cs + f.y * sn, f.y * cs - f.x * sn);
             }
-            step = (p + 1 - p_begin) % kScreenSteps != 0 && p + 1 < p_end;
+            __syncthreads();
         }
+        const bool step = (p + 1 - p_begin) % kScreenSteps != 0 && p + 1 < p_end;   // uniform: advance g
         auto load = [&](int, int J) -> float2 {
             if (!in_crop(J, half, Np)) return make_float2(0.f, 0.f);
             const int jj = grid_to_crop(J, half, Np);
-            if constexpr (!STEP) {
-                return screened(jj);
-            } else {
-                const float2 g = grow[jj];
-                if (step) {
-                    const float2 e = erow[jj];
-                    grow[jj] = make_float2(g.x * e.x - g.y * e.y, g.x * e.y + g.y * e.x);
-                }
-                return g;
+            const float2 g = grow[jj];
+            if (step) {
+                const float2 e = erow[jj];
+                grow[jj] = make_float2(g.x * e.x - g.y * e.y, g.x * e.y + g.y * e.x);
             }
+            return g;
         };
         // columns of this plane's t-tile that no footprint touches are never read
         auto store = [&](int, int R, float2 v) {
@@ -169,7 +171,7 @@ fwd_rows_kernel(Launch L, FftPlan F, const float2 *__restrict__ tw, const float2
         if constexpr (NP >= 512)
             fft_static_row<NP, row_threads_max<NP>(), CROP ? fftst::PRUNE_IN : 0>(sbuf, false, tid, load, store, rt);
         else
-            fft_many<1, false>(sbuf, F, tw, tid, kRowThreads, load, store);
+            fft_many<1, false>(sbuf, F, tw, tid, T, load, store);
     }
 }
 
@@ -275,19 +277,23 @@ struct RowsSmem {
     size_t buf, bytes;
 };
 inline RowsSmem rows_smem(const FftPlan &F, int N) {
-    RowsSmem r{2, 1, ((size_t)F.stride * sizeof(float2) + 127) / 128 * 128, 0};
-    auto need = [&] {
-        return 128 + r.buffers * r.buf + (size_t)N * (sizeof(float4) + (r.keep_z ? sizeof(float2) : 0)) + 32;
+    const size_t buf = ((size_t)F.stride * sizeof(float2) + 127) / 128 * 128;
+    auto layout = [&](int buffers, int keep_z) {
+        return RowsSmem{buffers, keep_z, buf,
+                        128 + buffers * buf + (size_t)N * (sizeof(float4) + (keep_z ? sizeof(float2) : 0)) + 32};
     };
-    // Two CTAs per SM come first: with one, nothing covers a CTA's barriers.  Where
-    // both buffers and the z row leave no room for a second CTA, one buffer and z
-    // from global memory do (N = 4096, N' = 5600).
-    if (need() > kTwoCtaSmem) {
-        r.keep_z = 0;
-        if (need() > kTwoCtaSmem) r.buffers = 1;
+    // As many CTAs per SM as registers allow come first: they cover each other's
+    // barriers and waits.  For that the z row goes to global memory (a CTA reads the
+    // same row on every plane, from L1 mostly) and then the second buffer goes, if the
+    // last stage's inputs fit in registers (dit_last_held).
+    const int last = F.nstages - 1;
+    const bool held = compile_time_size(F.n) || F.nb[last] <= F.row_threads * (32 / F.radix[last]);
+    for (int ctas = row_cta_limit(F); ctas > 1; --ctas) {
+        for (const RowsSmem &r : {layout(2, 1), layout(2, 0)})
+            if (r.bytes <= cta_smem(ctas)) return r;
+        if (held && layout(1, 0).bytes <= cta_smem(ctas)) return layout(1, 0);
     }
-    r.bytes = need();
-    return r;
+    return layout(2, 1).bytes <= cta_smem(1) ? layout(2, 1) : layout(2, 0);
 }
 
 // One CTA owns image row ii and an equal share of the chunk's planes (share
@@ -299,18 +305,20 @@ inline RowsSmem rows_smem(const FftPlan &F, int N) {
 //
 // The rows come by TMA in boxes of up to 256 column blocks (8 KB), all
 // completing on the buffer's mbarrier: with two buffers, plane p + 1's row is
-// copied while plane p is transformed.  Strips no footprint touched hold stale
+// copied while plane p is transformed; with one (ONE_BUFFER) it is copied while
+// the last stage, whose inputs are in registers by then, finishes plane p.  Strips no footprint touched hold stale
 // data; the first FFT stage masks them to zero.  Every wait is bounded; a CTA
 // that gives up waits (bounded) for the copy in flight and ends; *timeouts
 // counts the rows left incomplete.
-template <int NP, bool CROP>
+template <int NP, bool CROP, bool ONE_BUFFER>
 __global__ void __launch_bounds__(row_threads_max<NP>(), row_ctas<NP>())
 inv_rows_kernel(Launch L, FftPlan F, const float2 *__restrict__ tw, const __grid_constant__ CUtensorMap row_map,
-                const uint8_t *__restrict__ col_occ, int plane0, int planes, int buffers, int keep_z, int buf_slots,
+                const uint8_t *__restrict__ col_occ, int plane0, int planes, int keep_z, int buf_slots,
                 const float2 *__restrict__ zsplit, const float *__restrict__ corr, float4 *__restrict__ acc,
                 unsigned *__restrict__ rows_done, int first, int last, float2 *__restrict__ dirty,
                 unsigned long long *__restrict__ timeouts, int wait_polls) {
     extern __shared__ __align__(16) float2 sbuf[];
+    constexpr int buffers = ONE_BUFFER ? 1 : 2;
     const int Np = L.Np, N = L.N, half = N / 2;
     const int ii = blockIdx.x, tid = threadIdx.x, T = NP ? row_threads_max<NP>() : (int)blockDim.x;
     const int R0 = NP ? fftst::Radices<NP ? NP : 512>::r0 : F.radix[0], nb = NP ? NP / 16 : F.nb[0];
@@ -387,15 +395,14 @@ inv_rows_kernel(Launch L, FftPlan F, const float2 *__restrict__ tw, const __grid
             kahan_add(sum, comp, cmul_rot(v, make_float2(cs, sn), make_float2(-sn, cs)));
             srow[jj] = make_float4(sum.x, sum.y, comp.x, comp.y);
         };
+        auto between = [&] {
+            if (warp == 0 && k + 1 < count) issue(k + 1);
+        };
         if constexpr (NP >= 512)
-            fft_static_inplace<NP, row_threads_max<NP>(), CROP ? fftst::PRUNE_OUT : 0>(row_buf(k), true, tid, store,
-                                                                                     rt, live);
+            fft_static_inplace<NP, row_threads_max<NP>(), ONE_BUFFER, CROP ? fftst::PRUNE_OUT : 0>(
+                row_buf(k), true, tid, between, store, rt, live);
         else
-            fft_inplace(row_buf(k), F, tw, tid, T, store, live);
-        if (buffers == 1 && k + 1 < count) {
-            __syncthreads();
-            if (warp == 0) issue(k + 1);
-        }
+            fft_inplace<ONE_BUFFER>(row_buf(k), F, tw, tid, T, between, store, live);
     }
     __syncthreads();
     if (shares == 1 || !last) {
@@ -442,12 +449,16 @@ inv_rows_kernel(Launch L, FftPlan F, const float2 *__restrict__ tw, const __grid
 
 // transform buffers + one occupancy byte per strip (at most N'/16 or N'/32 of them)
 inline size_t smem2(const FftPlan &F) { return (size_t)kPerCta * F.stride * sizeof(float2) + F.n / TU + 16; }
-inline size_t smem_fwd_rows(const FftPlan &F, int N, bool step) {
-    return (size_t)F.stride * sizeof(float2) + (size_t)N * (step ? 4 : 2) * sizeof(float2) + F.n / TU + 16;
+inline size_t smem_fwd_rows(const FftPlan &F, int N, bool keep_rows) {
+    return (size_t)F.stride * sizeof(float2) + (size_t)N * (keep_rows ? 4 : 2) * sizeof(float2) + F.n / TU + 16;
 }
-// fwd_rows steps its screen where the two extra rows still leave room for two
-// CTAs per SM
-inline bool fwd_rows_step(const FftPlan &F, int N) { return smem_fwd_rows(F, N, true) <= kTwoCtaSmem; }
+// fwd_rows keeps the image row and z in shared memory where that costs no resident CTA
+inline bool fwd_rows_keep(const FftPlan &F, int N) {
+    auto fit = [&](bool keep) {
+        return std::min<size_t>(row_cta_limit(F), 228 * 1024 / (smem_fwd_rows(F, N, keep) + 1024));
+    };
+    return smem_fwd_rows(F, N, true) <= cta_smem(1) && fit(true) == fit(false);
+}
 // CTAs per image row in fwd_rows (each takes an equal share of the planes):
 // enough rows x groups for about 32 CTAs per SM over the launch,
 // so the SMs that finish first in the last round idle for a short CTA, not a long one
@@ -477,23 +488,23 @@ template <int NP>
 struct Transforms {
     static cudaError_t setup(const FftPlan &F, const FftPlan &inv, int N) {
         cudaError_t e;
-        const bool step = fwd_rows_step(F, N);
-        if ((e = allow_smem(fwd_rows_kernel<NP, false, false>, smem_fwd_rows(F, N, false))) != cudaSuccess) return e;
-        if (step && (e = allow_smem(fwd_rows_kernel<NP, true, false>, smem_fwd_rows(F, N, true))) != cudaSuccess)
-            return e;
-        if constexpr (NP != 0) {
-            if ((e = allow_smem(fwd_rows_kernel<NP, false, true>, smem_fwd_rows(F, N, false))) != cudaSuccess) return e;
-            if (step && (e = allow_smem(fwd_rows_kernel<NP, true, true>, smem_fwd_rows(F, N, true))) != cudaSuccess)
-                return e;
-        }
+        const size_t rows = smem_fwd_rows(F, N, fwd_rows_keep(F, N));
+        if ((e = allow_smem(fwd_rows_kernel<NP, false>, rows)) != cudaSuccess) return e;
+        if constexpr (NP != 0)
+            if ((e = allow_smem(fwd_rows_kernel<NP, true>, rows)) != cudaSuccess) return e;
         if ((e = allow_smem(fwd_cols_kernel<NP, false>, smem2(F))) != cudaSuccess) return e;
         if constexpr (NP != 0)
             if ((e = allow_smem(fwd_cols_kernel<NP, true>, smem2(F))) != cudaSuccess) return e;
         if ((e = allow_smem(inv_cols_kernel<NP, false>, smem2(inv))) != cudaSuccess) return e;
         if constexpr (NP != 0)
             if ((e = allow_smem(inv_cols_kernel<NP, true>, smem2(inv))) != cudaSuccess) return e;
-        if ((e = allow_smem(inv_rows_kernel<NP, false>, rows_smem(inv, N).bytes)) != cudaSuccess) return e;
-        if constexpr (NP != 0) e = allow_smem(inv_rows_kernel<NP, true>, rows_smem(inv, N).bytes);
+        const size_t inv_rows = rows_smem(inv, N).bytes;
+        if ((e = allow_smem(inv_rows_kernel<NP, false, false>, inv_rows)) != cudaSuccess) return e;
+        if ((e = allow_smem(inv_rows_kernel<NP, false, true>, inv_rows)) != cudaSuccess) return e;
+        if constexpr (NP != 0) {
+            if ((e = allow_smem(inv_rows_kernel<NP, true, false>, inv_rows)) != cudaSuccess) return e;
+            e = allow_smem(inv_rows_kernel<NP, true, true>, inv_rows);
+        }
         return e;
     }
     // Runs go(std::bool_constant): whether the crop is the centred half (compile-time plans only).
@@ -510,17 +521,13 @@ struct Transforms {
     static int row_threads(const FftPlan &F) { return NP ? row_threads_max<NP>() : F.row_threads; }
     static int col_threads(const FftPlan &F) { return NP ? col_threads_max<NP>() : F.col_threads; }
     static cudaError_t fwd_rows(const ws_plan_s *p, int chunk, int planes, cudaStream_t s) {
-        const bool step = fwd_rows_step(p->fft_fwd, p->L.N);
-        const int T = row_threads(p->fft_fwd);
+        const bool keep = fwd_rows_keep(p->fft_fwd, p->L.N);
         const dim3 grid(p->L.N, row_groups(p->L.N, planes, p->sms));
-        const size_t smem = smem_fwd_rows(p->fft_fwd, p->L.N, step);
-        auto go = [&](auto kernel) {
-            kernel<<<grid, T, smem, s>>>(p->L, p->fft_fwd, p->d_tw, p->d_img, p->d_zsplit, p->d_col_occ, chunk * p->P,
-                                         planes, p->d_stack);
-        };
         with_crop(p->L, [&](auto crop) {
-            constexpr bool C = decltype(crop)::value;
-            step ? go(fwd_rows_kernel<NP, true, C>) : go(fwd_rows_kernel<NP, false, C>);
+            fwd_rows_kernel<NP, decltype(crop)::value>
+                <<<grid, row_threads(p->fft_fwd), smem_fwd_rows(p->fft_fwd, p->L.N, keep), s>>>(
+                    p->L, p->fft_fwd, p->d_tw, p->d_img, p->d_zsplit, p->d_col_occ, chunk * p->P, planes, keep ? 1 : 0,
+                    p->d_stack);
         });
         return cudaGetLastError();
     }
@@ -546,12 +553,15 @@ struct Transforms {
         const cudaError_t e = row_tensor_map(p, &map);
         if (e != cudaSuccess) return e;
         const RowsSmem sm = rows_smem(p->fft_inv, p->L.N);
+        auto go = [&](auto kernel) {
+            kernel<<<dim3(p->L.N, p->row_shares), row_threads(p->fft_inv), sm.bytes, s>>>(
+                p->L, p->fft_inv, p->d_tw, map, p->d_col_occ, chunk * p->P, planes, sm.keep_z,
+                (int)(sm.buf / sizeof(float2)), p->d_zsplit, p->d_corr, p->d_acc, p->d_rows_done, first ? 1 : 0,
+                last ? 1 : 0, dirty, p->d_drop + 2, p->wait_polls);
+        };
         with_crop(p->L, [&](auto crop) {
-            inv_rows_kernel<NP, decltype(crop)::value>
-                <<<dim3(p->L.N, p->row_shares), row_threads(p->fft_inv), sm.bytes, s>>>(
-                    p->L, p->fft_inv, p->d_tw, map, p->d_col_occ, chunk * p->P, planes, sm.buffers, sm.keep_z,
-                    (int)(sm.buf / sizeof(float2)), p->d_zsplit, p->d_corr, p->d_acc, p->d_rows_done, first ? 1 : 0,
-                    last ? 1 : 0, dirty, p->d_drop + 2, p->wait_polls);
+            constexpr bool C = decltype(crop)::value;
+            sm.buffers == 1 ? go(inv_rows_kernel<NP, C, true>) : go(inv_rows_kernel<NP, C, false>);
         });
         return cudaGetLastError();
     }
