@@ -933,105 +933,111 @@ __global__ void unfold_kernel(const double *__restrict__ uvw, int64_t M, float2 
 // ---------------------------------------------------------------------------
 constexpr int kDegridThreads = 256;
 
-// Degridding: Algorithm 6 steps 4-5.  One warp per visibility (visiting them
-// in tile order for cache reuse); lanes over the W x W (a, b) columns of the
-// footprint (W^2 / 32 rounded up per lane), W planes each.  All of a lane's
-// gathers are issued before any is used, so a warp keeps up to 2 W loads in
-// flight.  The polynomial table sits in shared memory for the weights.  Each
-// chunk adds its planes' share to vis, in chunk order.
+// Degridding: Algorithm 6 steps 4-5.  One warp per visibility; lanes over the
+// W x W (a, b) columns of the footprint (W^2 / 32 rounded up per lane), W planes
+// each.  All of a lane's gathers are issued before any is used, so a warp keeps
+// up to 2 W loads in flight.  Each chunk adds its planes' share to vis, in chunk order.
+//
+// The kernel waits for its gathers, and they share the L1's data pipe with the
+// weights.  So a CTA takes up to kDegridRun x 8 consecutive visibilities of the
+// tile-sorted list at a time: their footprints overlap and meet in its L1 (with
+// consecutive visibilities dealt to different SMs, each SM fetched the same lines).
+// The polynomial table sits in shared memory coefficient by coefficient, so a
+// step of Horner's rule reads consecutive words, and the steps start at the
+// table's degree.  A warp has the next visibility's record under way while it
+// works on one.
+constexpr int kDegridRun = 8;
+
 template <int W>
 __global__ void __launch_bounds__(kDegridThreads, W <= 6 ? 5 : (W <= 8 ? 3 : 1))
 degrid3d_kernel(Launch L, const float *__restrict__ coef, int deg, const VisRec *__restrict__ rec,
                 const uint32_t *__restrict__ order, const uint32_t *__restrict__ n_order,
                 const float2 *__restrict__ stack, int plane0, int planes, float2 *__restrict__ vis) {
-    constexpr int kPasses = (W * W + 31) / 32;
-    __shared__ float swt[kDegridThreads / 32][3 * W];
-    // the (u, v) table, then the w table: 2W rows of kCoefStride coefficients, zero past deg
-    __shared__ __align__(16) float scoef[2 * W * kCoefStride];
-    for (int i = threadIdx.x; i < 2 * W * kCoefStride; i += kDegridThreads) {
-        const int row = i / kCoefStride, m = i - row * kCoefStride;
-        scoef[i] = m <= deg ? coef[row * (deg + 1) + m] : 0.f;
+    constexpr int kPasses = (W * W + 31) / 32, kWarps = kDegridThreads / 32, S = 3 * W;
+    __shared__ float swt[kWarps][S];
+    __shared__ float scoef[(kMaxDeg + 1) * S];              // [m][u taps, v taps, w taps]
+    for (int i = threadIdx.x; i < (deg + 1) * S; i += kDegridThreads) {
+        const int m = i / S, l = i - m * S;
+        scoef[i] = coef[(l < W ? l : l - W) * (deg + 1) + m];   // rows: the (u, v) table, then the w table
     }
     __syncthreads();
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int64_t n = (int64_t)*n_order;                   // entries of the sorted list (dropped ones excluded)
-    const int64_t nwarps = (int64_t)gridDim.x * (kDegridThreads / 32);
     const int Np = L.Np;
     const size_t plane = (size_t)Np * Np;
     float *wt = swt[warp];
-    // a grid of resident CTAs: each warp takes every nwarps-th visibility of the
-    // tile-sorted list, so the warps in flight still gather from neighbouring cells
-    for (int64_t widx = ((int64_t)blockIdx.x * kDegridThreads + threadIdx.x) >> 5; widx < n; widx += nwarps) {
-        const uint32_t k = order[widx];
-        const VisRec r = rec[k];
-        if (r.t0 < 0) continue;
-        const int c_lo = max(0, plane0 - r.t0);
-        const int c_hi = min(W - 1, plane0 + planes - 1 - r.t0);
-        if (c_lo > c_hi) continue;
-        __syncwarp();                                       // the previous visibility's weights are read
-        for (int l = lane; l < 3 * W; l += 32) {             // 3W > 32 for W >= 11
-            const int axis = l / W, i = l - axis * W;
-            const float nu = axis == 0 ? r.nux : (axis == 1 ? r.nuy : r.nuz);
-            const float4 *c = reinterpret_cast<const float4 *>(scoef + ((axis == 2 ? W : 0) + i) * kCoefStride);
-            float acc = c[4].x;                              // Horner from nu^16 down
+    // visibilities per warp and run: short runs while there are too few to go round
+    const int64_t nwarps = (int64_t)gridDim.x * kWarps;
+    const int run = (int)max((int64_t)1, min((int64_t)kDegridRun, n / (4 * nwarps)));
+    for (int64_t base = (int64_t)blockIdx.x * kWarps * run; base < n; base += nwarps * run) {
+        const int mine = (int)max((int64_t)0, min((int64_t)run, (n - base - warp + kWarps - 1) / kWarps));
+        uint32_t ids = 0;                                   // lane i: this warp's i-th visibility
+        if (lane < mine) ids = order[base + warp + kWarps * lane];
+        VisRec next{};
+        if (mine > 0) next = rec[__shfl_sync(0xffffffffu, ids, 0)];
+        for (int i = 0; i < mine; ++i) {
+            const uint32_t k = __shfl_sync(0xffffffffu, ids, i);
+            const VisRec r = next;
+            if (i + 1 < mine) next = rec[__shfl_sync(0xffffffffu, ids, i + 1)];
+            if (r.t0 < 0) continue;
+            const int c_lo = max(0, plane0 - r.t0);
+            const int c_hi = min(W - 1, plane0 + planes - 1 - r.t0);
+            if (c_lo > c_hi) continue;
+            const int64_t t_rel = (int64_t)r.t0 - plane0;       // stack plane of tap c is t_rel + c
+            const bool all_planes = c_lo == 0 && c_hi == W - 1; // uniform: the whole footprint is in the chunk
+            float2 f[kPasses][W];
 #pragma unroll
-            for (int b = 3; b >= 0; --b) {
-                const float4 c4 = c[b];
-                acc = fmaf(acc, nu, c4.w);
-                acc = fmaf(acc, nu, c4.z);
-                acc = fmaf(acc, nu, c4.y);
-                acc = fmaf(acc, nu, c4.x);
-            }
-            wt[l] = acc;
-        }
-        __syncwarp();
-        const int64_t t_rel = (int64_t)r.t0 - plane0;       // stack plane of tap c is t_rel + c
-        const bool all_planes = c_lo == 0 && c_hi == W - 1; // uniform: the whole footprint is in the chunk
-        float2 f[kPasses][W];
+            for (int ps = 0; ps < kPasses; ++ps) {
+                const int pair = lane + 32 * ps;
+                const int a = pair % W, b = pair / W;
+                const bool live = pair < W * W;
+                const float2 *cell = stack + tiled_index(wrap_add(r.s0, live ? b : 0, Np), wrap_add(r.r0, a, Np), Np) +
+                                     t_rel * (int64_t)plane;
+                if (all_planes) {
 #pragma unroll
-        for (int ps = 0; ps < kPasses; ++ps) {
-            const int pair = lane + 32 * ps;
-            const int a = pair % W, b = pair / W;
-            const bool live = pair < W * W;
-            const float2 *cell = stack + tiled_index(wrap_add(r.s0, live ? b : 0, Np), wrap_add(r.r0, a, Np), Np) +
-                                 (size_t)t_rel * plane;
-            if (all_planes) {
+                    for (int c = 0; c < W; ++c)
+                        f[ps][c] = live ? __ldg(cell + (size_t)c * plane) : make_float2(0.f, 0.f);
+                } else {
 #pragma unroll
-                for (int c = 0; c < W; ++c) f[ps][c] = live ? __ldg(cell + (size_t)c * plane) : make_float2(0.f, 0.f);
-            } else {
-#pragma unroll
-                for (int c = 0; c < W; ++c) {
-                    f[ps][c] = make_float2(0.f, 0.f);
-                    if (live && c >= c_lo && c <= c_hi) f[ps][c] = __ldg(cell + (size_t)c * plane);
+                    for (int c = 0; c < W; ++c) {
+                        f[ps][c] = make_float2(0.f, 0.f);
+                        if (live && c >= c_lo && c <= c_hi) f[ps][c] = __ldg(cell + (int64_t)c * (int64_t)plane);
+                    }
                 }
             }
-        }
-        float ar = 0.f, ai = 0.f;
+            __syncwarp();                                       // the previous visibility's weights are read
+            for (int l = lane; l < S; l += 32) {                // S > 32 for W >= 11
+                const float nu = l < W ? r.nux : (l < 2 * W ? r.nuy : r.nuz);
+                float acc = 0.f;                                // Horner from nu^deg down
 #pragma unroll
-        for (int ps = 0; ps < kPasses; ++ps) {
-            const int pair = lane + 32 * ps;
-            if (pair >= W * W) break;
-            const int a = pair % W, b = pair / W;
-            float sr = 0.f, si = 0.f;
-#pragma unroll
-            for (int c = 0; c < W; ++c) {
-                const float wc = wt[2 * W + c];
-                sr = fmaf(wc, f[ps][c].x, sr);
-                si = fmaf(wc, f[ps][c].y, si);
+                for (int m = kMaxDeg; m >= 0; --m)
+                    if (m <= deg) acc = fmaf(acc, nu, scoef[m * S + l]);
+                wt[l] = acc;
             }
-            const float wab = wt[a] * wt[W + b];
-            ar = fmaf(wab, sr, ar);
-            ai = fmaf(wab, si, ai);
-        }
-        for (int o = 16; o > 0; o >>= 1) {
-            ar += __shfl_xor_sync(0xffffffffu, ar, o);
-            ai += __shfl_xor_sync(0xffffffffu, ai, o);
-        }
-        if (lane == 0) {
-            float2 out = vis[k];
-            out.x += ar * r.vre - ai * r.vim;
-            out.y += ar * r.vim + ai * r.vre;
-            vis[k] = out;
+            __syncwarp();
+            float ar = 0.f, ai = 0.f;
+#pragma unroll
+            for (int ps = 0; ps < kPasses; ++ps) {
+                const int pair = lane + 32 * ps;
+                if (pair >= W * W) break;
+                const int a = pair % W, b = pair / W;
+                float2 s = make_float2(0.f, 0.f);
+#pragma unroll
+                for (int c = 0; c < W; ++c) s = fma2(dup2(wt[2 * W + c]), f[ps][c], s);
+                const float wab = wt[a] * wt[W + b];
+                ar = fmaf(wab, s.x, ar);
+                ai = fmaf(wab, s.y, ai);
+            }
+            for (int o = 16; o > 0; o >>= 1) {
+                ar += __shfl_xor_sync(0xffffffffu, ar, o);
+                ai += __shfl_xor_sync(0xffffffffu, ai, o);
+            }
+            if (lane == 0) {
+                float2 out = vis[k];
+                out.x += ar * r.vre - ai * r.vim;
+                out.y += ar * r.vim + ai * r.vre;
+                vis[k] = out;
+            }
         }
     }
 }
