@@ -811,7 +811,7 @@ ws_status plan_create(ws_plan_s **out, int32_t N, double x0, int32_t W, double f
     size_t budget = (size_t)(0.6 * (double)free_b);
     if (const char *env = std::getenv("WS_STACK_BYTES")) budget = (size_t)std::strtoull(env, nullptr, 10);
     int P = fp64 ? 0 : L.ntt * TT;
-    if (fp64) own_stack = false;                  // FP64 plans work one plane at a time
+    if (fp64) own_stack = false;                  // FP64 plans have planes of their own (fp64_planes)
     if (const char *env = std::getenv("WS_PLANES_PER_CHUNK")) {
         int want = std::atoi(env);
         if (want > 0) P = std::min(P, std::max(TT, (want / TT) * TT));
@@ -888,7 +888,13 @@ ws_status plan_create(ws_plan_s **out, int32_t N, double x0, int32_t W, double f
         WS_TRY(dev_alloc(&p->d_tw64, tw64.size(), &p->bytes), "allocating FP64 twiddles");
         WS_TRY(cudaMemcpy(p->d_tw64, tw64.data(), tw64.size() * sizeof(double2), cudaMemcpyHostToDevice),
                "uploading FP64 twiddles");
-        WS_TRY(dev_alloc(&p->d_plane64, (size_t)Np * Np, &p->bytes), "allocating the FP64 plane");
+        p->planes64 = fp64_planes((int)Np, L.Nw);
+        if (const char *env = std::getenv("WS_PLANES_PER_CHUNK")) {
+            const int want = std::atoi(env);
+            if (want > 0) p->planes64 = std::min(p->planes64, want);
+        }
+        WS_TRY(fp64_setup((int)Np), "configuring the FP64 transforms");
+        WS_TRY(dev_alloc(&p->d_plane64, (size_t)p->planes64 * Np * Np, &p->bytes), "allocating the FP64 planes");
         WS_TRY(dev_alloc(&p->d_acc64, (size_t)N * N, &p->bytes), "allocating the FP64 accumulator");
         p->fft64_log = 0;
         while ((1LL << p->fft64_log) < Np) ++p->fft64_log;

@@ -163,12 +163,13 @@ struct ws_plan_s {
     uint8_t *d_btile_occ = nullptr;         // ntiles
     uint8_t *d_bcol_occ = nullptr;          // ntt x ntu
     unsigned long long *d_bdrop = nullptr;  // kCounters: the bound set's drop counts
-    // FP64 plans (WS_FLAG_FP64): their own tables and one plane of workspace
+    // FP64 plans (WS_FLAG_FP64): their own tables and a chunk of planes
     bool fp64 = false;
     double *d_cheb64 = nullptr;             // 2 x W x (degree+1): Chebyshev series of c_i(nu), (u, v) then w
     double *d_corr64 = nullptr;             // N x N
     double *d_z64 = nullptr;                // N x N
-    double2 *d_plane64 = nullptr;           // N' x N'
+    int planes64 = 1;                       // planes per chunk
+    double2 *d_plane64 = nullptr;           // planes64 x N' x N'
     double2 *d_acc64 = nullptr;             // N x N
     double2 *d_tw64 = nullptr;              // N': exp(-2 pi i m / N')
     int fft64_log = 0;
@@ -222,6 +223,8 @@ bool tune_store(const char *path, const std::string &key, int tile_rows, const i
 
 // FP64 path (fp64.cu).
 size_t fp64_record_bytes();
+int fp64_planes(int Np, int Nw);
+cudaError_t fp64_setup(int Np);
 ws_status enqueue_grid64(ws_plan_s *p, const double *uvw, const double2 *vis, int64_t M, double2 *dirty,
                          cudaStream_t s);
 ws_status enqueue_degrid64(ws_plan_s *p, const double2 *image, const double *uvw, int64_t M, double2 *vis,
