@@ -93,7 +93,7 @@ extern "C" ws_status ws_degrid_noalloc(ws_plan_t plan, const void *image, const 
     uint32_t *counts = reinterpret_cast<uint32_t *>(take((size_t)(p->ntiles + 1) * sizeof(uint32_t)));
     uint32_t *offsets = reinterpret_cast<uint32_t *>(take((size_t)(p->ntiles + 1) * sizeof(uint32_t)));
     uint32_t *blocksums = reinterpret_cast<uint32_t *>(take(4096 * sizeof(uint32_t)));
-    unsigned long long *drop = reinterpret_cast<unsigned long long *>(take(2 * sizeof(unsigned long long)));
+    unsigned long long *drop = reinterpret_cast<unsigned long long *>(take(kCounters * sizeof(unsigned long long)));
     uint8_t *tile_occ = take((size_t)p->ntiles);
     uint8_t *col_occ = take((size_t)p->L.ntt * p->L.ntu);
     float2 *img = reinterpret_cast<float2 *>(take(n_img * sizeof(float2)));
@@ -133,14 +133,14 @@ extern "C" ws_status ws_degrid_noalloc(ws_plan_t plan, const void *image, const 
     v.d_col_occ = col_occ;
 
     cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
-    cudaError_t e = cudaMemsetAsync(drop, 0, 2 * sizeof(unsigned long long), s);
-    if (e != cudaSuccess) return cuda_fail(e, "ws_degrid_noalloc: clearing counters");
+    cudaError_t e = cudaSuccess;
+    if (M == 0 && (e = cudaMemsetAsync(drop, 0, kCounters * sizeof(unsigned long long), s)) != cudaSuccess)
+        return cuda_fail(e, "ws_degrid_noalloc: clearing counters");
     if (M > 0) {
-        if ((e = cudaMemsetAsync(vis, 0, (size_t)M * sizeof(float2), s)) != cudaSuccess)
-            return cuda_fail(e, "ws_degrid_noalloc: clearing the output");
-        if ((e = launch_prep(&v, uvw, nullptr, M, false, s)) != cudaSuccess)
-            return cuda_fail(e, "ws_degrid_noalloc: prep kernel");
-        if ((e = launch_bin(&v, M, false, s)) != cudaSuccess)
+        if ((e = launch_clear_bins(&v, drop, s)) != cudaSuccess ||
+            (e = launch_prep_count(&v, uvw, nullptr, M, false, static_cast<float2 *>(vis), s)) != cudaSuccess)
+            return cuda_fail(e, "ws_degrid_noalloc: prep kernels");
+        if ((e = launch_sort(&v, M, false, s)) != cudaSuccess)
             return cuda_fail(e, "ws_degrid_noalloc: binning kernels");
         if ((e = launch_correct_image(&v, static_cast<const float2 *>(image), s)) != cudaSuccess)
             return cuda_fail(e, "ws_degrid_noalloc: correction kernel");

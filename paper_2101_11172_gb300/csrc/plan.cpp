@@ -966,23 +966,25 @@ bool is_bound(const ws_plan_s *p, const double *uvw, int64_t M) {
 ws_status enqueue_grid(ws_plan_s *p, const double *uvw, const float2 *vis, int64_t M, float2 *dirty,
                        cudaStream_t s) {
     const bool bound = is_bound(p, uvw, M);
-    cudaError_t e = bound ? cudaMemcpyAsync(p->d_drop, p->d_bdrop, kCounters * sizeof(unsigned long long),
-                                            cudaMemcpyDeviceToDevice, s)
-                          : cudaMemsetAsync(p->d_drop, 0, kCounters * sizeof(unsigned long long), s);
-    if (e != cudaSuccess) return cuda_fail(e, "ws_grid: clearing counters");
+    cudaError_t e = cudaSuccess;
     p->stats.calls += 1;
     if (bound) {
+        if ((e = cudaMemcpyAsync(p->d_drop, p->d_bdrop, kCounters * sizeof(unsigned long long),
+                                 cudaMemcpyDeviceToDevice, s)) != cudaSuccess)
+            return cuda_fail(e, "ws_grid: clearing counters");
         // the bound set's records, with this call's values and the gridding pre-phase
         StageTimer t(p, s, WS_STAGE_PREP, M > 0 ? 1 : 0);
         if ((e = launch_bound_grid_records(p, uvw, vis, M, s)) != cudaSuccess)
             return cuda_fail(e, "ws_grid: bound records kernel");
     } else {
         {
-            StageTimer t(p, s, WS_STAGE_PREP, M > 0 ? 1 : 0);
-            if ((e = launch_prep(p, uvw, vis, M, true, s)) != cudaSuccess) return cuda_fail(e, "ws_grid: prep kernel");
+            StageTimer t(p, s, WS_STAGE_PREP, M > 0 ? 2 : 1);
+            if ((e = launch_clear_bins(p, p->d_drop, s)) != cudaSuccess ||
+                (e = launch_prep_count(p, uvw, vis, M, true, nullptr, s)) != cudaSuccess)
+                return cuda_fail(e, "ws_grid: prep kernels");
         }
-        StageTimer t(p, s, WS_STAGE_BIN, (M > 0 ? 6 : 3) + ((p->flags & WS_FLAG_TIMING) ? 1 : 0));
-        if ((e = launch_bin(p, M, true, s)) != cudaSuccess) return cuda_fail(e, "ws_grid: binning kernels");
+        StageTimer t(p, s, WS_STAGE_BIN, sort_launches(p, M) + ((p->flags & WS_FLAG_TIMING) ? 1 : 0));
+        if ((e = launch_sort(p, M, true, s)) != cudaSuccess) return cuda_fail(e, "ws_grid: binning kernels");
     }
     BoundView view(p, bound, true);
     if ((e = copy_occ_counts(p, s)) != cudaSuccess) return cuda_fail(e, "ws_grid: occupancy statistics");
@@ -1018,22 +1020,27 @@ ws_status enqueue_grid(ws_plan_s *p, const double *uvw, const float2 *vis, int64
 ws_status enqueue_degrid(ws_plan_s *p, const float2 *image, const double *uvw, int64_t M, float2 *vis,
                          cudaStream_t s) {
     const bool bound = is_bound(p, uvw, M);
-    cudaError_t e = bound ? cudaMemcpyAsync(p->d_drop, p->d_bdrop, kCounters * sizeof(unsigned long long),
-                                            cudaMemcpyDeviceToDevice, s)
-                          : cudaMemsetAsync(p->d_drop, 0, kCounters * sizeof(unsigned long long), s);
-    if (e != cudaSuccess) return cuda_fail(e, "ws_degrid: clearing counters");
+    cudaError_t e = cudaSuccess;
+    if (bound || M == 0) {
+        e = bound ? cudaMemcpyAsync(p->d_drop, p->d_bdrop, kCounters * sizeof(unsigned long long),
+                                    cudaMemcpyDeviceToDevice, s)
+                  : cudaMemsetAsync(p->d_drop, 0, kCounters * sizeof(unsigned long long), s);
+        if (e != cudaSuccess) return cuda_fail(e, "ws_degrid: clearing counters");
+    }
     if (M == 0) return WS_OK;
-    if ((e = cudaMemsetAsync(vis, 0, (size_t)M * sizeof(float2), s)) != cudaSuccess)
-        return cuda_fail(e, "ws_degrid: clearing the output");
     p->stats.calls += 1;
-    if (!bound) {
+    if (bound) {
+        if ((e = cudaMemsetAsync(vis, 0, (size_t)M * sizeof(float2), s)) != cudaSuccess)
+            return cuda_fail(e, "ws_degrid: clearing the output");
+    } else {
         {
-            StageTimer t(p, s, WS_STAGE_PREP, 1);
-            if ((e = launch_prep(p, uvw, nullptr, M, false, s)) != cudaSuccess)
-                return cuda_fail(e, "ws_degrid: prep kernel");
+            StageTimer t(p, s, WS_STAGE_PREP, 2);
+            if ((e = launch_clear_bins(p, p->d_drop, s)) != cudaSuccess ||
+                (e = launch_prep_count(p, uvw, nullptr, M, false, vis, s)) != cudaSuccess)
+                return cuda_fail(e, "ws_degrid: prep kernels");
         }
-        StageTimer t(p, s, WS_STAGE_BIN, 6 + ((p->flags & WS_FLAG_TIMING) ? 1 : 0));
-        if ((e = launch_bin(p, M, false, s)) != cudaSuccess) return cuda_fail(e, "ws_degrid: binning kernels");
+        StageTimer t(p, s, WS_STAGE_BIN, sort_launches(p, M) + ((p->flags & WS_FLAG_TIMING) ? 1 : 0));
+        if ((e = launch_sort(p, M, false, s)) != cudaSuccess) return cuda_fail(e, "ws_degrid: binning kernels");
     }
     BoundView view(p, bound, false);
     if ((e = copy_occ_counts(p, s)) != cudaSuccess) return cuda_fail(e, "ws_degrid: occupancy statistics");
@@ -1209,11 +1216,13 @@ ws_status ws_plan_bind_uvw(ws_plan_t plan, const double *uvw, int64_t M, ws_stre
         p->d_offsets = p->d_boff_g;
         p->d_tile_occ = p->d_btile_occ;
         p->d_col_occ = p->d_bcol_occ;
-        e = launch_prep(p, uvw, nullptr, M, false, s);
-        if (e == cudaSuccess) e = launch_bin(p, M, true, s);
+        e = launch_prep(p, uvw, M, s);
+        if (e == cudaSuccess) e = launch_count(p, M, true, s);
+        if (e == cudaSuccess) e = launch_sort(p, M, true, s);
         p->d_list = p->d_blist_d;
         p->d_offsets = p->d_boff_d;
-        if (e == cudaSuccess) e = launch_bin(p, M, false, s);
+        if (e == cudaSuccess) e = launch_count(p, M, false, s);
+        if (e == cudaSuccess) e = launch_sort(p, M, false, s);
         p->d_rec = rec;
         p->d_list = list;
         p->d_offsets = offsets;

@@ -231,13 +231,21 @@ ws_status enqueue_degrid64(ws_plan_s *p, const double2 *image, const double *uvw
                            cudaStream_t s);
 
 // Launchers (wstack.cu).
-cudaError_t launch_prep(const ws_plan_s *p, const double *uvw, const float2 *vis, int64_t M,
-                        bool grid, cudaStream_t s);
+// Records of a visibility set in the degridding form, and nothing else.
+cudaError_t launch_prep(const ws_plan_s *p, const double *uvw, int64_t M, cudaStream_t s);
+// One call's records, bin counts and tile marks in one pass, after launch_clear_bins
+// (which zeroes the drop counters too, if given).  Degridding also zeroes its output.
+cudaError_t launch_clear_bins(const ws_plan_s *p, unsigned long long *drop, cudaStream_t s);
+cudaError_t launch_prep_count(const ws_plan_s *p, const double *uvw, const float2 *vis, int64_t M, bool grid,
+                              float2 *zeroed, cudaStream_t s);
 cudaError_t launch_bound_grid_records(const ws_plan_s *p, const double *uvw, const float2 *vis, int64_t M,
                                       cudaStream_t s);
 // Binning (gridding: by tile column and first-tap t-tile; degridding: by
-// first-tap tile) and the stack's occupancy maps, from the records d_rec.
-cudaError_t launch_bin(ws_plan_s *p, int64_t M, bool grid, cudaStream_t s);
+// first-tap tile): the counts and tile marks of the records d_rec, cleared first;
+// then the offsets, the lists and the strips' occupancy from the counts.
+cudaError_t launch_count(const ws_plan_s *p, int64_t M, bool grid, cudaStream_t s);
+cudaError_t launch_sort(const ws_plan_s *p, int64_t M, bool grid, cudaStream_t s);
+int sort_launches(const ws_plan_s *p, int64_t M);
 cudaError_t launch_occ_count(const ws_plan_s *p, cudaStream_t s);
 cudaError_t launch_grid_chunk(const ws_plan_s *p, int chunk, int planes, cudaStream_t s);
 cudaError_t launch_correct_image(const ws_plan_s *p, const float2 *image, cudaStream_t s);

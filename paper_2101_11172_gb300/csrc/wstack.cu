@@ -1,9 +1,9 @@
 // CUDA kernels of the improved W-stacking hot path (sm_103a).
 //
-// Gridding (Algorithm 5):   prep -> bin -> per plane chunk: grid3d -> inv_cols -> inv_rows
+// Gridding (Algorithm 5):   prep and count -> sort -> per plane chunk: grid3d -> inv_cols -> inv_rows
 //                           (transforms.cu: inverse DFTs, crop, x exp(2 pi i t z), sum over t,
 //                           x h_x h_y h_z)
-// Degridding (Algorithm 6): prep -> bin -> correct_image (x h_x h_y h_z) -> per plane chunk:
+// Degridding (Algorithm 6): prep and count -> sort -> correct_image (x h_x h_y h_z) -> per plane chunk:
 //                           fwd_rows -> fwd_cols (transforms.cu: x exp(-2 pi i t z), zero pad,
 //                           forward DFTs) -> degrid3d (3-D correlation with C_x C_y C_z,
 //                           x exp(-2 pi i w (n0-1)))
@@ -34,87 +34,6 @@ __device__ __forceinline__ int wrap_index(double x, int n) {
     if (i < 0) i += n;
     if (i >= n) i -= n;
     return (int)i;
-}
-
-// ---------------------------------------------------------------------------
-// Pre-processing (Section 3.3 tap rule, Section 5.2 scaling and pre-phase)
-// ---------------------------------------------------------------------------
-__global__ void prep_kernel(Launch L, const double *__restrict__ uvw, const float2 *__restrict__ vis,
-                            int64_t M, int grid, VisRec *__restrict__ rec,
-                            unsigned long long *__restrict__ drop) {
-    // a grid-stride loop: the plan's constants in FP64 (W / 2, offsets) are formed
-    // once per thread, not once per visibility (FP64 arithmetic is slow here)
-    const int W = L.W;
-    const double half_w = 0.5 * W, half_wm1 = 0.5 * (W - 1), t_off = (double)(W - 1) + L.t_lo;
-    const double t_max = (double)(L.Nw - W);
-    for (int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; k < M; k += (int64_t)gridDim.x * blockDim.x) {
-        double u = uvw[3 * k], v = uvw[3 * k + 1], w = uvw[3 * k + 2];
-        // Section 5.4, real sky: V(u, v, w) = conj V(-u, -v, -w), so w < 0 is gridded at
-        // -(u, v, w) with the conjugate value (and degridded there, conjugated afterwards)
-        const bool folded = L.fold && w < 0.0;
-        if (folded) {
-            u = -u;
-            v = -v;
-            w = -w;
-        }
-        VisRec r;
-        r.r0 = r.s0 = 0;
-        r.t0 = -1;
-        r.nux = r.nuy = r.nuz = 0.f;
-        r.vre = r.vim = 0.f;
-        const double up = u * L.uv_scale, vp = v * L.uv_scale, wp = w * L.nscale;
-        if (!(fabs(up) < 1e15) || !(fabs(vp) < 1e15)) {   // also catches NaN
-            atomicAdd(&drop[0], 1ull);
-            rec[k] = r;
-            continue;
-        }
-        const double ft = floor(wp + half_w);
-        const double t0 = ft - t_off;
-        if (!(t0 >= 0.0 && t0 <= t_max)) {                 // NaN w fails too
-            atomicAdd(&drop[1], 1ull);
-            rec[k] = r;
-            continue;
-        }
-        const double fu = floor(up + half_w), fv = floor(vp + half_w);
-        const double ru = fu - (W - 1), rv = fv - (W - 1);
-        r.r0 = wrap_index(ru, L.Np);
-        r.s0 = wrap_index(rv, L.Np);
-        r.t0 = (int)t0;
-        r.nux = (float)(up + half_wm1 - fu);
-        r.nuy = (float)(vp + half_wm1 - fv);
-        r.nuz = (float)(wp + half_wm1 - ft);
-        // pre-phase exp(+2 pi i w (n0 - 1)), argument reduced in FP64
-        double turns = w * L.n0m1;
-        turns -= rint(turns);
-        float s, c;
-        sincospif(2.0f * (float)turns, &s, &c);
-        if (grid) {
-            float2 V = vis[k];
-            if (folded) V.y = -V.y;
-            r.vre = V.x * c - V.y * s;
-            r.vim = V.x * s + V.y * c;
-        } else {
-            r.vre = c;          // conjugate phase applied after degridding
-            r.vim = -s;
-        }
-        rec[k] = r;
-    }
-}
-
-// Gridding records of a bound visibility set: the set's records hold the
-// degridding factor exp(-2 pi i w (n0 - 1)); gridding needs V exp(+2 pi i w
-// (n0 - 1)), with V conjugated where a real-sky plan folded w < 0.
-__global__ void bound_grid_records_kernel(Launch L, const double *__restrict__ uvw, const float2 *__restrict__ vis,
-                                          int64_t M, const VisRec *__restrict__ brec, VisRec *__restrict__ rec) {
-    int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (k >= M) return;
-    VisRec r = brec[k];
-    float2 V = vis[k];
-    if (L.fold && uvw[3 * k + 2] < 0.0) V.y = -V.y;
-    const float c = r.vre, s = -r.vim;      // exp(+2 pi i w (n0 - 1)) = (c, s)
-    r.vre = V.x * c - V.y * s;
-    r.vim = V.x * s + V.y * c;
-    rec[k] = r;
 }
 
 // ---------------------------------------------------------------------------
@@ -164,11 +83,8 @@ constexpr int kMaxKeys = 2 * 2;
 // Every other cell of the stack is zero when gridding and never read when
 // degridding, so the plane kernels skip it.
 template <bool GRID>
-__global__ void count_kernel(Launch L, const VisRec *__restrict__ rec, int64_t M, uint32_t *__restrict__ counts,
-                             uint8_t *__restrict__ tile_occ) {
-    int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (k >= M) return;
-    const VisRec r = rec[k];
+__device__ __forceinline__ void count_record(const Launch &L, const VisRec &r, uint32_t *__restrict__ counts,
+                                             uint8_t *__restrict__ tile_occ) {
     uint32_t keys[kMaxKeys];
     const int n = record_keys<GRID>(L, r, keys);
     for (int i = 0; i < n; ++i) atomicAdd(&counts[keys[i]], 1u);
@@ -181,24 +97,168 @@ __global__ void count_kernel(Launch L, const VisRec *__restrict__ rec, int64_t M
             for (int a = 0; a < nu_; ++a) tile_occ[tile_id(L, tt, tv[b], tu[a])] = 1;   // stores only: no waits
 }
 
+// ---------------------------------------------------------------------------
+// Pre-processing (Section 3.3 tap rule, Section 5.2 scaling and pre-phase)
+// ---------------------------------------------------------------------------
+// What prep_kernel makes of a record once it has it: nothing more (the bound
+// set's records), or its degridding or gridding bins counted and its tiles marked.
+enum : int { kPrepOnly = 0, kPrepDegrid = 1, kPrepGrid = 2 };
+
+// floor(x) for |x| < 2^51, by adding and taking off 1.5 x 2^52: the sum rounds x
+// to the nearest integer, in its low bits.  FP64 adds run at 2 a clock and SM;
+// floor and the FP64-to-integer conversions at a fraction of that.
+__device__ __forceinline__ double floor_int(double x, int *low) {
+    constexpr double kRound = 6755399441055744.0;
+    double s = x + kRound, f = s - kRound;
+    if (f > x) {
+        s -= 1.0;
+        f -= 1.0;
+    }
+    *low = __double2loint(s);
+    return f;
+}
+
+// A grid index i (|i| < 2^31) modulo n: with the division only for the rare points more than a grid away.
+__device__ __forceinline__ int wrap_small(int i, int n) {
+    if (i < -n || i >= 2 * n) i %= n;
+    if (i < 0) i += n;
+    return i >= n ? i - n : i;
+}
+
+// The loop bound: M records, 8 CTAs per SM in a grid-stride loop, so that the
+// plan's constants in FP64 (W / 2, offsets) are formed once per thread, not once
+// per visibility.  FP64 arithmetic is what bounds this kernel (GB300 adds and
+// multiplies 0.6 T FP64 numbers a second).
+template <int BIN>
+__global__ void prep_kernel(Launch L, const double *__restrict__ uvw, const float2 *__restrict__ vis,
+                            int64_t M, VisRec *__restrict__ rec, unsigned long long *__restrict__ drop,
+                            uint32_t *__restrict__ counts, uint8_t *__restrict__ tile_occ, float2 *__restrict__ zeroed) {
+    const int W = L.W;
+    const double half_w = 0.5 * W, half_wm1 = 0.5 * (W - 1), t_off = (double)(W - 1) + L.t_lo;
+    const double t_max = (double)(L.Nw - W);
+    for (int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; k < M; k += (int64_t)gridDim.x * blockDim.x) {
+        double u = uvw[3 * k], v = uvw[3 * k + 1], w = uvw[3 * k + 2];
+        if (BIN == kPrepDegrid) zeroed[k] = make_float2(0.f, 0.f);      // the output that degridding adds to
+        // Section 5.4, real sky: V(u, v, w) = conj V(-u, -v, -w), so w < 0 is gridded at
+        // -(u, v, w) with the conjugate value (and degridded there, conjugated afterwards)
+        const bool folded = L.fold && w < 0.0;
+        if (folded) {
+            u = -u;
+            v = -v;
+            w = -w;
+        }
+        VisRec r;
+        r.r0 = r.s0 = 0;
+        r.t0 = -1;
+        r.nux = r.nuy = r.nuz = 0.f;
+        r.vre = r.vim = 0.f;
+        const double up = u * L.uv_scale, vp = v * L.uv_scale, wp = w * L.nscale;
+        if (!(fabs(up) < 1e15) || !(fabs(vp) < 1e15)) {   // also catches NaN
+            atomicAdd(&drop[0], 1ull);
+            rec[k] = r;
+            continue;
+        }
+        const double xt = wp + half_w;
+        // (the planes' range is below 2^12, so a w within it is within floor_int's range)
+        int it, iu, iv;
+        const double ft = floor_int(xt, &it);
+        const double t0 = ft - t_off;
+        if (!(fabs(xt) < 1e9 && t0 >= 0.0 && t0 <= t_max)) {   // NaN w fails too
+            atomicAdd(&drop[1], 1ull);
+            rec[k] = r;
+            continue;
+        }
+        const double xu = up + half_w, xv = vp + half_w;
+        double fu, fv;
+        if (fabs(xu) < 1e9 && fabs(xv) < 1e9) {
+            fu = floor_int(xu, &iu);
+            fv = floor_int(xv, &iv);
+            r.r0 = wrap_small(iu - (W - 1), L.Np);
+            r.s0 = wrap_small(iv - (W - 1), L.Np);
+        } else {
+            fu = floor(xu);
+            fv = floor(xv);
+            r.r0 = wrap_index(fu - (W - 1), L.Np);
+            r.s0 = wrap_index(fv - (W - 1), L.Np);
+        }
+        r.t0 = it - (W - 1) - L.t_lo;
+        r.nux = (float)(up + half_wm1 - fu);
+        r.nuy = (float)(vp + half_wm1 - fv);
+        r.nuz = (float)(wp + half_wm1 - ft);
+        // pre-phase exp(+2 pi i w (n0 - 1)), argument reduced in FP64
+        double turns = w * L.n0m1;
+        turns -= rint(turns);
+        float s, c;
+        sincospif(2.0f * (float)turns, &s, &c);
+        if (BIN == kPrepGrid) {
+            float2 V = vis[k];
+            if (folded) V.y = -V.y;
+            r.vre = V.x * c - V.y * s;
+            r.vim = V.x * s + V.y * c;
+        } else {
+            r.vre = c;          // conjugate phase applied after degridding
+            r.vim = -s;
+        }
+        rec[k] = r;
+        if (BIN == kPrepGrid) count_record<true>(L, r, counts, tile_occ);
+        if (BIN == kPrepDegrid) count_record<false>(L, r, counts, tile_occ);
+    }
+}
+
+// Zeroes the counts and the occupancy maps, and the drop counters if there are any.
+__global__ void clear_bins_kernel(uint32_t *__restrict__ counts, int64_t n, uint8_t *__restrict__ tile_occ, int64_t nt,
+                                  uint8_t *__restrict__ col_occ, int64_t nc, unsigned long long *__restrict__ drop) {
+    const int64_t i0 = (int64_t)blockIdx.x * blockDim.x + threadIdx.x, step = (int64_t)gridDim.x * blockDim.x;
+    for (int64_t i = i0; i < n; i += step) counts[i] = 0u;
+    for (int64_t i = i0; i < nt / 16; i += step) reinterpret_cast<uint4 *>(tile_occ)[i] = make_uint4(0u, 0u, 0u, 0u);
+    for (int64_t i = nt / 16 * 16 + i0; i < nt; i += step) tile_occ[i] = 0;
+    for (int64_t i = i0; i < nc; i += step) col_occ[i] = 0;
+    if (drop && i0 < kCounters) drop[i0] = 0ull;
+}
+
+// The counting pass over records that are there already (the bound set's).
 template <bool GRID>
-__global__ void scatter_kernel(Launch L, const VisRec *__restrict__ rec, int64_t M,
-                               const uint32_t *__restrict__ offsets, uint32_t *__restrict__ fill,
-                               uint32_t *__restrict__ list) {
+__global__ void count_kernel(Launch L, const VisRec *__restrict__ rec, int64_t M, uint32_t *__restrict__ counts,
+                             uint8_t *__restrict__ tile_occ) {
+    int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (k < M) count_record<GRID>(L, rec[k], counts, tile_occ);
+}
+
+// Gridding records of a bound visibility set: the set's records hold the
+// degridding factor exp(-2 pi i w (n0 - 1)); gridding needs V exp(+2 pi i w
+// (n0 - 1)), with V conjugated where a real-sky plan folded w < 0.
+__global__ void bound_grid_records_kernel(Launch L, const double *__restrict__ uvw, const float2 *__restrict__ vis,
+                                          int64_t M, const VisRec *__restrict__ brec, VisRec *__restrict__ rec) {
+    int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (k >= M) return;
+    VisRec r = brec[k];
+    float2 V = vis[k];
+    if (L.fold && uvw[3 * k + 2] < 0.0) V.y = -V.y;
+    const float c = r.vre, s = -r.vim;      // exp(+2 pi i w (n0 - 1)) = (c, s)
+    r.vre = V.x * c - V.y * s;
+    r.vim = V.x * s + V.y * c;
+    rec[k] = r;
+}
+
+// Lists the pairs: a bin's next place is its cursor, which starts at the bin's
+// offset.  The CTAs from vis_blocks on mark the occupied (t-tile, u-tile) strips
+// of N' rows (any tile of the strip touched) on the side.
+template <bool GRID>
+__global__ void scatter_kernel(Launch L, const VisRec *__restrict__ rec, int64_t M, int vis_blocks,
+                               uint32_t *__restrict__ cursor, uint32_t *__restrict__ list,
+                               const uint8_t *__restrict__ tile_occ, int64_t ntiles, uint8_t *__restrict__ col_occ) {
+    if ((int)blockIdx.x >= vis_blocks) {
+        const int64_t t = (int64_t)(blockIdx.x - vis_blocks) * blockDim.x + threadIdx.x;
+        if (t >= ntiles || !tile_occ[t]) return;
+        const int64_t c = (t / ((int64_t)L.ntu * L.ntv)) * L.ntu + t % L.ntu;
+        if (!col_occ[c]) col_occ[c] = 1;
+        return;
+    }
     int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (k >= M) return;
     uint32_t keys[kMaxKeys];
     int n = record_keys<GRID>(L, rec[k], keys);
-    for (int i = 0; i < n; ++i) list[offsets[keys[i]] + atomicAdd(&fill[keys[i]], 1u)] = (uint32_t)k;
-}
-
-// Occupancy of the (t-tile, u-tile) strips of N' rows: any tile of the strip touched.
-__global__ void strip_occ_kernel(Launch L, const uint8_t *__restrict__ tile_occ, int64_t ntiles,
-                                 uint8_t *__restrict__ col_occ) {
-    const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (t >= ntiles || !tile_occ[t]) return;
-    const int64_t c = (t / ((int64_t)L.ntu * L.ntv)) * L.ntu + t % L.ntu;
-    if (!col_occ[c]) col_occ[c] = 1;
+    for (int i = 0; i < n; ++i) list[atomicAdd(&cursor[keys[i]], 1u)] = (uint32_t)k;
 }
 
 // Statistics only (WS_FLAG_TIMING): occupied tiles and occupied (t-tile,
@@ -250,16 +310,17 @@ __device__ __forceinline__ uint32_t block_exclusive_scan(uint32_t v, uint32_t *t
     return before;
 }
 
-__global__ void __launch_bounds__(kScanThreads) scan_block_kernel(const uint32_t *__restrict__ in,
+// (the counts are replaced by a copy of the offsets, the scatter's cursors)
+__global__ void __launch_bounds__(kScanThreads) scan_block_kernel(uint32_t *__restrict__ counts,
                                                                   uint32_t *__restrict__ out,
                                                                   uint32_t *__restrict__ sums, int64_t n) {
     const int64_t base = (int64_t)blockIdx.x * kScanPerBlock + 4 * threadIdx.x;
     uint32_t a[4];
-    for (int i = 0; i < 4; ++i) a[i] = base + i < n ? in[base + i] : 0u;
+    for (int i = 0; i < 4; ++i) a[i] = base + i < n ? counts[base + i] : 0u;
     uint32_t local = a[0] + a[1] + a[2] + a[3], total;
     uint32_t run = block_exclusive_scan(local, &total);
     for (int i = 0; i < 4; ++i) {
-        if (base + i < n) out[base + i] = run;
+        if (base + i < n) out[base + i] = counts[base + i] = run;
         run += a[i];
     }
     if (threadIdx.x == 0) sums[blockIdx.x] = total;
@@ -277,9 +338,10 @@ __global__ void __launch_bounds__(kScanThreads) scan_sums_kernel(uint32_t *sums,
     }
 }
 
-__global__ void scan_add_kernel(uint32_t *__restrict__ out, const uint32_t *__restrict__ sums, int64_t n) {
+__global__ void scan_add_kernel(uint32_t *__restrict__ out, uint32_t *__restrict__ cursor,
+                                const uint32_t *__restrict__ sums, int64_t n) {
     int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < n) out[i] += sums[i / kScanPerBlock];
+    if (i < n) out[i] = cursor[i] = out[i] + sums[i / kScanPerBlock];
 }
 
 // ---------------------------------------------------------------------------
@@ -1049,11 +1111,31 @@ inline unsigned blocks_for(int64_t n, int threads) { return (unsigned)((n + thre
 // ---------------------------------------------------------------------------
 // Launchers
 // ---------------------------------------------------------------------------
-cudaError_t launch_prep(const ws_plan_s *p, const double *uvw, const float2 *vis, int64_t M, bool grid,
-                        cudaStream_t s) {
+cudaError_t launch_prep(const ws_plan_s *p, const double *uvw, int64_t M, cudaStream_t s) {
     if (M == 0) return cudaSuccess;
     const unsigned blocks = (unsigned)std::min<int64_t>(blocks_for(M, 256), (int64_t)p->sms * 8);
-    prep_kernel<<<blocks, 256, 0, s>>>(p->L, uvw, vis, M, grid ? 1 : 0, p->d_rec, p->d_drop);
+    prep_kernel<kPrepOnly><<<blocks, 256, 0, s>>>(p->L, uvw, nullptr, M, p->d_rec, p->d_drop, nullptr, nullptr, nullptr);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_clear_bins(const ws_plan_s *p, unsigned long long *drop, cudaStream_t s) {
+    const int64_t n = p->ntiles + 1;
+    const unsigned blocks = (unsigned)std::min<int64_t>(blocks_for(n, 256), (int64_t)p->sms * 8);
+    clear_bins_kernel<<<blocks, 256, 0, s>>>(p->d_counts, n, p->d_tile_occ, p->ntiles, p->d_col_occ,
+                                             (int64_t)p->L.ntt * p->L.ntu, drop);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_prep_count(const ws_plan_s *p, const double *uvw, const float2 *vis, int64_t M, bool grid,
+                              float2 *zeroed, cudaStream_t s) {
+    if (M == 0) return cudaSuccess;
+    const unsigned blocks = (unsigned)std::min<int64_t>(blocks_for(M, 256), (int64_t)p->sms * 8);
+    if (grid)
+        prep_kernel<kPrepGrid><<<blocks, 256, 0, s>>>(p->L, uvw, vis, M, p->d_rec, p->d_drop, p->d_counts,
+                                                      p->d_tile_occ, nullptr);
+    else
+        prep_kernel<kPrepDegrid><<<blocks, 256, 0, s>>>(p->L, uvw, nullptr, M, p->d_rec, p->d_drop, p->d_counts,
+                                                        p->d_tile_occ, zeroed);
     return cudaGetLastError();
 }
 
@@ -1064,30 +1146,34 @@ cudaError_t launch_bound_grid_records(const ws_plan_s *p, const double *uvw, con
     return cudaGetLastError();
 }
 
-cudaError_t launch_bin(ws_plan_s *p, int64_t M, bool grid, cudaStream_t s) {
-    const int64_t n = p->ntiles + 1;
-    cudaError_t e = cudaMemsetAsync(p->d_counts, 0, n * sizeof(uint32_t), s);
-    if (e == cudaSuccess) e = cudaMemsetAsync(p->d_tile_occ, 0, (size_t)p->ntiles, s);
-    if (e == cudaSuccess) e = cudaMemsetAsync(p->d_col_occ, 0, (size_t)p->L.ntt * p->L.ntu, s);
-    if (e != cudaSuccess) return e;
-    if (M > 0 && grid)
+cudaError_t launch_count(const ws_plan_s *p, int64_t M, bool grid, cudaStream_t s) {
+    cudaError_t e = launch_clear_bins(p, nullptr, s);
+    if (e != cudaSuccess || M == 0) return e;
+    if (grid)
         count_kernel<true><<<blocks_for(M, 256), 256, 0, s>>>(p->L, p->d_rec, M, p->d_counts, p->d_tile_occ);
-    else if (M > 0)
+    else
         count_kernel<false><<<blocks_for(M, 256), 256, 0, s>>>(p->L, p->d_rec, M, p->d_counts, p->d_tile_occ);
+    return cudaGetLastError();
+}
+
+int sort_launches(const ws_plan_s *p, int64_t M) { return (p->ntiles + 1 > kScanPerBlock ? 3 : 1) + (M > 0 ? 1 : 0); }
+
+cudaError_t launch_sort(const ws_plan_s *p, int64_t M, bool grid, cudaStream_t s) {
+    const int64_t n = p->ntiles + 1;
     const int nb = (int)((n + kScanPerBlock - 1) / kScanPerBlock);
     scan_block_kernel<<<nb, kScanThreads, 0, s>>>(p->d_counts, p->d_offsets, p->d_blocksums, n);
-    scan_sums_kernel<<<1, kScanThreads, 0, s>>>(p->d_blocksums, nb);
-    scan_add_kernel<<<blocks_for(n, 256), 256, 0, s>>>(p->d_offsets, p->d_blocksums, n);
+    if (nb > 1) {                                // one block's scan is the whole one
+        scan_sums_kernel<<<1, kScanThreads, 0, s>>>(p->d_blocksums, nb);
+        scan_add_kernel<<<blocks_for(n, 256), 256, 0, s>>>(p->d_offsets, p->d_counts, p->d_blocksums, n);
+    }
     if (M == 0) return cudaGetLastError();
-    e = cudaMemsetAsync(p->d_counts, 0, n * sizeof(uint32_t), s);
-    if (e != cudaSuccess) return e;
+    const unsigned vis_blocks = blocks_for(M, 256), blocks = vis_blocks + blocks_for(p->ntiles, 256);
     if (grid)
-        scatter_kernel<true><<<blocks_for(M, 256), 256, 0, s>>>(p->L, p->d_rec, M, p->d_offsets, p->d_counts,
-                                                               p->d_list);
+        scatter_kernel<true><<<blocks, 256, 0, s>>>(p->L, p->d_rec, M, (int)vis_blocks, p->d_counts, p->d_list,
+                                                    p->d_tile_occ, p->ntiles, p->d_col_occ);
     else
-        scatter_kernel<false><<<blocks_for(M, 256), 256, 0, s>>>(p->L, p->d_rec, M, p->d_offsets,
-                                                                p->d_counts, p->d_list);
-    strip_occ_kernel<<<blocks_for(p->ntiles, 256), 256, 0, s>>>(p->L, p->d_tile_occ, p->ntiles, p->d_col_occ);
+        scatter_kernel<false><<<blocks, 256, 0, s>>>(p->L, p->d_rec, M, (int)vis_blocks, p->d_counts, p->d_list,
+                                                     p->d_tile_occ, p->ntiles, p->d_col_occ);
     return cudaGetLastError();
 }
 
