@@ -353,11 +353,72 @@ __device__ __forceinline__ void dit_stage(float2 *buf, const FftPlan &P, int s, 
         if (kq > 0) twiddle_powers<R>(v, v1, v4);
         dft<R>(v, inv);
         if constexpr (LAST) {
-#pragma unroll
-            for (int m = 0; m < R; ++m) store(t, b + m * L, v[m]);
+            store(std::false_type{}, t, b, L, v);
         } else {
 #pragma unroll
             for (int m = 0; m < R; ++m) x[m * step] = v[m];
+        }
+    }
+}
+
+// Stages s (radix A) and s + 1 (radix B) in one pass: a thread holds the A B
+// elements k + m1 L + m2 A L of a block, does the B butterflies of the first stage
+// and then the A butterflies of the second, whose twiddles are those of k + m1 L.
+// For one transform (the rows; for the columns' pairs it was slower: N' = 2016, rows
+// 746 -> 650 us, columns 856 -> 896, on 68 planes).
+// The arithmetic is that of the two stages; one trip through shared memory and one
+// barrier less.
+template <int A, int B, bool LAST, class Store>
+__device__ __forceinline__ void dit_pair(float2 *buf, const FftPlan &P, int s, const float2 *__restrict__ tw, bool inv,
+                                         int tid, int nthr, Store &store) {
+    static_assert(B < 8, "the second radix takes its twiddles from w alone");
+    const int L = P.L[s], total = P.nb[s] / B, step_a = P.step[s], step_b = P.step[s + 1];
+    float2 w1, w4;
+    int base = 0, k = 0;
+    auto fetch = [&](int q) {                // as in dit_stage, for the first of the two stages
+        const int bq = min(q, total - 1);
+        const int blk = LAST ? 0 : div_small(bq, P.L_mul[s]);
+        k = bq - blk * L;
+        base = blk * A * B * L + k;
+        w1 = twiddle(tw, k * P.twstep[s], inv);
+        w4 = A >= 8 ? twiddle(tw, 4 * k * P.twstep[s], inv) : make_float2(1.f, 0.f);
+    };
+    fetch(tid);
+    __syncthreads();
+    for (int q = tid; q < total; q += nthr) {
+        const int b = base, kq = k;
+        const float2 v1 = w1, v4 = w4;
+        float2 *x = buf + b + div_small(b, P.chunk_mul);
+        float2 v[A * B], w[A];
+#pragma unroll
+        for (int m1 = 0; m1 < A; ++m1) w[m1] = twiddle(tw, (kq + m1 * L) * P.twstep[s + 1], inv);
+#pragma unroll
+        for (int m2 = 0; m2 < B; ++m2)
+#pragma unroll
+            for (int m1 = 0; m1 < A; ++m1) v[m1 + A * m2] = x[m1 * step_a + m2 * step_b];
+        fetch(q + nthr);
+#pragma unroll
+        for (int m2 = 0; m2 < B; ++m2) {
+            if (kq > 0) twiddle_powers<A>(v + A * m2, v1, v4);
+            dft<A>(v + A * m2, inv);
+        }
+#pragma unroll
+        for (int m1 = 0; m1 < A; ++m1) {
+            float2 c[B];
+#pragma unroll
+            for (int m2 = 0; m2 < B; ++m2) c[m2] = v[m1 + A * m2];
+            if (m1 > 0 || kq > 0) twiddle_powers<B>(c, w[m1], w[m1]);
+            dft<B>(c, inv);
+#pragma unroll
+            for (int m2 = 0; m2 < B; ++m2) v[m1 + A * m2] = c[m2];
+        }
+        if constexpr (LAST) {
+            store(std::false_type{}, 0, b, L, v);
+        } else {
+#pragma unroll
+            for (int m2 = 0; m2 < B; ++m2)
+#pragma unroll
+                for (int m1 = 0; m1 < A; ++m1) x[m1 * step_a + m2 * step_b] = v[m1 + A * m2];
         }
     }
 }
@@ -393,8 +454,7 @@ __device__ __forceinline__ void dit_last_held(float2 *buf, const FftPlan &P, con
         if (k >= nb) break;
         if (k > 0) twiddle_powers<R>(v[i], w1[i], w4[i]);
         dft<R>(v[i], inv);
-#pragma unroll
-        for (int m = 0; m < R; ++m) store(0, k + m * L, v[i][m]);
+        store(std::false_type{}, 0, k, L, v[i]);
     }
 }
 
@@ -419,8 +479,7 @@ __device__ __forceinline__ void dit_first(float2 *buf, const FftPlan &P, bool in
     for (int q = tid; q < total; q += nthr) {
         const int t = q % COUNT, j = q / COUNT;
         float2 v[R];
-#pragma unroll
-        for (int m = 0; m < R; ++m) v[m] = load(t, m * nb + j);
+        load(std::false_type{}, t, j, nb, v);
         dft<R>(v, inv);
         float2 *x = buf + t * P.stride + first_slot(P, j);
 #pragma unroll
@@ -473,6 +532,20 @@ __device__ __forceinline__ void with_forward_later(int r, F f) {
         default: f(Radix<3>{}); break;
     }
 }
+// The pairs of consecutive forward radices that run as one pass (fft_make_plan): f(Radix<A>, Radix<B>).
+template <class F>
+__device__ __forceinline__ void with_forward_pair(int a, int b, F f) {
+    switch (16 * a + b) {
+        case 16 * 4 + 7: f(Radix<4>{}, Radix<7>{}); break;
+        case 16 * 4 + 5: f(Radix<4>{}, Radix<5>{}); break;
+        case 16 * 4 + 3: f(Radix<4>{}, Radix<3>{}); break;
+        case 16 * 7 + 3: f(Radix<7>{}, Radix<3>{}); break;
+        case 16 * 5 + 5: f(Radix<5>{}, Radix<5>{}); break;
+        case 16 * 5 + 3: f(Radix<5>{}, Radix<3>{}); break;
+        case 16 * 8 + 3: f(Radix<8>{}, Radix<3>{}); break;
+        default: f(Radix<3>{}, Radix<3>{}); break;
+    }
+}
 template <class F>
 __device__ __forceinline__ void with_first_radix(int r, F f) {
     switch (r) {
@@ -515,38 +588,62 @@ __device__ __forceinline__ void with_last_radix(int r, F f) {
 
 }  // namespace fftdev
 
-// Transform COUNT sequences of length P.n from load(t, e) to store(t, e, v)
-// (t < COUNT), using the shared buffers buf + t * P.stride between stages.
+// Transform COUNT sequences of length P.n, using the shared buffers buf + t * P.stride between stages.
 // All threads of the CTA must call it; shared buffers may be reused after the
 // caller's next barrier.
+// The stages between the first and the last pass; returns the last pass's (first) stage.
 template <int COUNT, bool INV>
-__device__ __forceinline__ void fft_middle_stages(float2 *buf, const FftPlan &P, const float2 *__restrict__ tw, int tid,
-                                                  int nthr) {
-    auto none = [](int, int, float2) {};
-    for (int s = 1; s < P.nstages - 1; ++s) {
+__device__ __forceinline__ int fft_middle_stages(float2 *buf, const FftPlan &P, const float2 *__restrict__ tw, int tid,
+                                                 int nthr) {
+    auto none = [](auto, int, int, int, auto &) {};
+    int s = 1;
+    auto fused = [&](int i) { return COUNT == 1 && !INV ? P.fuse[i] : 0; };     // rows only (FftPlan)
+    while (s + fused(s) < P.nstages - 1) {
         auto stage = [&](auto r) {
             fftdev::dit_stage<decltype(r)::value, COUNT, false>(buf, P, s, tw, INV, tid, nthr, none);
         };
-        if constexpr (INV)
+        if constexpr (INV) {
             fftdev::with_middle_radix(P.radix[s], stage);
-        else
+        } else if (fused(s)) {
+            if constexpr (COUNT == 1)
+                fftdev::with_forward_pair(P.radix[s], P.radix[s + 1], [&](auto ra, auto rb) {
+                    fftdev::dit_pair<decltype(ra)::value, decltype(rb)::value, false>(buf, P, s, tw, INV, tid, nthr, none);
+                });
+        } else {
             fftdev::with_forward_later(P.radix[s], stage);
+        }
+        s += 1 + fused(s);
     }
+    return s;
 }
 
 template <int COUNT, bool INV, class Store>
-__device__ __forceinline__ void fft_last_stage(float2 *buf, const FftPlan &P, const float2 *__restrict__ tw, int tid,
-                                               int nthr, Store &store) {
-    const int last = P.nstages - 1;
+__device__ __forceinline__ void fft_last_stage(float2 *buf, const FftPlan &P, const float2 *__restrict__ tw, int last,
+                                               int tid, int nthr, Store &store) {
     auto stage = [&](auto r) {
         fftdev::dit_stage<decltype(r)::value, COUNT, true>(buf, P, last, tw, INV, tid, nthr, store);
     };
-    if constexpr (INV)
+    if constexpr (INV) {
         fftdev::with_last_radix(P.radix[last], stage);
-    else
+    } else {
+        if constexpr (COUNT == 1)
+            if (P.fuse[last]) {
+                fftdev::with_forward_pair(P.radix[last], P.radix[last + 1], [&](auto ra, auto rb) {
+                    fftdev::dit_pair<decltype(ra)::value, decltype(rb)::value, true>(buf, P, last, tw, INV, tid, nthr, store);
+                });
+                return;
+            }
         fftdev::with_forward_later(P.radix[last], stage);
+    }
 }
 
+//
+// load(t, e0, step, v) fills a first-stage butterfly's inputs v[m], element e0 +
+// m step of transform t (t < COUNT), and store(t, e0, step, v) takes a last-stage
+// butterfly's outputs; both get a whole butterfly, so that what they read from
+// shared memory is under way before what they write (element by element, each
+// read waited for the write before it).  Under PRUNE_IN / PRUNE_OUT only the
+// first and last quarter of v counts (first argument: whether that is so).
 template <int COUNT, bool INV, class Load, class Store>
 __device__ __forceinline__ void fft_many(float2 *buf, const FftPlan &P, const float2 *__restrict__ tw, int tid,
                                          int nthr, Load load, Store store) {
@@ -557,8 +654,8 @@ __device__ __forceinline__ void fft_many(float2 *buf, const FftPlan &P, const fl
         fftdev::with_first_radix(P.radix[0], first);
     else
         fftdev::with_forward_first(P.radix[0], first);
-    fft_middle_stages<COUNT, INV>(buf, P, tw, tid, nthr);
-    fft_last_stage<COUNT, INV>(buf, P, tw, tid, nthr, store);
+    const int last = fft_middle_stages<COUNT, INV>(buf, P, tw, tid, nthr);
+    fft_last_stage<COUNT, INV>(buf, P, tw, last, tid, nthr, store);
 }
 
 // One inverse transform whose input sits in buf in natural order (see
@@ -570,13 +667,13 @@ __device__ __forceinline__ void fft_inplace(float2 *buf, const FftPlan &P, const
     fftdev::with_first_radix(P.radix[0], [&](auto r) {
         fftdev::dit_first_inplace<decltype(r)::value>(buf, P, true, tid, live);
     });
-    fft_middle_stages<1, true>(buf, P, tw, tid, nthr);
+    const int last = fft_middle_stages<1, true>(buf, P, tw, tid, nthr);
     if constexpr (HELD)
-        fftdev::with_last_radix(P.radix[P.nstages - 1], [&](auto r) {
+        fftdev::with_last_radix(P.radix[last], [&](auto r) {
             fftdev::dit_last_held<decltype(r)::value>(buf, P, tw, true, tid, nthr, between, store);
         });
     else
-        fft_last_stage<1, true>(buf, P, tw, tid, nthr, store);
+        fft_last_stage<1, true>(buf, P, tw, last, tid, nthr, store);
 }
 
 // -- compile-time plans for the power-of-two sizes -----------------------------
@@ -622,9 +719,7 @@ __device__ __forceinline__ void first(float2 *buf, bool inv, int tid, Load &load
     for (int q = tid; q < total; q += T) {
         const int t = q % COUNT, j = q / COUNT;
         float2 v[R];
-#pragma unroll
-        for (int m = 0; m < R; ++m)
-            if (!pin || m < R / 4 || m >= 3 * R / 4) v[m] = load(t, m * nb + j);
+        load(std::bool_constant<pin>{}, t, j, nb, v);
         if constexpr (pin)
             fftdev::dft16_zero_middle(v, inv);
         else
@@ -714,9 +809,7 @@ __device__ __forceinline__ void later(float2 *buf, const float2 *__restrict__ tw
         if (k > 0) fftdev::twiddle_powers<R>(v, v1, v4);
         fftdev::dft<R>(v, inv);
         if constexpr (LAST) {
-#pragma unroll
-            for (int m = 0; m < R; ++m)
-                if (!pout || m < R / 4 || m >= 3 * R / 4) store(t, base + m * L, v[m]);
+            store(std::bool_constant<pout>{}, t, base, L, v);
         } else {
 #pragma unroll
             for (int m = 0; m < R; ++m) x[at(pbase, base, m)] = v[m];
@@ -747,9 +840,7 @@ __device__ __forceinline__ void last_held(float2 *buf, int tid, bool inv, const 
         const int k = tid + i * T;
         if (k > 0) fftdev::twiddle_powers<R>(v[i], pre.w1[Pre::kept == 1 ? 0 : i], pre.w4[Pre::kept == 1 ? 0 : i]);
         fftdev::dft<R>(v[i], inv);
-#pragma unroll
-        for (int m = 0; m < R; ++m)
-            if (!pout || m < R / 4 || m >= 3 * R / 4) store(0, k + m * L, v[i][m]);
+        store(std::bool_constant<pout>{}, 0, k, L, v[i]);
     }
 }
 
@@ -788,7 +879,155 @@ struct RowTw {
     }
 };
 
+// -- two-stage transforms of 4096 = 64 x 64 points ------------------------------
+//
+// A thread transforms 64 points in registers (128 of them), so a sequence goes
+// through shared memory once instead of twice and a CTA has one barrier:
+//   X[k1 + 64 k2] = sum_j w64^(j k2) w4096^(j k1) sum_m x[j + 64 m] w64^(m k1)
+// with thread j in the first stage and thread k1 in the second.  Radix 64 is 8 x 8.
+
+// cos and sin of 2 pi m / 64 for m = 0..63 (decimal expansions over an eighth of the circle)
+__host__ __device__ constexpr double cos64(int m) {
+    constexpr double c[9] = {1.0, 0.99518472667219688624, 0.98078528040323044913, 0.95694033573220886494,
+                             0.92387953251128675613, 0.88192126434835502971, 0.83146961230254523708,
+                             0.77301045336273696081, 0.70710678118654752440};
+    constexpr double s[9] = {0.0, 0.09801714032956060199, 0.19509032201612826785, 0.29028467725446236764,
+                             0.38268343236508977173, 0.47139673682599764856, 0.55557023301960222474,
+                             0.63439328416364549822, 0.70710678118654752440};
+    const int r = m & 63, q = r >= 32 ? 64 - r : r;                  // cos is even about 0 and 32
+    const int h = q > 16 ? 32 - q : q;                               // and odd about 16
+    const double v = h <= 8 ? c[h] : s[16 - h];
+    return q > 16 ? -v : v;
+}
+__host__ __device__ constexpr double sin64(int m) { return cos64(m + 48); }
+
+// v[8 b + q] *= w64^(b q), forward or inverse, for the constants of one b
+template <int B, int Q = 1>
+__device__ __forceinline__ void mul_w64(float2 *v, bool inv) {
+    if constexpr (Q < 8) {
+        constexpr float c = (float)cos64(B * Q), s = (float)sin64(B * Q);
+        v[8 * B + Q] = inv ? cmul_rot(v[8 * B + Q], make_float2(c, s), make_float2(-s, c))
+                           : cmul_rot(v[8 * B + Q], make_float2(c, -s), make_float2(s, c));
+        mul_w64<B, Q + 1>(v, inv);
+    }
+}
+template <int B = 1>
+__device__ __forceinline__ void mul_w64_all(float2 *v, bool inv) {
+    if constexpr (B < 8) {
+        mul_w64<B>(v, inv);
+        mul_w64_all<B + 1>(v, inv);
+    }
+}
+
+// 8-point DFT of (a0, a1, 0, 0, 0, 0, a6, a7) (v[2..5] need not be set)
+__device__ __forceinline__ void dft8_zero_middle(float2 *v, bool inv) {
+    // even inputs (v0, 0, 0, v6), odd inputs (v1, 0, 0, v7)
+    const float2 e0 = cadd(v[0], v[6]), e2 = csub(v[0], v[6]), e1 = sub_rot(v[0], v[6], inv), e3 = add_rot(v[0], v[6], inv);
+    const float2 o0 = cadd(v[1], v[7]), o2 = csub(v[1], v[7]);
+    const float2 o1 = fftdev::mul_w16(sub_rot(v[1], v[7], inv), 2, inv);
+    const float2 o3 = fftdev::mul_w16(add_rot(v[1], v[7], inv), 6, inv);
+    v[0] = cadd(e0, o0);
+    v[4] = csub(e0, o0);
+    v[1] = cadd(e1, o1);
+    v[5] = csub(e1, o1);
+    v[2] = add_rot(e2, o2, inv);
+    v[6] = sub_rot(e2, o2, inv);
+    v[3] = cadd(e3, o3);
+    v[7] = csub(e3, o3);
+}
+
+// In-register 64-point DFT: v[8 a + b], a, b < 8, becomes output q + 8 p in v[8 q + p].
+// PIN: only a = 0, 1, 6, 7 are non-zero (the others need not be set).
+template <bool PIN>
+__device__ __forceinline__ void dft64_over_a(float2 *v, bool inv) {
+    float2 o[64];
+#pragma unroll
+    for (int b = 0; b < 8; ++b) {
+        float2 c[8];
+#pragma unroll
+        for (int a = 0; a < 8; ++a)
+            if (!PIN || a < 2 || a > 5) c[a] = v[8 * a + b];
+        if constexpr (PIN)
+            dft8_zero_middle(c, inv);
+        else
+            fftdev::dft<8>(c, inv);
+#pragma unroll
+        for (int q = 0; q < 8; ++q) o[8 * b + q] = c[q];
+    }
+#pragma unroll
+    for (int i = 0; i < 64; ++i) v[i] = o[i];           // v[8 b + q]
+}
+__device__ __forceinline__ void dft64_over_b(float2 *v, bool inv) {
+    mul_w64_all(v, inv);
+    float2 o[64];
+#pragma unroll
+    for (int q = 0; q < 8; ++q) {
+        float2 c[8];
+#pragma unroll
+        for (int b = 0; b < 8; ++b) c[b] = v[8 * b + q];
+        fftdev::dft<8>(c, inv);
+#pragma unroll
+        for (int p = 0; p < 8; ++p) o[8 * q + p] = c[p];
+    }
+#pragma unroll
+    for (int i = 0; i < 64; ++i) v[i] = o[i];
+}
+
+// v[8 r + i] *= w^r for r = 1..7, all i (the powers are products at most three deep)
+__device__ __forceinline__ void mul_rows(float2 *v, float2 w) {
+    const fftdev::Tw t1(w), t2(t1.times(w)), t4(t2.times(t2.w));
+    auto row = [&](int r, const fftdev::Tw &t) {
+#pragma unroll
+        for (int i = 0; i < 8; ++i) v[8 * r + i] = t.times(v[8 * r + i]);
+    };
+    row(1, t1);
+    row(2, t2);
+    row(4, t4);
+    row(5, fftdev::Tw(t1.times(t4.w)));
+    row(6, fftdev::Tw(t2.times(t4.w)));
+    const fftdev::Tw t3(t1.times(t2.w));
+    row(3, t3);
+    row(7, fftdev::Tw(t3.times(t4.w)));
+}
+
+constexpr int kPitch64 = 65;                             // row pitch of the exchange, in points
+constexpr int kStride64 = 64 * kPitch64 + 8;             // points per sequence; 8 (mod 16)
+
 }  // namespace fftst
+
+// COUNT sequences of 4096 points by 64 COUNT threads (load and store as for
+// fft_many, 64 points each; under PRUNE_IN / PRUNE_OUT the first and last quarter).
+template <int COUNT, int PRUNE, class Load, class Store>
+__device__ __forceinline__ void fft_4096_two_stage(float2 *buf, const float2 *__restrict__ tw, bool inv, int tid,
+                                                   Load load, Store store) {
+    using namespace fftst;
+    const int t = tid % COUNT, j = tid / COUNT;
+    float2 *x = buf + t * kStride64;
+    // w^1 and w^8 of this thread's second stage
+    const float2 w1 = fftdev::twiddle(tw, j, inv), w8 = fftdev::twiddle(tw, 8 * j, inv);
+    float2 v[64];
+    load(std::bool_constant<(PRUNE & PRUNE_IN) != 0>{}, t, j, 64, v);
+    dft64_over_a<(PRUNE & PRUNE_IN) != 0>(v, inv);
+    dft64_over_b(v, inv);
+#pragma unroll
+    for (int q = 0; q < 8; ++q)
+#pragma unroll
+        for (int p = 0; p < 8; ++p) x[(q + 8 * p) * kPitch64 + j] = v[8 * q + p];
+    __syncthreads();
+#pragma unroll
+    for (int i = 0; i < 64; ++i) v[i] = x[j * kPitch64 + i];
+    // w^(8 a + b) = (w^8)^a w^b: the first factor before the DFTs over a, the second after
+    mul_rows(v, w8);
+    dft64_over_a<false>(v, inv);
+    mul_rows(v, w1);
+    dft64_over_b(v, inv);
+    float2 o[64];
+#pragma unroll
+    for (int q = 0; q < 8; ++q)
+#pragma unroll
+        for (int p = 0; p < 8; ++p) o[q + 8 * p] = v[8 * q + p];
+    store(std::bool_constant<(PRUNE & PRUNE_OUT) != 0>{}, t, j, 64, o);
+}
 
 // One transform of the compile-time size N by T threads: input in buf in
 // natural order (see first_inplace for live; HELD as in fft_inplace), or read through load.

@@ -25,6 +25,7 @@ struct FftPlan {
     int nb[kMaxFftStages];          // butterflies of stage s: n / radix[s]
     int twstep[kMaxFftStages];      // n / (radix[s] L[s])
     int step[kMaxFftStages];        // slots from one element of a butterfly to the next
+    int fuse[kMaxFftStages];        // 1: this stage and the next run as one pass (rows of forward plans)
     int gw[kMaxFftStages];          // first-stage digit reversal: gw[i] = radix[1] * ... * radix[i-1]
     // div_mul of: L[s]; the digit weight radix[s+1] * ...; radix[s]; and of chunk.
     // x / d = umulhi(x, mul) exactly for 0 <= x < 2^16 and d < 2^13, since

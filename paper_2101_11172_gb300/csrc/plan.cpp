@@ -171,7 +171,10 @@ double butterfly_cost(int r) {
         case 6: dft = 22; break;
         case 7: dft = 36; break;
         case 8: dft = 26; break;
+        case 9: dft = 60; break;
         case 10: dft = 46; break;
+        case 15: dft = 140; break;
+        case 25: dft = 330; break;
         case 12: dft = 56; break;
         case 14: dft = 86; break;
         case 16: dft = 80; break;
@@ -300,6 +303,28 @@ int inverse_radices(int n, int *best) {
     return nbest;
 }
 
+// Which forward stages run as one pass with the next in the rows (dit_pair): the pairs that
+// fft.cuh has, chosen for the fewest passes after the first stage, e.g. 2016 = 8 (4 7)
+// (3 3), 3072 = 16 8 (8 3), 1344 = 8 8 (7 3).  The arithmetic is the stages' own.
+void fuse_stages(const int *radix, int ns, int *fuse) {
+    auto pair = [](int a, int b) {
+        return (a == 4 && (b == 7 || b == 5 || b == 3)) || (b == 5 && a == 5) ||
+               (b == 3 && (a == 3 || a == 5 || a == 7 || a == 8));
+    };
+    int passes[kMaxFftStages + 2] = {};                  // fewest passes from stage s on
+    for (int s = ns - 1; s >= 1; --s) {
+        passes[s] = 1 + passes[s + 1];
+        fuse[s] = 0;
+        if (s + 1 < ns && pair(radix[s], radix[s + 1]) && 1 + passes[s + 2] < passes[s]) {
+            passes[s] = 1 + passes[s + 2];
+            fuse[s] = 1;
+        }
+    }
+    fuse[0] = 0;
+    for (int s = 1; s < ns; ++s)
+        if (fuse[s]) fuse[++s] = 0;                      // a pair's second stage starts none
+}
+
 // Bank conflicts of a plan's shared-memory accesses by `count` interleaved
 // transforms: the sum over all half-warp accesses (16 lanes of 8 bytes) of the
 // lanes on the fullest bank pair.
@@ -308,7 +333,9 @@ long fft_conflicts(const FftPlan &F, int chunk, int stride, int count) {
     auto slot = [&](int e) { return e + e / chunk; };
     long total = 0;
     for (int s = 0; s < ns; ++s) {
-        const int R = F.radix[s], L = F.L[s], items = std::min(count * F.nb[s], 512);
+        const bool fused = count == 1 && F.fuse[s];
+        const int R = F.radix[s] * (fused ? F.radix[s + 1] : 1), L = F.L[s];
+        const int items = std::min(count * (F.n / R), 512);
         for (int q0 = 0; q0 < items; q0 += 16) {
             int at[16], n = std::min(16, items - q0);
             for (int i = 0; i < n; ++i) {
@@ -320,7 +347,7 @@ long fft_conflicts(const FftPlan &F, int chunk, int stride, int count) {
                         g += (rest % F.radix[k]) * F.gw[k];
                         rest /= F.radix[k];
                     }
-                    e = g * R;
+                    e = g * F.radix[0];
                 } else {
                     e = b / L * R * L + b % L;
                 }
@@ -330,6 +357,7 @@ long fft_conflicts(const FftPlan &F, int chunk, int stride, int count) {
             for (int i = 0; i < n; ++i) worst = std::max(worst, ++bank[at[i] % 16]);
             total += (long)worst * R;
         }
+        s += fused;
     }
     return total;
 }
@@ -342,6 +370,10 @@ bool fft_make_plan(int n, bool inverse, FftPlan *F) {
     if (ns < 2) return false;
     F->n = n;
     F->nstages = ns;
+    for (int &f : F->fuse) f = 0;
+    if (!inverse) fuse_stages(radix, ns, F->fuse);
+    int passes[kMaxFftStages] = {}, np = 0;              // the radix of each pass of a row
+    for (int s = 0; s < ns; s += 1 + F->fuse[s]) passes[np++] = radix[s] * (F->fuse[s] ? radix[s + 1] : 1);
     int L = 1, gw = 1;
     for (int s = 0; s < ns; ++s) {
         const int r = radix[s];
@@ -373,7 +405,7 @@ bool fft_make_plan(int n, bool inverse, FftPlan *F) {
     for (int s = 0; s < ns; ++s) F->step[s] = F->L[s] >= chunk ? F->L[s] + F->L[s] / chunk : F->L[s];
     // the compile-time plans of fft.cuh pad at most 17 slots
     F->stride = stride_of(std::max(n + n / chunk, n + 17));
-    F->row_threads = best_threads(radix, ns, n, 1, row_smem(n, inverse), inverse ? F->nb[0] : 32, nullptr);
+    F->row_threads = best_threads(passes, np, n, 1, row_smem(n, inverse), inverse ? F->nb[0] : 32, nullptr);
     F->col_threads = best_threads(radix, ns, n, 2, 16 * (size_t)n, 32, nullptr);
     // boxes of at most 256 column blocks whose size keeps shared-memory addresses 128-byte aligned
     const int blocks = n / 4;

@@ -35,7 +35,7 @@ WS_HD constexpr int row_threads_max() {
 }
 template <int NP>
 WS_HD constexpr int col_threads_max() {
-    return NP ? (NP > 2048 ? 256 : NP / 8) : kMaxFftThreads;
+    return NP ? (NP > 2048 ? 128 : NP / 8) : kMaxFftThreads;
 }
 template <int NP>
 WS_HD constexpr int row_ctas() {
@@ -43,7 +43,7 @@ WS_HD constexpr int row_ctas() {
 }
 template <int NP>
 WS_HD constexpr int col_ctas() {
-    return NP ? 768 / col_threads_max<NP>() : 2;
+    return NP == 4096 ? 3 : NP ? 768 / col_threads_max<NP>() : 2;
 }
 // Row CTAs that an SM can hold by threads and registers, and the shared memory
 // that each may have for `ctas` of them to fit (228 KB per SM, 1 KB of it reserved per CTA).
@@ -63,8 +63,22 @@ __device__ __forceinline__ void column_fft(float2 *buf, const FftPlan &F, const 
                                            Store store) {
     if constexpr (NP == 0)
         fft_many<kPerCta, INV>(buf, F, tw, threadIdx.x, blockDim.x, load, store);
+    else if constexpr (NP == 4096)
+        fft_4096_two_stage<kPerCta, PRUNE>(buf, tw, INV, threadIdx.x, load, store);
     else
         fft_static<NP, kPerCta, col_threads_max<NP>(), PRUNE>(buf, tw, INV, threadIdx.x, load, store);
+}
+
+// Calls f(m) for the elements of a butterfly of R that count: all of them, or the first and last quarter.
+template <int R, bool PRUNED, class F>
+__device__ __forceinline__ void for_live(F f) {
+#pragma unroll
+    for (int m = 0; m < R; ++m)
+        if (!PRUNED || m < R / 4 || m >= 3 * R / 4) f(m);
+}
+template <class A>
+__device__ __forceinline__ constexpr int length_of() {
+    return (int)std::extent<std::remove_reference_t<A>>::value;
 }
 
 // The twiddle bases a row kernel's thread keeps across planes.
@@ -85,6 +99,12 @@ template <int NP>
 inline bool crop_half(const Launch &L) { return NP >= 512 && 2 * L.N == L.Np; }
 
 // -- degridding --------------------------------------------------------------
+
+// g times e, the screened value one plane on, with the products rounded in a fixed
+// order: (g.x e.x - g.y e.y, g.y e.x + g.x e.y), those with e.y first.
+__device__ __forceinline__ float2 step_screen(float2 g, float2 e) {
+    return fma2(g, dup2(e.x), mul2(swap2(g), make_float2(-e.y, e.y)));
+}
 
 // Planes per exact evaluation of the screen in fwd_rows: in between, each
 // pixel's screened value advances one plane by a product with exp(-2 pi i z).
@@ -154,19 +174,50 @@ fwd_rows_kernel(Launch L, FftPlan F, const float2 *__restrict__ tw, const float2
             __syncthreads();
         }
         const bool step = (p + 1 - p_begin) % kScreenSteps != 0 && p + 1 < p_end;   // uniform: advance g
-        auto load = [&](int, int J) -> float2 {
-            if (!in_crop(J, half, Np)) return make_float2(0.f, 0.f);
-            const int jj = grid_to_crop(J, half, Np);
-            const float2 g = grow[jj];
-            if (step) {
-                const float2 e = erow[jj];
-                grow[jj] = make_float2(g.x * e.x - g.y * e.y, g.x * e.y + g.y * e.x);
+        auto load = [&](auto pruned, int, int J0, int dJ, auto &v) {
+            constexpr int R = length_of<decltype(v)>();
+            constexpr bool P = decltype(pruned)::value;
+            if constexpr (NP == 0) {
+                // (runtime plans: reading all steps first took more registers than it saved time)
+                for_live<R, P>([&](int m) {
+                    const int J = J0 + m * dJ, jj = grid_to_crop(J, half, Np);
+                    v[m] = make_float2(0.f, 0.f);
+                    if (!in_crop(J, half, Np)) return;
+                    v[m] = grow[jj];
+                    if (step) grow[jj] = step_screen(v[m], erow[jj]);
+                });
+                return;
             }
-            return g;
+            for_live<R, P>([&](int m) {
+                const int J = J0 + m * dJ;
+                v[m] = in_crop(J, half, Np) ? grow[grid_to_crop(J, half, Np)] : make_float2(0.f, 0.f);
+            });
+            if (!step) return;
+            float2 e[R];
+            for_live<R, P>([&](int m) {
+                const int J = J0 + m * dJ;
+                if (in_crop(J, half, Np)) e[m] = erow[grid_to_crop(J, half, Np)];
+            });
+            for_live<R, P>([&](int m) {
+                const int J = J0 + m * dJ;
+                if (in_crop(J, half, Np)) grow[grid_to_crop(J, half, Np)] = step_screen(v[m], e[m]);
+            });
         };
         // columns of this plane's t-tile that no footprint touches are never read
-        auto store = [&](int, int R, float2 v) {
-            if (occ[R / TU]) __stcs(plane + tiled_index(ii, R, Np), v);
+        auto store = [&](auto, int, int R0, int dR, auto &v) {
+            if (NP == 0 && dR % TU == 0) {                       // whole strips apart: one address and a stride
+                float2 *at = plane + tiled_index(ii, R0, Np);
+                const size_t stride = (size_t)(dR / CB) * Np * CB;
+                const uint8_t *strip = occ + R0 / TU;
+                for_live<length_of<decltype(v)>(), false>([&](int m) {
+                    if (strip[m * (dR / TU)]) __stcs(at + m * stride, v[m]);
+                });
+                return;
+            }
+            for_live<length_of<decltype(v)>(), false>([&](int m) {
+                const int R = R0 + m * dR;
+                if (occ[R / TU]) __stcs(plane + tiled_index(ii, R, Np), v[m]);
+            });
         };
         if constexpr (NP >= 512)
             fft_static_row<NP, row_threads_max<NP>(), CROP ? fftst::PRUNE_IN : 0>(sbuf, false, tid, load, store, rt);
@@ -175,27 +226,55 @@ fwd_rows_kernel(Launch L, FftPlan F, const float2 *__restrict__ tw, const float2
     }
 }
 
+// A column CTA is short and waits for its columns' loads at DRAM latency.  In the
+// forward direction, whose loads are the N rows of a block in one run, the CTA of
+// a block's first column pair asks L2 for the rows of the block `ahead` CTAs later
+// (about the CTAs resident at once; 0: it does not).  Worth it from N = 2048 on (366
+// planes of N' = 4096: 10.98 -> 10.40 ms; N = 1024: 1.41 -> 1.43); inverse, where the
+// loads are the occupied tiles, 512 bytes each, it cost more than it gave (10.96 -> 11.27).
+constexpr int kAheadMinImage = 2048;
+__device__ __forceinline__ void fetch_columns_ahead(const Launch &L, const uint8_t *__restrict__ col_occ, int plane0,
+                                                    int ahead, const float2 *__restrict__ stack) {
+    if (ahead == 0 || (blockIdx.x & 1) || threadIdx.x >= 4) return;      // a quarter of the rows each
+    const unsigned x = blockIdx.x + (unsigned)ahead, pair = x % gridDim.x, plane = blockIdx.y + x / gridDim.x;
+    if (plane >= gridDim.y || plane0 + (int)plane >= L.Nw) return;
+    if (!col_occ[(plane0 + (int)plane) / TT * L.ntu + (int)pair * kPerCta / TU]) return;
+    const unsigned bytes = (unsigned)(L.N / 4 * CB * sizeof(float2));
+    const char *block = reinterpret_cast<const char *>(stack + (size_t)plane * L.Np * L.Np +
+                                                       (size_t)(pair * kPerCta / CB) * L.Np * CB);
+    asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(
+                     __cvta_generic_to_global(block + (size_t)threadIdx.x * bytes)),
+                 "r"(bytes)
+                 : "memory");
+}
+
 template <int NP, bool CROP>
 __global__ void __launch_bounds__(col_threads_max<NP>(), col_ctas<NP>())
 fwd_cols_kernel(Launch L, FftPlan F, const float2 *__restrict__ tw, const uint8_t *__restrict__ tile_occ,
-                const uint8_t *__restrict__ col_occ, int plane0, float2 *__restrict__ stack) {
+                const uint8_t *__restrict__ col_occ, int plane0, int ahead, float2 *__restrict__ stack) {
     extern __shared__ __align__(16) float2 sbuf[];
     const int Np = L.Np, half = L.N / 2;
+    fetch_columns_ahead(L, col_occ, plane0, ahead, stack);
     const int R0 = blockIdx.x * kPerCta;                  // two of the four columns of a block
     const int tt = (plane0 + (int)blockIdx.y) / TT, tu = R0 / TU;
     if (plane0 + (int)blockIdx.y >= L.Nw) return;         // padding planes of the last t-tile: never read
     if (!col_occ[tt * L.ntu + tu]) return;                // no visibility reads these columns of this plane
     float2 *blk = stack + (size_t)blockIdx.y * Np * Np + (size_t)(R0 >> 2) * Np * CB + (R0 & 3);
-    uint8_t *occ = reinterpret_cast<uint8_t *>(sbuf + kPerCta * F.stride);
+    uint8_t *occ = reinterpret_cast<uint8_t *>(sbuf + kPerCta * (NP == 4096 ? fftst::kStride64 : F.stride));
     for (int i = threadIdx.x; i < L.ntv; i += blockDim.x) occ[i] = tile_occ[((size_t)tt * L.ntv + i) * L.ntu + tu];
     __syncthreads();
     // rows 0..N-1 hold the N transformed image rows; every other row is zero padding
-    auto load = [&](int b, int S) -> float2 {
-        if (!in_crop(S, half, Np)) return make_float2(0.f, 0.f);
-        return __ldcs(blk + (size_t)grid_to_crop(S, half, Np) * CB + b);
+    auto load = [&](auto pruned, int b, int S0, int dS, auto &v) {
+        for_live<length_of<decltype(v)>(), decltype(pruned)::value>([&](int m) {
+            const int S = S0 + m * dS;
+            v[m] = in_crop(S, half, Np) ? __ldcs(blk + (size_t)grid_to_crop(S, half, Np) * CB + b) : make_float2(0.f, 0.f);
+        });
     };
-    auto store = [&](int b, int S, float2 v) {
-        if (occ[S >> L.tv_log]) blk[(size_t)S * CB + b] = v;     // only tiles the gather reads
+    auto store = [&](auto, int b, int S0, int dS, auto &v) {
+        for_live<length_of<decltype(v)>(), false>([&](int m) {
+            const int S = S0 + m * dS;
+            if (occ[S >> L.tv_log]) blk[(size_t)S * CB + b] = v[m];     // only tiles the gather reads
+        });
     };
     column_fft<NP, false, CROP ? fftst::PRUNE_IN : 0>(sbuf, F, tw, load, store);
 }
@@ -213,16 +292,22 @@ inv_cols_kernel(Launch L, FftPlan F, const float2 *__restrict__ tw, const uint8_
     if (plane0 + (int)blockIdx.y >= L.Nw) return;         // padding planes of the last t-tile: inv_rows skips them
     if (!col_occ[tt * L.ntu + tu]) return;                // all-zero columns: inv_rows skips them too
     float2 *blk = stack + (size_t)blockIdx.y * Np * Np + (size_t)(R0 >> 2) * Np * CB + (R0 & 3);
-    uint8_t *occ = reinterpret_cast<uint8_t *>(sbuf + kPerCta * F.stride);
+    uint8_t *occ = reinterpret_cast<uint8_t *>(sbuf + kPerCta * (NP == 4096 ? fftst::kStride64 : F.stride));
     for (int i = threadIdx.x; i < L.ntv; i += blockDim.x) occ[i] = tile_occ[((size_t)tt * L.ntv + i) * L.ntu + tu];
     __syncthreads();
     // gridding wrote only occupied tiles; every other cell is zero
-    auto load = [&](int b, int S) -> float2 {
-        return occ[S >> L.tv_log] ? __ldcs(blk + (size_t)S * CB + b) : make_float2(0.f, 0.f);
+    auto load = [&](auto, int b, int S0, int dS, auto &v) {
+        for_live<length_of<decltype(v)>(), false>([&](int m) {
+            const int S = S0 + m * dS;
+            v[m] = occ[S >> L.tv_log] ? __ldcs(blk + (size_t)S * CB + b) : make_float2(0.f, 0.f);
+        });
     };
     // keep the N crop rows, compacted into rows 0..N-1 (all reads precede these writes)
-    auto store = [&](int b, int S, float2 v) {
-        if (in_crop(S, half, Np)) blk[(size_t)grid_to_crop(S, half, Np) * CB + b] = v;
+    auto store = [&](auto pruned, int b, int S0, int dS, auto &v) {
+        for_live<length_of<decltype(v)>(), decltype(pruned)::value>([&](int m) {
+            const int S = S0 + m * dS;
+            if (in_crop(S, half, Np)) blk[(size_t)grid_to_crop(S, half, Np) * CB + b] = v[m];
+        });
     };
     column_fft<NP, true, CROP ? fftst::PRUNE_OUT : 0>(sbuf, F, tw, load, store);
 }
@@ -270,32 +355,37 @@ __device__ __forceinline__ void tma_row_box(float2 *dst, const CUtensorMap *map,
 }
 
 // Shared memory of inv_rows: one or two 128-byte aligned row buffers (TMA
-// destinations), the compensated sums, the z row (kept where it fits), two mbarriers and a flag.
+// destinations), the compensated sums, the half rows of z and screen (where they fit), two mbarriers and a flag.
 struct RowsSmem {
     int buffers;          // 2: the next plane's row is copied while this one is transformed
-    int keep_z;           // 0: the screen reads z from global memory
+    int half;             // 1: half rows of z and of the screen; 0: z from global memory
     size_t buf, bytes;
 };
 inline RowsSmem rows_smem(const FftPlan &F, int N) {
     const size_t buf = ((size_t)F.stride * sizeof(float2) + 127) / 128 * 128;
-    auto layout = [&](int buffers, int keep_z) {
-        return RowsSmem{buffers, keep_z, buf,
-                        128 + buffers * buf + (size_t)N * (sizeof(float4) + (keep_z ? sizeof(float2) : 0)) + 32};
+    auto layout = [&](int buffers, int half) {
+        return RowsSmem{buffers, half, buf,
+                        128 + buffers * buf + (size_t)N * sizeof(float4) + (half ? (N + 2) * sizeof(float2) : 0) + 32};
     };
     // As many CTAs per SM as registers allow come first: they cover each other's
-    // barriers and waits.  For that the z row goes to global memory (a CTA reads the
-    // same row on every plane, from L1 mostly) and then the second buffer goes, if the
-    // last stage's inputs fit in registers (dit_last_held).
+    // barriers and waits.  For that the second buffer goes, if the last stage's inputs
+    // fit in registers (dit_last_held), and then the half rows.
     const int last = F.nstages - 1;
     const bool held = compile_time_size(F.n) || F.nb[last] <= F.row_threads * (32 / F.radix[last]);
     for (int ctas = row_cta_limit(F); ctas > 1; --ctas) {
-        for (const RowsSmem &r : {layout(2, 1), layout(2, 0)})
-            if (r.bytes <= cta_smem(ctas)) return r;
-        if (held && layout(1, 0).bytes <= cta_smem(ctas)) return layout(1, 0);
+        for (const RowsSmem &r : {layout(2, 1), layout(1, 1), layout(2, 0), layout(1, 0)})
+            if ((held || r.buffers == 2) && r.bytes <= cta_smem(ctas)) return r;
     }
     return layout(2, 1).bytes <= cta_smem(1) ? layout(2, 1) : layout(2, 0);
 }
 
+// HALF: shared memory keeps half a row of z and of the plane's screen exp(2 pi i t
+// z).  z depends on l^2, so a pixel and its mirror image share both: the N/2 + 1
+// screens are evaluated together as the plane begins, half the evaluations of one
+// per output (which were a quarter of the kernel's instructions), in the room that
+// a whole row of z took.  (Stepping the screen from plane to plane as fwd_rows does is
+// cheaper still, but raised the error against the exact DFT from 2.7e-7 to 3.0e-7.)
+//
 // One CTA owns image row ii and an equal share of the chunk's planes (share
 // blockIdx.y of gridDim.y): it sums them into a compensated accumulator in
 // shared memory; the last FFT stage screens and accumulates.  Where a row is
@@ -310,10 +400,10 @@ inline RowsSmem rows_smem(const FftPlan &F, int N) {
 // data; the first FFT stage masks them to zero.  Every wait is bounded; a CTA
 // that gives up waits (bounded) for the copy in flight and ends; *timeouts
 // counts the rows left incomplete.
-template <int NP, bool CROP, bool ONE_BUFFER>
+template <int NP, bool CROP, bool ONE_BUFFER, bool HALF>
 __global__ void __launch_bounds__(row_threads_max<NP>(), row_ctas<NP>())
 inv_rows_kernel(Launch L, FftPlan F, const float2 *__restrict__ tw, const __grid_constant__ CUtensorMap row_map,
-                const uint8_t *__restrict__ col_occ, int plane0, int planes, int keep_z, int buf_slots,
+                const uint8_t *__restrict__ col_occ, int plane0, int planes, int buf_slots,
                 const float2 *__restrict__ zsplit, const float *__restrict__ corr, float4 *__restrict__ acc,
                 unsigned *__restrict__ rows_done, int first, int last, float2 *__restrict__ dirty,
                 unsigned long long *__restrict__ timeouts, int wait_polls) {
@@ -332,10 +422,10 @@ inv_rows_kernel(Launch L, FftPlan F, const float2 *__restrict__ tw, const __grid
     float2 *base = sbuf + ((128u - (smem_addr(sbuf) & 127u)) & 127u) / sizeof(float2);
     auto row_buf = [&](int k) { return base + (k & (buffers - 1)) * buf_slots; };
     float4 *srow = reinterpret_cast<float4 *>(base + buffers * buf_slots);   // N: (sum re, sum im, comp re, comp im)
-    float2 *zrow = reinterpret_cast<float2 *>(srow + N);                     // N if keep_z
-    uint64_t *bar = reinterpret_cast<uint64_t *>(zrow + (keep_z ? N : 0));   // 2
+    float2 *scr = reinterpret_cast<float2 *>(srow + N);                      // N/2 + 1 if HALF: exp(2 pi i t z)
+    float2 *zhalf = scr + N / 2 + 1;                                         // N/2 + 1 if HALF: z
+    uint64_t *bar = reinterpret_cast<uint64_t *>(scr + (HALF ? N + 2 : 0));  // 2
     volatile int &finisher = *reinterpret_cast<int *>(bar + 2);              // shared by the CTA
-    const float2 *zsrc = keep_z ? zrow : zsplit + pix0;
     const int warp = tid >> 5, lane = tid & 31;
     // warp 0: copy row ii of the share's k-th plane into buffer k mod buffers
     auto issue = [&](int k) {
@@ -351,8 +441,9 @@ inv_rows_kernel(Launch L, FftPlan F, const float2 *__restrict__ tw, const __grid
         mbar_init(&bar[1], 1);
         mbar_init_fence();
     }
+    if (HALF)
+        for (int h = tid; h <= N / 2; h += T) zhalf[h] = zsplit[pix0 + N / 2 - h];
     for (int jj = tid; jj < N; jj += T) {
-        if (keep_z) zrow[jj] = zsplit[pix0 + jj];
         srow[jj] = first ? make_float4(0.f, 0.f, 0.f, 0.f) : own_acc[pix0 + jj];
     }
     const typename RowTwOf<NP>::type rt(tw, true, tid);
@@ -385,15 +476,45 @@ inv_rows_kernel(Launch L, FftPlan F, const float2 *__restrict__ tw, const __grid
         }
         // every thread is past plane k - 1, so its buffer is free for plane k + 1
         if (warp == 0 && buffers == 2 && k + 1 < count) issue(k + 1);
-        auto store = [&](int, int J, float2 v) {
-            if (!in_crop(J, half, Np)) return;
-            const int jj = grid_to_crop(J, half, Np);
-            float sn, cs;
-            phase_tz(t, zsrc[jj], &sn, &cs);
-            const float4 a = srow[jj];
-            float2 sum = make_float2(a.x, a.y), comp = make_float2(a.z, a.w);
-            kahan_add(sum, comp, cmul_rot(v, make_float2(cs, sn), make_float2(-sn, cs)));
-            srow[jj] = make_float4(sum.x, sum.y, comp.x, comp.y);
+        // the screen of this plane, read by the last stage (the stages' barriers lie between)
+        if (HALF)
+            for (int h = tid; h <= N / 2; h += T) {
+                float sn, cs;
+                phase_tz(t, zhalf[h], &sn, &cs);
+                scr[h] = make_float2(cs, sn);
+            }
+        // a few outputs at a time: their screens and sums are read before any sum is written
+        auto store = [&](auto pruned, int, int J0, int dJ, auto &v) {
+            constexpr int R = length_of<decltype(v)>(), G = NP == 0 && ONE_BUFFER ? 2 : 4;
+            constexpr bool P = decltype(pruned)::value;
+#pragma unroll
+            for (int m0 = 0; m0 < R; m0 += G) {
+                if (P && m0 >= R / 4 && m0 + G <= 3 * R / 4) continue;
+                // (runtime plans: keep the compiler from reading every group's z and sums first)
+                if (NP == 0) asm volatile("" ::: "memory");
+                float2 z[G];
+                float4 a[G];
+                int at[G];
+#pragma unroll
+                for (int i = 0; i < G; ++i) {
+                    const int m = m0 + i, J = J0 + m * dJ;
+                    at[i] = m < R && !(P && m >= R / 4 && m < 3 * R / 4) && in_crop(J, half, Np)
+                                ? grid_to_crop(J, half, Np) : -1;
+                    z[i] = HALF ? scr[abs(max(at[i], 0) - half)] : __ldg(zsplit + pix0 + max(at[i], 0));
+                }
+#pragma unroll
+                for (int i = 0; i < G; ++i)
+                    a[i] = srow[max(at[i], 0)];
+#pragma unroll
+                for (int i = 0; i < G; ++i) {
+                    if (m0 + i >= R || at[i] < 0) continue;
+                    float sn = z[i].y, cs = z[i].x;
+                    if (!HALF) phase_tz(t, z[i], &sn, &cs);
+                    float2 sum = make_float2(a[i].x, a[i].y), comp = make_float2(a[i].z, a[i].w);
+                    kahan_add(sum, comp, cmul_rot(v[m0 + i], make_float2(cs, sn), make_float2(-sn, cs)));
+                    srow[at[i]] = make_float4(sum.x, sum.y, comp.x, comp.y);
+                }
+            }
         };
         auto between = [&] {
             if (warp == 0 && k + 1 < count) issue(k + 1);
@@ -448,7 +569,10 @@ inv_rows_kernel(Launch L, FftPlan F, const float2 *__restrict__ tw, const __grid
 }
 
 // transform buffers + one occupancy byte per strip (at most N'/16 or N'/32 of them)
-inline size_t smem2(const FftPlan &F) { return (size_t)kPerCta * F.stride * sizeof(float2) + F.n / TU + 16; }
+inline size_t smem2(const FftPlan &F) {
+    const int slots = F.n == 4096 ? std::max(F.stride, fftst::kStride64) : F.stride;
+    return (size_t)kPerCta * slots * sizeof(float2) + F.n / TU + 16;
+}
 inline size_t smem_fwd_rows(const FftPlan &F, int N, bool keep_rows) {
     return (size_t)F.stride * sizeof(float2) + (size_t)N * (keep_rows ? 4 : 2) * sizeof(float2) + F.n / TU + 16;
 }
@@ -499,12 +623,16 @@ struct Transforms {
         if constexpr (NP != 0)
             if ((e = allow_smem(inv_cols_kernel<NP, true>, smem2(inv))) != cudaSuccess) return e;
         const size_t inv_rows = rows_smem(inv, N).bytes;
-        if ((e = allow_smem(inv_rows_kernel<NP, false, false>, inv_rows)) != cudaSuccess) return e;
-        if ((e = allow_smem(inv_rows_kernel<NP, false, true>, inv_rows)) != cudaSuccess) return e;
-        if constexpr (NP != 0) {
-            if ((e = allow_smem(inv_rows_kernel<NP, true, false>, inv_rows)) != cudaSuccess) return e;
-            e = allow_smem(inv_rows_kernel<NP, true, true>, inv_rows);
-        }
+        auto allow = [&](auto crop) {
+            constexpr bool C = decltype(crop)::value;
+            cudaError_t r = allow_smem(inv_rows_kernel<NP, C, false, true>, inv_rows);
+            if (r == cudaSuccess) r = allow_smem(inv_rows_kernel<NP, C, false, false>, inv_rows);
+            if (r == cudaSuccess) r = allow_smem(inv_rows_kernel<NP, C, true, true>, inv_rows);
+            return r == cudaSuccess ? allow_smem(inv_rows_kernel<NP, C, true, false>, inv_rows) : r;
+        };
+        e = allow(std::false_type{});
+        if constexpr (NP != 0)
+            if (e == cudaSuccess) e = allow(std::true_type{});
         return e;
     }
     // Runs go(std::bool_constant): whether the crop is the centred half (compile-time plans only).
@@ -517,6 +645,11 @@ struct Transforms {
             }
         }
         go(std::false_type{});
+    }
+    // column CTAs resident on the GPU, a multiple of the two of a block
+    static int columns_ahead(const FftPlan &F, int sms) {
+        const int by_smem = (int)(228 * 1024 / (smem2(F) + 1024)), by_regs = col_ctas<NP>() * col_threads_max<NP>() / col_threads(F);
+        return std::max(1, std::min(by_smem, by_regs)) * sms / 2 * 2;
     }
     static int row_threads(const FftPlan &F) { return NP ? row_threads_max<NP>() : F.row_threads; }
     static int col_threads(const FftPlan &F) { return NP ? col_threads_max<NP>() : F.col_threads; }
@@ -535,7 +668,8 @@ struct Transforms {
         const dim3 grid(p->L.Np / kPerCta, planes);
         with_crop(p->L, [&](auto crop) {
             fwd_cols_kernel<NP, decltype(crop)::value><<<grid, col_threads(p->fft_fwd), smem2(p->fft_fwd), s>>>(
-                p->L, p->fft_fwd, p->d_tw, p->d_tile_occ, p->d_col_occ, chunk * p->P, p->d_stack);
+                p->L, p->fft_fwd, p->d_tw, p->d_tile_occ, p->d_col_occ, chunk * p->P,
+                p->L.N >= kAheadMinImage ? columns_ahead(p->fft_fwd, p->sms) : 0, p->d_stack);
         });
         return cudaGetLastError();
     }
@@ -555,13 +689,15 @@ struct Transforms {
         const RowsSmem sm = rows_smem(p->fft_inv, p->L.N);
         auto go = [&](auto kernel) {
             kernel<<<dim3(p->L.N, p->row_shares), row_threads(p->fft_inv), sm.bytes, s>>>(
-                p->L, p->fft_inv, p->d_tw, map, p->d_col_occ, chunk * p->P, planes, sm.keep_z,
-                (int)(sm.buf / sizeof(float2)), p->d_zsplit, p->d_corr, p->d_acc, p->d_rows_done, first ? 1 : 0,
+                p->L, p->fft_inv, p->d_tw, map, p->d_col_occ, chunk * p->P, planes, (int)(sm.buf / sizeof(float2)), p->d_zsplit, p->d_corr, p->d_acc, p->d_rows_done, first ? 1 : 0,
                 last ? 1 : 0, dirty, p->d_drop + 2, p->wait_polls);
         };
         with_crop(p->L, [&](auto crop) {
             constexpr bool C = decltype(crop)::value;
-            sm.buffers == 1 ? go(inv_rows_kernel<NP, C, true>) : go(inv_rows_kernel<NP, C, false>);
+            if (sm.buffers == 1)
+                sm.half ? go(inv_rows_kernel<NP, C, true, true>) : go(inv_rows_kernel<NP, C, true, false>);
+            else
+                sm.half ? go(inv_rows_kernel<NP, C, false, true>) : go(inv_rows_kernel<NP, C, false, false>);
         });
         return cudaGetLastError();
     }
