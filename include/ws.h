@@ -94,8 +94,8 @@ enum {
     WS_STAGE_COLS_INV,      /* Alg. 5 steps 3b-3c, first half: inverse DFT along v, crop rows */
     WS_STAGE_ROWS_INV,      /* Alg. 5 steps 3b-5, second half: inverse DFT along u, crop,
                                w-screen, sum over planes, correction */
-    WS_STAGE_CORRECT,       /* Alg. 6 step 2: image x correction */
-    WS_STAGE_ROWS_FWD,      /* Alg. 6 steps 3a-3c, first half: w-screen, zero pad, DFT along l */
+    WS_STAGE_CORRECT,       /* Alg. 6 step 2, image x correction: done by the next stage, no launches of its own */
+    WS_STAGE_ROWS_FWD,      /* Alg. 6 steps 2-3c, first half: correction, w-screen, zero pad, DFT along l */
     WS_STAGE_COLS_FWD,      /* Alg. 6 step 3c, second half: zero pad, DFT along m */
     WS_STAGE_DEGRID3D,      /* Alg. 6 steps 4-5: 3-D correlation with C, post-phase */
     WS_NSTAGES

@@ -6,8 +6,7 @@
 // device allocations) or code that must not trigger the implicit device
 // synchronisation an allocation can cause.  For them this file runs the same
 // degridding kernels as ws_degrid, but takes every per-call scratch buffer
-// (visibility records, bin lists, counts and occupancy, the corrected
-// image, the w-plane chunk and the drop counters) from one fixed, file-scope device
+// (visibility records, bin lists, counts and occupancy, the w-plane chunk and the drop counters) from one fixed, file-scope device
 // array instead of the plan's workspace.  The plan itself (tables made by
 // ws_plan) and the caller's inputs and outputs are used as they are.
 #include <cuda_runtime.h>
@@ -96,7 +95,7 @@ extern "C" ws_status ws_degrid_noalloc(ws_plan_t plan, const void *image, const 
     unsigned long long *drop = reinterpret_cast<unsigned long long *>(take(kCounters * sizeof(unsigned long long)));
     uint8_t *tile_occ = take((size_t)p->ntiles);
     uint8_t *col_occ = take((size_t)p->L.ntt * p->L.ntu);
-    float2 *img = reinterpret_cast<float2 *>(take(n_img * sizeof(float2)));
+    take(n_img * sizeof(float2));       // room for an image: not used, but what fits the scratch stays what it was
     if (off > kScratchBytes || (kScratchBytes - off) / plane < (size_t)TT) {
         set_error("ws_degrid_noalloc: the problem needs more than the 64 MiB of fixed scratch (visibility "
                   "records, image and at least 8 w-planes of N' x N'); use ws_degrid");
@@ -127,7 +126,6 @@ extern "C" ws_status ws_degrid_noalloc(ws_plan_t plan, const void *image, const 
     v.d_counts = counts;
     v.d_offsets = offsets;
     v.d_blocksums = blocksums;
-    v.d_img = img;
     v.d_drop = drop;
     v.d_tile_occ = tile_occ;
     v.d_col_occ = col_occ;
@@ -142,12 +140,10 @@ extern "C" ws_status ws_degrid_noalloc(ws_plan_t plan, const void *image, const 
             return cuda_fail(e, "ws_degrid_noalloc: prep kernels");
         if ((e = launch_sort(&v, M, false, s)) != cudaSuccess)
             return cuda_fail(e, "ws_degrid_noalloc: binning kernels");
-        if ((e = launch_correct_image(&v, static_cast<const float2 *>(image), s)) != cudaSuccess)
-            return cuda_fail(e, "ws_degrid_noalloc: correction kernel");
         const int nchunks = (total + P - 1) / P;
         for (int c = 0; c < nchunks; ++c) {
             const int planes = std::min(P, total - c * P);
-            if ((e = launch_fwd_rows(&v, c, planes, s)) != cudaSuccess)
+            if ((e = launch_fwd_rows(&v, static_cast<const float2 *>(image), c, planes, s)) != cudaSuccess)
                 return cuda_fail(e, "ws_degrid_noalloc: fwd_rows kernel");
             if ((e = launch_fwd_cols(&v, c, planes, s)) != cudaSuccess)
                 return cuda_fail(e, "ws_degrid_noalloc: fwd_cols kernel");

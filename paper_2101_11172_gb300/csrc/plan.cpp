@@ -87,7 +87,6 @@ void release(ws_plan_s *p) {
     cudaFree(p->d_rows_done);
     cudaFree(p->d_tile_occ);
     cudaFree(p->d_col_occ);
-    cudaFree(p->d_img);
     cudaFree(p->d_drop);
     cudaFree(p->d_occ_counts);
     cudaFree(p->d_brec);
@@ -444,8 +443,7 @@ void add_occupied_bytes(ws_plan_s *p, bool grid, int64_t M) {
                                 (nchunks - 1) * img * 2 * sizeof(float4);
     } else {
         b[WS_STAGE_PREP] += (double)M * (24 + sizeof(VisRec));
-        b[WS_STAGE_CORRECT] += img * (sizeof(float2) + sizeof(float) + sizeof(float2));
-        b[WS_STAGE_ROWS_FWD] += nchunks * img * 2 * sizeof(float2) + s_valid * strip_plane;
+        b[WS_STAGE_ROWS_FWD] += nchunks * img * (2 * sizeof(float2) + sizeof(float)) + s_valid * strip_plane;
         b[WS_STAGE_COLS_FWD] += s_valid * strip_plane + t_valid * tile_plane;
         b[WS_STAGE_DEGRID3D] += t_valid * tile_plane + entries * (sizeof(uint32_t) + sizeof(VisRec)) +
                                 nchunks * (double)M * 2 * sizeof(float2);
@@ -893,7 +891,6 @@ ws_status plan_create(ws_plan_s **out, int32_t N, double x0, int32_t W, double f
     WS_TRY(cudaMemset(p->d_rows_done, 0, (size_t)N * sizeof(unsigned)), "clearing row counters");
     WS_TRY(dev_alloc(&p->d_tile_occ, (size_t)p->ntiles, &p->bytes), "allocating tile occupancy");
     WS_TRY(dev_alloc(&p->d_col_occ, (size_t)L.ntt * L.ntu, &p->bytes), "allocating strip occupancy");
-    WS_TRY(dev_alloc(&p->d_img, (size_t)N * N, &p->bytes), "allocating the corrected image");
     WS_TRY(dev_alloc(&p->d_drop, (size_t)kCounters, &p->bytes), "allocating drop counters");
     WS_TRY(cudaMallocHost((void **)&p->h_drop, kCounters * sizeof(unsigned long long)), "allocating pinned counters");
     std::memset(p->h_drop, 0, kCounters * sizeof(unsigned long long));
@@ -1076,18 +1073,13 @@ ws_status enqueue_degrid(ws_plan_s *p, const float2 *image, const double *uvw, i
     }
     BoundView view(p, bound, false);
     if ((e = copy_occ_counts(p, s)) != cudaSuccess) return cuda_fail(e, "ws_degrid: occupancy statistics");
-    {
-        StageTimer t(p, s, WS_STAGE_CORRECT, 1);
-        if ((e = launch_correct_image(p, image, s)) != cudaSuccess)
-            return cuda_fail(e, "ws_degrid: correction kernel");
-    }
     const int total = p->L.ntt * TT;
     const int nchunks = (total + p->P - 1) / p->P;
     for (int c = 0; c < nchunks; ++c) {
         const int planes = std::min(p->P, total - c * p->P);
         {
             StageTimer t(p, s, WS_STAGE_ROWS_FWD, 1);
-            if ((e = launch_fwd_rows(p, c, planes, s)) != cudaSuccess)
+            if ((e = launch_fwd_rows(p, image, c, planes, s)) != cudaSuccess)
                 return cuda_fail(e, "ws_degrid: fwd_rows kernel");
         }
         {

@@ -1,10 +1,10 @@
 // Fused plane transforms of the improved W-stacking method (sm_103a).
 //
-// Degridding (Algorithm 6 steps 3a-3c) for plane t:
+// Degridding (Algorithm 6 steps 2-3c) for plane t:
 //   Q_t = pad_{N'}( g exp(-2 pi i t z) ),  g = h_x h_y h_z f   (image, N x N)
 //   F_t[S][R] = sum_{I,J} Q_t[I][J] exp(-2 pi i (S I + R J) / N')
 // is split into
-//   fwd_rows  (screen + zero pad + DFT over J, only the N image rows I)
+//   fwd_rows  (correction + screen + zero pad + DFT over J, only the N image rows I)
 //   fwd_cols  (zero pad in I + DFT over I, every column R, all N' outputs S).
 // Gridding (Algorithm 5 steps 3b-5) for plane t:
 //   P_t[I][J] = sum_{S,R} G_t[S][R] exp(+2 pi i (S I + R J) / N'), kept on the crop
@@ -101,8 +101,8 @@ cudaError_t setup_transform_kernels(const FftPlan &fwd, const FftPlan &inv, int 
     return ops_for(fwd.n).setup(fwd, inv, N);
 }
 
-cudaError_t launch_fwd_rows(const ws_plan_s *p, int chunk, int planes, cudaStream_t s) {
-    return ops_for(p->L.Np).fwd_rows(p, chunk, planes, s);
+cudaError_t launch_fwd_rows(const ws_plan_s *p, const float2 *image, int chunk, int planes, cudaStream_t s) {
+    return ops_for(p->L.Np).fwd_rows(p, image, chunk, planes, s);
 }
 
 cudaError_t launch_fwd_cols(const ws_plan_s *p, int chunk, int planes, cudaStream_t s) {

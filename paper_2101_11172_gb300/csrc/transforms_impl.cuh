@@ -123,7 +123,7 @@ constexpr int kScreenSteps = 8;
 template <int NP, bool CROP>
 __global__ void __launch_bounds__(row_threads_max<NP>(), row_ctas<NP>())
 fwd_rows_kernel(Launch L, FftPlan F, const float2 *__restrict__ tw, const float2 *__restrict__ img,
-                const float2 *__restrict__ zsplit, const uint8_t *__restrict__ col_occ, int plane0, int planes,
+                const float *__restrict__ corr, const float2 *__restrict__ zsplit, const uint8_t *__restrict__ col_occ, int plane0, int planes,
                 int keep_rows, float2 *__restrict__ stack) {
     extern __shared__ __align__(16) float2 sbuf[];
     const int Np = L.Np, N = L.N, half = N / 2;
@@ -139,17 +139,22 @@ fwd_rows_kernel(Launch L, FftPlan F, const float2 *__restrict__ tw, const float2
     const int p_begin = (int)blockIdx.y * per, p_end = min(nvalid, p_begin + per);
     if (p_begin >= p_end) return;
     const size_t pix0 = (size_t)ii * N;
+    // Algorithm 6 step 2, image x h_x h_y h_z (a real-sky plan reads only the image's real part)
+    auto corrected = [&](int jj) {
+        const float h = corr[pix0 + jj];
+        const float2 f = img[pix0 + jj];
+        return make_float2(h * f.x, L.fold ? 0.f : h * f.y);
+    };
     for (int jj = tid; jj < N; jj += T) {
         const float2 z = zsplit[pix0 + jj];
         if (keep_rows) {
-            irow[jj] = img[pix0 + jj];
+            irow[jj] = corrected(jj);
             zrow[jj] = z;
         }
         float sn, cs;
         phase_tz(1.f, z, &sn, &cs);
         erow[jj] = make_float2(cs, -sn);
     }
-    const float2 *isrc = keep_rows ? irow : img + pix0, *zsrc = keep_rows ? zrow : zsplit + pix0;
     int occ_tt = -1;
     const typename RowTwOf<NP>::type rt(tw, false, tid);        // the thread's twiddle bases, read once
     for (int p = p_begin; p < p_end; ++p) {
@@ -165,11 +170,11 @@ fwd_rows_kernel(Launch L, FftPlan F, const float2 *__restrict__ tw, const float2
         }
         if ((p - p_begin) % kScreenSteps == 0) {
             for (int jj = tid; jj < N; jj += T) {
-                // row x exp(-i phi), phi = 2 pi t z
-                const float2 f = isrc[jj];
+                // row x exp(-i phi), phi = 2 pi t z: (f.x cs + f.y sn, f.y cs - f.x sn), the products with f.x rounded first
+                const float2 f = keep_rows ? irow[jj] : corrected(jj);
                 float sn, cs;
-                phase_tz(t, zsrc[jj], &sn, &cs);
-                grow[jj] = make_float2(f.x * cs + f.y * sn, f.y * cs - f.x * sn);
+                phase_tz(t, keep_rows ? zrow[jj] : zsplit[pix0 + jj], &sn, &cs);
+                grow[jj] = fma2(dup2(f.y), make_float2(sn, cs), mul2(dup2(f.x), make_float2(cs, -sn)));
             }
             __syncthreads();
         }
@@ -653,13 +658,13 @@ struct Transforms {
     }
     static int row_threads(const FftPlan &F) { return NP ? row_threads_max<NP>() : F.row_threads; }
     static int col_threads(const FftPlan &F) { return NP ? col_threads_max<NP>() : F.col_threads; }
-    static cudaError_t fwd_rows(const ws_plan_s *p, int chunk, int planes, cudaStream_t s) {
+    static cudaError_t fwd_rows(const ws_plan_s *p, const float2 *image, int chunk, int planes, cudaStream_t s) {
         const bool keep = fwd_rows_keep(p->fft_fwd, p->L.N);
         const dim3 grid(p->L.N, row_groups(p->L.N, planes, p->sms));
         with_crop(p->L, [&](auto crop) {
             fwd_rows_kernel<NP, decltype(crop)::value>
                 <<<grid, row_threads(p->fft_fwd), smem_fwd_rows(p->fft_fwd, p->L.N, keep), s>>>(
-                    p->L, p->fft_fwd, p->d_tw, p->d_img, p->d_zsplit, p->d_col_occ, chunk * p->P, planes, keep ? 1 : 0,
+                    p->L, p->fft_fwd, p->d_tw, image, p->d_corr, p->d_zsplit, p->d_col_occ, chunk * p->P, planes, keep ? 1 : 0,
                     p->d_stack);
         });
         return cudaGetLastError();
@@ -707,7 +712,7 @@ struct Transforms {
 // instantiates it (so every kernel is compiled exactly once).
 struct Ops {
     cudaError_t (*setup)(const FftPlan &, const FftPlan &, int);
-    cudaError_t (*fwd_rows)(const ws_plan_s *, int, int, cudaStream_t);
+    cudaError_t (*fwd_rows)(const ws_plan_s *, const float2 *, int, int, cudaStream_t);
     cudaError_t (*fwd_cols)(const ws_plan_s *, int, int, cudaStream_t);
     cudaError_t (*inv_cols)(const ws_plan_s *, int, int, cudaStream_t);
     cudaError_t (*inv_rows)(const ws_plan_s *, int, int, bool, bool, float2 *, cudaStream_t);

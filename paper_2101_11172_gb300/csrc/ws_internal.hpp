@@ -144,7 +144,6 @@ struct ws_plan_s {
     int row_shares = 1;            // shares of the planes per image row in inv_rows (transforms.cu)
     float4 *d_acc = nullptr;       // row_shares x N x N: (sum re, sum im, comp re, comp im)
     unsigned *d_rows_done = nullptr;   // N: shares of the row that are done, zero between calls
-    float2 *d_img = nullptr;       // N x N: corrected image (degridding)
     unsigned long long *d_drop = nullptr;   // kCounters: [0] non-finite uv, [1] w out of range, [2] timed-out waits
     unsigned long long *h_drop = nullptr;   // pinned mirror
     int wait_polls = ws::kWaitPolls;        // limit of inv_rows' first wait per plane (WS_WAIT_POLLS)
@@ -248,7 +247,6 @@ cudaError_t launch_sort(const ws_plan_s *p, int64_t M, bool grid, cudaStream_t s
 int sort_launches(const ws_plan_s *p, int64_t M);
 cudaError_t launch_occ_count(const ws_plan_s *p, cudaStream_t s);
 cudaError_t launch_grid_chunk(const ws_plan_s *p, int chunk, int planes, cudaStream_t s);
-cudaError_t launch_correct_image(const ws_plan_s *p, const float2 *image, cudaStream_t s);
 cudaError_t launch_unfold(const ws_plan_s *p, const double *uvw, int64_t M, float2 *vis, cudaStream_t s);
 cudaError_t launch_degrid_chunk(const ws_plan_s *p, int chunk, int planes, int64_t M,
                                 float2 *vis, cudaStream_t s);
@@ -257,7 +255,7 @@ cudaError_t launch_degrid_chunk(const ws_plan_s *p, int chunk, int planes, int64
 size_t transform_smem_bytes(const FftPlan &fwd, const FftPlan &inv, int N);
 int inv_row_shares(const FftPlan &F, int N, int planes, int sms);
 cudaError_t setup_transform_kernels(const FftPlan &fwd, const FftPlan &inv, int N);
-cudaError_t launch_fwd_rows(const ws_plan_s *p, int chunk, int planes, cudaStream_t s);
+cudaError_t launch_fwd_rows(const ws_plan_s *p, const float2 *image, int chunk, int planes, cudaStream_t s);
 cudaError_t launch_fwd_cols(const ws_plan_s *p, int chunk, int planes, cudaStream_t s);
 cudaError_t launch_inv_cols(const ws_plan_s *p, int chunk, int planes, cudaStream_t s);
 cudaError_t launch_inv_rows(const ws_plan_s *p, int chunk, int planes, bool first, bool last, float2 *dirty,

@@ -3,9 +3,8 @@
 // Gridding (Algorithm 5):   prep and count -> sort -> per plane chunk: grid3d -> inv_cols -> inv_rows
 //                           (transforms.cu: inverse DFTs, crop, x exp(2 pi i t z), sum over t,
 //                           x h_x h_y h_z)
-// Degridding (Algorithm 6): prep and count -> sort -> correct_image (x h_x h_y h_z) -> per plane chunk:
-//                           fwd_rows -> fwd_cols (transforms.cu: x exp(-2 pi i t z), zero pad,
-//                           forward DFTs) -> degrid3d (3-D correlation with C_x C_y C_z,
+// Degridding (Algorithm 6): prep and count -> sort -> per plane chunk: fwd_rows -> fwd_cols
+//                           (transforms.cu: x h_x h_y h_z, x exp(-2 pi i t z), zero pad, forward DFTs) -> degrid3d (3-D correlation with C_x C_y C_z,
 //                           x exp(-2 pi i w (n0-1)))
 //
 // Grid indices: row s (v direction) and column r (u direction) of a plane are
@@ -104,19 +103,27 @@ __device__ __forceinline__ void count_record(const Launch &L, const VisRec &r, u
 // set's records), or its degridding or gridding bins counted and its tiles marked.
 enum : int { kPrepOnly = 0, kPrepDegrid = 1, kPrepGrid = 2 };
 
-// floor(x) for |x| < 2^51, by adding and taking off 1.5 x 2^52: the sum rounds x
-// to the nearest integer, in its low bits.  FP64 adds run at 2 a clock and SM;
-// floor and the FP64-to-integer conversions at a fraction of that.
-__device__ __forceinline__ double floor_int(double x, int *low) {
+// The tap rule's floor(x + W/2) for |x| < 2^51 and, in nu, the offset x + (W-1)/2 -
+// floor(x + W/2) in [-1/2, 1/2), from FP64 adds alone: the nearest integer to x +
+// (W-1)/2 comes from adding 1.5 x 2^52 (it is left in the sum's low bits), and
+// differs from the floor only where x + W/2 is an integer and the tie went down.
+// FP64 arithmetic is what bounds the kernel (GB300 does 0.6 T FP64 operations a
+// second), floor and the conversions to integers more so.
+__device__ __forceinline__ void tap_floor(double x, double half_wm1, int *floor_low, float *nu) {
     constexpr double kRound = 6755399441055744.0;
-    double s = x + kRound, f = s - kRound;
-    if (f > x) {
-        s -= 1.0;
-        f -= 1.0;
+    const double y = x + half_wm1, s = y + kRound;
+    double d = y - (s - kRound);
+    int low = __double2loint(s);
+    if (d == 0.5) {
+        d = -0.5;
+        ++low;
     }
-    *low = __double2loint(s);
-    return f;
+    *floor_low = low;
+    *nu = (float)d;
 }
+
+// |x| below about 10^9 (an exponent below 30), by integer comparison: false for NaN and infinities too.
+__device__ __forceinline__ bool small_enough(double x) { return (__double2hiint(x) & 0x7fffffff) < ((1023 + 30) << 20); }
 
 // A grid index i (|i| < 2^31) modulo n: with the division only for the rare points more than a grid away.
 __device__ __forceinline__ int wrap_small(int i, int n) {
@@ -134,8 +141,7 @@ __global__ void prep_kernel(Launch L, const double *__restrict__ uvw, const floa
                             int64_t M, VisRec *__restrict__ rec, unsigned long long *__restrict__ drop,
                             uint32_t *__restrict__ counts, uint8_t *__restrict__ tile_occ, float2 *__restrict__ zeroed) {
     const int W = L.W;
-    const double half_w = 0.5 * W, half_wm1 = 0.5 * (W - 1), t_off = (double)(W - 1) + L.t_lo;
-    const double t_max = (double)(L.Nw - W);
+    const double half_w = 0.5 * W, half_wm1 = 0.5 * (W - 1);
     for (int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; k < M; k += (int64_t)gridDim.x * blockDim.x) {
         double u = uvw[3 * k], v = uvw[3 * k + 1], w = uvw[3 * k + 2];
         if (BIN == kPrepDegrid) zeroed[k] = make_float2(0.f, 0.f);      // the output that degridding adds to
@@ -153,41 +159,39 @@ __global__ void prep_kernel(Launch L, const double *__restrict__ uvw, const floa
         r.nux = r.nuy = r.nuz = 0.f;
         r.vre = r.vim = 0.f;
         const double up = u * L.uv_scale, vp = v * L.uv_scale, wp = w * L.nscale;
-        if (!(fabs(up) < 1e15) || !(fabs(vp) < 1e15)) {   // also catches NaN
+        const bool near = small_enough(up) && small_enough(vp);
+        if (!near && (!(fabs(up) < 1e15) || !(fabs(vp) < 1e15))) {   // also catches NaN
             atomicAdd(&drop[0], 1ull);
             rec[k] = r;
             continue;
         }
-        const double xt = wp + half_w;
-        // (the planes' range is below 2^12, so a w within it is within floor_int's range)
-        int it, iu, iv;
-        const double ft = floor_int(xt, &it);
-        const double t0 = ft - t_off;
-        if (!(fabs(xt) < 1e9 && t0 >= 0.0 && t0 <= t_max)) {   // NaN w fails too
+        int it;
+        float nuz;
+        tap_floor(wp, half_wm1, &it, &nuz);
+        const int t0 = it - (W - 1) - L.t_lo;
+        if (!small_enough(wp) || t0 < 0 || t0 > L.Nw - W) {          // NaN w is not small
             atomicAdd(&drop[1], 1ull);
             rec[k] = r;
             continue;
         }
-        const double xu = up + half_w, xv = vp + half_w;
-        double fu, fv;
-        if (fabs(xu) < 1e9 && fabs(xv) < 1e9) {
-            fu = floor_int(xu, &iu);
-            fv = floor_int(xv, &iv);
+        r.t0 = t0;
+        r.nuz = nuz;
+        if (near) {
+            int iu, iv;
+            tap_floor(up, half_wm1, &iu, &r.nux);
+            tap_floor(vp, half_wm1, &iv, &r.nuy);
             r.r0 = wrap_small(iu - (W - 1), L.Np);
             r.s0 = wrap_small(iv - (W - 1), L.Np);
         } else {
-            fu = floor(xu);
-            fv = floor(xv);
+            const double fu = floor(up + half_w), fv = floor(vp + half_w);
             r.r0 = wrap_index(fu - (W - 1), L.Np);
             r.s0 = wrap_index(fv - (W - 1), L.Np);
+            r.nux = (float)(up + half_wm1 - fu);
+            r.nuy = (float)(vp + half_wm1 - fv);
         }
-        r.t0 = it - (W - 1) - L.t_lo;
-        r.nux = (float)(up + half_wm1 - fu);
-        r.nuy = (float)(vp + half_wm1 - fv);
-        r.nuz = (float)(wp + half_wm1 - ft);
         // pre-phase exp(+2 pi i w (n0 - 1)), argument reduced in FP64
         double turns = w * L.n0m1;
-        turns -= rint(turns);
+        turns -= (turns + 6755399441055744.0) - 6755399441055744.0;      // |turns| < 2^51: rint by 1.5 x 2^52
         float s, c;
         sincospif(2.0f * (float)turns, &s, &c);
         if (BIN == kPrepGrid) {
@@ -973,17 +977,6 @@ grid3d_mma_kernel(Launch L, const float *__restrict__ coef, int deg, const VisRe
     flush(cur + 1);
 }
 
-// Algorithm 6 step 2: image x h_x h_y h_z.
-// A real-sky plan (fold) reads only the real part of the image.
-__global__ void correct_image_kernel(int64_t n, const float *__restrict__ corr,
-                                     const float2 *__restrict__ image, int fold, float2 *__restrict__ out) {
-    int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    const float h = corr[i];
-    const float2 f = image[i];
-    out[i] = make_float2(h * f.x, fold ? 0.f : h * f.y);
-}
-
 // Section 5.4: a visibility with w < 0 was degridded at -(u, v, w); the real
 // sky's visibility at (u, v, w) is the conjugate of that.
 __global__ void unfold_kernel(const double *__restrict__ uvw, int64_t M, float2 *__restrict__ vis) {
@@ -1235,12 +1228,6 @@ cudaError_t launch_grid_chunk(const ws_plan_s *p, int chunk, int planes, cudaStr
         case 12: return width(std::integral_constant<int, 12>{});
         default: return cudaErrorInvalidValue;
     }
-}
-
-cudaError_t launch_correct_image(const ws_plan_s *p, const float2 *image, cudaStream_t s) {
-    const int64_t n = (int64_t)p->L.N * p->L.N;
-    correct_image_kernel<<<blocks_for(n, 256), 256, 0, s>>>(n, p->d_corr, image, p->L.fold, p->d_img);
-    return cudaGetLastError();
 }
 
 cudaError_t launch_unfold(const ws_plan_s *p, const double *uvw, int64_t M, float2 *vis, cudaStream_t s) {
