@@ -43,6 +43,22 @@ __device__ __forceinline__ float2 twiddle(const float2 *__restrict__ tw, int m, 
     return inv ? make_float2(w.x, -w.y) : w;
 }
 
+// The bases of butterfly offset k of a runtime plan's stage of radix R, from the
+// stage's own table (fft_tables): w^k and, from R = 8 on, w^4k beside it.
+// Read from the N'-entry table, a warp's w^4k fell into as many sectors as
+// lanes, and a stage's table is small enough for the L1 that the buffers leave.
+template <int R>
+__device__ __forceinline__ void twiddle_bases(const float2 *__restrict__ bases, int k, bool inv, float2 &w1, float2 &w4) {
+    if (R >= 8) {
+        const float4 w = __ldg(reinterpret_cast<const float4 *>(bases) + k);
+        w1 = make_float2(w.x, inv ? -w.y : w.y);
+        w4 = make_float2(w.z, inv ? -w.w : w.w);
+    } else {
+        w1 = twiddle(bases, k, inv);
+        w4 = make_float2(1.f, 0.f);
+    }
+}
+
 __device__ __forceinline__ void dft4(float2 &a0, float2 &a1, float2 &a2, float2 &a3, bool inv) {
     const float2 t0 = cadd(a0, a2), t1 = csub(a0, a2), t2 = cadd(a1, a3), d = csub(a1, a3);
     a0 = cadd(t0, t2);
@@ -328,8 +344,8 @@ __device__ __forceinline__ int div_small(int x, unsigned mul) {
 template <int R, int COUNT, bool LAST, class Store>
 __device__ __forceinline__ void dit_stage(float2 *buf, const FftPlan &P, int s, const float2 *__restrict__ tw,
                                           bool inv, int tid, int nthr, Store &store) {
-    const int L = P.L[s], total = COUNT * P.nb[s], twstep = P.twstep[s];
-    const int step = P.step[s];
+    const int L = P.L[s], total = COUNT * P.nb[s], step = P.step[s];
+    tw += P.bases[s];
     float2 w1, w4;
     int base = 0, k = 0;
     auto fetch = [&](int q) {                // butterfly q's first position and twiddles (q past the end: the last one's)
@@ -337,8 +353,7 @@ __device__ __forceinline__ void dit_stage(float2 *buf, const FftPlan &P, int s, 
         const int blk = LAST ? 0 : div_small(bq, P.L_mul[s]);
         k = bq - blk * L;
         base = blk * R * L + k;
-        w1 = twiddle(tw, k * twstep, inv);
-        w4 = R >= 8 ? twiddle(tw, 4 * k * twstep, inv) : make_float2(1.f, 0.f);
+        twiddle_bases<R>(tw, k, inv, w1, w4);
     };
     fetch(tid);
     __syncthreads();
@@ -380,8 +395,7 @@ __device__ __forceinline__ void dit_pair(float2 *buf, const FftPlan &P, int s, c
         const int blk = LAST ? 0 : div_small(bq, P.L_mul[s]);
         k = bq - blk * L;
         base = blk * A * B * L + k;
-        w1 = twiddle(tw, k * P.twstep[s], inv);
-        w4 = A >= 8 ? twiddle(tw, 4 * k * P.twstep[s], inv) : make_float2(1.f, 0.f);
+        twiddle_bases<A>(tw + P.bases[s], k, inv, w1, w4);
     };
     fetch(tid);
     __syncthreads();
@@ -391,7 +405,7 @@ __device__ __forceinline__ void dit_pair(float2 *buf, const FftPlan &P, int s, c
         float2 *x = buf + b + div_small(b, P.chunk_mul);
         float2 v[A * B], w[A];
 #pragma unroll
-        for (int m1 = 0; m1 < A; ++m1) w[m1] = twiddle(tw, (kq + m1 * L) * P.twstep[s + 1], inv);
+        for (int m1 = 0; m1 < A; ++m1) w[m1] = twiddle(tw + P.bases[s + 1], kq + m1 * L, inv);
 #pragma unroll
         for (int m2 = 0; m2 < B; ++m2)
 #pragma unroll
@@ -434,9 +448,7 @@ __device__ __forceinline__ void dit_last_held(float2 *buf, const FftPlan &P, con
     float2 v[ROUNDS][R], w1[ROUNDS], w4[ROUNDS];
 #pragma unroll
     for (int i = 0; i < ROUNDS; ++i) {
-        const int e = min(tid + i * nthr, nb - 1) * P.twstep[s];
-        w1[i] = twiddle(tw, e, inv);
-        w4[i] = R >= 8 ? twiddle(tw, 4 * e, inv) : make_float2(1.f, 0.f);
+        twiddle_bases<R>(tw + P.bases[s], min(tid + i * nthr, nb - 1), inv, w1[i], w4[i]);
     }
     __syncthreads();
 #pragma unroll
@@ -459,29 +471,26 @@ __device__ __forceinline__ void dit_last_held(float2 *buf, const FftPlan &P, con
 }
 
 // The slot where butterfly j of the first stage puts its R outputs: that of
-// position g*R, g = the digits of j in reverse order.
-__device__ __forceinline__ int first_slot(const FftPlan &P, int j) {
-    int g = 0;
-    for (int i = 1; i < P.nstages; ++i) {
-        const int a = div_small(j, P.xw_mul[i]);
-        g += (a - div_small(a, P.r_mul[i]) * P.radix[i]) * P.gw[i];
-    }
-    g *= P.radix[0];
-    return g + div_small(g, P.chunk_mul);
+// position g*R, g = the digits of j in reverse order (from the plan's table: the
+// digits took a dozen instructions per stage, five per element of a radix-8 stage).
+__device__ __forceinline__ int first_slot(const FftPlan &P, const float2 *__restrict__ tw, int j) {
+    return __ldg(reinterpret_cast<const int *>(tw) + P.slots + j);
 }
 
 // First stage: butterfly j of each transform reads inputs m*(n/R) + j, m < R,
 // straight from load(t, e), and writes them to the digit-reversed positions
 // g*R + m that the later in-place stages expect.
 template <int R, int COUNT, class Load>
-__device__ __forceinline__ void dit_first(float2 *buf, const FftPlan &P, bool inv, int tid, int nthr, Load &load) {
+__device__ __forceinline__ void dit_first(float2 *buf, const FftPlan &P, const float2 *__restrict__ tw, bool inv, int tid,
+                                          int nthr, Load &load) {
     const int nb = P.nb[0], total = COUNT * nb;
     for (int q = tid; q < total; q += nthr) {
         const int t = q % COUNT, j = q / COUNT;
+        const int slot = first_slot(P, tw, j);
         float2 v[R];
         load(std::false_type{}, t, j, nb, v);
         dft<R>(v, inv);
-        float2 *x = buf + t * P.stride + first_slot(P, j);
+        float2 *x = buf + t * P.stride + slot;
 #pragma unroll
         for (int m = 0; m < R; ++m) x[m] = v[m];
     }
@@ -491,10 +500,11 @@ __device__ __forceinline__ void dit_first(float2 *buf, const FftPlan &P, bool in
 // at 0..n-1 (n / R <= nthr: one butterfly per thread); input m of a thread is
 // zero where bit m of live is clear, whatever the buffer holds.
 template <int R>
-__device__ __forceinline__ void dit_first_inplace(float2 *buf, const FftPlan &P, bool inv, int tid, uint32_t live) {
+__device__ __forceinline__ void dit_first_inplace(float2 *buf, const FftPlan &P, const float2 *__restrict__ tw, bool inv, int tid,
+                                                  uint32_t live) {
     // threads past nb read the last butterfly's inputs and drop them: a value that
     // exists only under a condition, kept across the barrier, made the compiler spill
-    const int nb = P.nb[0], at = min(tid, nb - 1);
+    const int nb = P.nb[0], at = min(tid, nb - 1), slot = first_slot(P, tw, at);
     float2 v[R];
 #pragma unroll
     for (int m = 0; m < R; ++m) {
@@ -504,7 +514,7 @@ __device__ __forceinline__ void dit_first_inplace(float2 *buf, const FftPlan &P,
     __syncthreads();
     if (tid < nb) {
         dft<R>(v, inv);
-        float2 *x = buf + first_slot(P, tid);
+        float2 *x = buf + slot;
 #pragma unroll
         for (int m = 0; m < R; ++m) x[m] = v[m];
     }
@@ -648,7 +658,7 @@ template <int COUNT, bool INV, class Load, class Store>
 __device__ __forceinline__ void fft_many(float2 *buf, const FftPlan &P, const float2 *__restrict__ tw, int tid,
                                          int nthr, Load load, Store store) {
     auto first = [&](auto r) {
-        fftdev::dit_first<decltype(r)::value, COUNT>(buf, P, INV, tid, nthr, load);
+        fftdev::dit_first<decltype(r)::value, COUNT>(buf, P, tw, INV, tid, nthr, load);
     };
     if constexpr (INV)
         fftdev::with_first_radix(P.radix[0], first);
@@ -665,7 +675,7 @@ template <bool HELD, class Between, class Store>
 __device__ __forceinline__ void fft_inplace(float2 *buf, const FftPlan &P, const float2 *__restrict__ tw, int tid,
                                             int nthr, Between between, Store store, uint32_t live) {
     fftdev::with_first_radix(P.radix[0], [&](auto r) {
-        fftdev::dit_first_inplace<decltype(r)::value>(buf, P, true, tid, live);
+        fftdev::dit_first_inplace<decltype(r)::value>(buf, P, tw, true, tid, live);
     });
     const int last = fft_middle_stages<1, true>(buf, P, tw, tid, nthr);
     if constexpr (HELD)

@@ -24,13 +24,14 @@ struct FftPlan {
     int L[kMaxFftStages];           // radix[0] * ... * radix[s-1]
     int nb[kMaxFftStages];          // butterflies of stage s: n / radix[s]
     int twstep[kMaxFftStages];      // n / (radix[s] L[s])
+    int bases[kMaxFftStages];       // the stage's twiddle bases in the twiddle buffer (fft_tables)
     int step[kMaxFftStages];        // slots from one element of a butterfly to the next
     int fuse[kMaxFftStages];        // 1: this stage and the next run as one pass (rows of forward plans)
-    int gw[kMaxFftStages];          // first-stage digit reversal: gw[i] = radix[1] * ... * radix[i-1]
-    // div_mul of: L[s]; the digit weight radix[s+1] * ...; radix[s]; and of chunk.
+    int slots;                      // the first stage's output slots, as integers in the twiddle buffer (fft_tables)
+    // div_mul of L[s] and of chunk.
     // x / d = umulhi(x, mul) exactly for 0 <= x < 2^16 and d < 2^13, since
     // x (mul d - 2^32) < 2^32 (div_small in fft.cuh)
-    unsigned L_mul[kMaxFftStages], xw_mul[kMaxFftStages], r_mul[kMaxFftStages], chunk_mul;
+    unsigned L_mul[kMaxFftStages], chunk_mul;
     int stride;                     // float2 slots per transform buffer (== 8 mod 16)
     int row_threads, col_threads;   // threads per CTA: one transform (rows), two (columns)
     int box_blocks, boxes;          // TMA row copies: boxes of box_blocks column blocks

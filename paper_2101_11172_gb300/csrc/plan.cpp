@@ -324,6 +324,18 @@ void fuse_stages(const int *radix, int ns, int *fuse) {
         if (fuse[s]) fuse[++s] = 0;                      // a pair's second stage starts none
 }
 
+// The position of the first stage's butterfly j in the order of the later stages: its
+// digits (radices 1, 2, ...) reversed.
+int first_position(const FftPlan &F, int j) {
+    int g = 0, weight = 1;
+    for (int s = 1, rest = F.nb[0]; s < F.nstages; ++s) {
+        rest /= F.radix[s];
+        g += j / rest % F.radix[s] * weight;
+        weight *= F.radix[s];
+    }
+    return g * F.radix[0];
+}
+
 // Bank conflicts of a plan's shared-memory accesses by `count` interleaved
 // transforms: the sum over all half-warp accesses (16 lanes of 8 bytes) of the
 // lanes on the fullest bank pair.
@@ -341,12 +353,7 @@ long fft_conflicts(const FftPlan &F, int chunk, int stride, int count) {
                 const int t = (q0 + i) % count, b = (q0 + i) / count;
                 int e;
                 if (s == 0) {
-                    int g = 0, rest = b;
-                    for (int k = ns - 1; k >= 1; --k) {
-                        g += (rest % F.radix[k]) * F.gw[k];
-                        rest /= F.radix[k];
-                    }
-                    e = g * F.radix[0];
+                    e = first_position(F, b);
                 } else {
                     e = b / L * R * L + b % L;
                 }
@@ -373,20 +380,14 @@ bool fft_make_plan(int n, bool inverse, FftPlan *F) {
     if (!inverse) fuse_stages(radix, ns, F->fuse);
     int passes[kMaxFftStages] = {}, np = 0;              // the radix of each pass of a row
     for (int s = 0; s < ns; s += 1 + F->fuse[s]) passes[np++] = radix[s] * (F->fuse[s] ? radix[s + 1] : 1);
-    int L = 1, gw = 1;
+    int L = 1;
     for (int s = 0; s < ns; ++s) {
         const int r = radix[s];
-        int xw = 1;
-        for (int l = s + 1; l < ns; ++l) xw *= radix[l];
         F->radix[s] = r;
         F->L[s] = L;
         F->nb[s] = n / r;
         F->twstep[s] = n / (r * L);
-        F->gw[s] = s == 0 ? 0 : gw;
         F->L_mul[s] = div_mul(L);
-        F->xw_mul[s] = div_mul(xw);
-        F->r_mul[s] = div_mul(r);
-        if (s > 0) gw *= r;
         L *= r;
     }
     auto stride_of = [&](int len) { return len + ((8 - len % 16) + 16) % 16; };     // == 8 (mod 16)
@@ -412,6 +413,31 @@ bool fft_make_plan(int n, bool inverse, FftPlan *F) {
     while (blocks % F->boxes || (blocks / F->boxes) % 4) ++F->boxes;
     F->box_blocks = blocks / F->boxes;
     return true;
+}
+
+// Appends to the twiddles (the first n entries, exp(-2 pi i m / n)) each later
+// stage's bases in the order its butterflies take them: w^k, k < L, and beside
+// it w^4k where the radix is 8 or more (fft.cuh: twiddle_bases), and then the slots
+// where the first stage's butterflies put their outputs (first_slot).
+void fft_tables(FftPlan *F, std::vector<float2> *tw) {
+    for (int s = 1; s < F->nstages; ++s) {
+        F->bases[s] = (int)(tw->size() + 1) / 2 * 2;         // 16-byte aligned
+        tw->resize((size_t)F->bases[s]);
+        for (int k = 0; k < F->L[s]; ++k) {
+            const float2 w1 = (*tw)[(size_t)k * F->twstep[s]];
+            tw->push_back(w1);
+            if (F->radix[s] >= 8) {
+                const float2 w4 = (*tw)[(size_t)4 * k * F->twstep[s]];
+                tw->push_back(w4);
+            }
+        }
+    }
+    F->slots = (int)tw->size() * 2;
+    tw->resize(tw->size() + (size_t)(F->nb[0] + 1) / 2);
+    for (int j = 0; j < F->nb[0]; ++j) {
+        const int e = first_position(*F, j), slot = e + (F->chunk_mul ? (int)((unsigned long long)e * F->chunk_mul >> 32) : 0);
+        std::memcpy(reinterpret_cast<int *>(tw->data()) + F->slots + j, &slot, sizeof(int));
+    }
 }
 
 // Occupied algorithmic bytes of one call per stage, from the occupancy counts
@@ -877,6 +903,8 @@ ws_status plan_create(ws_plan_s **out, int32_t N, double x0, int32_t W, double f
             const double ang = 2.0 * 3.14159265358979323846 * (double)m / (double)Np;
             tw[m] = make_float2((float)std::cos(ang), (float)-std::sin(ang));
         }
+        fft_tables(&p->fft_fwd, &tw);
+        fft_tables(&p->fft_inv, &tw);
         WS_TRY(dev_alloc(&p->d_tw, tw.size(), &p->bytes), "allocating twiddles");
         WS_TRY(cudaMemcpy(p->d_tw, tw.data(), tw.size() * sizeof(float2), cudaMemcpyHostToDevice),
                "uploading twiddles");

@@ -51,8 +51,13 @@ inline int row_threads_of(const FftPlan &F) { return compile_time_size(F.n) ? F.
 inline int row_cta_limit(const FftPlan &F) { return 512 / row_threads_of(F); }
 inline size_t cta_smem(int ctas) { return (size_t)228 * 1024 / ctas - 1024; }
 
-__device__ __forceinline__ int grid_to_crop(int g, int half, int Np) { return g < half ? g + half : g - (Np - half); }
-__device__ __forceinline__ bool in_crop(int g, int half, int Np) { return g < half || g >= Np - half; }
+// The crop index of grid index g (0 <= g < N'): below N = 2 half inside the centred
+// crop, at least N outside it.  One minimum for both: g + half - N' wraps to a huge
+// value unless g is in the grid's last half columns.
+__device__ __forceinline__ unsigned grid_to_crop(int g, int half, int Np) {
+    const unsigned c = (unsigned)(g + half);
+    return min(c, c - (unsigned)Np);
+}
 
 // The column kernels' transforms (two columns).  PRUNE (fftst::PRUNE_IN /
 // PRUNE_OUT, compile-time plans with N' = 2N only): the inputs outside the
@@ -155,6 +160,12 @@ fwd_rows_kernel(Launch L, FftPlan F, const float2 *__restrict__ tw, const float2
         phase_tz(1.f, z, &sn, &cs);
         erow[jj] = make_float2(cs, -sn);
     }
+    // Runtime plans whose last-stage butterflies take whole strips apart keep a mask per
+    // strip of their first elements instead: one load for all of a butterfly's strips
+    // (they span ntu strips in mask_span steps; at least 4, so the masks fit in occ's room).
+    unsigned *mask = reinterpret_cast<unsigned *>(occ);
+    const int last_L = F.L[F.nstages - (F.nstages > 2 && F.fuse[F.nstages - 2] ? 2 : 1)];
+    const int mask_span = NP == 0 && last_L % TU == 0 && 4 * last_L <= Np ? last_L / TU : 0;
     int occ_tt = -1;
     const typename RowTwOf<NP>::type rt(tw, false, tid);        // the thread's twiddle bases, read once
     for (int p = p_begin; p < p_end; ++p) {
@@ -164,7 +175,15 @@ fwd_rows_kernel(Launch L, FftPlan F, const float2 *__restrict__ tw, const float2
         const int tt = pl / TT;
         __syncthreads();                     // row and z visible; the previous plane's last stage is done
         if (tt != occ_tt) {                  // uniform across the CTA
-            for (int i = tid; i < L.ntu; i += T) occ[i] = col_occ[tt * L.ntu + i];
+            const uint8_t *strips = col_occ + tt * L.ntu;
+            if (mask_span > 0)
+                for (int i = tid; i < mask_span; i += T) {
+                    unsigned bits = 0u;
+                    for (int m = 0; m * mask_span < L.ntu; ++m) bits |= (unsigned)(strips[i + m * mask_span] != 0) << m;
+                    mask[i] = bits;
+                }
+            else
+                for (int i = tid; i < L.ntu; i += T) occ[i] = strips[i];
             occ_tt = tt;
             __syncthreads();
         }
@@ -185,37 +204,37 @@ fwd_rows_kernel(Launch L, FftPlan F, const float2 *__restrict__ tw, const float2
             if constexpr (NP == 0) {
                 // (runtime plans: reading all steps first took more registers than it saved time)
                 for_live<R, P>([&](int m) {
-                    const int J = J0 + m * dJ, jj = grid_to_crop(J, half, Np);
+                    const unsigned jj = grid_to_crop(J0 + m * dJ, half, Np);
                     v[m] = make_float2(0.f, 0.f);
-                    if (!in_crop(J, half, Np)) return;
+                    if (jj >= (unsigned)N) return;
                     v[m] = grow[jj];
                     if (step) grow[jj] = step_screen(v[m], erow[jj]);
                 });
                 return;
             }
             for_live<R, P>([&](int m) {
-                const int J = J0 + m * dJ;
-                v[m] = in_crop(J, half, Np) ? grow[grid_to_crop(J, half, Np)] : make_float2(0.f, 0.f);
+                const unsigned jj = grid_to_crop(J0 + m * dJ, half, Np);
+                v[m] = jj < (unsigned)N ? grow[jj] : make_float2(0.f, 0.f);
             });
             if (!step) return;
             float2 e[R];
             for_live<R, P>([&](int m) {
-                const int J = J0 + m * dJ;
-                if (in_crop(J, half, Np)) e[m] = erow[grid_to_crop(J, half, Np)];
+                const unsigned jj = grid_to_crop(J0 + m * dJ, half, Np);
+                if (jj < (unsigned)N) e[m] = erow[jj];
             });
             for_live<R, P>([&](int m) {
-                const int J = J0 + m * dJ;
-                if (in_crop(J, half, Np)) grow[grid_to_crop(J, half, Np)] = step_screen(v[m], e[m]);
+                const unsigned jj = grid_to_crop(J0 + m * dJ, half, Np);
+                if (jj < (unsigned)N) grow[jj] = step_screen(v[m], e[m]);
             });
         };
         // columns of this plane's t-tile that no footprint touches are never read
         auto store = [&](auto, int, int R0, int dR, auto &v) {
-            if (NP == 0 && dR % TU == 0) {                       // whole strips apart: one address and a stride
+            if (NP == 0 && mask_span > 0) {                      // one address and a stride
                 float2 *at = plane + tiled_index(ii, R0, Np);
                 const size_t stride = (size_t)(dR / CB) * Np * CB;
-                const uint8_t *strip = occ + R0 / TU;
+                const unsigned strips = mask[R0 / TU];
                 for_live<length_of<decltype(v)>(), false>([&](int m) {
-                    if (strip[m * (dR / TU)]) __stcs(at + m * stride, v[m]);
+                    if (strips >> m & 1u) __stcs(at + m * stride, v[m]);
                 });
                 return;
             }
@@ -271,8 +290,8 @@ fwd_cols_kernel(Launch L, FftPlan F, const float2 *__restrict__ tw, const uint8_
     // rows 0..N-1 hold the N transformed image rows; every other row is zero padding
     auto load = [&](auto pruned, int b, int S0, int dS, auto &v) {
         for_live<length_of<decltype(v)>(), decltype(pruned)::value>([&](int m) {
-            const int S = S0 + m * dS;
-            v[m] = in_crop(S, half, Np) ? __ldcs(blk + (size_t)grid_to_crop(S, half, Np) * CB + b) : make_float2(0.f, 0.f);
+            const unsigned c = grid_to_crop(S0 + m * dS, half, Np);
+            v[m] = c < 2u * half ? __ldcs(blk + (size_t)c * CB + b) : make_float2(0.f, 0.f);
         });
     };
     auto store = [&](auto, int b, int S0, int dS, auto &v) {
@@ -310,8 +329,8 @@ inv_cols_kernel(Launch L, FftPlan F, const float2 *__restrict__ tw, const uint8_
     // keep the N crop rows, compacted into rows 0..N-1 (all reads precede these writes)
     auto store = [&](auto pruned, int b, int S0, int dS, auto &v) {
         for_live<length_of<decltype(v)>(), decltype(pruned)::value>([&](int m) {
-            const int S = S0 + m * dS;
-            if (in_crop(S, half, Np)) blk[(size_t)grid_to_crop(S, half, Np) * CB + b] = v[m];
+            const unsigned c = grid_to_crop(S0 + m * dS, half, Np);
+            if (c < 2u * half) blk[(size_t)c * CB + b] = v[m];
         });
     };
     column_fft<NP, true, CROP ? fftst::PRUNE_OUT : 0>(sbuf, F, tw, load, store);
@@ -499,20 +518,19 @@ inv_rows_kernel(Launch L, FftPlan F, const float2 *__restrict__ tw, const __grid
                 if (NP == 0) asm volatile("" ::: "memory");
                 float2 z[G];
                 float4 a[G];
-                int at[G];
+                unsigned at[G];                                  // outputs outside the crop read the row's last pixel
+                auto wanted = [&](int i) { return m0 + i < R && !(P && m0 + i >= R / 4 && m0 + i < 3 * R / 4); };
 #pragma unroll
                 for (int i = 0; i < G; ++i) {
-                    const int m = m0 + i, J = J0 + m * dJ;
-                    at[i] = m < R && !(P && m >= R / 4 && m < 3 * R / 4) && in_crop(J, half, Np)
-                                ? grid_to_crop(J, half, Np) : -1;
-                    z[i] = HALF ? scr[abs(max(at[i], 0) - half)] : __ldg(zsplit + pix0 + max(at[i], 0));
+                    if (!wanted(i)) continue;
+                    at[i] = grid_to_crop(J0 + (m0 + i) * dJ, half, Np);
+                    const int jj = (int)min(at[i], (unsigned)N - 1u);
+                    z[i] = HALF ? scr[abs(jj - half)] : __ldg(zsplit + pix0 + jj);
+                    a[i] = srow[jj];
                 }
 #pragma unroll
-                for (int i = 0; i < G; ++i)
-                    a[i] = srow[max(at[i], 0)];
-#pragma unroll
                 for (int i = 0; i < G; ++i) {
-                    if (m0 + i >= R || at[i] < 0) continue;
+                    if (!wanted(i) || at[i] >= (unsigned)N) continue;
                     float sn = z[i].y, cs = z[i].x;
                     if (!HALF) phase_tz(t, z[i], &sn, &cs);
                     float2 sum = make_float2(a[i].x, a[i].y), comp = make_float2(a[i].z, a[i].w);

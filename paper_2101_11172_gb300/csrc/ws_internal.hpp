@@ -128,7 +128,7 @@ struct ws_plan_s {
     // stack workspace
     int P = 0;                     // planes per chunk (multiple of TT)
     float2 *d_stack = nullptr;     // P x N' x N', column-block layout (common.cuh)
-    float2 *d_tw = nullptr;        // N' twiddles exp(-2 pi i m / N')
+    float2 *d_tw = nullptr;        // N' twiddles exp(-2 pi i m / N'), then the stages' bases (FftPlan)
     ws::FftPlan fft_fwd{}, fft_inv{};   // the N'-point plane transforms
     // per-call buffers (grow on demand)
     ws::VisRec *d_rec = nullptr;
