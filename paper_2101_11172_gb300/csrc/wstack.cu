@@ -381,14 +381,14 @@ static_assert(ring_planes(kMaxW) <= 31, "ring slots are packed in 5 bits");
 constexpr int kGeneral = -1;                       // item shape: the part wraps an axis of a small grid
 
 // Dynamic shared memory of grid3d<W, R, DET> (grid_smem_bytes): the ring (re,
-// im; FP32 sums, or 64-bit fixed-point sums for the deterministic mode), the
+// im; FP32 sums, or the low and high words of 64-bit fixed-point sums for the deterministic mode), the
 // weight table, and per warp the staged chunk (weights, items, values, nu).
 template <int W, int R, bool DET>
 struct GridSmem {
     static constexpr int S = 3 * W;                // weight slots per entry: u taps, v taps, w taps
     static constexpr int WX = wx_span(W);          // staged u weights, from the part's first tap
     static constexpr int SP = stage_stride(W);     // entry stride of the staged weights: u, v, w
-    static constexpr int ES = DET ? 8 : 4;         // bytes per cell component
+    static constexpr int HI = ring_planes(W) * plane_stride(R) * 4;    // DET: from a sum's low word to its high word
     static constexpr int RP = ring_planes(W);      // ring planes
     static constexpr int PS = plane_stride(R);     // cells per ring plane (padded)
     static constexpr size_t re = 0;
@@ -429,34 +429,74 @@ __device__ __forceinline__ void red_shared_at(unsigned addr, float v) {
     asm volatile("red.shared.add.f32 [%0+%1], %2;" ::"r"(addr), "n"(OFF), "f"(v) : "memory");
 }
 
-// The deterministic mode's shared-memory add: a contribution v becomes the
-// 64-bit integer nearest v 2^scale, and integer sums do not depend on the
-// order of their terms.
+// The 64-bit integer nearest v (ties to even), |v| < 2^62.  The conversion to 64 bits
+// goes at the rate of FP64 arithmetic, and bounded the deterministic mode (120,960
+// visibilities, W = 7, N = 512: 350 us with it, 274 so); this takes the two words of |v| by 32-bit conversions, both exact
+// but for the low word's rounding (below 2^24 |v| is all in the low word; from there on it is an integer).
+__device__ __forceinline__ long long nearest_int64(float v) {
+    const float a = fabsf(v), x = a * 0x1p-32f;
+    const unsigned hi = __float2uint_rz(x), lo = __float2uint_rn(fmaf(truncf(x), -0x1p32f, a));
+    const long long q = (long long)((unsigned long long)hi << 32 | lo);
+    return v < 0.f ? -q : q;
+}
+// The deterministic mode's shared-memory add: a contribution, in units of the
+// column's 2^-scale, becomes the nearest 64-bit integer, and integer sums do not
+// depend on the order of their terms.  A sum is kept as two 32-bit words `HI` bytes
+// apart: shared memory adds 32-bit integers itself, while a 64-bit add is a loop of
+// compare-and-swap.  Every addition to the low word adds its carry to the high
+// word, so the pair is the 64-bit sum once all have arrived.
+// add_low returns the low word before the addition; add_high takes it.
 template <int OFF>
-__device__ __forceinline__ void red_shared_fixed_at(unsigned addr, float v, int scale) {
-    const unsigned long long q = (unsigned long long)__float2ll_rn(ldexpf(v, scale));
-    asm volatile("red.shared.add.u64 [%0+%1], %2;" ::"r"(addr), "n"(OFF), "l"(q) : "memory");
+__device__ __forceinline__ unsigned add_low(unsigned addr, long long q) {
+    unsigned old;
+    asm volatile("atom.shared.add.u32 %0, [%1+%2], %3;" : "=r"(old) : "r"(addr), "n"(OFF), "r"((unsigned)q) : "memory");
+    return old;
+}
+template <int OFF>
+__device__ __forceinline__ void add_high(unsigned addr, long long q, unsigned old) {
+    const unsigned carry = old + (unsigned)q < old ? 1u : 0u;
+    asm volatile("red.shared.add.u32 [%0+%1], %2;" ::"r"(addr), "n"(OFF), "r"((unsigned)(q >> 32) + carry) : "memory");
 }
 
-// One contribution to a ring cell component at byte address addr + OFF.
-template <bool DET, int OFF>
-__device__ __forceinline__ void add_cell(unsigned addr, float v, int scale) {
-    if constexpr (DET)
-        red_shared_fixed_at<OFF>(addr, v, scale);
-    else
-        red_shared_at<OFF>(addr, v);
+// One contribution to a ring cell component at byte address addr (the general path: any v).
+template <bool DET, int HI>
+__device__ __forceinline__ void add_cell(unsigned addr, float v) {
+    if constexpr (DET) {
+        const long long q = __float2ll_rn(v);
+        add_high<HI>(addr, q, add_low<0>(addr, q));
+    } else {
+        red_shared_at<0>(addr, v);
+    }
 }
 
-// Adds (pr, pi) x wx[a] to cells a = 0 .. na - 1 of a ring row (re and im at byte addresses).
-template <int W, bool DET, int A = 0>
-__device__ __forceinline__ void add_row(unsigned re, unsigned im, const float (&wx)[wx_span(W)], int na, float pr, float pi,
-                                        int scale) {
+// Adds p x wx[a] to cells a = 0 .. na - 1 of a ring row (byte address `addr`).
+template <int W, int A = 0>
+__device__ __forceinline__ void add_row(unsigned addr, const float (&wx)[wx_span(W)], int na, float p) {
     if constexpr (A < W) {
         if (A < na) {
-            constexpr int ES = DET ? 8 : 4;
-            add_cell<DET, ES * A>(re, pr * wx[A], scale);
-            add_cell<DET, ES * A>(im, pi * wx[A], scale);
-            add_row<W, DET, A + 1>(re, im, wx, na, pr, pi, scale);
+            red_shared_at<4 * A>(addr, p * wx[A]);
+            add_row<W, A + 1>(addr, wx, na, p);
+        }
+    }
+}
+// The same in fixed point: all low words first, so their returns are waited for once.
+template <int W, int HI, int A = 0>
+__device__ __forceinline__ void add_row_low(unsigned addr, const float (&wx)[wx_span(W)], int na, float p,
+                                            long long (&q)[W], unsigned (&old)[W]) {
+    if constexpr (A < W) {
+        if (A < na) {
+            q[A] = nearest_int64(p * wx[A]);
+            old[A] = add_low<4 * A>(addr, q[A]);
+            add_row_low<W, HI, A + 1>(addr, wx, na, p, q, old);
+        }
+    }
+}
+template <int W, int HI, int A = 0>
+__device__ __forceinline__ void add_row_high(unsigned addr, int na, const long long (&q)[W], const unsigned (&old)[W]) {
+    if constexpr (A < W) {
+        if (A < na) {
+            add_high<HI + 4 * A>(addr, q[A], old[A]);
+            add_row_high<W, HI, A + 1>(addr, na, q, old);
         }
     }
 }
@@ -495,12 +535,13 @@ __device__ __forceinline__ void flush_slices(int from, int to, const Launch &L, 
             if (t < ring_end) {
                 const int cell = (t % RP) * PS + lr * kRowPad + lc;
                 if constexpr (DET) {
-                    long long *qre = reinterpret_cast<long long *>(smem + Sm::re);
-                    long long *qim = reinterpret_cast<long long *>(smem + Sm::im);
-                    v = make_float4(ldexpf(__ll2float_rn(qre[cell]), -scale), ldexpf(__ll2float_rn(qim[cell]), -scale),
-                                    ldexpf(__ll2float_rn(qre[cell + 1]), -scale),
-                                    ldexpf(__ll2float_rn(qim[cell + 1]), -scale));
-                    if (clear) qre[cell] = qim[cell] = qre[cell + 1] = qim[cell + 1] = 0;
+                    auto sum = [&](size_t ring, int c) {
+                        unsigned *lo = reinterpret_cast<unsigned *>(smem + ring) + c, *hi = lo + Sm::HI / 4;
+                        const long long q = (long long)((unsigned long long)*hi << 32 | *lo);
+                        if (clear) *lo = *hi = 0u;
+                        return ldexpf(__ll2float_rn(q), -scale);
+                    };
+                    v = make_float4(sum(Sm::re, cell), sum(Sm::im, cell), sum(Sm::re, cell + 1), sum(Sm::im, cell + 1));
                 } else {
                     float *sre = reinterpret_cast<float *>(smem + Sm::re);
                     float *sim = reinterpret_cast<float *>(smem + Sm::im);
@@ -528,7 +569,7 @@ grid3d_kernel(Launch L, const float *__restrict__ coef, int deg, const VisRec *_
               const uint8_t *__restrict__ tile_occ, int chunk_tt0, int chunk_ntt, float wbound,
               float2 *__restrict__ stack) {
     using Sm = GridSmem<W, R, DET>;
-    constexpr int PS = Sm::PS, RP = Sm::RP, ES = Sm::ES, S = Sm::S, SP = Sm::SP, WX = Sm::WX;
+    constexpr int PS = Sm::PS, RP = Sm::RP, HI = Sm::HI, S = Sm::S, SP = Sm::SP, WX = Sm::WX;
     extern __shared__ __align__(16) unsigned char smem[];
     __shared__ unsigned col_max;                      // DET: max |V~| of the column's entries (float bits)
     const int tu = centre_first(blockIdx.x % L.ntu, L.ntu);
@@ -584,6 +625,9 @@ grid3d_kernel(Launch L, const float *__restrict__ coef, int deg, const VisRec *_
             scale = 62 - ex;
         }
     }
+    // 2^scale in two factors that FP32 holds; the staged values are multiplied by it
+    // (exactly), so a contribution needs no scaling of its own
+    const float up0 = ldexpf(1.f, scale / 2), up1 = ldexpf(1.f, scale - scale / 2);
     int cur = -1;                                    // t-tile of the ring's first plane; -1: none yet
     for (int k = k_lo; k < k_hi; ++k) {
         const uint32_t beg = off[k], end = off[k + 1];
@@ -610,7 +654,10 @@ grid3d_kernel(Launch L, const float *__restrict__ coef, int deg, const VisRec *_
                 const int nsv = tile_spans(v_org, r.s0, Np, W, R, sv[0], sv[1]);
                 const int c0 = max(0, plo - r.t0), c1 = min(W, phi - r.t0);
                 int4 it;
-                if (nsu == 1 && nsv == 1) {
+                const float2 V = DET ? make_float2(r.vre * up0 * up1, r.vim * up0 * up1) : make_float2(r.vre, r.vim);
+                // (values that are not finite keep the conversion that saturates)
+                const bool finite = !DET || (fabsf(V.x) <= 0x1p126f && fabsf(V.y) <= 0x1p126f);
+                if (nsu == 1 && nsv == 1 && finite) {
                     const int na = su[0].a1 - su[0].a0, nb = sv[0].a1 - sv[0].a0, nc = max(c1 - c0, 0);
                     const int slot = (r.t0 + c0) % RP;      // ring slot of the part's first plane
                     it.x = (sv[0].a0 - sv[0].off) * kRowPad + (su[0].a0 - su[0].off);
@@ -623,7 +670,7 @@ grid3d_kernel(Launch L, const float *__restrict__ coef, int deg, const VisRec *_
                 }
                 it.w = (int)kv;
                 items[lane] = it;
-                vals[lane] = make_float2(r.vre, r.vim);
+                vals[lane] = V;
                 nus[lane] = make_float4(r.nux, r.nuy, r.nuz, 0.f);
             }
             __syncwarp();
@@ -679,11 +726,21 @@ grid3d_kernel(Launch L, const float *__restrict__ coef, int deg, const VisRec *_
                         const float wyz = wt[WX + b0 + bb] * wt[WX + W + cw0 + cc];
                         int slot = slot0 + cc;
                         if (slot >= RP) slot -= RP;
-                        const unsigned o = (unsigned)(it.x + slot * PS + bb * kRowPad) * ES;
-                        add_row<W, DET>(re_base + o, im_base + o, wx, na, V.x * wyz, V.y * wyz, scale);
+                        const unsigned o = (unsigned)(it.x + slot * PS + bb * kRowPad) * 4;
+                        if constexpr (DET) {
+                            long long qre[W], qim[W];
+                            unsigned ore[W], oim[W];
+                            add_row_low<W, HI>(re_base + o, wx, na, V.x * wyz, qre, ore);
+                            add_row_low<W, HI>(im_base + o, wx, na, V.y * wyz, qim, oim);
+                            add_row_high<W, HI>(re_base + o, na, qre, ore);
+                            add_row_high<W, HI>(im_base + o, na, qim, oim);
+                        } else {
+                            add_row<W>(re_base + o, wx, na, V.x * wyz);
+                            add_row<W>(im_base + o, wx, na, V.y * wyz);
+                        }
                     }
                 } else {
-                    // the part wraps around an axis (N' < W + R): every span pair, taps one by one
+                    // the part wraps around an axis (N' < W + R; or see above): every span pair, taps one by one
                     const VisRec r = rec[it.w];
                     Span su[2], sv[2];
                     const int nsu = tile_spans(u_org, r.r0, Np, W, TU, su[0], su[1]);
@@ -696,10 +753,9 @@ grid3d_kernel(Launch L, const float *__restrict__ coef, int deg, const VisRec *_
                                 const int a = su[iu].a0 + q % na, b = sv[iv].a0 + (q / na) % nb, c = c0 + q / (na * nb);
                                 const float w = wt[a] * wt[WX + b] * wt[WX + W + c];
                                 const unsigned o = (unsigned)(((r.t0 + c) % RP) * PS + (b - sv[iv].off) * kRowPad +
-                                                              (a - su[iu].off)) *
-                                                   ES;
-                                add_cell<DET, 0>(re_base + o, V.x * w, scale);
-                                add_cell<DET, 0>(im_base + o, V.y * w, scale);
+                                                              (a - su[iu].off)) * 4;
+                                add_cell<DET, HI>(re_base + o, V.x * w);
+                                add_cell<DET, HI>(im_base + o, V.y * w);
                             }
                         }
                 }
