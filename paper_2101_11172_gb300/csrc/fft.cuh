@@ -983,9 +983,11 @@ __device__ __forceinline__ void dft64_over_b(float2 *v, bool inv) {
     for (int i = 0; i < 64; ++i) v[i] = o[i];
 }
 
-// v[8 r + i] *= w^r for r = 1..7, all i (the powers are products at most three deep)
-__device__ __forceinline__ void mul_rows(float2 *v, float2 w) {
-    const fftdev::Tw t1(w), t2(t1.times(w)), t4(t2.times(t2.w));
+// v[8 r + i] *= w^r for r = 1..7, all i, given w, w^2 and w^4: the other powers are
+// products of these.  (All powers from w alone multiplied its rounding error by up to
+// seven: error against the exact DFT 3.3e-7 on the survey against 3.1e-7.)
+__device__ __forceinline__ void mul_rows(float2 *v, const float2 (&w)[3]) {
+    const fftdev::Tw t1(w[0]), t2(w[1]), t4(w[2]);
     auto row = [&](int r, const fftdev::Tw &t) {
 #pragma unroll
         for (int i = 0; i < 8; ++i) v[8 * r + i] = t.times(v[8 * r + i]);
@@ -1007,14 +1009,13 @@ constexpr int kStride64 = 64 * kPitch64 + 8;             // points per sequence;
 
 // COUNT sequences of 4096 points by 64 COUNT threads (load and store as for
 // fft_many, 64 points each; under PRUNE_IN / PRUNE_OUT the first and last quarter).
+// bases: w^j, w^2j, .. w^32j for each j < 64 (fft_tables).
 template <int COUNT, int PRUNE, class Load, class Store>
-__device__ __forceinline__ void fft_4096_two_stage(float2 *buf, const float2 *__restrict__ tw, bool inv, int tid,
+__device__ __forceinline__ void fft_4096_two_stage(float2 *buf, const float2 *__restrict__ bases, bool inv, int tid,
                                                    Load load, Store store) {
     using namespace fftst;
     const int t = tid % COUNT, j = tid / COUNT;
     float2 *x = buf + t * kStride64;
-    // w^1 and w^8 of this thread's second stage
-    const float2 w1 = fftdev::twiddle(tw, j, inv), w8 = fftdev::twiddle(tw, 8 * j, inv);
     float2 v[64];
     load(std::bool_constant<(PRUNE & PRUNE_IN) != 0>{}, t, j, 64, v);
     dft64_over_a<(PRUNE & PRUNE_IN) != 0>(v, inv);
@@ -1023,6 +1024,12 @@ __device__ __forceinline__ void fft_4096_two_stage(float2 *buf, const float2 *__
     for (int q = 0; q < 8; ++q)
 #pragma unroll
         for (int p = 0; p < 8; ++p) x[(q + 8 * p) * kPitch64 + j] = v[8 * q + p];
+    // the second stage's w, w^2, w^4 and w^8, w^16, w^32, asked for before the barrier
+    const float4 *row = reinterpret_cast<const float4 *>(bases) + 3 * j;
+    const float4 a = __ldg(row), b = __ldg(row + 1), c = __ldg(row + 2);
+    const float s = inv ? -1.f : 1.f;
+    const float2 w1[3] = {make_float2(a.x, s * a.y), make_float2(a.z, s * a.w), make_float2(b.x, s * b.y)};
+    const float2 w8[3] = {make_float2(b.z, s * b.w), make_float2(c.x, s * c.y), make_float2(c.z, s * c.w)};
     __syncthreads();
 #pragma unroll
     for (int i = 0; i < 64; ++i) v[i] = x[j * kPitch64 + i];

@@ -418,8 +418,18 @@ bool fft_make_plan(int n, bool inverse, FftPlan *F) {
 // Appends to the twiddles (the first n entries, exp(-2 pi i m / n)) each later
 // stage's bases in the order its butterflies take them: w^k, k < L, and beside
 // it w^4k where the radix is 8 or more (fft.cuh: twiddle_bases), and then the slots
-// where the first stage's butterflies put their outputs (first_slot).
+// where the first stage's butterflies put their outputs (first_slot).  For N' =
+// 4096, whose columns have two stages of 64, w^j, w^2j, .. w^32j of each j < 64 instead.
 void fft_tables(FftPlan *F, std::vector<float2> *tw) {
+    if (F->n == 4096) {
+        F->bases[1] = (int)tw->size();
+        for (int j = 0; j < 64; ++j)
+            for (int m = 1; m <= 32; m *= 2) {
+                const float2 w = (*tw)[(size_t)(m * j)];
+                tw->push_back(w);
+            }
+        return;
+    }
     for (int s = 1; s < F->nstages; ++s) {
         F->bases[s] = (int)(tw->size() + 1) / 2 * 2;         // 16-byte aligned
         tw->resize((size_t)F->bases[s]);

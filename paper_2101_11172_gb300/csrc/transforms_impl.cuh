@@ -69,7 +69,7 @@ __device__ __forceinline__ void column_fft(float2 *buf, const FftPlan &F, const 
     if constexpr (NP == 0)
         fft_many<kPerCta, INV>(buf, F, tw, threadIdx.x, blockDim.x, load, store);
     else if constexpr (NP == 4096)
-        fft_4096_two_stage<kPerCta, PRUNE>(buf, tw, INV, threadIdx.x, load, store);
+        fft_4096_two_stage<kPerCta, PRUNE>(buf, tw + F.bases[1], INV, threadIdx.x, load, store);
     else
         fft_static<NP, kPerCta, col_threads_max<NP>(), PRUNE>(buf, tw, INV, threadIdx.x, load, store);
 }

@@ -36,7 +36,7 @@ constexpr int kMaxDeg = 16;
 
 // Gridding kernel shape: 256 threads; each warp stages kChunk entries at a
 // time.  Shared memory holds a ring of TT + W - 1 w-planes of the tile column
-// (re and im, FP32 or, deterministic, 64-bit fixed point; rows padded to TU +
+// (re and im, FP32 or, deterministic, the two words of 64-bit fixed point; rows padded to TU +
 // 1 cells, planes to plane_stride cells), the weight table (3W slots of
 // kCoefStride coefficients) and the warps' staged chunks (per entry its u
 // weights from the first tap inside the tile, padded to a multiple of 4, then
@@ -67,9 +67,9 @@ WS_HD constexpr size_t grid_smem_bytes(int W, int rows, bool det) {
            + (size_t)kGridWarps * kChunk * (16 + 8 + 16);                         // items, values, nu
 }
 // CTAs of the gridding kernel that fit on one SM (1 KB reserved per CTA), at
-// most 6.  Gridding is latency-bound and gains from every CTA that fits: on the
-// survey (W = 7, 16-row tiles) 13.2 ms at 3 CTAs per SM, 11.0 at 4, 10.2 at 5 and
-// 10.1 at 6, where the 4-entry chunks and 40 registers just fit.
+// most 6.  The kernel is latency-bound and gains from every CTA that fits: on the
+// survey (W = 7, 16-row tiles, which now go to the tensor cores) 13.2 ms at 3 CTAs per
+// SM, 11.0 at 4, 10.2 at 5 and 10.1 at 6, where the 4-entry chunks and 40 registers just fit.
 WS_HD constexpr int grid_ctas_per_sm(int W, int rows, bool det) {
     return (int)(kSmemPerSM / (grid_smem_bytes(W, rows, det) + 1024)) < 1 ? 1
            : (int)(kSmemPerSM / (grid_smem_bytes(W, rows, det) + 1024)) > 6
