@@ -378,8 +378,11 @@ int fp64_planes(int Np, int Nw) {
     return (int)std::max<size_t>(1, std::min<size_t>(fit, (size_t)Nw));
 }
 
-cudaError_t fp64_setup(int Np) {
-    const int smem = (int)(fft_lines64(Np) * Np * sizeof(double2));
+// The limit belongs to the kernel and every plan on the device shares it, so it is raised to what the
+// largest line count needs (64 KB) whatever this plan's size: a limit set to one plan's need would
+// make the launches of a larger one fail.
+cudaError_t fp64_setup() {
+    const int smem = (int)(kFftPoints64 * sizeof(double2));
     cudaError_t e = cudaFuncSetAttribute(fwd_rows64_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     if (e == cudaSuccess) e = cudaFuncSetAttribute(cols64_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     if (e == cudaSuccess) e = cudaFuncSetAttribute(inv_rows64_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);

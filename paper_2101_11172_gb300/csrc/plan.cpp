@@ -960,7 +960,7 @@ ws_status plan_create(ws_plan_s **out, int32_t N, double x0, int32_t W, double f
             const int want = std::atoi(env);
             if (want > 0) p->planes64 = std::min(p->planes64, want);
         }
-        WS_TRY(fp64_setup((int)Np), "configuring the FP64 transforms");
+        WS_TRY(fp64_setup(), "configuring the FP64 transforms");
         WS_TRY(dev_alloc(&p->d_plane64, (size_t)p->planes64 * Np * Np, &p->bytes), "allocating the FP64 planes");
         WS_TRY(dev_alloc(&p->d_acc64, (size_t)N * N, &p->bytes), "allocating the FP64 accumulator");
         p->fft64_log = 0;

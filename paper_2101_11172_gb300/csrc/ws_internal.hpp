@@ -223,7 +223,7 @@ bool tune_store(const char *path, const std::string &key, int tile_rows, const i
 // FP64 path (fp64.cu).
 size_t fp64_record_bytes();
 int fp64_planes(int Np, int Nw);
-cudaError_t fp64_setup(int Np);
+cudaError_t fp64_setup();
 ws_status enqueue_grid64(ws_plan_s *p, const double *uvw, const double2 *vis, int64_t M, double2 *dirty,
                          cudaStream_t s);
 ws_status enqueue_degrid64(ws_plan_s *p, const double2 *image, const double *uvw, int64_t M, double2 *vis,
