@@ -9,7 +9,7 @@
 // and the sums -- so that its error against the exact DFT follows sqrt(3) E
 // down to W = 14.  It exists to measure the method's error, not for large
 // problems: the w-planes are taken a chunk at a time (planes64, as many as fit in
-// kPlaneBytes64), Algorithm 5 and Algorithm 6 step by step, with FP64 atomics
+// 2 GB and in the memory budget of a stack), Algorithm 5 and Algorithm 6 step by step, with FP64 atomics
 // for the spread and a shared-memory FFT per line.
 //
 // Work split.  A warp takes a visibility through all of a chunk's planes: its 3W
@@ -371,10 +371,10 @@ struct Fft64Launch {
 
 size_t fp64_record_bytes() { return sizeof(VisRec64); }
 
-// Planes per chunk: as many as fit in 2 GB, at least one.
-int fp64_planes(int Np, int Nw) {
+// Planes per chunk: as many as fit in 2 GB and in `budget` bytes, at least one.
+int fp64_planes(int Np, int Nw, size_t budget) {
     constexpr size_t kPlaneBytes64 = (size_t)2 << 30;
-    const size_t fit = kPlaneBytes64 / ((size_t)Np * Np * sizeof(double2));
+    const size_t fit = std::min(kPlaneBytes64, budget) / ((size_t)Np * Np * sizeof(double2));
     return (int)std::max<size_t>(1, std::min<size_t>(fit, (size_t)Nw));
 }
 

@@ -923,10 +923,12 @@ ws_status plan_create(ws_plan_s **out, int32_t N, double x0, int32_t W, double f
     WS_TRY(dev_alloc(&p->d_counts, (size_t)p->ntiles + 1, &p->bytes), "allocating tile counts");
     WS_TRY(dev_alloc(&p->d_offsets, (size_t)p->ntiles + 1, &p->bytes), "allocating tile offsets");
     WS_TRY(dev_alloc(&p->d_blocksums, (size_t)4096, &p->bytes), "allocating scan sums");
-    p->row_shares = inv_row_shares(p->fft_inv, N, p->P > 0 ? std::min(p->P, L.Nw) : L.Nw, p->sms);
-    WS_TRY(dev_alloc(&p->d_acc, (size_t)p->row_shares * N * N, &p->bytes), "allocating the accumulators");
-    WS_TRY(dev_alloc(&p->d_rows_done, (size_t)N, &p->bytes), "allocating row counters");
-    WS_TRY(cudaMemset(p->d_rows_done, 0, (size_t)N * sizeof(unsigned)), "clearing row counters");
+    if (!fp64) {                                  // FP64 plans have a sum of their own (d_acc64)
+        p->row_shares = inv_row_shares(p->fft_inv, N, p->P > 0 ? std::min(p->P, L.Nw) : L.Nw, p->sms);
+        WS_TRY(dev_alloc(&p->d_acc, (size_t)p->row_shares * N * N, &p->bytes), "allocating the accumulators");
+        WS_TRY(dev_alloc(&p->d_rows_done, (size_t)N, &p->bytes), "allocating row counters");
+        WS_TRY(cudaMemset(p->d_rows_done, 0, (size_t)N * sizeof(unsigned)), "clearing row counters");
+    }
     WS_TRY(dev_alloc(&p->d_tile_occ, (size_t)p->ntiles, &p->bytes), "allocating tile occupancy");
     WS_TRY(dev_alloc(&p->d_col_occ, (size_t)L.ntt * L.ntu, &p->bytes), "allocating strip occupancy");
     WS_TRY(dev_alloc(&p->d_drop, (size_t)kCounters, &p->bytes), "allocating drop counters");
@@ -955,7 +957,8 @@ ws_status plan_create(ws_plan_s **out, int32_t N, double x0, int32_t W, double f
         WS_TRY(dev_alloc(&p->d_tw64, tw64.size(), &p->bytes), "allocating FP64 twiddles");
         WS_TRY(cudaMemcpy(p->d_tw64, tw64.data(), tw64.size() * sizeof(double2), cudaMemcpyHostToDevice),
                "uploading FP64 twiddles");
-        p->planes64 = fp64_planes((int)Np, L.Nw);
+        // within the budget of the FP32 stack, and one plane whatever it is
+        p->planes64 = fp64_planes((int)Np, L.Nw, budget);
         if (const char *env = std::getenv("WS_PLANES_PER_CHUNK")) {
             const int want = std::atoi(env);
             if (want > 0) p->planes64 = std::min(p->planes64, want);

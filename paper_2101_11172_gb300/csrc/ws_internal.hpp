@@ -222,7 +222,7 @@ bool tune_store(const char *path, const std::string &key, int tile_rows, const i
 
 // FP64 path (fp64.cu).
 size_t fp64_record_bytes();
-int fp64_planes(int Np, int Nw);
+int fp64_planes(int Np, int Nw, size_t budget);
 cudaError_t fp64_setup();
 ws_status enqueue_grid64(ws_plan_s *p, const double *uvw, const double2 *vis, int64_t M, double2 *dirty,
                          cudaStream_t s);

@@ -38,3 +38,21 @@ def test_a_second_plan_leaves_the_first_usable(dev, first, second):
             again = _both(a, cs[0], dev)
     for x, y in zip(before, again):                    # gridding sums with FP64 atomics
         assert torch.linalg.norm(x - y) <= 1e-13 * torch.linalg.norm(x)
+
+
+def test_planes_stay_within_the_memory_budget(dev, monkeypatch):
+    """WS_STACK_BYTES bounds the chunk of planes down to one, and the result does not depend on it."""
+    c = case(N=128, M=300, W=6, wfac=16.0, seed=5)
+    plane = (2 * c["N"]) ** 2 * 16
+    out, used = [], []
+    for planes in (0, 5, 0.5):
+        if planes:
+            monkeypatch.setenv("WS_STACK_BYTES", str(int(planes * plane)))
+        with _plan(c, dev) as p:
+            used.append(p.workspace_bytes)
+            out.append(_both(p, c, dev))
+            assert p.Nw > 8
+    assert used[0] - used[1] == (p.Nw - 5) * plane and used[0] - used[2] == (p.Nw - 1) * plane
+    for o in out[1:]:
+        for x, y in zip(out[0], o):                    # the same terms, summed in another order
+            assert torch.linalg.norm(x - y) <= 1e-13 * torch.linalg.norm(x)
