@@ -82,7 +82,8 @@ enum {
                                       column in 64-bit fixed point (a power-of-two scale per column keeps
                                       every sum below 2^62, resolution about 1e-19 of the column's largest
                                       possible sum), so ws_grid's dirty image does not depend on the order
-                                      of the visibilities or of the GPU's atomics.  Slower gridding (twice
+                                      of the visibilities or of the GPU's atomics, nor on how many planes
+                                      are in memory at once (planes_per_chunk, a batch's slice).  Slower gridding (twice
                                       the shared memory per CTA); degridding is deterministic anyway.  For
                                       the FP32 path (not WS_FLAG_FP64 plans). */
 };

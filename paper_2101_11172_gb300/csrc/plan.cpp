@@ -924,7 +924,12 @@ ws_status plan_create(ws_plan_s **out, int32_t N, double x0, int32_t W, double f
     WS_TRY(dev_alloc(&p->d_offsets, (size_t)p->ntiles + 1, &p->bytes), "allocating tile offsets");
     WS_TRY(dev_alloc(&p->d_blocksums, (size_t)4096, &p->bytes), "allocating scan sums");
     if (!fp64) {                                  // FP64 plans have a sum of their own (d_acc64)
-        p->row_shares = inv_row_shares(p->fft_inv, N, p->P > 0 ? std::min(p->P, L.Nw) : L.Nw, p->sms);
+        if (flags & WS_FLAG_DETERMINISTIC) {
+            p->row_shares = inv_row_shares(p->fft_inv, N, L.Nw, kSharesSms);
+            p->share_planes = (L.Nw + p->row_shares - 1) / p->row_shares;
+        } else {
+            p->row_shares = inv_row_shares(p->fft_inv, N, p->P > 0 ? std::min(p->P, L.Nw) : L.Nw, p->sms);
+        }
         WS_TRY(dev_alloc(&p->d_acc, (size_t)p->row_shares * N * N, &p->bytes), "allocating the accumulators");
         WS_TRY(dev_alloc(&p->d_rows_done, (size_t)N, &p->bytes), "allocating row counters");
         WS_TRY(cudaMemset(p->d_rows_done, 0, (size_t)N * sizeof(unsigned)), "clearing row counters");

@@ -415,7 +415,9 @@ inline RowsSmem rows_smem(const FftPlan &F, int N) {
 // shared memory; the last FFT stage screens and accumulates.  Where a row is
 // shared, every share keeps its own sums in acc (N x N per share), and the CTA
 // that finishes the row last adds them up in share order, so the result does not
-// depend on which one that is.
+// depend on which one that is.  With share_planes > 0 (deterministic plans) share g
+// owns planes [g share_planes, (g + 1) share_planes) of the plan instead, in
+// whichever chunks they come, so that the sums do not depend on the chunks either.
 //
 // The rows come by TMA in boxes of up to 256 column blocks (8 KB), all
 // completing on the buffer's mbarrier: with two buffers, plane p + 1's row is
@@ -427,7 +429,7 @@ inline RowsSmem rows_smem(const FftPlan &F, int N) {
 template <int NP, bool CROP, bool ONE_BUFFER, bool HALF>
 __global__ void __launch_bounds__(row_threads_max<NP>(), row_ctas<NP>())
 inv_rows_kernel(Launch L, FftPlan F, const float2 *__restrict__ tw, const __grid_constant__ CUtensorMap row_map,
-                const uint8_t *__restrict__ col_occ, int plane0, int planes, int buf_slots,
+                const uint8_t *__restrict__ col_occ, int plane0, int planes, int share_planes, int buf_slots,
                 const float2 *__restrict__ zsplit, const float *__restrict__ corr, float4 *__restrict__ acc,
                 unsigned *__restrict__ rows_done, int first, int last, float2 *__restrict__ dirty,
                 unsigned long long *__restrict__ timeouts, int wait_polls) {
@@ -437,8 +439,10 @@ inv_rows_kernel(Launch L, FftPlan F, const float2 *__restrict__ tw, const __grid
     const int ii = blockIdx.x, tid = threadIdx.x, T = NP ? row_threads_max<NP>() : (int)blockDim.x;
     const int R0 = NP ? fftst::Radices<NP ? NP : 512>::r0 : F.radix[0], nb = NP ? NP / 16 : F.nb[0];
     const int shares = gridDim.y, nvalid = min(planes, L.Nw - plane0);
-    const int per = (nvalid + shares - 1) / shares;
-    const int p_begin = min(nvalid, (int)blockIdx.y * per), p_end = min(nvalid, p_begin + per);
+    const int per = share_planes > 0 ? share_planes : (nvalid + shares - 1) / shares;
+    const int own = (int)blockIdx.y * per - (share_planes > 0 ? plane0 : 0);
+    const int p_begin = min(nvalid, max(0, own)), p_end = min(nvalid, max(0, own + per));
+    if (p_begin == p_end && !first && !last) return;         // nothing to add in this chunk
     const size_t pix0 = (size_t)ii * N, image = (size_t)N * N;
     float4 *own_acc = acc + blockIdx.y * image;
     // 128-byte aligned start, by pointer arithmetic on sbuf so that every
@@ -712,7 +716,8 @@ struct Transforms {
         const RowsSmem sm = rows_smem(p->fft_inv, p->L.N);
         auto go = [&](auto kernel) {
             kernel<<<dim3(p->L.N, p->row_shares), row_threads(p->fft_inv), sm.bytes, s>>>(
-                p->L, p->fft_inv, p->d_tw, map, p->d_col_occ, chunk * p->P, planes, (int)(sm.buf / sizeof(float2)), p->d_zsplit, p->d_corr, p->d_acc, p->d_rows_done, first ? 1 : 0,
+                p->L, p->fft_inv, p->d_tw, map, p->d_col_occ, chunk * p->P, planes, p->share_planes,
+                (int)(sm.buf / sizeof(float2)), p->d_zsplit, p->d_corr, p->d_acc, p->d_rows_done, first ? 1 : 0,
                 last ? 1 : 0, dirty, p->d_drop + 2, p->wait_polls);
         };
         with_crop(p->L, [&](auto crop) {

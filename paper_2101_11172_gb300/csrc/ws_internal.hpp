@@ -142,6 +142,7 @@ struct ws_plan_s {
     uint8_t *d_tile_occ = nullptr; // ntiles: 1 if any visibility footprint touches the tile
     uint8_t *d_col_occ = nullptr;  // ntt x ntu: 1 if any tile of that (t-tile, u-tile) strip is touched
     int row_shares = 1;            // shares of the planes per image row in inv_rows (transforms.cu)
+    int share_planes = 0;          // planes of each share, cut at fixed planes of the plan; 0: equal parts of each chunk
     float4 *d_acc = nullptr;       // row_shares x N x N: (sum re, sum im, comp re, comp im)
     unsigned *d_rows_done = nullptr;   // N: shares of the row that are done, zero between calls
     unsigned long long *d_drop = nullptr;   // kCounters: [0] non-finite uv, [1] w out of range, [2] timed-out waits
@@ -253,6 +254,9 @@ cudaError_t launch_degrid_chunk(const ws_plan_s *p, int chunk, int planes, int64
 
 // Plane transforms (transforms.cu).
 size_t transform_smem_bytes(const FftPlan &fwd, const FftPlan &inv, int N);
+// Deterministic plans take their shares for this many SMs (a GB300's) and for all the plan's planes, whatever
+// GPU and chunk they get, so that the sums over the planes are the same everywhere.
+constexpr int kSharesSms = 152;
 int inv_row_shares(const FftPlan &F, int N, int planes, int sms);
 cudaError_t setup_transform_kernels(const FftPlan &fwd, const FftPlan &inv, int N);
 cudaError_t launch_fwd_rows(const ws_plan_s *p, const float2 *image, int chunk, int planes, cudaStream_t s);

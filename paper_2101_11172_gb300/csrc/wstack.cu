@@ -559,9 +559,9 @@ __device__ __forceinline__ void flush_slices(int from, int to, const Launch &L, 
 // fixed point with one scale 2^scale for the CTA, chosen so that no sum can
 // exceed 2^62: |sum| <= E max|V~| wbound for the column's E entries, wbound
 // bounding |C_x C_y C_z|.  The scale depends only on the column's set of
-// entries, and integer additions do not depend on their order, so the stack
-// -- and the dirty image -- come out bit for bit the same whatever order the
-// binning's atomics and the warps' schedule give the entries.
+// entries (all of them, whatever the chunk), and integer additions do not depend on
+// their order, so the stack -- and the dirty image -- come out bit for bit the same
+// whatever order the binning's atomics and the warps' schedule give the entries.
 template <int W, int R, bool DET>
 __global__ void __launch_bounds__(kGridThreads, grid_ctas_per_sm(W, R, DET))
 grid3d_kernel(Launch L, const float *__restrict__ coef, int deg, const VisRec *__restrict__ rec,
@@ -578,8 +578,8 @@ grid3d_kernel(Launch L, const float *__restrict__ coef, int deg, const VisRec *_
     const int k_lo = max(0, chunk_tt0 - (TT + W - 2) / TT), k_hi = chunk_tt0 + chunk_ntt;
     const int plo = chunk_tt0 * TT, phi = plo + chunk_ntt * TT;
     const uint32_t *__restrict__ off = offsets + ((size_t)tv * L.ntu + tu) * L.ntt;
-    const uint32_t all_beg = off[k_lo], all_end = off[k_hi];
-    if (all_beg == all_end) return;                  // untouched column: the transforms treat it as zero
+    if (off[k_lo] == off[k_hi]) return;              // untouched column: the transforms treat it as zero
+    const uint32_t all_beg = DET ? off[0] : 0u, all_end = DET ? off[L.ntt] : 0u;     // DET: the column's entries
     float *scoef = reinterpret_cast<float *>(smem + Sm::coef);
     {
         float4 *qre = reinterpret_cast<float4 *>(smem + Sm::re), *qim = reinterpret_cast<float4 *>(smem + Sm::im);

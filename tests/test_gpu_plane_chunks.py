@@ -1,0 +1,56 @@
+"""What a call gives when its planes come in several chunks (little free memory, a batch's slice)."""
+import numpy as np
+import pytest
+import torch
+
+from gpu_helpers import rel, tol_for
+from paper_2101_11172_gb300 import synth
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def dev():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    import __graft_entry__
+    __graft_entry__.build()
+    return torch.device("cuda", 0)
+
+
+def _case(N, M, w_half, seed, fov=0.2):
+    rng = synth.rng_for(0, 9000 + seed)
+    uvw = synth.disc_uvw(M, 0.45 * N / fov, w_half, rng)
+    return dict(N=N, fov=fov, uvw=uvw, vis=synth.complex_normal(M, rng), w_min=float(uvw[:, 2].min()),
+                w_max=float(uvw[:, 2].max()))
+
+
+def _plan(c, dev, W=7, x0=0.25, flags=0):
+    from paper_2101_11172_gb300.wstack import Plan
+    return Plan(c["N"], x0, W, c["fov"], c["w_min"], c["w_max"], flags=flags, device=dev)
+
+
+def _inputs(c, dev):
+    return torch.from_numpy(c["uvw"]).to(dev), torch.from_numpy(c["vis"]).to(torch.complex64).to(dev)
+
+
+@pytest.mark.parametrize("N,W,x0", [(64, 7, 0.25), (200, 10, 0.25), (256, 7, 0.25), (512, 4, 0.375)])
+def test_deterministic_image_does_not_depend_on_the_chunks(dev, monkeypatch, N, W, x0):
+    """Bit for bit, over chunks of 8 planes up to all of them and in a batch's small slice."""
+    from paper_2101_11172_gb300 import WS_FLAG_DETERMINISTIC
+    from paper_2101_11172_gb300.batch import Batch
+    c = _case(N, 3000, 6000.0 * x0, N)              # 67 planes
+    uvw, vis = _inputs(c, dev)
+    images = []
+    for chunk in (0, 8, 24, 64):
+        if chunk:
+            monkeypatch.setenv("WS_PLANES_PER_CHUNK", str(chunk))
+        with _plan(c, dev, W, x0, WS_FLAG_DETERMINISTIC) as p:
+            assert p.Nw > 64 and (p.planes_per_chunk == chunk or not chunk)
+            images.append(p.grid(uvw, vis))
+            Np = p.Np
+    with Batch([(N, c["fov"], c["w_min"], c["w_max"], 3000)], x0, W, branches=1, workspace_bytes=17 * Np * Np * 8,
+               flags=WS_FLAG_DETERMINISTIC, device=dev) as b:
+        images += b.grid([uvw], [vis])
+    for d in images[1:]:
+        assert torch.equal(d, images[0])
