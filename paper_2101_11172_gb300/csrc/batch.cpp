@@ -110,6 +110,9 @@ bool assign(ws_batch_s *b, int K) {
         const size_t fit = slice / plane_bytes(p);
         if (fit < (size_t)TT) return false;
         p->P = (int)std::min<size_t>((size_t)total, (fit / TT) * TT);
+        // shares for the planes that the slice holds, at most those allocated for all planes: with more shares
+        // than planes, each empty one still reads and writes its image of sums for every chunk
+        if (p->share_planes == 0) p->row_shares = inv_row_shares(p->fft_inv, p->L.N, std::min(p->P, p->L.Nw), p->sms);
         p->d_stack = reinterpret_cast<float2 *>(reinterpret_cast<char *>(b->workspace) + slice * b->branch_of[i]);
     }
     b->K = K;

@@ -1,9 +1,8 @@
 """What a call gives when its planes come in several chunks (little free memory, a batch's slice)."""
-import numpy as np
 import pytest
 import torch
 
-from gpu_helpers import rel, tol_for
+from gpu_helpers import rel
 from paper_2101_11172_gb300 import synth
 
 pytestmark = pytest.mark.gpu
@@ -54,3 +53,18 @@ def test_deterministic_image_does_not_depend_on_the_chunks(dev, monkeypatch, N, 
         images += b.grid([uvw], [vis])
     for d in images[1:]:
         assert torch.equal(d, images[0])
+
+
+@pytest.mark.parametrize("planes", [9, 17, 40])
+def test_batch_in_a_small_slice(dev, planes):
+    """Rows shared by no more CTAs than a chunk has planes give the plan's image to summation order."""
+    from paper_2101_11172_gb300.batch import Batch
+    c = _case(128, 3000, 1500.0, planes)
+    uvw, vis = _inputs(c, dev)
+    with _plan(c, dev) as p:
+        assert p.Nw > 60
+        whole, Np = p.grid(uvw, vis), p.Np
+    with Batch([(128, c["fov"], c["w_min"], c["w_max"], 3000)], 0.25, 7, branches=1,
+               workspace_bytes=planes * Np * Np * 8, device=dev) as b:
+        for _ in range(2):
+            assert rel(b.grid([uvw], [vis])[0].cpu().numpy(), whole.cpu().numpy()) < 1e-6
