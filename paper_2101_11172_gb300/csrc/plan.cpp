@@ -1071,22 +1071,28 @@ ws_status enqueue_grid(ws_plan_s *p, const double *uvw, const float2 *vis, int64
     }
     const int total = p->L.ntt * TT;
     const int nchunks = (total + p->P - 1) / p->P;
+    // a call that ends between its chunks must not leave rows marked for the next one
+    auto abandon = [&](const char *what) {
+        const ws_status st = cuda_fail(e, what);
+        cudaMemsetAsync(p->d_rows_done, 0, (size_t)p->L.N * sizeof(unsigned), s);
+        return st;
+    };
     for (int c = 0; c < nchunks; ++c) {
         const int planes = std::min(p->P, total - c * p->P);
         {
             StageTimer t(p, s, WS_STAGE_GRID3D, 1);
             if ((e = launch_grid_chunk(p, c, planes, s)) != cudaSuccess)
-                return cuda_fail(e, "ws_grid: grid3d kernel");
+                return abandon("ws_grid: grid3d kernel");
         }
         {
             StageTimer t(p, s, WS_STAGE_COLS_INV, 1);
             if ((e = launch_inv_cols(p, c, planes, s)) != cudaSuccess)
-                return cuda_fail(e, "ws_grid: inv_cols kernel");
+                return abandon("ws_grid: inv_cols kernel");
         }
         {
             StageTimer t(p, s, WS_STAGE_ROWS_INV, 1);
             if ((e = launch_inv_rows(p, c, planes, c == 0, c == nchunks - 1, dirty, s)) != cudaSuccess)
-                return cuda_fail(e, "ws_grid: inv_rows kernel");
+                return abandon("ws_grid: inv_rows kernel");
         }
     }
     return WS_OK;

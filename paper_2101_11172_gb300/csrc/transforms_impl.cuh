@@ -425,7 +425,9 @@ inline RowsSmem rows_smem(const FftPlan &F, int N) {
 // the last stage, whose inputs are in registers by then, finishes plane p.  Strips no footprint touched hold stale
 // data; the first FFT stage masks them to zero.  Every wait is bounded; a CTA
 // that gives up waits (bounded) for the copy in flight and ends; *timeouts
-// counts the rows left incomplete.
+// counts the rows left incomplete, once each however many shares and chunks
+// gave up, and they are not written.
+constexpr unsigned kRowIncomplete = 0x10000u;      // above the count of a row's finished shares
 template <int NP, bool CROP, bool ONE_BUFFER, bool HALF>
 __global__ void __launch_bounds__(row_threads_max<NP>(), row_ctas<NP>())
 inv_rows_kernel(Launch L, FftPlan F, const float2 *__restrict__ tw, const __grid_constant__ CUtensorMap row_map,
@@ -553,35 +555,29 @@ inv_rows_kernel(Launch L, FftPlan F, const float2 *__restrict__ tw, const __grid
             fft_inplace<ONE_BUFFER>(row_buf(k), F, tw, tid, T, between, store, live);
     }
     __syncthreads();
-    if (shares == 1 || !last) {
-        if (gave_up) {
-            if (tid == 0) atomicAdd(timeouts, 1ull);
-            return;
-        }
-    }
-    if (!(last && shares == 1))
+    // a row that misses a plane of any chunk is marked in its counter
+    if (gave_up && tid == 0) atomicOr(&rows_done[ii], kRowIncomplete);
+    if (!gave_up && !(last && shares == 1))
         for (int jj = tid; jj < N; jj += T) own_acc[pix0 + jj] = srow[jj];
     if (!last) return;
-    if (shares > 1) {
-        // the row's counter holds the finished shares and, above bit 16, those that
-        // gave up; the last one to finish leaves it zero for the next call
-        __threadfence();
-        __syncthreads();
-        if (tid == 0) {
-            const unsigned mine = gave_up ? 0x10001u : 1u, all = atomicAdd(&rows_done[ii], mine) + mine;
-            finisher = (all & 0xffffu) == (unsigned)shares ? 1 : 0;
-            if (finisher) {
-                rows_done[ii] = 0u;
-                if (all >> 16) {                 // an incomplete row counts once
-                    atomicAdd(timeouts, 1ull);
-                    finisher = 0;
-                }
+    // the counter's low bits hold the finished shares; the last one to finish leaves it
+    // zero for the next call, counts an incomplete row once and does not write it
+    __threadfence();
+    __syncthreads();
+    if (tid == 0) {
+        const unsigned all = atomicAdd(&rows_done[ii], 1u) + 1u;
+        finisher = (all & (kRowIncomplete - 1u)) == (unsigned)shares ? 1 : 0;
+        if (finisher) {
+            rows_done[ii] = 0u;
+            if (all & kRowIncomplete) {
+                atomicAdd(timeouts, 1ull);
+                finisher = 0;
             }
-            __threadfence();
         }
-        __syncthreads();
-        if (!finisher) return;
+        __threadfence();
     }
+    __syncthreads();
+    if (!finisher) return;
     for (int jj = tid; jj < N; jj += T) {
         float4 a = shares == 1 ? srow[jj] : __ldcg(acc + pix0 + jj);
         float2 sum = make_float2(a.x, a.y), comp = make_float2(a.z, a.w);

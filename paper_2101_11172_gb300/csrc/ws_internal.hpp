@@ -144,7 +144,7 @@ struct ws_plan_s {
     int row_shares = 1;            // shares of the planes per image row in inv_rows (transforms.cu)
     int share_planes = 0;          // planes of each share, cut at fixed planes of the plan; 0: equal parts of each chunk
     float4 *d_acc = nullptr;       // row_shares x N x N: (sum re, sum im, comp re, comp im)
-    unsigned *d_rows_done = nullptr;   // N: shares of the row that are done, zero between calls
+    unsigned *d_rows_done = nullptr;   // N: shares of the row that are done and a mark if it is incomplete, zero between calls
     unsigned long long *d_drop = nullptr;   // kCounters: [0] non-finite uv, [1] w out of range, [2] timed-out waits
     unsigned long long *h_drop = nullptr;   // pinned mirror
     int wait_polls = ws::kWaitPolls;        // limit of inv_rows' first wait per plane (WS_WAIT_POLLS)

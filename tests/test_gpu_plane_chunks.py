@@ -68,3 +68,28 @@ def test_batch_in_a_small_slice(dev, planes):
                workspace_bytes=planes * Np * Np * 8, device=dev) as b:
         for _ in range(2):
             assert rel(b.grid([uvw], [vis])[0].cpu().numpy(), whole.cpu().numpy()) < 1e-6
+
+
+@pytest.mark.parametrize("N,chunk,flags", [(64, 0, 0), (64, 24, 0), (200, 16, 0), (256, 24, 1 << 6)])
+def test_incomplete_rows_count_once(dev, monkeypatch, N, chunk, flags):
+    """Waits that give up at once (host knob, every copy still lands) in rows shared by several CTAs and
+    planes in several chunks: one count per row, no row written, and the next call is complete."""
+    from paper_2101_11172_gb300 import _lib
+    c = _case(N, 3000, 1500.0, N + chunk)
+    uvw, vis = _inputs(c, dev)
+    if chunk:
+        monkeypatch.setenv("WS_PLANES_PER_CHUNK", str(chunk))
+    with _plan(c, dev, flags=flags) as p:
+        assert p.Nw > 60
+        want = p.grid(uvw, vis)
+        p.stats(reset=True)
+        out = torch.full_like(want, 7.0)
+        monkeypatch.setenv("WS_WAIT_POLLS", "0")
+        with pytest.raises(_lib.WsError) as err:
+            p.grid(uvw, vis, out=out)
+        assert err.value.status == _lib.WS_ERR_TIMEOUT
+        assert p.stats(reset=True)["waits_timed_out"] == N
+        assert bool((out == 7.0).all())
+        monkeypatch.delenv("WS_WAIT_POLLS")
+        assert rel(p.grid(uvw, vis, out=out).cpu().numpy(), want.cpu().numpy()) < 1e-6
+        assert p.stats()["waits_timed_out"] == 0
