@@ -980,6 +980,9 @@ ws_status plan_create(ws_plan_s **out, int32_t N, double x0, int32_t W, double f
                "allocating pinned occupancy counts");
         std::memset(p->h_occ_counts, 0, ((size_t)2 * L.ntt + 1) * sizeof(uint32_t));
     }
+    // the tables and the cleared row counters are there before any call, on whatever stream: the clearing is
+    // work on the legacy stream, which streams made with cudaStreamNonBlocking do not wait for
+    WS_TRY(cudaStreamSynchronize(nullptr), "waiting for the plan's tables");
 #undef WS_TRY
     // the tuned tile rows for this (GPU, N', W), when a tuning cache is named
     if (const char *cache = std::getenv("WS_TUNE_CACHE")) {

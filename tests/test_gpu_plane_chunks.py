@@ -93,3 +93,20 @@ def test_incomplete_rows_count_once(dev, monkeypatch, N, chunk, flags):
         monkeypatch.delenv("WS_WAIT_POLLS")
         assert rel(p.grid(uvw, vis, out=out).cpu().numpy(), want.cpu().numpy()) < 1e-6
         assert p.stats()["waits_timed_out"] == 0
+
+
+def test_new_plans_on_a_stream_of_their_own(dev):
+    """A plan's first call, on a stream that is not ordered after the default one, finds its row counters cleared."""
+    c = _case(64, 3000, 1500.0, 3)
+    uvw, vis = _inputs(c, dev)
+    with _plan(c, dev) as p:
+        want = p.grid(uvw, vis).cpu().numpy()
+    side = torch.cuda.Stream(dev)
+    side.wait_stream(torch.cuda.current_stream(dev))
+    for _ in range(20):
+        torch.cuda.empty_cache()                       # the next plan's buffers may be memory that held anything
+        with _plan(c, dev) as p, torch.cuda.stream(side):
+            out = torch.zeros(64, 64, dtype=torch.complex64, device=dev)
+            p.grid(uvw, vis, out=out)
+            side.synchronize()
+            assert rel(out.cpu().numpy(), want) < 1e-6
