@@ -115,17 +115,23 @@ __device__ __forceinline__ float2 step_screen(float2 g, float2 e) {
 // pixel's screened value advances one plane by a product with exp(-2 pi i z).
 constexpr int kScreenSteps = 8;
 
-// One CTA owns image row ii for a run of planes.  Shared memory keeps the
-// screened row g = row x exp(-2 pi i t z) and the step exp(-2 pi i z), so each
-// plane costs the step, one FFT and the stores of the strips some footprint
-// reads.  g is evaluated exactly on every kScreenSteps-th plane of the CTA's
-// share; on the planes between, the FFT's first stage reads g and leaves g x step
-// in its place for the next plane.  Each pixel is read by the same thread on
-// every plane, so the update needs no barrier.  The exact evaluations read the
-// corrected row and its z from shared memory too (keep_rows), or, where that
-// would leave one CTA per SM, from global memory (N = 4096: evaluating the
-// screen exactly on every plane instead cost 12 % of the kernel there).
-template <int NP, bool CROP>
+// One CTA owns image row ii for a run of planes.
+//
+// STEP (fwd_rows_step): shared memory keeps the screened row g = row x exp(-2 pi i
+// t z) and the step exp(-2 pi i z), so each plane costs the step, one FFT and the
+// stores of the strips some footprint reads.  g is evaluated exactly on every
+// kScreenSteps-th plane of the CTA's share; on the planes between, the FFT's first
+// stage reads g and leaves g x step in its place for the next plane.  Each pixel is
+// read by the same thread on every plane, so the update needs no barrier.  The exact
+// evaluations read the corrected row and its z from shared memory too (keep_rows),
+// or, where that would cost a resident CTA, from global memory.
+//
+// Otherwise shared memory keeps the row and half a row of z and of the plane's
+// screen, evaluated exactly on every plane as in inv_rows: the N/2 + 1 screens that
+// a pixel and its mirror image share.  That takes the room of STEP's two rows.
+// Stepping these sizes too (N above about 2400) took 29.4 instead of 30.0 ms at N = 4096
+// (282 planes) but moved the error against the exact DFT: 2.07e-7 -> 2.35e-7 at N = 2560.
+template <int NP, bool CROP, bool STEP>
 __global__ void __launch_bounds__(row_threads_max<NP>(), row_ctas<NP>())
 fwd_rows_kernel(Launch L, FftPlan F, const float2 *__restrict__ tw, const float2 *__restrict__ img,
                 const float *__restrict__ corr, const float2 *__restrict__ zsplit, const uint8_t *__restrict__ col_occ, int plane0, int planes,
@@ -134,9 +140,12 @@ fwd_rows_kernel(Launch L, FftPlan F, const float2 *__restrict__ tw, const float2
     const int Np = L.Np, N = L.N, half = N / 2;
     float2 *grow = sbuf + F.stride;                              // N: the screened row (F.stride is even: 16-byte aligned)
     float2 *erow = grow + N;                                     // N: exp(-2 pi i z)
-    float2 *irow = erow + N;                                     // N if keep_rows
+    float2 *irow = STEP ? erow + N : grow;                       // N if keep_rows
     float2 *zrow = irow + N;                                     // N if keep_rows
-    uint8_t *occ = reinterpret_cast<uint8_t *>(erow + (keep_rows ? 3 : 1) * N);   // ntu: strips of the current t-tile
+    float2 *scr = irow + N;                                      // N/2 + 1 unless STEP: exp(2 pi i t z)
+    float2 *zhalf = scr + N / 2 + 1;                             // N/2 + 1 unless STEP: z
+    uint8_t *occ = reinterpret_cast<uint8_t *>(STEP ? erow + (keep_rows ? 3 : 1) * N
+                                                    : zhalf + N / 2 + 1);   // ntu: strips of the current t-tile
     const int ii = blockIdx.x, tid = threadIdx.x, T = NP ? row_threads_max<NP>() : (int)blockDim.x;
     // this CTA's planes: an equal share of the chunk's valid planes
     const int nvalid = min(planes, L.Nw - plane0);
@@ -151,6 +160,11 @@ fwd_rows_kernel(Launch L, FftPlan F, const float2 *__restrict__ tw, const float2
         return make_float2(h * f.x, L.fold ? 0.f : h * f.y);
     };
     for (int jj = tid; jj < N; jj += T) {
+        if (!STEP) {
+            irow[jj] = corrected(jj);
+            if (jj <= N / 2) zhalf[jj] = zsplit[pix0 + N / 2 - jj];
+            continue;
+        }
         const float2 z = zsplit[pix0 + jj];
         if (keep_rows) {
             irow[jj] = corrected(jj);
@@ -187,21 +201,39 @@ fwd_rows_kernel(Launch L, FftPlan F, const float2 *__restrict__ tw, const float2
             occ_tt = tt;
             __syncthreads();
         }
-        if ((p - p_begin) % kScreenSteps == 0) {
+        // row x exp(-i phi), phi = 2 pi t z: (f.x cs + f.y sn, f.y cs - f.x sn), the products with f.x rounded first
+        auto screened = [](float2 f, float sn, float cs) {
+            return fma2(dup2(f.y), make_float2(sn, cs), mul2(dup2(f.x), make_float2(cs, -sn)));
+        };
+        if (!STEP) {
+            for (int h = tid; h <= N / 2; h += T) {
+                float sn, cs;
+                phase_tz(t, zhalf[h], &sn, &cs);
+                scr[h] = make_float2(cs, sn);
+            }
+            __syncthreads();
+        } else if ((p - p_begin) % kScreenSteps == 0) {
             for (int jj = tid; jj < N; jj += T) {
-                // row x exp(-i phi), phi = 2 pi t z: (f.x cs + f.y sn, f.y cs - f.x sn), the products with f.x rounded first
-                const float2 f = keep_rows ? irow[jj] : corrected(jj);
                 float sn, cs;
                 phase_tz(t, keep_rows ? zrow[jj] : zsplit[pix0 + jj], &sn, &cs);
-                grow[jj] = fma2(dup2(f.y), make_float2(sn, cs), mul2(dup2(f.x), make_float2(cs, -sn)));
+                grow[jj] = screened(keep_rows ? irow[jj] : corrected(jj), sn, cs);
             }
             __syncthreads();
         }
-        const bool step = (p + 1 - p_begin) % kScreenSteps != 0 && p + 1 < p_end;   // uniform: advance g
+        const bool step = STEP && (p + 1 - p_begin) % kScreenSteps != 0 && p + 1 < p_end;   // uniform: advance g
         auto load = [&](auto pruned, int, int J0, int dJ, auto &v) {
             constexpr int R = length_of<decltype(v)>();
             constexpr bool P = decltype(pruned)::value;
-            if constexpr (NP == 0) {
+            if constexpr (!STEP) {
+                for_live<R, P>([&](int m) {
+                    const unsigned jj = grid_to_crop(J0 + m * dJ, half, Np);
+                    v[m] = make_float2(0.f, 0.f);
+                    if (jj >= (unsigned)N) return;
+                    const float2 s = scr[abs((int)jj - half)];
+                    v[m] = screened(irow[jj], s.y, s.x);
+                });
+                return;
+            } else if constexpr (NP == 0) {
                 // (runtime plans: reading all steps first took more registers than it saved time)
                 for_live<R, P>([&](int m) {
                     const unsigned jj = grid_to_crop(J0 + m * dJ, half, Np);
@@ -597,14 +629,17 @@ inline size_t smem2(const FftPlan &F) {
     return (size_t)kPerCta * slots * sizeof(float2) + F.n / TU + 16;
 }
 inline size_t smem_fwd_rows(const FftPlan &F, int N, bool keep_rows) {
-    return (size_t)F.stride * sizeof(float2) + (size_t)N * (keep_rows ? 4 : 2) * sizeof(float2) + F.n / TU + 16;
+    return (size_t)F.stride * sizeof(float2) + (size_t)N * (keep_rows ? 4 : 2) * sizeof(float2) + F.n / TU + 32;
 }
-// fwd_rows keeps the image row and z in shared memory where that costs no resident CTA
+// fwd_rows steps its screen where four rows leave room for two CTAs per SM: N up to
+// about 2400 at x0 = 1/4.  Larger sizes evaluate it on every plane (the reason: at the kernel).
+inline bool fwd_rows_step(const FftPlan &F, int N) { return smem_fwd_rows(F, N, true) <= cta_smem(2); }
+// a stepping fwd_rows keeps the image row and z in shared memory where that costs no resident CTA
 inline bool fwd_rows_keep(const FftPlan &F, int N) {
     auto fit = [&](bool keep) {
         return std::min<size_t>(row_cta_limit(F), 228 * 1024 / (smem_fwd_rows(F, N, keep) + 1024));
     };
-    return smem_fwd_rows(F, N, true) <= cta_smem(1) && fit(true) == fit(false);
+    return fwd_rows_step(F, N) && fit(true) == fit(false);
 }
 // CTAs per image row in fwd_rows (each takes an equal share of the planes):
 // enough rows x groups for about 32 CTAs per SM over the launch,
@@ -633,12 +668,16 @@ cudaError_t row_tensor_map(const ws_plan_s *p, CUtensorMap *map);
 // Launchers of one FFT variant.
 template <int NP>
 struct Transforms {
+    // N <= N' <= 2048 fits four rows in half an SM's shared memory, and so does N = N'/2 = 2048
+    static constexpr bool kMayNotStep = NP == 0 || NP == 4096;
     static cudaError_t setup(const FftPlan &F, const FftPlan &inv, int N) {
         cudaError_t e;
         const size_t rows = smem_fwd_rows(F, N, fwd_rows_keep(F, N));
-        if ((e = allow_smem(fwd_rows_kernel<NP, false>, rows)) != cudaSuccess) return e;
+        if ((e = allow_smem(fwd_rows_kernel<NP, false, true>, rows)) != cudaSuccess) return e;
         if constexpr (NP != 0)
-            if ((e = allow_smem(fwd_rows_kernel<NP, true>, rows)) != cudaSuccess) return e;
+            if ((e = allow_smem(fwd_rows_kernel<NP, true, true>, rows)) != cudaSuccess) return e;
+        if constexpr (kMayNotStep)
+            if ((e = allow_smem(fwd_rows_kernel<NP, false, false>, rows)) != cudaSuccess) return e;
         if ((e = allow_smem(fwd_cols_kernel<NP, false>, smem2(F))) != cudaSuccess) return e;
         if constexpr (NP != 0)
             if ((e = allow_smem(fwd_cols_kernel<NP, true>, smem2(F))) != cudaSuccess) return e;
@@ -679,12 +718,19 @@ struct Transforms {
     static cudaError_t fwd_rows(const ws_plan_s *p, const float2 *image, int chunk, int planes, cudaStream_t s) {
         const bool keep = fwd_rows_keep(p->fft_fwd, p->L.N);
         const dim3 grid(p->L.N, row_groups(p->L.N, planes, p->sms));
-        with_crop(p->L, [&](auto crop) {
-            fwd_rows_kernel<NP, decltype(crop)::value>
-                <<<grid, row_threads(p->fft_fwd), smem_fwd_rows(p->fft_fwd, p->L.N, keep), s>>>(
-                    p->L, p->fft_fwd, p->d_tw, image, p->d_corr, p->d_zsplit, p->d_col_occ, chunk * p->P, planes, keep ? 1 : 0,
-                    p->d_stack);
-        });
+        auto go = [&](auto kernel) {
+            kernel<<<grid, row_threads(p->fft_fwd), smem_fwd_rows(p->fft_fwd, p->L.N, keep), s>>>(
+                p->L, p->fft_fwd, p->d_tw, image, p->d_corr, p->d_zsplit, p->d_col_occ, chunk * p->P, planes,
+                keep ? 1 : 0, p->d_stack);
+        };
+        if (!fwd_rows_step(p->fft_fwd, p->L.N)) {
+            if constexpr (kMayNotStep)
+                go(fwd_rows_kernel<NP, false, false>);
+            else
+                return cudaErrorInvalidValue;
+            return cudaGetLastError();
+        }
+        with_crop(p->L, [&](auto crop) { go(fwd_rows_kernel<NP, decltype(crop)::value, true>); });
         return cudaGetLastError();
     }
     static cudaError_t fwd_cols(const ws_plan_s *p, int chunk, int planes, cudaStream_t s) {
