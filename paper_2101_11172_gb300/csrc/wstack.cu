@@ -769,54 +769,33 @@ grid3d_kernel(Launch L, const float *__restrict__ coef, int deg, const VisRec *_
 }
 
 // ---------------------------------------------------------------------------
-// Gridding on the tensor cores (W <= 9, 16-row tiles, FP32 sums in any order).
+// Gridding in registers (W <= 9, 16-row tiles, FP32 sums in any order).
 //
-// A bin's contribution to the 16 planes its footprints can reach (8 + W - 1 <=
-// 16) is a contraction over its entries e:
-//   G[t][v][u] += sum_e C_z[e][t] (C_y[e][v] C_x[e][u] V_e),
-// a matrix product of M = 16 planes, N = 512 (16 x 16 cells, re and im) and K =
-// the entries.  Each warp keeps the sums of its 4 x 8 cells for all 16 planes in
-// mma.m16n8k8 accumulators, plane t in fragment row t mod 16: a t-tile's planes are
-// registers 0 and 1 or 2 and 3, and moving on to the next bin writes out and clears
-// one half; there is no ring in shared memory, and there are no atomics.
+// A bin's footprints reach 16 planes (8 + W - 1 <= 16).  Each warp owns 4 x 8 of a
+// tile's 16 x 16 cells and a lane one of them, with its sums of all 16 planes in
+// registers, plane t in sum t mod 16: a t-tile's planes are sums 0..7 or 8..15, and
+// moving on to the next bin writes out and clears one half.  There is no ring in
+// shared memory, and there are no atomics.
 //
-// The CTA stages the column's entries kMmaEntries at a time, whatever their bins:
-// per entry its weights at the tile's 16 columns and 16 rows and at 16 planes, zero
-// where the footprint does not reach.  (A chunk per bin, 11 entries at the median,
-// spent most of its instructions on the staging's fixed part.)  A warp then takes only the entries that touch its cells (29 % of a
-// tile's for W = 7), eight at a time, and forms the B operand C_y C_x V in registers.
+// The CTA stages the column's entries kRegEntries at a time, whatever their bins: per
+// entry its weights at the tile's 16 columns and 16 rows and at 16 planes, zero where
+// the footprint does not reach.  (A chunk per bin, 11 entries at the median, spent
+// most of its instructions on the staging's fixed part.)  A warp then takes only the
+// entries that touch its cells (29 % of a tile's for W = 7): a lane forms C_x C_y V
+// for its cell once and adds C_z C_x C_y V to its 16 sums, one packed multiply-add
+// for both components of a plane.
 //
-// FP32 accuracy from TF32 operands: each factor is split into hi + lo (11 bits
-// and the rest), and lo hi + hi lo + hi hi is summed from zero for each group of
-// eight entries; the group's sum is then added to the accumulators in FP32.  The
-// tensor core truncates its sums, so a running sum kept there would lose more
-// than one kept by FP32 additions.
-constexpr int kMmaMaxW = TT + 1;
-constexpr int kMmaEntries = 64;                    // staged per chunk
-constexpr int kMmaStride = 72;                     // floats per staged entry: bank offset 8 between neighbours
-constexpr int kMmaMaxBins = 520;                   // t-tiles of a column: |t| < 2040, 8 planes each, and two more
-enum : int { kEntU = 0, kEntV = 16, kEntT = 32, kEntVal = 64, kEntMask = 66, kEntNu = 67, kEntOff = 70 };
-
-__device__ __forceinline__ float tf32_near(float x) {      // nearest value with 11 significant bits
-    return __uint_as_float((__float_as_uint(x) + 0x1000u) & 0xffffe000u);
-}
-__device__ __forceinline__ float tf32_cut(float x) { return __uint_as_float(__float_as_uint(x) & 0xffffe000u); }
-
-__device__ __forceinline__ void mma_tf32(float (&d)[4], const float (&a)[4], float b0, float b1) {
-    asm("mma.sync.aligned.m16n8k8.row.col.f32.tf32.tf32.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, {%0, %1, %2, "
-        "%3};"
-        : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
-        : "r"(__float_as_uint(a[0])), "r"(__float_as_uint(a[1])), "r"(__float_as_uint(a[2])),
-          "r"(__float_as_uint(a[3])), "r"(__float_as_uint(b0)), "r"(__float_as_uint(b1)));
-}
-
-__device__ __forceinline__ void mma_tf32_from_zero(float (&d)[4], const float (&a)[4], float b0, float b1) {
-    asm("mma.sync.aligned.m16n8k8.row.col.f32.tf32.tf32.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, {%10, %10, "
-        "%10, %10};"
-        : "=f"(d[0]), "=f"(d[1]), "=f"(d[2]), "=f"(d[3])
-        : "r"(__float_as_uint(a[0])), "r"(__float_as_uint(a[1])), "r"(__float_as_uint(a[2])),
-          "r"(__float_as_uint(a[3])), "r"(__float_as_uint(b0)), "r"(__float_as_uint(b1)), "f"(0.f));
-}
+// Every product and sum is FP32, as in grid3d_kernel.  The same contraction on the
+// tensor cores (mma.m16n8k8, each factor split into two TF32 terms) took 6.63 ms on the
+// survey (18.9 M entries) where this takes 5.29 and grid3d_kernel 9.8, and was less exact:
+// 1.92e-7 from an FP64 plan where these two stay at 1.64e-7 (1,000 visibilities, N = 256,
+// W = 7), and values near 2^-115 lost digits, their low terms below the tensor core's smallest.
+// (The 80 registers that three CTAs an SM allow spill 32 bytes in the staging, 64 for W <= 4.)
+constexpr int kRegMaxW = TT + 1;
+constexpr int kRegEntries = 64;                    // staged per chunk
+constexpr int kRegStride = 60;                     // floats per staged entry: weights read as float4
+constexpr int kRegMaxBins = 520;                   // t-tiles of a column: |t| < 2040, 8 planes each, and two more
+enum : int { kEntU = 0, kEntV = 16, kEntT = 32, kEntVal = 48, kEntOff = 50, kEntNu = 51 };
 
 // Cells 0..15 of a tile axis that a footprint starting `off` cells after the
 // tile's origin (mod n) covers, as bits.
@@ -829,15 +808,15 @@ __device__ __forceinline__ unsigned axis_mask(int off, int n, int W) {
 
 template <int W>
 __global__ void __launch_bounds__(kGridThreads, 3)
-grid3d_mma_kernel(Launch L, const float *__restrict__ coef, int deg, const VisRec *__restrict__ rec,
-                  const uint32_t *__restrict__ offsets, const uint32_t *__restrict__ list, int chunk_tt0,
-                  int chunk_ntt, float2 *__restrict__ stack) {
-    static_assert(W <= kMmaMaxW, "a bin's footprints stay within 16 planes");
-    __shared__ __align__(16) float ents[2][(kMmaEntries + 1) * kMmaStride];
+grid3d_cells_kernel(Launch L, const float *__restrict__ coef, int deg, const VisRec *__restrict__ rec,
+                    const uint32_t *__restrict__ offsets, const uint32_t *__restrict__ list,
+                    const uint8_t *__restrict__ tile_occ, int chunk_tt0, int chunk_ntt, float2 *__restrict__ stack) {
+    static_assert(W <= kRegMaxW, "a bin's footprints stay within 16 planes");
+    __shared__ __align__(16) float ents[2][kRegEntries * kRegStride];
+    __shared__ unsigned masks[2][kRegEntries];     // the entries' cells: columns in bits 0..15, rows in 16..31
     __shared__ __align__(16) float scoef[3 * W * kCoefStride];
-    __shared__ uint32_t soff[kMmaMaxBins];
-    __shared__ uint8_t picks[kGridWarps][kMmaEntries + 8];
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, g = lane >> 2, t4 = lane & 3;
+    __shared__ uint32_t soff[kRegMaxBins];
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int Np = L.Np;
     const int tu = centre_first(blockIdx.x % L.ntu, L.ntu);
     const int tv = centre_first(blockIdx.x / L.ntu, L.ntv);
@@ -853,61 +832,57 @@ grid3d_mma_kernel(Launch L, const float *__restrict__ coef, int deg, const VisRe
         const int l = i / kCoefStride, m = i - l * kCoefStride, axis = l / W;
         scoef[i] = m <= deg ? coef[((axis == 2 ? W : 0) + l - axis * W) * (deg + 1) + m] : 0.f;
     }
-    // entry kMmaEntries of either buffer is the zero that fills up a group of eight
-    for (int i = tid; i < 2 * kMmaStride; i += kGridThreads)
-        ents[i / kMmaStride][kMmaEntries * kMmaStride + i % kMmaStride] = 0.f;
     __syncthreads();
 
     // lanes 0..7 of a warp hold the records of entries warp + 8 lane of the next chunk
     VisRec r{};
     auto fetch = [&] {
         const uint32_t p = pos + warp + kGridWarps * lane;
-        if (lane < kMmaEntries / kGridWarps && p < all_end) r = rec[list[p]];
+        if (lane < kRegEntries / kGridWarps && p < all_end) r = rec[list[p]];
     };
     fetch();
     const int row0 = 4 * (warp >> 1), col0 = 8 * (warp & 1);         // this warp's cells
+    const int row = row0 + (lane >> 3), col = col0 + (lane & 7);     // this lane's
     const unsigned my_cells = (0xffu << col0) | (0xfu << (16 + row0));
-    float c[4][2][4];                                                // [row][re, im][fragment]
+    float2 c[16];
 #pragma unroll
-    for (int i = 0; i < 32; ++i) c[i >> 3][(i >> 2) & 1][i & 3] = 0.f;
+    for (int i = 0; i < 16; ++i) c[i] = make_float2(0.f, 0.f);
     const size_t plane = (size_t)Np * Np;
-    // writes out t-tile s, if the chunk owns it, and zeroes its sums: plane t sits in
-    // fragment row t mod 16, so a tile's planes are registers 0, 1 or 2, 3
-    auto flush = [&](int s) {
-        float2 *dst = stack + (size_t)((s - chunk_tt0) * TT + g) * plane +
-                      tiled_index(v_org + row0, u_org + col0 + 2 * t4, Np);
-        const bool odd = s & 1, own = s >= chunk_tt0 && s < k_hi;
+    // writes out t-tile s, if the chunk owns it, and zeroes its sums
+    auto flush = [&](int s, bool touched) {
+        float2 *dst = stack + (size_t)(s - chunk_tt0) * TT * plane + tiled_index(v_org + row, u_org + col, Np);
+        const bool own = touched && s >= chunk_tt0 && s < k_hi;
+        auto half = [&](int first) {
 #pragma unroll
-        for (int j = 0; j < 4; ++j) {
-            float *re = c[j][0], *im = c[j][1];
-            if (own)
-                *reinterpret_cast<float4 *>(dst + j * CB) = make_float4(odd ? re[2] : re[0], odd ? im[2] : im[0],
-                                                                        odd ? re[3] : re[1], odd ? im[3] : im[1]);
-#pragma unroll
-            for (int i = 0; i < 4; ++i) {
-                const bool gone = odd == (i >= 2);
-                re[i] = gone ? 0.f : re[i];
-                im[i] = gone ? 0.f : im[i];
+            for (int i = 0; i < TT; ++i) {
+                if (own) dst[i * plane] = c[first + i];
+                c[first + i] = make_float2(0.f, 0.f);
             }
-        }
+        };
+        if (s & 1)
+            half(8);
+        else
+            half(0);
     };
+    // the planes past bin k's t-tile, where some footprint of the bin or the bins before may have reached
+    auto flush_next = [&](int s) { flush(s, s < k_hi && tile_occ[((size_t)s * L.ntv + tv) * L.ntu + tu]); };
     const int axis = lane / W < 3 ? lane / W : 2, tap = lane - axis * W;     // staging: this lane's weight slot
-    const int off_shift = 13 * axis, axis_len = axis == 2 ? 16 : Np, axis_base = 16 * axis, axis_log = axis == 2 ? 1 : 0;
+    const int off_shift = 13 * axis, axis_len = axis == 2 ? 16 : Np, axis_base = 16 * axis;
     const unsigned off_mask = axis == 2 ? 15u : 0x1fffu;
     int k = k_lo, cur = -1, buf = 0;
     while (pos < all_end) {
-        const int n = (int)min((uint32_t)kMmaEntries, all_end - pos);
+        const int n = (int)min((uint32_t)kRegEntries, all_end - pos);
         float *ent = ents[buf];
         // 1. staging: this warp's entries warp, warp + 8, ...
         const int mine = n > warp ? (n - warp + kGridWarps - 1) / kGridWarps : 0;
         if (lane < mine) {
-            float *e = ent + (warp + kGridWarps * lane) * kMmaStride;
+            float *e = ent + (warp + kGridWarps * lane) * kRegStride;
             int du = r.r0 - u_org, dv = r.s0 - v_org;
             if (du < 0) du += Np;
             if (dv < 0) dv += Np;
             e[kEntVal] = r.vre;
             e[kEntVal + 1] = r.vim;
-            e[kEntMask] = __uint_as_float(axis_mask(du, Np, W) | axis_mask(dv, Np, W) << 16);
+            masks[buf][warp + kGridWarps * lane] = axis_mask(du, Np, W) | axis_mask(dv, Np, W) << 16;
             e[kEntNu] = r.nux;
             e[kEntNu + 1] = r.nuy;
             e[kEntNu + 2] = r.nuz;
@@ -915,8 +890,8 @@ grid3d_mma_kernel(Launch L, const float *__restrict__ coef, int deg, const VisRe
         }
         for (int i = 0; i < mine; i += 2) {            // zero the weights: 16 lanes an entry
             const int j = i + (lane >> 4);
-            if (j < mine)
-                *reinterpret_cast<float4 *>(ent + (warp + kGridWarps * j) * kMmaStride + 4 * (lane & 15)) =
+            if (j < mine && (lane & 15) < 12)
+                *reinterpret_cast<float4 *>(ent + (warp + kGridWarps * j) * kRegStride + 4 * (lane & 15)) =
                     make_float4(0.f, 0.f, 0.f, 0.f);
         }
         __syncwarp();
@@ -933,8 +908,8 @@ grid3d_mma_kernel(Launch L, const float *__restrict__ coef, int deg, const VisRe
             }
             cf[16] = c4[4].x;
             for (int i = 0; i < mine; i += 2) {        // Horner from nu^16 down, two entries at a time
-                float *e0 = ent + (warp + kGridWarps * i) * kMmaStride;
-                float *e1 = i + 1 < mine ? e0 + kGridWarps * kMmaStride : e0;
+                float *e0 = ent + (warp + kGridWarps * i) * kRegStride;
+                float *e1 = i + 1 < mine ? e0 + kGridWarps * kRegStride : e0;
                 const float2 nu = make_float2(e0[kEntNu + axis], e1[kEntNu + axis]);
                 float2 w = dup2(cf[16]);
 #pragma unroll
@@ -945,12 +920,9 @@ grid3d_mma_kernel(Launch L, const float *__restrict__ coef, int deg, const VisRe
 #pragma unroll
                 for (int h = 0; h < 2; ++h) {          // the same steps for every axis: no divergence
                     float *e = h ? e1 : e0;
-                    const float wt = h ? w.y : w.x, hi = tf32_near(wt);
                     int p = (int)((__float_as_uint(e[kEntOff]) >> off_shift) & off_mask) + tap;
                     if (p >= axis_len) p -= axis_len;
-                    float *at = e + axis_base + (p << axis_log);
-                    if (p < 16) *at = axis == 2 ? hi : wt;
-                    if (axis == 2) at[1] = tf32_near(wt - hi);
+                    if (p < 16) e[axis_base + p] = h ? w.y : w.x;
                 }
             }
         }
@@ -966,71 +938,38 @@ grid3d_mma_kernel(Launch L, const float *__restrict__ coef, int deg, const VisRe
             // 2. the window moves to bin k: planes it has left behind are final
             if (k != cur) {
                 if (cur >= 0) {
-                    flush(cur);
-                    if (k > cur + 1) flush(cur + 1);
+                    flush(cur, true);
+                    if (k > cur + 1) flush_next(cur + 1);
                 }
                 cur = k;
             }
-            // 3. the entries that touch this warp's cells, in groups of eight
-            int cnt = 0;
+            // 3. the entries that touch this warp's cells, one after the other
             for (int b = (int)(b0 - chunk0); b < (int)(b1 - chunk0); b += 32) {
                 bool hit = false;
                 if (b + lane < (int)(b1 - chunk0)) {
-                    const unsigned m = __float_as_uint(ent[(b + lane) * kMmaStride + kEntMask]) & my_cells;
+                    const unsigned m = masks[buf][b + lane] & my_cells;
                     hit = (m & 0xffffu) && (m >> 16);
                 }
-                const unsigned bal = __ballot_sync(0xffffffffu, hit);
-                if (hit) picks[warp][cnt + __popc(bal & ((1u << lane) - 1u))] = (uint8_t)(b + lane);
-                cnt += __popc(bal);
-            }
-            b0 = b1;
-            if (cnt == 0) continue;
-            if (lane < 8) picks[warp][cnt + lane] = (uint8_t)kMmaEntries;
-            __syncwarp();
-            for (int q = 0; q < cnt; q += 8) {
-                const float *e0 = ent + (int)picks[warp][q + t4] * kMmaStride;
-                const float *e1 = ent + (int)picks[warp][q + t4 + 4] * kMmaStride;
-                float ah[4], al[4];
-                {
-                    const float2 w0 = *reinterpret_cast<const float2 *>(e0 + kEntT + 2 * g);
-                    const float2 w1 = *reinterpret_cast<const float2 *>(e0 + kEntT + 2 * (g + 8));
-                    const float2 w2 = *reinterpret_cast<const float2 *>(e1 + kEntT + 2 * g);
-                    const float2 w3 = *reinterpret_cast<const float2 *>(e1 + kEntT + 2 * (g + 8));
-                    ah[0] = w0.x, al[0] = w0.y, ah[1] = w1.x, al[1] = w1.y;
-                    ah[2] = w2.x, al[2] = w2.y, ah[3] = w3.x, al[3] = w3.y;
-                }
-                // packed over the two entries: a fragment of B is one register pair
-                const float2 u = make_float2(e0[kEntU + col0 + g], e1[kEntU + col0 + g]);
-                const float2 x_re = mul2(make_float2(e0[kEntVal], e1[kEntVal]), u);
-                const float2 x_im = mul2(make_float2(e0[kEntVal + 1], e1[kEntVal + 1]), u);
+                for (unsigned hits = __ballot_sync(0xffffffffu, hit); hits; hits &= hits - 1u) {
+                    const float *e = ent + (b + __ffs(hits) - 1) * kRegStride;
+                    const float2 V = *reinterpret_cast<const float2 *>(e + kEntVal);
+                    const float2 p = mul2(V, dup2(e[kEntU + col] * e[kEntV + row]));
 #pragma unroll
-                for (int j = 0; j < 4; ++j) {
-                    const float2 y = make_float2(e0[kEntV + row0 + j], e1[kEntV + row0 + j]);
-#pragma unroll
-                    for (int comp = 0; comp < 2; ++comp) {
-                        const float2 p = mul2(comp ? x_im : x_re, y);
-                        const float2 h = make_float2(tf32_near(p.x), tf32_near(p.y));
-                        const float2 l = csub(p, h);
-                        float d[4];
-                        mma_tf32_from_zero(d, al, h.x, h.y);
-                        mma_tf32(d, ah, tf32_cut(l.x), tf32_cut(l.y));
-                        mma_tf32(d, ah, h.x, h.y);
-#pragma unroll
-                        for (int i = 0; i < 4; i += 2) {
-                            float *f = c[j][comp] + i;
-                            const float2 sum = cadd(make_float2(f[0], f[1]), make_float2(d[i], d[i + 1]));
-                            f[0] = sum.x;
-                            f[1] = sum.y;
-                        }
+                    for (int q = 0; q < 4; ++q) {
+                        const float4 z = *reinterpret_cast<const float4 *>(e + kEntT + 4 * q);
+                        c[4 * q] = fma2(dup2(z.x), p, c[4 * q]);
+                        c[4 * q + 1] = fma2(dup2(z.y), p, c[4 * q + 1]);
+                        c[4 * q + 2] = fma2(dup2(z.z), p, c[4 * q + 2]);
+                        c[4 * q + 3] = fma2(dup2(z.w), p, c[4 * q + 3]);
                     }
                 }
             }
-            __syncwarp();                              // the picks are read before the next bin's
+            b0 = b1;
         }
         buf ^= 1;
     }
-    flush(cur);
-    flush(cur + 1);
+    flush(cur, true);
+    flush_next(cur + 1);
 }
 
 // Section 5.4: a visibility with w < 0 was degridded at -(u, v, w); the real
@@ -1247,12 +1186,12 @@ cudaError_t launch_grid_chunk(const ws_plan_s *p, int chunk, int planes, cudaStr
                                                    p->d_tile_occ, chunk_tt0, chunk_ntt, p->wbound, p->d_stack);
         return cudaGetLastError();
     };
-    // 16-row tiles of widths up to 9 go to the tensor cores; wider footprints reach
-    // past the 16 planes of a fragment, and taller tiles and the deterministic mode
+    // 16-row tiles of widths up to 9 keep their sums in registers; wider footprints reach
+    // past the 16 planes that a lane holds, and taller tiles and the deterministic mode
     // keep their sums in shared memory
-    auto mma = [&](auto kernel) -> cudaError_t {
+    auto cells = [&](auto kernel) -> cudaError_t {
         kernel<<<nblocks, kGridThreads, 0, s>>>(p->L, p->d_wcoef, p->wdeg, p->d_rec, p->d_offsets, p->d_list,
-                                                chunk_tt0, chunk_ntt, p->d_stack);
+                                                p->d_tile_occ, chunk_tt0, chunk_ntt, p->d_stack);
         return cudaGetLastError();
     };
     auto width = [&](auto wc) -> cudaError_t {
@@ -1264,8 +1203,8 @@ cudaError_t launch_grid_chunk(const ws_plan_s *p, int chunk, int planes, cudaStr
         }
         if (R == 64) return go(grid3d_kernel<w, 64, false>, GridSmem<w, 64, false>::bytes);
         if (R == 32) return go(grid3d_kernel<w, 32, false>, GridSmem<w, 32, false>::bytes);
-        if constexpr (w <= kMmaMaxW)
-            return mma(grid3d_mma_kernel<w>);
+        if constexpr (w <= kRegMaxW)
+            return cells(grid3d_cells_kernel<w>);
         else
             return go(grid3d_kernel<w, 16, false>, GridSmem<w, 16, false>::bytes);
     };

@@ -41,3 +41,42 @@ def test_large_rows_screen_every_plane_exactly(dev, monkeypatch, N, x0):
     whole = first % 24 <= 24 - W
     assert 0.5 < whole.mean() < 1.0
     assert np.array_equal(out[0][whole], out[1][whole])
+
+
+def _grid(p, uvw, vis):
+    return p.grid(uvw, vis.to(p.cdtype)).to(torch.complex128).cpu().numpy()
+
+
+@pytest.mark.parametrize("N,W,M", [(64, 7, 1000), (256, 7, 10), (256, 7, 1000), (256, 8, 10_000), (256, 4, 1000), (128, 9, 3000)])
+def test_gridding_products_are_fp32(dev, N, W, M):
+    """Against an FP64 plan, the default mode is no further off than the deterministic one, whose contributions
+    are FP32 products (three roundings each) summed exactly: here one rounding fewer a product and a sum or two
+    per cell, so 5 % is left for the sums."""
+    from paper_2101_11172_gb300 import WS_FLAG_DETERMINISTIC, WS_FLAG_FP64
+    from paper_2101_11172_gb300.wstack import Plan
+    sq = np.zeros(2)
+    for seed in range(4):
+        rng = synth.rng_for(0, 9200 + 10 * W + seed)
+        uvw = torch.from_numpy(synth.disc_uvw(M, 0.45 * N / 0.2, 1.0, rng)).to(dev)
+        vis = torch.from_numpy(synth.complex_normal(M, rng).astype(np.complex64).astype(np.complex128)).to(dev)
+        d = []
+        for flags in (WS_FLAG_FP64, 0, WS_FLAG_DETERMINISTIC):
+            with Plan(N, 0.25, W, 0.2, -1.0, 1.0, flags=flags, device=dev) as p:
+                d.append(_grid(p, uvw, vis))
+        sq += rel(d[1], d[0]) ** 2, rel(d[2], d[0]) ** 2
+    print(N, W, M, np.sqrt(sq / 4))
+    assert sq[0] <= 1.05 ** 2 * sq[1]
+
+
+@pytest.mark.parametrize("power", [-110, 90])
+def test_gridding_keeps_its_digits_at_every_scale(dev, power):
+    """Visibilities scaled by a power of two give the image scaled by it, up to the order of the sums
+    (about 1e-7): only contributions below 2^-126, 2^-16 of these visibilities, lose digits."""
+    from paper_2101_11172_gb300.wstack import Plan
+    N, W, M = 256, 7, 5000
+    rng = synth.rng_for(0, 9300)
+    uvw = torch.from_numpy(synth.disc_uvw(M, 0.45 * N / 0.2, 1.0, rng)).to(dev)
+    vis = torch.from_numpy(synth.complex_normal(M, rng).astype(np.complex64).astype(np.complex128)).to(dev)
+    with Plan(N, 0.25, W, 0.2, -1.0, 1.0, device=dev) as p:
+        one, scaled = _grid(p, uvw, vis), _grid(p, uvw, vis * 2.0 ** power)
+    assert rel(scaled * 2.0 ** -power, one) < 1.4e-7
