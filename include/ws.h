@@ -231,14 +231,14 @@ ws_status ws_plan_tune(ws_plan_t plan, const double *uvw, const void *vis, const
  * host application owns every allocation, code that must not trigger the
  * synchronisation an allocation can imply).  It computes the same result as
  * ws_degrid, with the same arguments and status codes, but takes all of its
- * per-call scratch (visibility records, bin lists, the corrected image, the
- * w-plane chunk) from one 64 MiB array in device memory that the library
+ * per-call scratch (visibility records, bin lists, the w-plane chunk) from one 64 MiB array in device memory that the library
  * holds on every device that loads it, until the process exits.  It calls no
  * cudaMalloc or cudaFree and allocates nothing else on the device.
  *   - The plan (made earlier by ws_plan, which does allocate) supplies the
  *     tables; the caller supplies inputs and outputs as for ws_degrid.
- *   - Problems whose records, image and at least 8 w-planes of N' x N' do not
- *     fit in the 64 MiB are rejected with WS_ERR_ARG and a message.
+ *   - Problems whose records, room for an image and at least 8 w-planes of
+ *     N' x N' do not fit in the 64 MiB are rejected with WS_ERR_ARG and a
+ *     message.
  *   - The first call on a device looks up the array's device address (a
  *     runtime symbol query that may load the module); make that first call
  *     before capturing the stream into a graph.

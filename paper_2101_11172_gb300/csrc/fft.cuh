@@ -85,7 +85,8 @@ constexpr float kR2 = 0.70710678118654752f;   // sqrt(1/2)
 __device__ __forceinline__ float2 mul_w16(float2 a, int m, bool inv) {
     const float c = m == 1 ? kC1 : m == 2 ? kR2 : m == 3 ? kS1 : m == 6 ? -kR2 : -kC1;
     const float s = m == 1 ? kS1 : m == 2 ? kR2 : m == 3 ? kC1 : m == 6 ? kR2 : -kS1;
-    return inv ? cmul_rot(a, make_float2(c, s), make_float2(-s, c)) : cmul_rot(a, make_float2(c, -s), make_float2(s, c));
+    return inv ? cmul_rot(a, make_float2(c, s), make_float2(-s, c))
+               : cmul_rot(a, make_float2(c, -s), make_float2(s, c));
 }
 
 template <int R>
@@ -316,7 +317,8 @@ __device__ __forceinline__ void twiddle_powers(float2 *v, float2 w1, float2 w4) 
                 if (a == 4) base = Tw(w8).times(w8);
                 v[4 * a] = Tw(base).times(v[4 * a]);
                 if (4 * a + 1 < R) v[4 * a + 1] = Tw(t1.times(base)).times(v[4 * a + 1]);
-                if (4 * a + 2 < R) v[4 * a + 2] = Tw(R == 7 ? t3.times(t3.w) : t2.times(base)).times(v[4 * a + 2]);
+                if (4 * a + 2 < R)
+                    v[4 * a + 2] = Tw(R == 7 ? t3.times(t3.w) : t2.times(base)).times(v[4 * a + 2]);
                 if (4 * a + 3 < R) v[4 * a + 3] = Tw(t3.times(base)).times(v[4 * a + 3]);
             }
         }
@@ -348,7 +350,7 @@ __device__ __forceinline__ void dit_stage(float2 *buf, const FftPlan &P, int s, 
     tw += P.bases[s];
     float2 w1, w4;
     int base = 0, k = 0;
-    auto fetch = [&](int q) {                // butterfly q's first position and twiddles (q past the end: the last one's)
+    auto fetch = [&](int q) {                // butterfly q's first position and twiddles (past the end: the last one's)
         const int bq = min(q, total - 1) / COUNT;
         const int blk = LAST ? 0 : div_small(bq, P.L_mul[s]);
         k = bq - blk * L;
@@ -481,8 +483,8 @@ __device__ __forceinline__ int first_slot(const FftPlan &P, const float2 *__rest
 // straight from load(t, e), and writes them to the digit-reversed positions
 // g*R + m that the later in-place stages expect.
 template <int R, int COUNT, class Load>
-__device__ __forceinline__ void dit_first(float2 *buf, const FftPlan &P, const float2 *__restrict__ tw, bool inv, int tid,
-                                          int nthr, Load &load) {
+__device__ __forceinline__ void dit_first(float2 *buf, const FftPlan &P, const float2 *__restrict__ tw, bool inv,
+                                          int tid, int nthr, Load &load) {
     const int nb = P.nb[0], total = COUNT * nb;
     for (int q = tid; q < total; q += nthr) {
         const int t = q % COUNT, j = q / COUNT;
@@ -500,8 +502,8 @@ __device__ __forceinline__ void dit_first(float2 *buf, const FftPlan &P, const f
 // at 0..n-1 (n / R <= nthr: one butterfly per thread); input m of a thread is
 // zero where bit m of live is clear, whatever the buffer holds.
 template <int R>
-__device__ __forceinline__ void dit_first_inplace(float2 *buf, const FftPlan &P, const float2 *__restrict__ tw, bool inv, int tid,
-                                                  uint32_t live) {
+__device__ __forceinline__ void dit_first_inplace(float2 *buf, const FftPlan &P, const float2 *__restrict__ tw,
+                                                  bool inv, int tid, uint32_t live) {
     // threads past nb read the last butterfly's inputs and drop them: a value that
     // exists only under a condition, kept across the barrier, made the compiler spill
     const int nb = P.nb[0], at = min(tid, nb - 1), slot = first_slot(P, tw, at);
@@ -547,7 +549,6 @@ template <class F>
 __device__ __forceinline__ void with_forward_pair(int a, int b, F f) {
     switch (16 * a + b) {
         case 16 * 4 + 7: f(Radix<4>{}, Radix<7>{}); break;
-        case 16 * 4 + 5: f(Radix<4>{}, Radix<5>{}); break;
         case 16 * 4 + 3: f(Radix<4>{}, Radix<3>{}); break;
         case 16 * 7 + 3: f(Radix<7>{}, Radix<3>{}); break;
         case 16 * 5 + 5: f(Radix<5>{}, Radix<5>{}); break;
@@ -932,7 +933,8 @@ __device__ __forceinline__ void mul_w64_all(float2 *v, bool inv) {
 // 8-point DFT of (a0, a1, 0, 0, 0, 0, a6, a7) (v[2..5] need not be set)
 __device__ __forceinline__ void dft8_zero_middle(float2 *v, bool inv) {
     // even inputs (v0, 0, 0, v6), odd inputs (v1, 0, 0, v7)
-    const float2 e0 = cadd(v[0], v[6]), e2 = csub(v[0], v[6]), e1 = sub_rot(v[0], v[6], inv), e3 = add_rot(v[0], v[6], inv);
+    const float2 e0 = cadd(v[0], v[6]), e2 = csub(v[0], v[6]);
+    const float2 e1 = sub_rot(v[0], v[6], inv), e3 = add_rot(v[0], v[6], inv);
     const float2 o0 = cadd(v[1], v[7]), o2 = csub(v[1], v[7]);
     const float2 o1 = fftdev::mul_w16(sub_rot(v[1], v[7], inv), 2, inv);
     const float2 o3 = fftdev::mul_w16(add_rot(v[1], v[7], inv), 6, inv);

@@ -138,7 +138,8 @@ spread64_kernel(Launch L, const double *__restrict__ cheb, int deg, const VisRec
         for (int q = lane; q < W * W; q += 32) {
             const int b = q / W, a = q - b * W;
             const double wab = w[a] * w[W + b], xr = vr * wab, xi = vi * wab;
-            double2 *cell = stack + (size_t)((r.s0 + b) % Np) * Np + (r.r0 + a) % Np + (size_t)(r.t0 + c_lo - p0) * plane;
+            double2 *cell =
+                stack + (size_t)((r.s0 + b) % Np) * Np + (r.r0 + a) % Np + (size_t)(r.t0 + c_lo - p0) * plane;
             for (int c = c_lo; c <= c_hi; ++c, cell += plane) {
                 const double wz = w[2 * W + c];
                 atomicAdd(&cell->x, xr * wz);
@@ -385,7 +386,8 @@ cudaError_t fp64_setup() {
     const int smem = (int)(kFftPoints64 * sizeof(double2));
     cudaError_t e = cudaFuncSetAttribute(fwd_rows64_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     if (e == cudaSuccess) e = cudaFuncSetAttribute(cols64_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(inv_rows64_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    if (e == cudaSuccess)
+        e = cudaFuncSetAttribute(inv_rows64_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     return e;
 }
 

@@ -10,6 +10,7 @@
 #include <cmath>
 #include <cstdlib>
 #include <cstring>
+#include <initializer_list>
 #include <new>
 #include <string>
 
@@ -273,9 +274,10 @@ size_t row_smem(int n, bool inverse) { return inverse ? 28 * (size_t)n : 24 * (s
 // through shared memory.
 int inverse_radices(int n, int *best) {
     // what the kernels have as a first, middle and last radix
-    auto first = [](int r) { return r == 28 || r == 24 || r == 20 || r == 16 || r == 14 || r == 12 || r == 10 || r == 8; };
-    auto middle = [](int r) { return r == 21 || r == 20 || r == 16 || r == 14 || r == 12 || r == 10 || r == 8 || r == 6; };
-    auto last = [](int r) { return r == 16 || r == 14 || r == 12 || r == 10 || r == 8 || r == 7 || r == 6 || r == 4; };
+    auto among = [](int r, std::initializer_list<int> set) { return std::find(set.begin(), set.end(), r) != set.end(); };
+    auto first = [&](int r) { return among(r, {28, 24, 20, 16, 14, 12, 10, 8}); };
+    auto middle = [&](int r) { return among(r, {21, 20, 16, 14, 12, 10, 8, 6}); };
+    auto last = [&](int r) { return among(r, {16, 14, 12, 10, 8, 7, 6, 4}); };
     const int radices[] = {28, 24, 21, 20, 16, 14, 12, 10, 8, 7, 6, 4};
     int cur[kMaxFftStages] = {}, nbest = 0;
     double best_time = 0.0;
@@ -307,7 +309,7 @@ int inverse_radices(int n, int *best) {
 // (3 3), 3072 = 16 8 (8 3), 1344 = 8 8 (7 3).  The arithmetic is the stages' own.
 void fuse_stages(const int *radix, int ns, int *fuse) {
     auto pair = [](int a, int b) {
-        return (a == 4 && (b == 7 || b == 5 || b == 3)) || (b == 5 && a == 5) ||
+        return (a == 4 && (b == 7 || b == 3)) || (b == 5 && a == 5) ||
                (b == 3 && (a == 3 || a == 5 || a == 7 || a == 8));
     };
     int passes[kMaxFftStages + 2] = {};                  // fewest passes from stage s on
@@ -445,7 +447,8 @@ void fft_tables(FftPlan *F, std::vector<float2> *tw) {
     F->slots = (int)tw->size() * 2;
     tw->resize(tw->size() + (size_t)(F->nb[0] + 1) / 2);
     for (int j = 0; j < F->nb[0]; ++j) {
-        const int e = first_position(*F, j), slot = e + (F->chunk_mul ? (int)((unsigned long long)e * F->chunk_mul >> 32) : 0);
+        const int e = first_position(*F, j);
+        const int slot = e + (F->chunk_mul ? (int)((unsigned long long)e * F->chunk_mul >> 32) : 0);
         std::memcpy(reinterpret_cast<int *>(tw->data()) + F->slots + j, &slot, sizeof(int));
     }
 }

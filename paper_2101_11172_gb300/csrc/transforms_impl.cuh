@@ -134,11 +134,12 @@ constexpr int kScreenSteps = 8;
 template <int NP, bool CROP, bool STEP>
 __global__ void __launch_bounds__(row_threads_max<NP>(), row_ctas<NP>())
 fwd_rows_kernel(Launch L, FftPlan F, const float2 *__restrict__ tw, const float2 *__restrict__ img,
-                const float *__restrict__ corr, const float2 *__restrict__ zsplit, const uint8_t *__restrict__ col_occ, int plane0, int planes,
-                int keep_rows, float2 *__restrict__ stack) {
+                const float *__restrict__ corr, const float2 *__restrict__ zsplit,
+                const uint8_t *__restrict__ col_occ, int plane0, int planes, int keep_rows,
+                float2 *__restrict__ stack) {
     extern __shared__ __align__(16) float2 sbuf[];
     const int Np = L.Np, N = L.N, half = N / 2;
-    float2 *grow = sbuf + F.stride;                              // N: the screened row (F.stride is even: 16-byte aligned)
+    float2 *grow = sbuf + F.stride;                              // N: the screened row (16-byte aligned)
     float2 *erow = grow + N;                                     // N: exp(-2 pi i z)
     float2 *irow = STEP ? erow + N : grow;                       // N if keep_rows
     float2 *zrow = irow + N;                                     // N if keep_rows
@@ -710,7 +711,8 @@ struct Transforms {
     }
     // column CTAs resident on the GPU, a multiple of the two of a block
     static int columns_ahead(const FftPlan &F, int sms) {
-        const int by_smem = (int)(228 * 1024 / (smem2(F) + 1024)), by_regs = col_ctas<NP>() * col_threads_max<NP>() / col_threads(F);
+        const int by_smem = (int)(228 * 1024 / (smem2(F) + 1024));
+        const int by_regs = col_ctas<NP>() * col_threads_max<NP>() / col_threads(F);
         return std::max(1, std::min(by_smem, by_regs)) * sms / 2 * 2;
     }
     static int row_threads(const FftPlan &F) { return NP ? row_threads_max<NP>() : F.row_threads; }

@@ -142,9 +142,9 @@ struct ws_plan_s {
     uint8_t *d_tile_occ = nullptr; // ntiles: 1 if any visibility footprint touches the tile
     uint8_t *d_col_occ = nullptr;  // ntt x ntu: 1 if any tile of that (t-tile, u-tile) strip is touched
     int row_shares = 1;            // shares of the planes per image row in inv_rows (transforms.cu)
-    int share_planes = 0;          // planes of each share, cut at fixed planes of the plan; 0: equal parts of each chunk
+    int share_planes = 0;          // planes of a share, cut at fixed planes of the plan; 0: equal parts of a chunk
     float4 *d_acc = nullptr;       // row_shares x N x N: (sum re, sum im, comp re, comp im)
-    unsigned *d_rows_done = nullptr;   // N: shares of the row that are done and a mark if it is incomplete, zero between calls
+    unsigned *d_rows_done = nullptr;   // N, zero between calls: shares of the row done, and a mark if it is incomplete
     unsigned long long *d_drop = nullptr;   // kCounters: [0] non-finite uv, [1] w out of range, [2] timed-out waits
     unsigned long long *h_drop = nullptr;   // pinned mirror
     int wait_polls = ws::kWaitPolls;        // limit of inv_rows' first wait per plane (WS_WAIT_POLLS)

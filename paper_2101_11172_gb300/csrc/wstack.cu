@@ -4,8 +4,8 @@
 //                           (transforms.cu: inverse DFTs, crop, x exp(2 pi i t z), sum over t,
 //                           x h_x h_y h_z)
 // Degridding (Algorithm 6): prep and count -> sort -> per plane chunk: fwd_rows -> fwd_cols
-//                           (transforms.cu: x h_x h_y h_z, x exp(-2 pi i t z), zero pad, forward DFTs) -> degrid3d (3-D correlation with C_x C_y C_z,
-//                           x exp(-2 pi i w (n0-1)))
+//                           (transforms.cu: x h_x h_y h_z, x exp(-2 pi i t z), zero pad, forward DFTs)
+//                           -> degrid3d (3-D correlation with C_x C_y C_z, x exp(-2 pi i w (n0-1)))
 //
 // Grid indices: row s (v direction) and column r (u direction) of a plane are
 // stored modulo N'.  Because exp(2 pi i r j / N') is N'-periodic in r, a tap
@@ -123,7 +123,9 @@ __device__ __forceinline__ void tap_floor(double x, double half_wm1, int *floor_
 }
 
 // |x| below about 10^9 (an exponent below 30), by integer comparison: false for NaN and infinities too.
-__device__ __forceinline__ bool small_enough(double x) { return (__double2hiint(x) & 0x7fffffff) < ((1023 + 30) << 20); }
+__device__ __forceinline__ bool small_enough(double x) {
+    return (__double2hiint(x) & 0x7fffffff) < ((1023 + 30) << 20);
+}
 
 // A grid index i (|i| < 2^31) modulo n: with the division only for the rare points more than a grid away.
 __device__ __forceinline__ int wrap_small(int i, int n) {
@@ -431,8 +433,9 @@ __device__ __forceinline__ void red_shared_at(unsigned addr, float v) {
 
 // The 64-bit integer nearest v (ties to even), |v| < 2^62.  The conversion to 64 bits
 // goes at the rate of FP64 arithmetic, and bounded the deterministic mode (120,960
-// visibilities, W = 7, N = 512: 350 us with it, 274 so); this takes the two words of |v| by 32-bit conversions, both exact
-// but for the low word's rounding (below 2^24 |v| is all in the low word; from there on it is an integer).
+// visibilities, W = 7, N = 512: 350 us with it, 274 so); this takes the two words of |v|
+// by 32-bit conversions, both exact but for the low word's rounding (below 2^24 |v| is
+// all in the low word; from there on it is an integer).
 __device__ __forceinline__ long long nearest_int64(float v) {
     const float a = fabsf(v), x = a * 0x1p-32f;
     const unsigned hi = __float2uint_rz(x), lo = __float2uint_rn(fmaf(truncf(x), -0x1p32f, a));

@@ -47,7 +47,8 @@ def _grid(p, uvw, vis):
     return p.grid(uvw, vis.to(p.cdtype)).to(torch.complex128).cpu().numpy()
 
 
-@pytest.mark.parametrize("N,W,M", [(64, 7, 1000), (256, 7, 10), (256, 7, 1000), (256, 8, 10_000), (256, 4, 1000), (128, 9, 3000)])
+@pytest.mark.parametrize("N,W,M", [(64, 7, 1000), (256, 7, 10), (256, 7, 1000), (256, 8, 10_000), (256, 4, 1000),
+                                   (128, 9, 3000)])
 def test_gridding_products_are_fp32(dev, N, W, M):
     """Against an FP64 plan, the default mode is no further off than the deterministic one, whose contributions
     are FP32 products (three roundings each) summed exactly: here one rounding fewer a product and a sum or two
