@@ -43,19 +43,34 @@ __device__ __forceinline__ float2 twiddle(const float2 *__restrict__ tw, int m, 
     return inv ? make_float2(w.x, -w.y) : w;
 }
 
-// The bases of butterfly offset k of a runtime plan's stage of radix R, from the
-// stage's own table (fft_tables): w^k and, from R = 8 on, w^4k beside it.
+// Powers of a butterfly's twiddle w: those its table holds (the others are not set).
+struct Bases {
+    float2 w1, w2, w4, w8;
+};
+
+// The bases of butterfly offset k of a runtime plan's stage of radix R, from row k of the
+// stage's own table (fft_tables, base_row).
 // Read from the N'-entry table, a warp's w^4k fell into as many sectors as
 // lanes, and a stage's table is small enough for the L1 that the buffers leave.
-template <int R>
-__device__ __forceinline__ void twiddle_bases(const float2 *__restrict__ bases, int k, bool inv, float2 &w1, float2 &w4) {
-    if (R >= 8) {
-        const float4 w = __ldg(reinterpret_cast<const float4 *>(bases) + k);
-        w1 = make_float2(w.x, inv ? -w.y : w.y);
-        w4 = make_float2(w.z, inv ? -w.w : w.w);
+template <int R, bool INV>
+__device__ __forceinline__ Bases twiddle_bases(const float2 *__restrict__ bases, int k) {
+    constexpr int ROW = base_row(R, INV);
+    Bases b{};
+    if constexpr (ROW == 1) {
+        b.w1 = twiddle(bases, k, INV);
+        return b;
     } else {
-        w1 = twiddle(bases, k, inv);
-        w4 = make_float2(1.f, 0.f);
+        const float4 w = __ldg(reinterpret_cast<const float4 *>(bases + ROW * k));
+        b.w1 = make_float2(w.x, INV ? -w.y : w.y);
+        (INV ? b.w2 : b.w4) = make_float2(w.z, INV ? -w.w : w.w);
+        if constexpr (ROW == 4 && R > 8) {
+            const float4 h = __ldg(reinterpret_cast<const float4 *>(bases + ROW * k) + 1);
+            b.w4 = make_float2(h.x, -h.y);
+            b.w8 = make_float2(h.z, -h.w);
+        } else if constexpr (ROW == 4) {
+            b.w4 = twiddle(bases, ROW * k + 2, INV);
+        }
+        return b;
     }
 }
 
@@ -292,38 +307,48 @@ struct Tw {
     __device__ __forceinline__ float2 times(float2 a) const { return cmul_rot(a, w, rot); }
 };
 
-// v[m] *= w^m for m = 1..R-1, w = exp(-+ 2 pi i e / n), given w and w^4.  The
-// table holds w^m to half an ulp, but a warp's loads of w^m for m > 1 scatter
-// over many sectors; so only w and, from R = 8 on, w^4 are read and the
-// other powers are products of them (at most five roundings: RMS error about 7e-8 against 2e-8
-// for the table, far below the FP32 transform's own rounding).
-template <int R>
-__device__ __forceinline__ void twiddle_powers(float2 *v, float2 w1, float2 w4) {
-    static_assert(R >= 3 && R <= 28, "powers up to w^27");
-    const Tw t1(w1);
+// v[m] *= w^m for m = 1..R-1, w = exp(-+ 2 pi i e / n), given the powers that
+// base_row<R, INV> names.  The table holds w^m to half an ulp, but a warp's loads of
+// w^m for m > 1 scatter over many sectors; so only those powers are read and the
+// others are products of them (forward, at most five roundings: RMS error about 7e-8
+// against 2e-8 for the table).
+template <int R, bool INV>
+__device__ __forceinline__ void twiddle_powers(float2 *v, const Bases &b) {
+    static_assert(R >= 3 && R <= 21, "powers up to w^20");
+    constexpr bool W4 = base_row(R, INV) == (INV ? 4 : 2), W8 = base_row(R, INV) == 4;
+    const Tw t1(b.w1);
     v[1] = t1.times(v[1]);
-    const Tw t2(t1.times(w1));
+    const Tw t2(INV ? b.w2 : t1.times(b.w1));
     v[2] = t2.times(v[2]);
     if constexpr (R >= 4) {
         const Tw t3(t1.times(t2.w));
         v[3] = t3.times(v[3]);
         if constexpr (R > 4) {
-            const Tw t4(R <= 7 ? t2.times(t2.w) : w4);
+            const Tw t4(W4 ? b.w4 : t2.times(t2.w));
             float2 base = t4.w, w8 = t4.w;
 #pragma unroll
             for (int a = 1; 4 * a < R; ++a) {
-                if (a == 2) base = w8 = t4.times(t4.w);
-                if (a == 3 || a >= 5) base = t4.times(base);
+                if (a == 2) base = w8 = W8 ? b.w8 : t4.times(t4.w);
+                if (a == 3 || a == 5) base = t4.times(base);
                 if (a == 4) base = Tw(w8).times(w8);
                 v[4 * a] = Tw(base).times(v[4 * a]);
                 if (4 * a + 1 < R) v[4 * a + 1] = Tw(t1.times(base)).times(v[4 * a + 1]);
                 if (4 * a + 2 < R)
-                    v[4 * a + 2] = Tw(R == 7 ? t3.times(t3.w) : t2.times(base)).times(v[4 * a + 2]);
+                    v[4 * a + 2] = Tw(R == 7 && !W4 ? t3.times(t3.w) : t2.times(base)).times(v[4 * a + 2]);
                 if (4 * a + 3 < R) v[4 * a + 3] = Tw(t3.times(base)).times(v[4 * a + 3]);
             }
         }
     }
 }
+// The same with w and, from R = 8 on, w^4 given, as the compile-time plans keep them in either direction.
+template <int R>
+__device__ __forceinline__ void twiddle_powers(float2 *v, float2 w1, float2 w4) {
+    Bases b{};
+    b.w1 = w1;
+    b.w4 = w4;
+    twiddle_powers<R, false>(v, b);
+}
+
 // x / d for 0 <= x < 2^16, 1 <= d < 2^13, with mul = div_mul(d) (fft_plan.hpp)
 __device__ __forceinline__ int div_small(int x, unsigned mul) {
     return mul ? (int)__umulhi((unsigned)x, mul) : x;
@@ -343,32 +368,32 @@ __device__ __forceinline__ int div_small(int x, unsigned mul) {
 // twiddles have been asked for, and each round asks for the next one's: the table
 // mostly comes from L2 (the buffers leave little L1), and a stage that waited for
 // it after the barrier spent a third of its time there.
-template <int R, int COUNT, bool LAST, class Store>
-__device__ __forceinline__ void dit_stage(float2 *buf, const FftPlan &P, int s, const float2 *__restrict__ tw,
-                                          bool inv, int tid, int nthr, Store &store) {
+template <int R, int COUNT, bool LAST, bool INV, class Store>
+__device__ __forceinline__ void dit_stage(float2 *buf, const FftPlan &P, int s, const float2 *__restrict__ tw, int tid,
+                                          int nthr, Store &store) {
     const int L = P.L[s], total = COUNT * P.nb[s], step = P.step[s];
     tw += P.bases[s];
-    float2 w1, w4;
+    Bases w{};
     int base = 0, k = 0;
     auto fetch = [&](int q) {                // butterfly q's first position and twiddles (past the end: the last one's)
         const int bq = min(q, total - 1) / COUNT;
         const int blk = LAST ? 0 : div_small(bq, P.L_mul[s]);
         k = bq - blk * L;
         base = blk * R * L + k;
-        twiddle_bases<R>(tw, k, inv, w1, w4);
+        w = twiddle_bases<R, INV>(tw, k);
     };
     fetch(tid);
     __syncthreads();
     for (int q = tid; q < total; q += nthr) {
         const int t = q % COUNT, b = base, kq = k;
-        const float2 v1 = w1, v4 = w4;
+        const Bases wq = w;
         float2 *x = buf + t * P.stride + b + div_small(b, P.chunk_mul);
         float2 v[R];
 #pragma unroll
         for (int m = 0; m < R; ++m) v[m] = x[m * step];
         fetch(q + nthr);
-        if (kq > 0) twiddle_powers<R>(v, v1, v4);
-        dft<R>(v, inv);
+        if (kq > 0) twiddle_powers<R, INV>(v, wq);
+        dft<R>(v, INV);
         if constexpr (LAST) {
             store(std::false_type{}, t, b, L, v);
         } else {
@@ -386,24 +411,25 @@ __device__ __forceinline__ void dit_stage(float2 *buf, const FftPlan &P, int s, 
 // The arithmetic is that of the two stages; one trip through shared memory and one
 // barrier less.
 template <int A, int B, bool LAST, class Store>
-__device__ __forceinline__ void dit_pair(float2 *buf, const FftPlan &P, int s, const float2 *__restrict__ tw, bool inv,
-                                         int tid, int nthr, Store &store) {
+__device__ __forceinline__ void dit_pair(float2 *buf, const FftPlan &P, int s, const float2 *__restrict__ tw, int tid,
+                                         int nthr, Store &store) {
+    constexpr bool inv = false;
     static_assert(B < 8, "the second radix takes its twiddles from w alone");
     const int L = P.L[s], total = P.nb[s] / B, step_a = P.step[s], step_b = P.step[s + 1];
-    float2 w1, w4;
+    Bases w_a{};
     int base = 0, k = 0;
     auto fetch = [&](int q) {                // as in dit_stage, for the first of the two stages
         const int bq = min(q, total - 1);
         const int blk = LAST ? 0 : div_small(bq, P.L_mul[s]);
         k = bq - blk * L;
         base = blk * A * B * L + k;
-        twiddle_bases<A>(tw + P.bases[s], k, inv, w1, w4);
+        w_a = twiddle_bases<A, inv>(tw + P.bases[s], k);
     };
     fetch(tid);
     __syncthreads();
     for (int q = tid; q < total; q += nthr) {
         const int b = base, kq = k;
-        const float2 v1 = w1, v4 = w4;
+        const Bases wq = w_a;
         float2 *x = buf + b + div_small(b, P.chunk_mul);
         float2 v[A * B], w[A];
 #pragma unroll
@@ -415,7 +441,7 @@ __device__ __forceinline__ void dit_pair(float2 *buf, const FftPlan &P, int s, c
         fetch(q + nthr);
 #pragma unroll
         for (int m2 = 0; m2 < B; ++m2) {
-            if (kq > 0) twiddle_powers<A>(v + A * m2, v1, v4);
+            if (kq > 0) twiddle_powers<A, inv>(v + A * m2, wq);
             dft<A>(v + A * m2, inv);
         }
 #pragma unroll
@@ -443,14 +469,16 @@ __device__ __forceinline__ void dit_pair(float2 *buf, const FftPlan &P, int s, c
 // (the buffer is free from then on): up to ROUNDS butterflies a thread in
 // registers, R ROUNDS <= 32.
 template <int R, class Between, class Store>
-__device__ __forceinline__ void dit_last_held(float2 *buf, const FftPlan &P, const float2 *__restrict__ tw, bool inv,
-                                              int tid, int nthr, Between &between, Store &store) {
+__device__ __forceinline__ void dit_last_held(float2 *buf, const FftPlan &P, const float2 *__restrict__ tw, int tid,
+                                              int nthr, Between &between, Store &store) {
+    constexpr bool inv = true;
     constexpr int ROUNDS = 32 / R;
     const int s = P.nstages - 1, L = P.L[s], nb = P.nb[s], step = P.step[s];
-    float2 v[ROUNDS][R], w1[ROUNDS], w4[ROUNDS];
+    float2 v[ROUNDS][R];
+    Bases w[ROUNDS];
 #pragma unroll
     for (int i = 0; i < ROUNDS; ++i) {
-        twiddle_bases<R>(tw + P.bases[s], min(tid + i * nthr, nb - 1), inv, w1[i], w4[i]);
+        w[i] = twiddle_bases<R, inv>(tw + P.bases[s], min(tid + i * nthr, nb - 1));
     }
     __syncthreads();
 #pragma unroll
@@ -466,7 +494,7 @@ __device__ __forceinline__ void dit_last_held(float2 *buf, const FftPlan &P, con
     for (int i = 0; i < ROUNDS; ++i) {
         const int k = tid + i * nthr;
         if (k >= nb) break;
-        if (k > 0) twiddle_powers<R>(v[i], w1[i], w4[i]);
+        if (k > 0) twiddle_powers<R, inv>(v[i], w[i]);
         dft<R>(v[i], inv);
         store(std::false_type{}, 0, k, L, v[i]);
     }
@@ -611,14 +639,14 @@ __device__ __forceinline__ int fft_middle_stages(float2 *buf, const FftPlan &P, 
     auto fused = [&](int i) { return COUNT == 1 && !INV ? P.fuse[i] : 0; };     // rows only (FftPlan)
     while (s + fused(s) < P.nstages - 1) {
         auto stage = [&](auto r) {
-            fftdev::dit_stage<decltype(r)::value, COUNT, false>(buf, P, s, tw, INV, tid, nthr, none);
+            fftdev::dit_stage<decltype(r)::value, COUNT, false, INV>(buf, P, s, tw, tid, nthr, none);
         };
         if constexpr (INV) {
             fftdev::with_middle_radix(P.radix[s], stage);
         } else if (fused(s)) {
             if constexpr (COUNT == 1)
                 fftdev::with_forward_pair(P.radix[s], P.radix[s + 1], [&](auto ra, auto rb) {
-                    fftdev::dit_pair<decltype(ra)::value, decltype(rb)::value, false>(buf, P, s, tw, INV, tid, nthr, none);
+                    fftdev::dit_pair<decltype(ra)::value, decltype(rb)::value, false>(buf, P, s, tw, tid, nthr, none);
                 });
         } else {
             fftdev::with_forward_later(P.radix[s], stage);
@@ -632,7 +660,7 @@ template <int COUNT, bool INV, class Store>
 __device__ __forceinline__ void fft_last_stage(float2 *buf, const FftPlan &P, const float2 *__restrict__ tw, int last,
                                                int tid, int nthr, Store &store) {
     auto stage = [&](auto r) {
-        fftdev::dit_stage<decltype(r)::value, COUNT, true>(buf, P, last, tw, INV, tid, nthr, store);
+        fftdev::dit_stage<decltype(r)::value, COUNT, true, INV>(buf, P, last, tw, tid, nthr, store);
     };
     if constexpr (INV) {
         fftdev::with_last_radix(P.radix[last], stage);
@@ -640,7 +668,7 @@ __device__ __forceinline__ void fft_last_stage(float2 *buf, const FftPlan &P, co
         if constexpr (COUNT == 1)
             if (P.fuse[last]) {
                 fftdev::with_forward_pair(P.radix[last], P.radix[last + 1], [&](auto ra, auto rb) {
-                    fftdev::dit_pair<decltype(ra)::value, decltype(rb)::value, true>(buf, P, last, tw, INV, tid, nthr, store);
+                    fftdev::dit_pair<decltype(ra)::value, decltype(rb)::value, true>(buf, P, last, tw, tid, nthr, store);
                 });
                 return;
             }
@@ -681,7 +709,7 @@ __device__ __forceinline__ void fft_inplace(float2 *buf, const FftPlan &P, const
     const int last = fft_middle_stages<1, true>(buf, P, tw, tid, nthr);
     if constexpr (HELD)
         fftdev::with_last_radix(P.radix[last], [&](auto r) {
-            fftdev::dit_last_held<decltype(r)::value>(buf, P, tw, true, tid, nthr, between, store);
+            fftdev::dit_last_held<decltype(r)::value>(buf, P, tw, tid, nthr, between, store);
         });
     else
         fft_last_stage<1, true>(buf, P, tw, last, tid, nthr, store);

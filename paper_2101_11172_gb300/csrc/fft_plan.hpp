@@ -37,6 +37,17 @@ struct FftPlan {
     int box_blocks, boxes;          // TMA row copies: boxes of box_blocks column blocks
 };
 
+// Powers of a butterfly's twiddle w that a later stage's table holds (in a row of that many
+// pairs); the other powers are products of these.  Forward: w, and w^4 from radix 8 on, as
+// ever, which keeps the model visibilities' last bits.  Inverse: w, w^2 and, above radix 4,
+// w^4 and w^8: the inverse plans have radices 6, 12, 16 or 20 where the forward ones have 3s and
+// 8s, and with w and w^4 alone (w alone at radix 6) their powers' rounding moved the error
+// against the exact DFT: N' = 4320 (20 6 6 6) 1.96e-7 -> 2.50e-7, 1536 (16 16 6)
+// 1.97e-7 -> 2.21e-7, 3072 (16 16 12) 2.08e-7 -> 2.27e-7.
+WS_HD constexpr int base_row(int radix, bool inverse) {
+    return inverse ? (radix > 4 ? 4 : 2) : (radix >= 8 ? 2 : 1);
+}
+
 // ceil(2^32 / d), or 0 for d = 1
 WS_HD constexpr unsigned div_mul(int d) {
     return d <= 1 ? 0u : (unsigned)((4294967296ull + (unsigned long long)d - 1ull) / (unsigned long long)d);
