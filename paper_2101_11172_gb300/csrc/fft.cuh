@@ -271,9 +271,27 @@ template <>
 __device__ __forceinline__ void dft<6>(float2 *v, bool inv) {
     dft_pfa<2, 3>(v, inv);
 }
+// Forward, radix 10 keeps the 5 x 2 form with the twiddles w10^k that it always had: the prime
+// factor form, which the inverse takes, moved the model visibilities' error by up to 2 %
+// (N' = 2560: 2.06e-7 -> 2.10e-7).
 template <>
 __device__ __forceinline__ void dft<10>(float2 *v, bool inv) {
-    dft_pfa<2, 5>(v, inv);
+    if (inv) {
+        dft_pfa<2, 5>(v, true);
+        return;
+    }
+    float2 e[5] = {v[0], v[2], v[4], v[6], v[8]}, o[5] = {v[1], v[3], v[5], v[7], v[9]};
+    dft_odd<5>(e, false);
+    dft_odd<5>(o, false);
+    // cos and sin of 2 pi k / 10 from those of fifths of a turn
+    constexpr float c[5] = {1.f, (float)-odd_cos(5, 2), (float)odd_cos(5, 1), (float)-odd_cos(5, 1), (float)odd_cos(5, 2)};
+    constexpr float sn[5] = {0.f, (float)odd_sin(5, 2), (float)odd_sin(5, 1), (float)odd_sin(5, 1), (float)odd_sin(5, 2)};
+#pragma unroll
+    for (int k = 0; k < 5; ++k) {
+        const float2 t = k == 0 ? o[0] : cmul_rot(o[k], make_float2(c[k], -sn[k]), make_float2(sn[k], c[k]));
+        v[k] = cadd(e[k], t);
+        v[k + 5] = csub(e[k], t);
+    }
 }
 template <>
 __device__ __forceinline__ void dft<12>(float2 *v, bool inv) {
