@@ -616,8 +616,7 @@ inv_rows_kernel(Launch L, FftPlan F, const float2 *__restrict__ tw, const __grid
         float2 sum = make_float2(a.x, a.y), comp = make_float2(a.z, a.w);
         for (int g = 1; g < shares; ++g) {
             a = __ldcg(acc + g * image + pix0 + jj);
-            kahan_add(sum, comp, make_float2(a.x, a.y));
-            kahan_add(sum, comp, make_float2(-a.z, -a.w));
+            add_sums(sum, comp, a);
         }
         const float h = corr[pix0 + jj];
         dirty[pix0 + jj] = make_float2(h * (sum.x - comp.x), L.fold ? 0.f : h * (sum.y - comp.y));
