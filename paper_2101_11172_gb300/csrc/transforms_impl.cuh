@@ -215,9 +215,10 @@ fwd_rows_kernel(Launch L, FftPlan F, const float2 *__restrict__ tw, const float2
             __syncthreads();
         } else if ((p - p_begin) % kScreenSteps == 0) {
             for (int jj = tid; jj < N; jj += T) {
+                const float2 f = keep_rows ? irow[jj] : corrected(jj);
                 float sn, cs;
                 phase_tz(t, keep_rows ? zrow[jj] : zsplit[pix0 + jj], &sn, &cs);
-                grow[jj] = screened(keep_rows ? irow[jj] : corrected(jj), sn, cs);
+                grow[jj] = screened(f, sn, cs);
             }
             __syncthreads();
         }
